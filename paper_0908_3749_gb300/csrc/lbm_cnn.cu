@@ -1,10 +1,17 @@
 // lbm_cnn.cu -- training and inference kernels of the coarse-grid corrector
 // (include/lbm_cnn.h).
 //
-// Activations are BF16, pixel-major (NHWC, one image): a[p][c], p = y W + x;
-// the input features stay FP32 and the first layer (4 -> 32) runs in FP32 on
-// the CUDA cores. The other 3 x 3 convolutions are implicit GEMMs on the tensor cores
-// (mma.sync m16n8k16, BF16 inputs, FP32 accumulation): rows are pixels, the
+// Activations and output gradients are BF16 in groups of 8 channels, row by
+// row: element (y, x, c) of a C-channel image at
+//   ((y * C/8 + c/8) * W + x) * 8 + c % 8,
+// so that a tile of pixels with its halo is one TMA box whose shared-memory
+// image holds, for every row and channel group, consecutive pixels 16 bytes
+// apart: 8 pixels x 8 channels are 128 contiguous bytes, the unit of ldmatrix
+// and of the tcgen05 operand layout, and a tap of the 3 x 3 stencil is an
+// address offset (pixels outside the image are the box's zero fill).
+// The input features stay FP32 and the first layer (4 -> 32) runs in FP32 on
+// the CUDA cores. The other 3 x 3 convolutions are implicit GEMMs on the tensor
+// cores (mma.sync m16n8k16, BF16 inputs, FP32 accumulation): rows are pixels, the
 // reduction index k = tap * CIN + ci runs over the 9 taps and the input
 // channels, columns are output channels. The weights of a layer are packed
 // once per update into [COUT][K] BF16 (K contiguous, the "col" operand) for
@@ -58,79 +65,231 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const unsigned (&a)[4],
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Two consecutive channels (k, k+1) of the patch element of pixel (y, x) for
-// reduction index k (k even, CIN even so both share a tap); zero outside the
-// image or beyond the real K.
-template <int CIN>
-__device__ __forceinline__ unsigned patch2(const __nv_bfloat16* __restrict__ in, int H, int W,
-                                           bool valid, int y, int x, int k) {
-  if (!valid || k >= 9 * CIN) return 0u;
-  const int tap = k / CIN, ci = k - tap * CIN;
-  const int yy = y + tap / 3 - 1, xx = x + tap % 3 - 1;
-  if (yy < 0 || yy >= H || xx < 0 || xx >= W) return 0u;
-  return *reinterpret_cast<const unsigned*>(in + ((long long)yy * W + xx) * CIN + ci);
+// Which values of a BF16 pair without negative numbers are positive, at bits 15
+// (low value) and 31 (high value): 0x7fff + x sets the top bit of its half for
+// every non-zero x, and no carry leaves the half.
+__device__ __forceinline__ unsigned positive_bits(__nv_bfloat162 v) {
+  return ((*reinterpret_cast<const unsigned*>(&v) & 0x7fff7fffu) + 0x7fff7fffu) & 0x80008000u;
+}
+// A pixel's word of 32 such bits: channels 8 j + 2 t, + 1 (j, t = 0..3) at bits
+// 15 - s and 31 - s, s = j + 4 t.
+
+// Tiles of CT_Y x CT_X output pixels; their inputs with a halo of one pixel
+// are one TMA box of CT_HY rows x channel groups x CT_HX pixels.
+constexpr int CT_X = 32, CT_Y = 8, CT_HX = CT_X + 2, CT_HY = CT_Y + 2;
+constexpr int CT_WARPS = 4, CT_T = 32 * CT_WARPS;  // a warp computes two rows
+constexpr int CONV_CTAS_PER_SM = 3;
+constexpr unsigned PX_BYTES = 16;                  // 8 BF16 channels of a pixel
+
+__device__ __forceinline__ void ldmatrix4(unsigned (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+__device__ __forceinline__ void ldmatrix2(unsigned& r0, unsigned& r1, unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];\n"
+               : "=r"(r0), "=r"(r1)
+               : "r"(addr));
+}
+__device__ __forceinline__ unsigned lds32(unsigned addr) {
+  unsigned v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr));
+  return v;
 }
 
-// out[p][c] (c < COUT) = epilogue(sum_k patch(p, k) * Wt[c][k]). Each warp
-// computes 16 pixels x COUTP columns; a block of 4 warps covers 64 pixels.
+// A box of `map` (3D: x in 32-bit words, channel group, row) whose first pixel
+// is (x, y), all channel groups.
+__device__ __forceinline__ void tma_load_box(void* dst, const CUtensorMap* map, int x, int y,
+                                             unsigned long long* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(gbtma::smem_addr(dst)),
+      "l"(reinterpret_cast<unsigned long long>(map)), "r"(4 * x), "r"(0), "r"(y),
+      "r"(gbtma::smem_addr(bar))
+      : "memory");
+}
+
+template <int CIN, int COUT>
+struct ConvShape {
+  static constexpr int NCG = CIN == 32 ? 4 : 1;      // channel groups of the input
+  static constexpr int KP = ru(9 * CIN, 16), KS = KP / 16;
+  static constexpr int COUTP = ru(COUT, 8), NF = COUTP / 8;
+  // Weight rows in shared memory, 16 bytes longer than K: the 8 rows that an
+  // 8 x 8 ldmatrix reads then start in different 16-byte bank groups.
+  static constexpr int WPITCH = KP + 8;
+  static constexpr unsigned ROW = NCG * CT_HX * PX_BYTES;  // bytes per tile row
+  static constexpr unsigned TILE = CT_HY * ROW;
+  static constexpr unsigned STAGE = (TILE + 127) / 128 * 128;
+  static constexpr unsigned SMEM = STAGE + COUTP * WPITCH * 2 + 128;
+};
+
+// out[p][c] (c < COUT) = epilogue(sum_k patch(p, k) * Wt[c][k]).
+//
+// Persistent CTAs of four warps, three per SM; a tile's input (10 x 34 pixels)
+// is copied by TMA while the CTA stores the previous tile's outputs and the
+// other CTAs compute, the packed weights stay in shared memory. A warp
+// computes two rows of 32 pixels (four 16-pixel M tiles) x COUTP channels: per
+// K step one ldmatrix.x4 per M tile (the tap is an offset into the tile), and
+// the B fragments serve all four. The K steps run in order, one accumulator per
+// fragment. Bound by the tensor pipe's mma.sync rate (8 us at 1024
+// multiply-adds per clock and SM) and the latencies around each tile.
+// Measured, 512 x 512, 32 -> 32 channels: 18 us with and without the mask;
+// reading the patches from global memory instead (four predicated 4-byte loads
+// per K step and M tile) was bound by L1 at 91 %: 67 us, and 72 us with the
+// mask read from the activations. Four and five CTAs per SM (128 and 96
+// registers, K loop partly unrolled) took 20 us, a second tile stage 18 us.
 template <int CIN, int COUT, int EPI>
-__global__ void __launch_bounds__(128) k_conv(const __nv_bfloat16* __restrict__ in, int H, int W,
-                                              const __nv_bfloat16* __restrict__ Wt,
-                                              const float* __restrict__ bias,
-                                              const __nv_bfloat16* __restrict__ mask,
-                                              __nv_bfloat16* __restrict__ out_bf,
-                                              float* __restrict__ out_f) {
-  constexpr int KP = ru(9 * CIN, 16), COUTP = ru(COUT, 8), NF = COUTP / 8, KS = KP / 16;
-  __shared__ __align__(16) __nv_bfloat16 sw[COUTP * KP];
-  for (int i = threadIdx.x; i < COUTP * KP / 2; i += blockDim.x)
-    reinterpret_cast<unsigned*>(sw)[i] = reinterpret_cast<const unsigned*>(Wt)[i];
-  __syncthreads();
+__global__ void __launch_bounds__(CT_T, CONV_CTAS_PER_SM)
+    k_conv(const __grid_constant__ CUtensorMap map, int H, int W, int tiles_x, int ntiles,
+           const __nv_bfloat16* __restrict__ Wt, const float* __restrict__ bias,
+           const unsigned* __restrict__ bits_in, __nv_bfloat16* __restrict__ out_bf,
+           float* __restrict__ out_f, unsigned* __restrict__ bits_out, int* __restrict__ timeout) {
+  using S = ConvShape<CIN, COUT>;
+  extern __shared__ __align__(128) unsigned char conv_raw[];
+  unsigned char* const base = conv_raw + ((128u - (gbtma::smem_addr(conv_raw) & 127u)) & 127u);
+  __shared__ unsigned long long bar;
+  const unsigned sw = gbtma::smem_addr(base) + S::STAGE;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, tig = lane & 3;
-  const int npix = H * W;
-  const int p0 = blockIdx.x * 64 + warp * 16;
-  const int pa = p0 + g, pb = p0 + g + 8;
-  const bool va = pa < npix, vb = pb < npix;
-  const int ya = va ? pa / W : 0, xa = va ? pa - ya * W : 0;
-  const int yb = vb ? pb / W : 0, xb = vb ? pb - yb * W : 0;
-  float acc[NF][4];
-#pragma unroll
-  for (int j = 0; j < NF; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-#pragma unroll 2
-  for (int ks = 0; ks < KS; ++ks) {
-    const int k0 = ks * 16 + tig * 2, k1 = k0 + 8;
-    unsigned a[4];
-    a[0] = patch2<CIN>(in, H, W, va, ya, xa, k0);
-    a[1] = patch2<CIN>(in, H, W, vb, yb, xb, k0);
-    a[2] = patch2<CIN>(in, H, W, va, ya, xa, k1);
-    a[3] = patch2<CIN>(in, H, W, vb, yb, xb, k1);
-#pragma unroll
-    for (int j = 0; j < NF; ++j) {
-      const __nv_bfloat16* col = sw + (j * 8 + g) * KP;
-      const unsigned b0 = *reinterpret_cast<const unsigned*>(col + k0);
-      const unsigned b1 = *reinterpret_cast<const unsigned*>(col + k1);
-      mma_bf16(acc[j], a, b0, b1);
-    }
+  const int G = (int)gridDim.x;
+  auto load = [&](int tile) {
+    gbtma::mbar_expect_tx(&bar, S::TILE);
+    tma_load_box(base, &map, (tile % tiles_x) * CT_X - 1, (tile / tiles_x) * CT_Y - 1, &bar);
+  };
+  if (threadIdx.x == 0) {
+    gbtma::mbar_init(&bar, 1);
+    load(blockIdx.x);  // the grid has at most ntiles CTAs
   }
+  constexpr int CHUNKS = S::KP / 8;  // 16-byte pieces of a weight row
+  for (int i = threadIdx.x; i < S::COUTP * CHUNKS; i += CT_T)
+    *reinterpret_cast<uint4*>(base + S::STAGE + (i / CHUNKS) * (S::WPITCH * 2) + (i % CHUNKS) * 16) =
+        __ldg(reinterpret_cast<const uint4*>(Wt) + i);
+  __syncthreads();
+
+  float bs[S::NF][2];
 #pragma unroll
-  for (int j = 0; j < NF; ++j) {
+  for (int j = 0; j < S::NF; ++j)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int p = h ? pb : pa;
-      if (!(h ? vb : va)) continue;
+    for (int e = 0; e < 2; ++e)
+      bs[j][e] = EPI != EPI_MASK_BF16 && j * 8 + tig * 2 + e < COUT ? __ldg(bias + j * 8 + tig * 2 + e) : 0.f;
+
+  for (int k = 0, tile = blockIdx.x; tile < ntiles; tile += G, ++k) {
+    const bool more = tile + G < ntiles;
+    const int x0 = (tile % tiles_x) * CT_X, y0 = (tile / tiles_x) * CT_Y + 2 * warp;
+    // The ReLU masks (which channels of a pixel are positive) of this
+    // thread's outputs, read while the tile's copy is in flight. Reading the
+    // activations themselves here or in the epilogue, 32 loads of 4 bytes per
+    // thread, took 25-27 us per layer.
+    unsigned keep[4][2];
+    if constexpr (EPI == EPI_MASK_BF16) {
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int c = j * 8 + tig * 2 + e;
-        if (c >= COUT) continue;
-        float v = acc[j][2 * h + e];
-        if (EPI == EPI_RELU_BF16) {
-          v = fmaxf(v + bias[c], 0.f);
-          out_bf[(long long)p * COUT + c] = __float2bfloat16(v);
-        } else if (EPI == EPI_LINEAR_F32) {
-          out_f[(long long)p * COUT + c] = v + bias[c];
+      for (int m = 0; m < 4; ++m)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int y = y0 + (m >> 1), x = x0 + (m & 1) * 16 + h * 8 + g;
+          keep[m][h] = y < H && x < W ? __ldg(bits_in + (long long)y * W + x) << (4 * tig) : 0u;
+        }
+    }
+    if (!__syncthreads_and(gbtma::mbar_wait_bounded(&bar, k & 1, gbtma::TMA_WAIT_CYCLES))) {
+      // The copy did not land in time: record it, wait once more (bounded), leave.
+      if (threadIdx.x == 0) {
+        atomicExch(timeout, 1);
+        gbtma::mbar_wait_bounded(&bar, k & 1, gbtma::TMA_WAIT_CYCLES);
+      }
+      return;
+    }
+    const unsigned in = gbtma::smem_addr(base);
+    float acc[4][S::NF][4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+      for (int j = 0; j < S::NF; ++j) acc[m][j][0] = acc[m][j][1] = acc[m][j][2] = acc[m][j][3] = 0.f;
+    // M tile m: row 2 warp + m / 2, pixels 16 (m % 2) .. + 15.
+    const unsigned arow = in + 2 * warp * S::ROW;
+    // ldmatrix row addresses: lane -> pixel lane % 16, channel group lane / 16
+    const unsigned a_lane = (lane & 15) * PX_BYTES + (lane >> 4) * (CT_HX * PX_BYTES);
+    const unsigned b_lane = S::NF == 1
+                                ? ((lane & 7) * S::WPITCH + ((lane >> 3) & 1) * 8) * 2
+                                : (((lane & 7) + (lane >> 4) * 8) * S::WPITCH + ((lane >> 3) & 1) * 8) * 2;
+#pragma unroll
+    for (int ks = 0; ks < S::KS; ++ks) {
+      unsigned b[S::NF][2];
+      if constexpr (S::NF == 1) {
+        ldmatrix2(b[0][0], b[0][1], sw + b_lane + ks * 32);
+      } else {
+#pragma unroll
+        for (int j = 0; j < S::NF; j += 2) {
+          unsigned r[4];
+          ldmatrix4(r, sw + b_lane + j * 8 * S::WPITCH * 2 + ks * 32);
+          b[j][0] = r[0]; b[j][1] = r[1]; b[j + 1][0] = r[2]; b[j + 1][1] = r[3];
+        }
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        unsigned a[4];
+        const unsigned mt = arow + (m >> 1) * S::ROW + (m & 1) * 16 * PX_BYTES;
+        if constexpr (CIN == 32) {
+          const int tap = ks >> 1;
+          ldmatrix4(a, mt + a_lane + (tap / 3) * S::ROW + (tap % 3) * PX_BYTES +
+                           (ks & 1) * 2 * (CT_HX * PX_BYTES));
         } else {
-          const float keep = __bfloat162float(mask[(long long)p * COUT + c]) > 0.f ? 1.f : 0.f;
-          out_bf[(long long)p * COUT + c] = __float2bfloat16(v * keep);
+          // k = tap * 4 + ci: the thread's channel pairs belong to taps
+          // 4 ks + tig / 2 and 4 ks + 2 + tig / 2 (zero beyond tap 8)
+          const int t0 = ks * 4 + (tig >> 1), t1 = t0 + 2;
+          const unsigned px = mt + g * PX_BYTES + (tig & 1) * 4;
+          const unsigned o0 = (t0 / 3) * S::ROW + (t0 % 3) * PX_BYTES;
+          const unsigned o1 = (t1 / 3) * S::ROW + (t1 % 3) * PX_BYTES;
+          a[0] = t0 < 9 ? lds32(px + o0) : 0u;
+          a[1] = t0 < 9 ? lds32(px + 8 * PX_BYTES + o0) : 0u;
+          a[2] = t1 < 9 ? lds32(px + o1) : 0u;
+          a[3] = t1 < 9 ? lds32(px + 8 * PX_BYTES + o1) : 0u;
+        }
+#pragma unroll
+        for (int j = 0; j < S::NF; ++j) mma_bf16(acc[m][j], a, b[j][0], b[j][1]);
+      }
+    }
+    __syncthreads();  // the tile is free again
+    if (threadIdx.x == 0 && more) load(tile + G);
+    // Thread (g, tig) holds channels j * 8 + 2 tig, + 1 of pixels g and g + 8
+    // of each M tile.
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const int y = y0 + (m >> 1);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int x = x0 + (m & 1) * 16 + h * 8 + g;
+        const bool in_image = y < H && x < W;
+        unsigned pos = 0u;  // positive channels of this pixel (this thread's)
+#pragma unroll
+        for (int j = 0; j < S::NF; ++j) {
+          if (!in_image) continue;
+          const float v0 = acc[m][j][2 * h], v1 = acc[m][j][2 * h + 1];
+          if constexpr (EPI == EPI_LINEAR_F32) {
+            const int c = j * 8 + tig * 2;
+            if (c < COUT)
+              *reinterpret_cast<float2*>(out_f + ((long long)y * W + x) * COUT + c) =
+                  make_float2(v0 + bs[j][0], v1 + bs[j][1]);
+          } else {
+            const long long o = (((long long)y * S::NF + j) * W + x) * 8 + tig * 2;
+            float r0, r1;
+            if constexpr (EPI == EPI_RELU_BF16) {
+              r0 = fmaxf(v0 + bs[j][0], 0.f);
+              r1 = fmaxf(v1 + bs[j][1], 0.f);
+            } else {
+              r0 = v0 * (keep[m][h] & (0x8000u >> j) ? 1.f : 0.f);
+              r1 = v1 * (keep[m][h] & (0x80000000u >> j) ? 1.f : 0.f);
+            }
+            const __nv_bfloat162 r = __floats2bfloat162_rn(r0, r1);
+            *reinterpret_cast<__nv_bfloat162*>(out_bf + o) = r;
+            if (EPI == EPI_RELU_BF16)
+              pos |= positive_bits(r) >> j;
+          }
+        }
+        if (EPI == EPI_RELU_BF16 && bits_out) {  // (uniform over the grid)
+          pos >>= 4 * tig;
+          pos |= __shfl_xor_sync(0xffffffffu, pos, 1);
+          pos |= __shfl_xor_sync(0xffffffffu, pos, 2);
+          if (tig == 0 && in_image) bits_out[(long long)y * W + x] = pos;
         }
       }
     }
@@ -272,7 +431,7 @@ __global__ void __launch_bounds__(WG_T, WG_CTAS_PER_SM)
           const int p = pbase + pg * 8 + j;
           const int y = p / W, x = p - y * W, yy = y + dy, xx = x + dx;
           v[j] = (p < npix && yy >= 0 && yy < H && xx >= 0 && xx < W)
-                     ? __ldg(reinterpret_cast<const uint4*>(act + ((long long)yy * W + xx) * 32 + cg * 8))
+                     ? __ldg(reinterpret_cast<const uint4*>(act + (((long long)yy * 4 + cg) * W + xx) * 8))
                      : make_uint4(0, 0, 0, 0);
         }
         uint4 o[8];
@@ -326,7 +485,8 @@ __global__ void __launch_bounds__(WG_T, WG_CTAS_PER_SM)
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const int p = pbase + pg * 8 + j;
-          v[j] = p < npix ? __ldg(reinterpret_cast<const uint4*>(dz + (long long)p * 32 + cg * 8))
+          const int y = p / W;
+          v[j] = p < npix ? __ldg(reinterpret_cast<const uint4*>(dz + ((long long)y * 4 + cg) * W * 8 + (long long)(p - y * W) * 8))
                           : make_uint4(0, 0, 0, 0);
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
@@ -345,7 +505,7 @@ __global__ void __launch_bounds__(WG_T, WG_CTAS_PER_SM)
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const int p = pbase + pg * 8 + j;
-          v[j] = p < npix ? __ldg(reinterpret_cast<const uint2*>(dz + (long long)p * 4))
+          v[j] = p < npix ? __ldg(reinterpret_cast<const uint2*>(dz + (long long)p * 8))
                           : make_uint2(0, 0);
           db[0] += bf_lo(v[j].x);
           db[1] += bf_hi(v[j].x);
@@ -455,14 +615,15 @@ constexpr size_t wg_smem() { return sizeof(WgSmem<CIN, COUT == 32 ? 32 : 16>); }
 
 // First layer (4 -> 32 channels) in FP32 on the CUDA cores, straight from the
 // FP32 input features [p][4]: 3 x 3 correlation with zero padding, bias,
-// ReLU, stored BF16 [p][32] for the tensor-core layers. Keeping the input in
+// ReLU, stored BF16 for the tensor-core layers. Keeping the input in
 // FP32 keeps differences between neighbouring nodes that are below one BF16
 // step of the fields (smooth regions of fine-grained coarse grids).
 // w: the layer's FP32 parameters, (3, 3, 4, 32) then 32 biases.
 constexpr int C0_T = 128;
 __global__ void __launch_bounds__(C0_T) k_conv0(const float* __restrict__ xf, int H, int W,
                                                 const float* __restrict__ w,
-                                                __nv_bfloat16* __restrict__ out) {
+                                                __nv_bfloat16* __restrict__ out,
+                                                unsigned* __restrict__ bits) {
   __shared__ float sw[9 * 4 * 32 + 32];
   for (int i = threadIdx.x; i < 9 * 4 * 32 + 32; i += C0_T) sw[i] = w[i];
   __syncthreads();
@@ -483,11 +644,19 @@ __global__ void __launch_bounds__(C0_T) k_conv0(const float* __restrict__ xf, in
 #pragma unroll
       for (int c = 0; c < 32; ++c) acc[c] += qi[ci] * sw[(tap * 4 + ci) * 32 + c];
   }
-  __nv_bfloat16* o = out + (long long)p * 32;
+  unsigned pos = 0u;
 #pragma unroll
-  for (int c = 0; c < 32; c += 2)
-    *reinterpret_cast<__nv_bfloat162*>(o + c) =
-        __floats2bfloat162_rn(fmaxf(acc[c], 0.f), fmaxf(acc[c + 1], 0.f));
+  for (int cg = 0; cg < 4; ++cg) {
+    __nv_bfloat162 q[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      q[k] = __floats2bfloat162_rn(fmaxf(acc[cg * 8 + 2 * k], 0.f), fmaxf(acc[cg * 8 + 2 * k + 1], 0.f));
+      pos |= positive_bits(q[k]) >> (cg + 4 * k);
+    }
+    *reinterpret_cast<uint4*>(out + (((long long)y * 4 + cg) * W + x) * 8) =
+        *reinterpret_cast<const uint4*>(q);
+  }
+  if (bits) bits[p] = pos;
 }
 
 // grad[i] = sum over blocks b (in order) of partial[b][i].
@@ -535,10 +704,10 @@ __global__ void k_loss(const float* __restrict__ xf, const float* __restrict__ z
     if (l1) {
       s = fabs((double)d);
       const float sg = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
-      if (dz) dz[i] = __float2bfloat16(k * sg / (float)n);
+      if (dz) dz[2 * (i & ~3) + (i & 3)] = __float2bfloat16(k * sg / (float)n);
     } else {
       s = (double)d * d;
-      if (dz) dz[i] = __float2bfloat16(2.f * k * d / (float)n);
+      if (dz) dz[2 * (i & ~3) + (i & 3)] = __float2bfloat16(2.f * k * d / (float)n);
     }
   }
   sm[threadIdx.x] = s;
@@ -695,7 +864,13 @@ struct lbm_cnn {
   __nv_bfloat16* wt[NL] = {};
   __nv_bfloat16* wb[NL] = {};
   __nv_bfloat16* act[NL] = {};  // act[l] = relu output of layer l-1 (act[0] unused)
-  __nv_bfloat16* dz[2] = {};    // ping-pong output gradients
+  unsigned* pos[NL] = {};       // pos[l]: which channels of act[l] are positive, a word per pixel
+  __nv_bfloat16* dz[2] = {};    // ping-pong output gradients (32 channels)
+  __nv_bfloat16* dz5 = nullptr; // output gradients of the last layer: 4 channels and 4 zeros
+  CUtensorMap m_act[NL], m_dz[2], m_dz5;  // tiles with halo of act[1..], dz[], dz5
+  int tiles_x = 0, ntiles = 0;  // convolution tiles
+  int sms = 0;
+  int* timeout = nullptr;       // a bounded wait of a convolution expired
   float* xf = nullptr;          // input features FP32 [p][4]
   float* tf = nullptr;          // target features FP32 [p][4]
   float* z = nullptr;           // last layer output FP32 [p][4]
@@ -739,22 +914,47 @@ int pack_all(lbm_cnn* n) {
   return LBM_OK;
 }
 
-template <int CIN, int COUT, int EPI>
-void conv(lbm_cnn* n, const __nv_bfloat16* in, const __nv_bfloat16* wt, const float* bias,
-          const __nv_bfloat16* mask, __nv_bfloat16* ob, float* of) {
-  k_conv<CIN, COUT, EPI><<<(n->npix + 63) / 64, 128, 0, n->stream>>>(in, n->H, n->W, wt, bias,
-                                                                      mask, ob, of);
+// After a synchronisation: whether a bounded wait of a convolution expired.
+int check_timeout(lbm_cnn* n, int flag) {
+  return flag ? cfail(n, LBM_ERR_TIMEOUT, "a tile load (TMA) did not complete within its time limit") : LBM_OK;
 }
 
-int forward(lbm_cnn* n, const double* coarse) {
+// Tensor map of a row-planar BF16 image of `ncg` channel groups: dims (x in
+// 32-bit words, channel group, row); box = one convolution tile with its halo.
+int encode_image(lbm_cnn* n, const void* p, int ncg, CUtensorMap* out) {
+  gbtma::EncodeTiledFn enc = gbtma::tensor_map_encoder();
+  if (!enc) return cfail(n, LBM_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
+  const cuuint64_t dims[3] = {(cuuint64_t)n->W * 4, (cuuint64_t)ncg, (cuuint64_t)n->H};
+  const cuuint64_t strides[2] = {(cuuint64_t)n->W * PX_BYTES, (cuuint64_t)n->W * PX_BYTES * ncg};
+  const cuuint32_t box[3] = {CT_HX * 4, (cuuint32_t)ncg, CT_HY};
+  const cuuint32_t es[3] = {1, 1, 1};
+  const CUresult r = enc(out, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<void*>(p), dims, strides, box,
+                         es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS)
+    return cfail(n, LBM_ERR_CUDA, "cuTensorMapEncodeTiled failed: " + std::to_string((int)r));
+  return LBM_OK;
+}
+
+template <int CIN, int COUT, int EPI>
+void conv(lbm_cnn* n, const CUtensorMap& in, const __nv_bfloat16* wt, const float* bias,
+          const unsigned* bits_in, __nv_bfloat16* ob, float* of, unsigned* bits_out = nullptr) {
+  const int grid = std::min(n->ntiles, CONV_CTAS_PER_SM * n->sms);
+  k_conv<CIN, COUT, EPI><<<grid, CT_T, ConvShape<CIN, COUT>::SMEM, n->stream>>>(
+      in, n->H, n->W, n->tiles_x, n->ntiles, wt, bias, bits_in, ob, of, bits_out, n->timeout);
+}
+
+// `train`: also store which activations are positive, for the backward pass.
+int forward(lbm_cnn* n, const double* coarse, bool train) {
+  auto bits = [&](int l) { return train ? n->pos[l] : nullptr; };
   k_features<<<(n->npix + 255) / 256, 256, 0, n->stream>>>(coarse, n->npix, n->xf);
   const float* w = n->w;
   k_conv0<<<(n->npix + C0_T - 1) / C0_T, C0_T, 0, n->stream>>>(n->xf, n->H, n->W,
-                                                               w + param_offset(0), n->act[1]);
-  conv<32, 32, EPI_RELU_BF16>(n, n->act[1], n->wt[1], w + param_offset(1) + wsize(1), nullptr, n->act[2], nullptr);
-  conv<32, 32, EPI_RELU_BF16>(n, n->act[2], n->wt[2], w + param_offset(2) + wsize(2), nullptr, n->act[3], nullptr);
-  conv<32, 32, EPI_RELU_BF16>(n, n->act[3], n->wt[3], w + param_offset(3) + wsize(3), nullptr, n->act[4], nullptr);
-  conv<32, 4, EPI_LINEAR_F32>(n, n->act[4], n->wt[4], w + param_offset(4) + wsize(4), nullptr, nullptr, n->z);
+                                                               w + param_offset(0), n->act[1], bits(1));
+  conv<32, 32, EPI_RELU_BF16>(n, n->m_act[1], n->wt[1], w + param_offset(1) + wsize(1), nullptr, n->act[2], nullptr, bits(2));
+  conv<32, 32, EPI_RELU_BF16>(n, n->m_act[2], n->wt[2], w + param_offset(2) + wsize(2), nullptr, n->act[3], nullptr, bits(3));
+  conv<32, 32, EPI_RELU_BF16>(n, n->m_act[3], n->wt[3], w + param_offset(3) + wsize(3), nullptr, n->act[4], nullptr, bits(4));
+  conv<32, 4, EPI_LINEAR_F32>(n, n->m_act[4], n->wt[4], w + param_offset(4) + wsize(4), nullptr, nullptr, n->z);
   CCK(n, cudaGetLastError());
   return LBM_OK;
 }
@@ -771,19 +971,19 @@ void wgrad(lbm_cnn* n, const void* act, const __nv_bfloat16* dzl, float* grad) {
 int loss_backward(lbm_cnn* n, const double* target) {
   k_features<<<(n->npix + 255) / 256, 256, 0, n->stream>>>(target, n->npix, n->tf);
   const int nel = 4 * n->npix, nb = (nel + 255) / 256;
-  k_loss<<<nb, 256, 0, n->stream>>>(n->xf, n->z, n->tf, nel, n->dz[0], n->dpart, n->scale,
+  k_loss<<<nb, 256, 0, n->stream>>>(n->xf, n->z, n->tf, nel, n->dz5, n->dpart, n->scale,
                                     n->loss_kind == LBM_CNN_LOSS_L1);
   k_sum_d<<<1, 32, 0, n->stream>>>(n->dpart, nb, 1.0 / nel, n->dloss);
   float* g = n->grad;
-  // layer 5 (32 -> 4): dz[0] holds d loss / d z5
-  wgrad<32, 4>(n, n->act[4], n->dz[0], g + param_offset(4));
-  conv<4, 32, EPI_MASK_BF16>(n, n->dz[0], n->wb[4], nullptr, n->act[4], n->dz[1], nullptr);
+  // layer 5 (32 -> 4): dz5 holds d loss / d z5
+  wgrad<32, 4>(n, n->act[4], n->dz5, g + param_offset(4));
+  conv<4, 32, EPI_MASK_BF16>(n, n->m_dz5, n->wb[4], nullptr, n->pos[4], n->dz[1], nullptr);
   wgrad<32, 32>(n, n->act[3], n->dz[1], g + param_offset(3));
-  conv<32, 32, EPI_MASK_BF16>(n, n->dz[1], n->wb[3], nullptr, n->act[3], n->dz[0], nullptr);
+  conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[1], n->wb[3], nullptr, n->pos[3], n->dz[0], nullptr);
   wgrad<32, 32>(n, n->act[2], n->dz[0], g + param_offset(2));
-  conv<32, 32, EPI_MASK_BF16>(n, n->dz[0], n->wb[2], nullptr, n->act[2], n->dz[1], nullptr);
+  conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[0], n->wb[2], nullptr, n->pos[2], n->dz[1], nullptr);
   wgrad<32, 32>(n, n->act[1], n->dz[1], g + param_offset(1));
-  conv<32, 32, EPI_MASK_BF16>(n, n->dz[1], n->wb[1], nullptr, n->act[1], n->dz[0], nullptr);
+  conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[1], n->wb[1], nullptr, n->pos[1], n->dz[0], nullptr);
   wgrad<4, 32>(n, n->xf, n->dz[0], g + param_offset(0));
   CCK(n, cudaGetLastError());
   return LBM_OK;
@@ -816,6 +1016,13 @@ int lbm_cnn_create(int H, int W, void* cuda_stream, lbm_cnn** out) {
   allow((const void*)k_wgrad_tc<32, 32>, wg_smem<32, 32>());
   allow((const void*)k_wgrad_tc<32, 4>, wg_smem<32, 4>());
   allow((const void*)k_wgrad_tc<4, 32>, wg_smem<4, 32>());
+  allow((const void*)k_conv<32, 32, EPI_RELU_BF16>, ConvShape<32, 32>::SMEM);
+  allow((const void*)k_conv<32, 32, EPI_MASK_BF16>, ConvShape<32, 32>::SMEM);
+  allow((const void*)k_conv<32, 4, EPI_LINEAR_F32>, ConvShape<32, 4>::SMEM);
+  allow((const void*)k_conv<4, 32, EPI_MASK_BF16>, ConvShape<4, 32>::SMEM);
+  n->sms = std::max(sms, 1);
+  n->tiles_x = (W + CT_X - 1) / CT_X;
+  n->ntiles = n->tiles_x * ((H + CT_Y - 1) / CT_Y);
   n->wblocks = (int)std::min<long long>((P + WG_CHUNK - 1) / WG_CHUNK,
                                         (long long)WG_CTAS_PER_SM * std::max(sms, 1));
   auto A = [&](void** p, size_t bytes) {
@@ -830,9 +1037,12 @@ int lbm_cnn_create(int H, int W, void* cuda_stream, lbm_cnn** out) {
     A((void**)&n->wt[l], 2 * (size_t)ru(cout_of(l), 8) * kp_of(l));
     A((void**)&n->wb[l], 2 * (size_t)ru(cin_of(l), 8) * kb_of(l));
     A((void**)&n->act[l], 2 * P * CH[l]);
+    A((void**)&n->pos[l], 4 * P);
   }
   A((void**)&n->dz[0], 2 * P * 32);
   A((void**)&n->dz[1], 2 * P * 32);
+  A((void**)&n->dz5, 2 * P * 8);
+  A((void**)&n->timeout, sizeof(int));
   A((void**)&n->xf, 4 * P * 4);
   A((void**)&n->tf, 4 * P * 4);
   A((void**)&n->z, 4 * P * 4);
@@ -845,7 +1055,11 @@ int lbm_cnn_create(int H, int W, void* cuda_stream, lbm_cnn** out) {
     lbm_cnn_destroy(n);
     return e == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA;
   }
-  if (pack_all(n) != LBM_OK) {
+  int rc = LBM_OK;
+  for (int l = 1; l < NL && rc == LBM_OK; ++l) rc = encode_image(n, n->act[l], 4, &n->m_act[l]);
+  for (int k = 0; k < 2 && rc == LBM_OK; ++k) rc = encode_image(n, n->dz[k], 4, &n->m_dz[k]);
+  if (rc == LBM_OK) rc = encode_image(n, n->dz5, 1, &n->m_dz5);
+  if (rc != LBM_OK || pack_all(n) != LBM_OK) {
     g_cnn_error = n->err;
     lbm_cnn_destroy(n);
     return LBM_ERR_CUDA;
@@ -858,13 +1072,14 @@ int lbm_cnn_destroy(lbm_cnn* n) {
   if (!n) return LBM_OK;
   if (n->stream) cudaStreamSynchronize(n->stream);
   void* ps[] = {n->w, n->m, n->v, n->grad, n->dz[0], n->dz[1], n->xf, n->tf, n->z,
-                n->wpartial, n->dpart, n->dloss};
+                n->wpartial, n->dpart, n->dloss, n->dz5, n->timeout};
   for (void* p : ps)
     if (p) cudaFree(p);
   for (int l = 0; l < NL; ++l) {
     if (n->wt[l]) cudaFree(n->wt[l]);
     if (n->wb[l]) cudaFree(n->wb[l]);
     if (n->act[l]) cudaFree(n->act[l]);
+    if (n->pos[l]) cudaFree(n->pos[l]);
   }
   if (n->own_stream && n->stream) cudaStreamDestroy(n->stream);
   delete n;
@@ -904,20 +1119,22 @@ int lbm_cnn_loss_grad(lbm_cnn* n, const double* coarse, const double* target, do
   if (!n || !coarse || !target) return cfail(n, LBM_ERR_INVALID, "NULL argument");
   nvtxRangePushA("lbm_cnn_train_step");
   struct Pop { ~Pop() { nvtxRangePop(); } } pop;
-  int rc = forward(n, coarse);
+  int rc = forward(n, coarse, true);
   if (rc == LBM_OK) rc = loss_backward(n, target);
   if (rc != LBM_OK) return rc;
   if (loss) CCK(n, cudaMemcpyAsync(loss, n->dloss, sizeof(double), cudaMemcpyDeviceToHost, n->stream));
   if (grads)
     CCK(n, cudaMemcpyAsync(grads, n->grad, sizeof(float) * LBM_CNN_NPARAMS, cudaMemcpyDeviceToHost,
                            n->stream));
+  int flag = 0;
+  CCK(n, cudaMemcpyAsync(&flag, n->timeout, sizeof(int), cudaMemcpyDeviceToHost, n->stream));
   CCK(n, cudaStreamSynchronize(n->stream));
-  return LBM_OK;
+  return check_timeout(n, flag);
 }
 
 int lbm_cnn_train_step(lbm_cnn* n, const double* coarse, const double* target, double* loss) {
   if (!n || !coarse || !target) return cfail(n, LBM_ERR_INVALID, "NULL argument");
-  int rc = forward(n, coarse);
+  int rc = forward(n, coarse, true);
   if (rc == LBM_OK) rc = loss_backward(n, target);
   if (rc != LBM_OK) return rc;
   n->step += 1;
@@ -929,8 +1146,11 @@ int lbm_cnn_train_step(lbm_cnn* n, const double* coarse, const double* target, d
   rc = pack_all(n);
   if (rc != LBM_OK) return rc;
   if (loss) {
+    int flag = 0;
     CCK(n, cudaMemcpyAsync(loss, n->dloss, sizeof(double), cudaMemcpyDeviceToHost, n->stream));
+    CCK(n, cudaMemcpyAsync(&flag, n->timeout, sizeof(int), cudaMemcpyDeviceToHost, n->stream));
     CCK(n, cudaStreamSynchronize(n->stream));
+    return check_timeout(n, flag);
   }
   return LBM_OK;
 }
@@ -979,7 +1199,7 @@ int lbm_cnn_residual_rms(lbm_cnn* n, const double* coarse, const double* target,
 int lbm_cnn_correct(lbm_cnn* n, const double* coarse, double* corrected, double mass_tol,
                     int* used_fallback) {
   if (!n || !coarse || !corrected) return cfail(n, LBM_ERR_INVALID, "NULL argument");
-  int rc = forward(n, coarse);
+  int rc = forward(n, coarse, false);
   if (rc != LBM_OK) return rc;
   const int nb = (n->npix + 255) / 256;
   k_apply<<<nb, 256, 0, n->stream>>>(n->xf, n->z, n->npix, corrected, coarse, n->dpart, n->scale);
@@ -987,7 +1207,10 @@ int lbm_cnn_correct(lbm_cnn* n, const double* coarse, double* corrected, double 
   std::vector<double> part(2 * (size_t)nb);
   CCK(n, cudaMemcpyAsync(part.data(), n->dpart, sizeof(double) * part.size(),
                          cudaMemcpyDeviceToHost, n->stream));
+  int flag = 0;
+  CCK(n, cudaMemcpyAsync(&flag, n->timeout, sizeof(int), cudaMemcpyDeviceToHost, n->stream));
   CCK(n, cudaStreamSynchronize(n->stream));
+  if ((rc = check_timeout(n, flag)) != LBM_OK) return rc;
   double m1 = 0, m0 = 0;
   for (int b = 0; b < nb; ++b) { m1 += part[2 * b]; m0 += part[2 * b + 1]; }
   const bool fallback = !std::isfinite(m1) || std::fabs(m1 - m0) > mass_tol * std::fabs(m0);

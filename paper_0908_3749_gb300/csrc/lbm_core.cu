@@ -394,24 +394,6 @@ int ensure_graph2(lbm_ctx* c, int from) {
 }
 static_assert(GRAPH_CHUNK % 4 == 0, "graphs of fused launches leave the buffer parity unchanged");
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
-                                  const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                                  const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn tensor_map_encoder() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                         &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = (EncodeTiledFn)p;
-  }
-  return fn;
-}
-
 // Tensor map of population buffer b: dims (pitch, ny, 16), box = one tile
 // with its halo (`rows` rows, Tile<R>::BXP columns, 16 populations).
 int encode_map(lbm_ctx* c, int b, cuuint32_t rows, CUtensorMap* out) {
