@@ -300,68 +300,54 @@ __global__ void __launch_bounds__(CT_T, CONV_CTAS_PER_SM)
 // Weight and bias gradients on the tensor cores (tcgen05)
 // ---------------------------------------------------------------------------
 // dW[tap][ci][co] = sum_p act[p + off(tap)][ci] dz[p][co] is a contraction
-// over the pixels: D (M x N) = A (M x K) B (K x N) with K = the pixels, N =
-// the output channels (32, or 4 padded to 16 with zero rows of B) and the
-// rows m of A:
-//   32-channel layers (BF16 activations): m = tap * 32 + ci, 288 rows as
-//     three M = 128 tiles (taps 0-3, taps 4-7, tap 8 and 96 zero rows);
-//   first layer (FP32 features, 4 channels): each feature split into three
-//     BF16 parts x = x0 + x1 + x2 (x0 = bf16(x), x1 = bf16(x - x0), x2 =
-//     bf16(x - x0 - x1), the differences exact in FP32; 24 significant bits
-//     together), m = part * 36 + tap * 4 + ci, 108 rows of one M = 128 tile;
-//     the epilogue adds the three parts' sums (x2 first), which gives the
-//     contraction of the FP32 features.
-// Persistent CTAs of 128 threads take chunks of WG_CHUNK pixels (WG_CHUNK /
-// 16 MMA steps of K = 16): the threads gather the chunk's shifted features
-// and output gradients as blocks of 8 channels x 8 consecutive pixels (eight
-// 16-byte loads, one per pixel, transposed in registers by byte permutes)
-// and store them in the canonical K-major layout; one thread issues the
-// chunk's MMAs into the CTA's TMEM accumulators and commits them to an
-// mbarrier, which every thread waits for (bounded) before the next chunk is
-// gathered. At the end each thread reads its rows of the accumulators
-// (tcgen05.ld) into the CTA's partial sums, with the bias gradient (sum_p
-// dz[p][co], FP32, a fixed order); k_sum_partials adds the partials of all
-// CTAs in a fixed order.
-constexpr int WG_T = 128, WG_CHUNK = 64, WG_KS = WG_CHUNK / 16;
-constexpr int WG_CTAS_PER_SM = 4;
+// over the pixels: D (M x N) = A (M x K) B (K x N), K = the pixels, N = the
+// output channels (32, or 4 padded to 16). Both operands are MN-major: a core
+// matrix is 8 pixels (K) x 8 channels, 128 contiguous bytes of the row-planar
+// tiles that TMA copies, so nothing is gathered or transposed by threads.
+//   A  the activations' tile with a halo of one pixel (10 x 34): its channel
+//      groups lie CT_HX pixels apart, and the tile's rows follow each other
+//      with the same stride, so the 16 core matrices of M = 128 run over
+//      (row offset dy, channel group) and a start address picks the column
+//      offset dx: three products (dx = -1, 0, 1) give the nine taps.
+//      32-channel layers: 4 row offsets x 4 groups, the fourth offset unused;
+//      first layer (FP32 features, 4 channels): each feature as three BF16
+//      parts x = x0 + x1 + x2 (x0 = bf16(x), x1 = bf16(x - x0), x2 = bf16(x -
+//      x0 - x1), the differences exact in FP32; 24 significant bits
+//      together), 12 channels padded to 16: 8 row offsets x 2 groups, three
+//      used; the epilogue adds the three parts' sums (x2 first), which gives
+//      the contraction of the FP32 features.
+//   B  the output gradients' tile (8 x 32, no halo). The last layer's 4
+//      channels are one group with 4 zeros; the second group of N = 16 is
+//      the box's zero fill.
+// Pixels outside the image are zero fill in both. Persistent CTAs, two per SM,
+// two stages: one thread issues a tile's 48 products (M = 128, K = 16) and
+// commits them to the stage's mbarrier, which it waits for before the stage is
+// copied into again; meanwhile the four warps add the tile's bias gradient
+// (sum_p dz[p][co], FP32, a fixed order). At the end each thread reads its rows
+// of the accumulators (tcgen05.ld) into the CTA's partial sums; k_update adds
+// the partials of all CTAs in a fixed order.
+// Bound by the tensor cores' reads of A and B from shared memory (5 KB per
+// product; about 10 us at 512 x 512, 32 -> 32). Measured: 15 us (32 -> 32),
+// 13 us (32 -> 4), 14 us (first layer); gathering and transposing the
+// operands with threads took 83, 55 and 34 us, bound by L1 (83 %).
+constexpr int WG_T = 128;
+constexpr int WG_CTAS_PER_SM = 2;
 constexpr unsigned WG_TMEM_COLS = 128;
-constexpr unsigned WG_A_TILE = 128 * 16 * 2;  // one M tile x one K step, BF16 (4 KB)
 
-template <int CIN>
-__host__ __device__ constexpr int wg_mt() { return CIN == 32 ? 3 : 1; }  // M tiles
-
-template <int CIN, int NP>
-struct WgSmem {
-  unsigned char a[wg_mt<CIN>() * WG_KS][WG_A_TILE];  // reused by the epilogue
-  unsigned char b[WG_KS][NP * 16 * 2];                // reused for the bias sums
-  unsigned long long bar;
-  unsigned tmem;
+template <int CG, int NP>
+struct WgShape {
+  static constexpr unsigned GROUP = CT_HX * PX_BYTES;   // bytes of one (row, group) of A
+  static constexpr unsigned ROW = CG * GROUP;           // bytes of one tile row of A
+  static constexpr int DY = 16 / CG;                    // row offsets that M = 128 spans
+  static constexpr unsigned A_TX = CT_HY * ROW;         // copied
+  static constexpr unsigned A_BYTES = ((CT_Y - 1 + DY) * ROW + 2 * PX_BYTES + 127) / 128 * 128;  // read
+  static constexpr int BG = NP / 8;                     // channel groups of B
+  static constexpr unsigned BGROUP = CT_X * PX_BYTES, BROW = BG * BGROUP;
+  static constexpr unsigned B_BYTES = CT_Y * BROW;
+  static constexpr unsigned STAGE = A_BYTES + B_BYTES;
+  static_assert(STAGE % 128 == 0 && A_BYTES >= A_TX, "stages");
+  static constexpr unsigned SMEM = 2 * STAGE + 128;
 };
-
-// Byte offset of element (row, k) of a rows x 16 BF16 operand tile in the
-// canonical K-major layout without swizzle (core matrices of 8 rows x 8
-// elements, 128 contiguous bytes; the next core matrix along K 128 bytes on,
-// the next 8-row group 256 bytes on).
-__device__ __forceinline__ unsigned wg_off(int row, int k) {
-  return (unsigned)((row >> 3) * 256 + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2);
-}
-
-// Transposes 8 pixels x 8 channels (v[j] = channels 0..7 of pixel j, two per
-// word) into 8 rows (channels) of 8 pixels: out[c] = pixels 0..7 of channel c.
-__device__ __forceinline__ void wg_transpose8(const uint4 (&v)[8], uint4 (&out)[8]) {
-#pragma unroll
-  for (int cp = 0; cp < 4; ++cp) {
-    unsigned lo[4], hi[4];
-#pragma unroll
-    for (int pp = 0; pp < 4; ++pp) {
-      const unsigned a = (&v[2 * pp].x)[cp], b = (&v[2 * pp + 1].x)[cp];
-      lo[pp] = __byte_perm(a, b, 0x5410);  // channel 2 cp of pixels 2 pp, 2 pp + 1
-      hi[pp] = __byte_perm(a, b, 0x7632);  // channel 2 cp + 1
-    }
-    out[2 * cp] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-    out[2 * cp + 1] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-  }
-}
 
 __device__ __forceinline__ float bf_lo(unsigned w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf_hi(unsigned w) { return __uint_as_float(w & 0xFFFF0000u); }
@@ -380,238 +366,168 @@ __device__ __forceinline__ void split3(float x, unsigned (&p)[3]) {
   p[2] = bf_bits(h2);
 }
 
-template <int CIN, int COUT>
+// CG: channel groups of A (4: a 32-channel layer, 2: the split features); COUT
+// output channels.
+template <int CG, int COUT>
 __global__ void __launch_bounds__(WG_T, WG_CTAS_PER_SM)
-    k_wgrad_tc(const void* __restrict__ act_, const __nv_bfloat16* __restrict__ dz, int H, int W,
-               float* __restrict__ partial) {
+    k_wgrad(const __grid_constant__ CUtensorMap act, const __grid_constant__ CUtensorMap dz,
+            int tiles_x, int ntiles, float* __restrict__ partial, int* __restrict__ timeout) {
   constexpr int NP = COUT == 32 ? 32 : 16;  // N of the MMA
-  constexpr int MT = wg_mt<CIN>();
-  constexpr int ROWS = CIN == 32 ? 9 * 32 : 3 * 36;  // used rows of A
+  constexpr int CIN = CG == 4 ? 32 : 4;
   constexpr int NOUT = 9 * CIN * COUT + COUT;
-  constexpr unsigned IDESC = tc05::idesc_f32acc(tc05::FMT_BF16, 128, NP);
-  static_assert(CIN == 32 || (CIN == 4 && COUT == 32), "layer shapes of the corrector");
-  extern __shared__ __align__(1024) unsigned char wg_raw[];
-  WgSmem<CIN, NP>& S = *reinterpret_cast<WgSmem<CIN, NP>*>(wg_raw);
-  const int t = threadIdx.x, warp = t >> 5;
-  const int npix = H * W, nchunks = (npix + WG_CHUNK - 1) / WG_CHUNK;
-  if (warp == 0) tc05::alloc(&S.tmem, WG_TMEM_COLS);
-  if (t == 0) gbtma::mbar_init(&S.bar, 1);
-  // Zero the rows that no gather writes: A rows ROWS .. MT * 128 - 1 (in the
-  // last M tile), B rows COUT .. NP - 1.
-  constexpr int AZ = MT * 128 - ROWS, AZ0 = 128 - AZ;
-  for (int i = t; i < WG_KS * AZ * 2; i += WG_T) {
-    const int ks = i / (AZ * 2), r = AZ0 + (i % (AZ * 2)) / 2, half = i & 1;
-    *reinterpret_cast<uint4*>(&S.a[(MT - 1) * WG_KS + ks][wg_off(r, 8 * half)]) = make_uint4(0, 0, 0, 0);
-  }
-  for (int i = t; i < WG_KS * (NP - COUT) * 2; i += WG_T) {
-    const int ks = i / ((NP - COUT) * 2), r = COUT + (i % ((NP - COUT) * 2)) / 2, half = i & 1;
-    *reinterpret_cast<uint4*>(&S.b[ks][wg_off(r, 8 * half)]) = make_uint4(0, 0, 0, 0);
+  using S = WgShape<CG, NP>;
+  constexpr unsigned IDESC = tc05::idesc_f32acc(tc05::FMT_BF16, 128, NP) | tc05::IDESC_A_MN | tc05::IDESC_B_MN;
+  extern __shared__ __align__(128) unsigned char wg_raw[];
+  unsigned char* const base = wg_raw + ((128u - (gbtma::smem_addr(wg_raw) & 127u)) & 127u);
+  __shared__ unsigned long long full[2], used[2];  // copies landed; products done
+  __shared__ unsigned s_tmem;
+  __shared__ float s_db[32];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int G = (int)gridDim.x;
+  auto load = [&](int tile, int st) {
+    const int x = (tile % tiles_x) * CT_X, y = (tile / tiles_x) * CT_Y;
+    unsigned char* const a = base + st * S::STAGE;
+    gbtma::mbar_expect_tx(&full[st], S::A_TX + S::B_BYTES);
+    tma_load_box(a, &act, x - 1, y - 1, &full[st]);
+    tma_load_box(a + S::A_BYTES, &dz, x, y, &full[st]);
+  };
+  if (warp == 0) tc05::alloc(&s_tmem, WG_TMEM_COLS);
+  if (t == 0) {
+    for (int k = 0; k < 2; ++k) {
+      gbtma::mbar_init(&full[k], 1);
+      gbtma::mbar_init(&used[k], 1);
+    }
+    load(blockIdx.x, 0);  // the grid has at most ntiles CTAs
   }
   tc05::fence_before();
   __syncthreads();
   tc05::fence_after();
-  const unsigned tmem = S.tmem;
+  const unsigned tmem = s_tmem;
 
-  float db[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // bias sums of this thread's B block
-  constexpr int NBB = COUT == 32 ? 32 : 8;                 // B blocks per chunk
-  unsigned done = 0;                                      // chunks whose MMAs completed
+  float db[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // bias sums: pixel column `lane`, group `warp`
   bool ok = true;
-  for (int ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-    const int pbase = ch * WG_CHUNK;
-    if constexpr (CIN == 32) {
-      // A: 288 blocks (tap, pixel group of 8, channel group of 8), channel
-      // group fastest so that neighbouring threads read one pixel's 64 bytes.
-      const __nv_bfloat16* act = static_cast<const __nv_bfloat16*>(act_);
-      for (int q = t; q < 288; q += WG_T) {
-        const int cg = q & 3, pg = (q >> 2) & 7, tap = q >> 5;
-        const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-        uint4 v[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int p = pbase + pg * 8 + j;
-          const int y = p / W, x = p - y * W, yy = y + dy, xx = x + dx;
-          v[j] = (p < npix && yy >= 0 && yy < H && xx >= 0 && xx < W)
-                     ? __ldg(reinterpret_cast<const uint4*>(act + (((long long)yy * 4 + cg) * W + xx) * 8))
-                     : make_uint4(0, 0, 0, 0);
-        }
-        uint4 o[8];
-        wg_transpose8(v, o);
-        const int mt = tap < 8 ? tap / 4 : 2, rbase = (tap < 8 ? (tap % 4) * 32 : 0) + cg * 8;
-        unsigned char* tile = S.a[mt * WG_KS + pg / 2];
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-          *reinterpret_cast<uint4*>(tile + wg_off(rbase + c, (pg & 1) * 8)) = o[c];
-      }
-    } else {
-      // A: 72 blocks (tap, pixel group of 8): 8 pixels x 4 features, each
-      // split into three BF16 parts, give rows part * 36 + tap * 4 + ci.
-      const float* act = static_cast<const float*>(act_);
-      if (t < 72) {
-        const int pg = t & 7, tap = t >> 3;
-        const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-        unsigned part[8][4][3];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int p = pbase + pg * 8 + j;
-          const int y = p / W, x = p - y * W, yy = y + dy, xx = x + dx;
-          const float4 v = (p < npix && yy >= 0 && yy < H && xx >= 0 && xx < W)
-                               ? __ldg(reinterpret_cast<const float4*>(act + ((long long)yy * W + xx) * 4))
-                               : make_float4(0.f, 0.f, 0.f, 0.f);
-          split3(v.x, part[j][0]);
-          split3(v.y, part[j][1]);
-          split3(v.z, part[j][2]);
-          split3(v.w, part[j][3]);
-        }
-        unsigned char* tile = S.a[pg / 2];
-#pragma unroll
-        for (int pt = 0; pt < 3; ++pt)
-#pragma unroll
-          for (int ci = 0; ci < 4; ++ci) {
-            uint4 o;
-            o.x = part[0][ci][pt] | (part[1][ci][pt] << 16);
-            o.y = part[2][ci][pt] | (part[3][ci][pt] << 16);
-            o.z = part[4][ci][pt] | (part[5][ci][pt] << 16);
-            o.w = part[6][ci][pt] | (part[7][ci][pt] << 16);
-            *reinterpret_cast<uint4*>(tile + wg_off(pt * 36 + tap * 4 + ci, (pg & 1) * 8)) = o;
-          }
-      }
+  int k = 0;
+  for (int tile = blockIdx.x; tile < ntiles; tile += G, ++k) {
+    const int st = k & 1;
+    if (t == 0) {
+      // Stage 1 - st: tile k - 1's products must have read it (the bias sums
+      // have, by the barrier at the end of the loop body).
+      if (k > 0) ok = gbtma::mbar_wait_bounded(&used[1 - st], ((k - 1) >> 1) & 1, gbtma::TMA_WAIT_CYCLES);
+      if (ok && tile + G < ntiles) load(tile + G, 1 - st);
     }
-    // B: the output gradients of the chunk's pixels (and the bias sums).
-    if (t < NBB) {
-      const int pg = COUT == 32 ? t >> 2 : t, cg = COUT == 32 ? t & 3 : 0;
-      unsigned char* tile = S.b[pg / 2];
-      if constexpr (COUT == 32) {
-        uint4 v[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int p = pbase + pg * 8 + j;
-          const int y = p / W;
-          v[j] = p < npix ? __ldg(reinterpret_cast<const uint4*>(dz + ((long long)y * 4 + cg) * W * 8 + (long long)(p - y * W) * 8))
-                          : make_uint4(0, 0, 0, 0);
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const unsigned w = (&v[j].x)[c];
-            db[2 * c] += bf_lo(w);
-            db[2 * c + 1] += bf_hi(w);
-          }
-        }
-        uint4 o[8];
-        wg_transpose8(v, o);
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-          *reinterpret_cast<uint4*>(tile + wg_off(cg * 8 + c, (pg & 1) * 8)) = o[c];
-      } else {
-        uint2 v[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int p = pbase + pg * 8 + j;
-          v[j] = p < npix ? __ldg(reinterpret_cast<const uint2*>(dz + (long long)p * 8))
-                          : make_uint2(0, 0);
-          db[0] += bf_lo(v[j].x);
-          db[1] += bf_hi(v[j].x);
-          db[2] += bf_lo(v[j].y);
-          db[3] += bf_hi(v[j].y);
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          unsigned w[4];
-#pragma unroll
-          for (int pp = 0; pp < 4; ++pp) {
-            const unsigned a = (&v[2 * pp].x)[c >> 1], b = (&v[2 * pp + 1].x)[c >> 1];
-            w[pp] = __byte_perm(a, b, (c & 1) ? 0x7632 : 0x5410);
-          }
-          *reinterpret_cast<uint4*>(tile + wg_off(c, (pg & 1) * 8)) = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-      }
-    }
-    tc05::fence_async_smem();
-    __syncthreads();
+    ok = __syncthreads_and(ok && gbtma::mbar_wait_bounded(&full[st], (k >> 1) & 1, gbtma::TMA_WAIT_CYCLES));
+    if (!ok) break;
+    const unsigned a = gbtma::smem_addr(base) + st * S::STAGE, b = a + S::A_BYTES;
     if (t == 0) {
       tc05::fence_after();
+#pragma unroll 1
+      for (int r = 0; r < CT_Y; ++r)
 #pragma unroll
-      for (int ks = 0; ks < WG_KS; ++ks)
+        for (int kg = 0; kg < CT_X / 16; ++kg)
 #pragma unroll
-        for (int mt = 0; mt < MT; ++mt)
-          tc05::mma_f16(tmem + mt * NP,
-                        tc05::smem_desc(gbtma::smem_addr(S.a[mt * WG_KS + ks]), 128, 256),
-                        tc05::smem_desc(gbtma::smem_addr(S.b[ks]), 128, 256), IDESC,
-                        (done > 0 || ks > 0) ? 1u : 0u);
-      tc05::commit(&S.bar);
+          for (int dx = 0; dx < 3; ++dx)
+            tc05::mma_f16(tmem + dx * NP,
+                          tc05::smem_desc(a + r * S::ROW + (kg * 16 + dx) * PX_BYTES, 128, S::GROUP),
+                          tc05::smem_desc(b + r * S::BROW + kg * 16 * PX_BYTES, 128, S::BGROUP), IDESC,
+                          (k > 0 || r > 0 || kg > 0) ? 1u : 0u);
+      tc05::commit(&used[st]);
     }
-    ok = __syncthreads_and(gbtma::mbar_wait_bounded(&S.bar, done & 1, gbtma::TMA_WAIT_CYCLES));
-    if (!ok) break;
-    ++done;
-    tc05::fence_after();
+    if (warp < COUT / 8 || warp == 0) {
+#pragma unroll
+      for (int r = 0; r < CT_Y; ++r) {
+        const uint4 v = *reinterpret_cast<const uint4*>(base + st * S::STAGE + S::A_BYTES + r * S::BROW +
+                                                        warp * S::BGROUP + lane * PX_BYTES);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const unsigned w = (&v.x)[c];
+          db[2 * c] += bf_lo(w);
+          db[2 * c + 1] += bf_hi(w);
+        }
+      }
+    }
+    __syncthreads();
   }
+  // The last tile's products (every earlier one was waited for).
+  if (ok) ok = gbtma::mbar_wait_bounded(&used[(k - 1) & 1], ((k - 1) >> 1) & 1, gbtma::TMA_WAIT_CYCLES);
+  ok = __syncthreads_and(ok);
+  float* out = partial + (long long)blockIdx.x * NOUT;
   if (!ok) {
-    // The products did not complete in time: wait once more (bounded), mark
-    // this CTA's partials not-a-number (the training loss turns non-finite
-    // and the host reports it), free tensor memory.
-    if (t == 0) gbtma::mbar_wait_bounded(&S.bar, done & 1, gbtma::TMA_WAIT_CYCLES);
-    for (int i = t; i < NOUT; i += WG_T) partial[(long long)blockIdx.x * NOUT + i] = __int_as_float(0x7fc00000);
+    // A copy or the products did not complete in time: record it, wait once
+    // more (bounded) for both, free tensor memory.
+    if (t == 0) {
+      atomicExch(timeout, 1);
+      const int st = k & 1;
+      gbtma::mbar_wait_bounded(&full[st], (k >> 1) & 1, gbtma::TMA_WAIT_CYCLES);
+      if (k > 0) gbtma::mbar_wait_bounded(&used[1 - st], ((k - 1) >> 1) & 1, gbtma::TMA_WAIT_CYCLES);
+    }
     tc05::fence_before();
     __syncthreads();
     if (warp == 0) tc05::dealloc(tmem, WG_TMEM_COLS);
     return;
   }
-  float* out = partial + (long long)blockIdx.x * NOUT;
-  if constexpr (CIN == 32) {
-#pragma unroll
-    for (int mt = 0; mt < MT; ++mt) {
-      const int row = mt * 128 + t;  // = tap * 32 + ci
-#pragma unroll
-      for (int cb = 0; cb < NP / 16; ++cb) {
-        float v[16];
-        tc05::ld16(tmem + ((unsigned)(warp * 32) << 16) + mt * NP + cb * 16, v);
-        if (row < ROWS)
-#pragma unroll
-          for (int c = 0; c < 16; ++c)
-            if (cb * 16 + c < COUT) out[row * COUT + cb * 16 + c] = done ? v[c] : 0.f;
-      }
-    }
-  } else {
-    // rows of the three parts through shared memory (the A tiles are free:
-    // every product has completed), then out[r][co] = D2 + D1 + D0.
-    float* sD = reinterpret_cast<float*>(S.a[0]);  // 128 x 32 FP32 = 16 KB
-    static_assert(sizeof(S.a) >= 128 * 32 * sizeof(float), "epilogue scratch");
-#pragma unroll
-    for (int cb = 0; cb < 2; ++cb) {
+  tc05::fence_after();
+  const unsigned trow = tmem + ((unsigned)(warp * 32) << 16);
+  if constexpr (COUT == 4) {  // D row = dy * 32 + ci: warp = dy, lane = ci
+    for (int dx = 0; dx < 3; ++dx) {
       float v[16];
-      tc05::ld16(tmem + ((unsigned)(warp * 32) << 16) + cb * 16, v);
+      tc05::ld16(trow + dx * NP, v);
+      if (warp < 3)
+        reinterpret_cast<float4*>(out)[(warp * 3 + dx) * 32 + lane] = make_float4(v[0], v[1], v[2], v[3]);
+    }
+  } else if constexpr (CG == 4) {
+    // The rows of 32 sums through shared memory (every product has completed;
+    // 16-byte pieces swizzled by row), so that a warp stores whole lines:
+    // storing them from the threads that hold them took 11 of 26 us.
+    float4* sD = reinterpret_cast<float4*>(base);
+    static_assert(2 * S::STAGE >= 288 * 32 * sizeof(float), "epilogue scratch");
+    for (int dx = 0; dx < 3; ++dx) {
+      float v[32];
+      tc05::ld32(trow + dx * NP, v);
+      if (warp < 3)
 #pragma unroll
-      for (int c = 0; c < 16; ++c) sD[t * 32 + ((cb * 16 + c + t) & 31)] = done ? v[c] : 0.f;
+        for (int c = 0; c < 8; ++c)
+          sD[((warp * 3 + dx) * 32 + lane) * 8 + (c ^ (lane & 7))] =
+              make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
     }
     __syncthreads();
-    for (int i = t; i < 36 * 32; i += WG_T) {
-      const int r = i >> 5, co = i & 31;
-      auto at = [&](int row) { return sD[row * 32 + ((co + row) & 31)]; };
-      out[r * 32 + co] = (at(72 + r) + at(36 + r)) + at(r);
+    for (int i = t; i < 288 * 8; i += WG_T)
+      reinterpret_cast<float4*>(out)[i] = sD[(i & ~7) + ((i & 7) ^ ((i >> 3) & 7))];
+  } else {
+    // D row = dy * 16 + part * 4 + ci, 48 rows used; the three parts are added
+    // through shared memory (every product has completed).
+    float* sD = reinterpret_cast<float*>(base);  // 64 rows x 33
+    static_assert(2 * S::STAGE >= 64 * 33 * sizeof(float), "epilogue scratch");
+    for (int dx = 0; dx < 3; ++dx) {
+#pragma unroll
+      for (int cb = 0; cb < 2; ++cb) {
+        float v[16];
+        tc05::ld16(trow + dx * NP + cb * 16, v);
+        if (t < 64)
+#pragma unroll
+          for (int c = 0; c < 16; ++c) sD[t * 33 + cb * 16 + c] = v[c];
+      }
+      __syncthreads();
+      for (int i = t; i < 3 * 4 * 32; i += WG_T) {
+        const int dy = i / 128, ci = (i >> 5) & 3, co = i & 31;
+        const float* d = sD + (dy * 16 + ci) * 33 + co;
+        out[((dy * 3 + dx) * 4 + ci) * 32 + co] = (d[8 * 33] + d[4 * 33]) + d[0];
+      }
+      __syncthreads();
     }
   }
-  // bias: thread t (t < NBB) holds 8 (COUT 32) or 4 (COUT 4) channel sums of
-  // pixel group pg; add the pixel groups in order.
-  float* sdb = reinterpret_cast<float*>(S.b[0]);  // the B tiles are free now
+  // bias: add the pixel columns (lanes) by a fixed butterfly; warp = group
+#pragma unroll
+  for (int c = 0; c < 8; ++c)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) db[c] += __shfl_xor_sync(0xffffffffu, db[c], o);
+  if (lane == 0)
+#pragma unroll
+    for (int c = 0; c < 8; ++c) s_db[warp * 8 + c] = db[c];
   tc05::fence_before();
   __syncthreads();
-  if (t < NBB)
-#pragma unroll
-    for (int c = 0; c < 8; ++c) sdb[t * 8 + c] = db[c];
-  __syncthreads();
-  if (t < COUT) {
-    float s = 0.f;
-    if constexpr (COUT == 32) {
-      const int cg = t >> 3, c = t & 7;
-      for (int pg = 0; pg < 8; ++pg) s += sdb[(pg * 4 + cg) * 8 + c];
-    } else {
-      for (int pg = 0; pg < 8; ++pg) s += sdb[pg * 8 + t];
-    }
-    out[9 * CIN * COUT + t] = s;
-  }
+  if (t < COUT) out[9 * CIN * COUT + t] = s_db[t];
   if (warp == 0) tc05::dealloc(tmem, WG_TMEM_COLS);
 }
-
-template <int CIN, int COUT>
-constexpr size_t wg_smem() { return sizeof(WgSmem<CIN, COUT == 32 ? 32 : 16>); }
 
 // First layer (4 -> 32 channels) in FP32 on the CUDA cores, straight from the
 // FP32 input features [p][4]: 3 x 3 correlation with zero padding, bias,
@@ -673,14 +589,27 @@ __global__ void k_sum_partials(const float* __restrict__ partial, int nblocks, i
 // Features, loss, Adam, packing, correction, restriction
 // ---------------------------------------------------------------------------
 // Planes [4][H][W] (rho, u, v, T) -> features (log rho, u, v, log T) in FP32
-// [p][4] and BF16 [p][4].
-__global__ void k_features(const double* __restrict__ f, int npix, float* __restrict__ xf) {
+// [p][4]; with `xs`, also their three BF16 parts (channel = part * 4 + feature,
+// 12 of 16 channels, row-planar; the other 4 stay zero).
+__global__ void k_features(const double* __restrict__ f, int npix, int W, float* __restrict__ xf,
+                           __nv_bfloat16* __restrict__ xs) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= npix) return;
-  xf[4 * p] = (float)log(f[p]);
-  xf[4 * p + 1] = (float)f[npix + p];
-  xf[4 * p + 2] = (float)f[2 * npix + p];
-  xf[4 * p + 3] = (float)log(f[3 * npix + p]);
+  const float4 q = make_float4((float)log(f[p]), (float)f[npix + p], (float)f[2 * npix + p],
+                               (float)log(f[3 * npix + p]));
+  reinterpret_cast<float4*>(xf)[p] = q;
+  if (xs) {
+    unsigned s[4][3];
+    split3(q.x, s[0]);
+    split3(q.y, s[1]);
+    split3(q.z, s[2]);
+    split3(q.w, s[3]);
+    const int y = p / W, x = p - y * W;
+    uint4* const o = reinterpret_cast<uint4*>(xs) + (long long)y * 2 * W + x;
+    o[0] = make_uint4(s[0][0] | s[1][0] << 16, s[2][0] | s[3][0] << 16,
+                      s[0][1] | s[1][1] << 16, s[2][1] | s[3][1] << 16);
+    o[W] = make_uint4(s[0][2] | s[1][2] << 16, s[2][2] | s[3][2] << 16, 0u, 0u);
+  }
 }
 
 // out = x + z; d = out - target; dz = 2 d / N (BF16); block partial of sum d^2.
@@ -867,7 +796,9 @@ struct lbm_cnn {
   unsigned* pos[NL] = {};       // pos[l]: which channels of act[l] are positive, a word per pixel
   __nv_bfloat16* dz[2] = {};    // ping-pong output gradients (32 channels)
   __nv_bfloat16* dz5 = nullptr; // output gradients of the last layer: 4 channels and 4 zeros
-  CUtensorMap m_act[NL], m_dz[2], m_dz5;  // tiles with halo of act[1..], dz[], dz5
+  __nv_bfloat16* xs = nullptr;  // input features as three BF16 parts (16 channels)
+  CUtensorMap m_act[NL], m_dz[2], m_dz5, m_xs;  // tiles with halo of act[1..], dz[], dz5, xs
+  CUtensorMap g_dz[2], g_dz5;   // the same tiles without halo
   int tiles_x = 0, ntiles = 0;  // convolution tiles
   int sms = 0;
   int* timeout = nullptr;       // a bounded wait of a convolution expired
@@ -920,13 +851,15 @@ int check_timeout(lbm_cnn* n, int flag) {
 }
 
 // Tensor map of a row-planar BF16 image of `ncg` channel groups: dims (x in
-// 32-bit words, channel group, row); box = one convolution tile with its halo.
-int encode_image(lbm_cnn* n, const void* p, int ncg, CUtensorMap* out) {
+// 32-bit words, channel group, row); box = one tile of `box_cg` groups (those
+// beyond ncg are zero fill), with its halo or without.
+int encode_image(lbm_cnn* n, const void* p, int ncg, int box_cg, bool halo, CUtensorMap* out) {
   gbtma::EncodeTiledFn enc = gbtma::tensor_map_encoder();
   if (!enc) return cfail(n, LBM_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
   const cuuint64_t dims[3] = {(cuuint64_t)n->W * 4, (cuuint64_t)ncg, (cuuint64_t)n->H};
   const cuuint64_t strides[2] = {(cuuint64_t)n->W * PX_BYTES, (cuuint64_t)n->W * PX_BYTES * ncg};
-  const cuuint32_t box[3] = {CT_HX * 4, (cuuint32_t)ncg, CT_HY};
+  const cuuint32_t box[3] = {4u * (halo ? CT_HX : CT_X), (cuuint32_t)box_cg,
+                             (cuuint32_t)(halo ? CT_HY : CT_Y)};
   const cuuint32_t es[3] = {1, 1, 1};
   const CUresult r = enc(out, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<void*>(p), dims, strides, box,
                          es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -947,7 +880,8 @@ void conv(lbm_cnn* n, const CUtensorMap& in, const __nv_bfloat16* wt, const floa
 // `train`: also store which activations are positive, for the backward pass.
 int forward(lbm_cnn* n, const double* coarse, bool train) {
   auto bits = [&](int l) { return train ? n->pos[l] : nullptr; };
-  k_features<<<(n->npix + 255) / 256, 256, 0, n->stream>>>(coarse, n->npix, n->xf);
+  k_features<<<(n->npix + 255) / 256, 256, 0, n->stream>>>(coarse, n->npix, n->W, n->xf,
+                                                           train ? n->xs : nullptr);
   const float* w = n->w;
   k_conv0<<<(n->npix + C0_T - 1) / C0_T, C0_T, 0, n->stream>>>(n->xf, n->H, n->W,
                                                                w + param_offset(0), n->act[1], bits(1));
@@ -959,32 +893,32 @@ int forward(lbm_cnn* n, const double* coarse, bool train) {
   return LBM_OK;
 }
 
-template <int CIN, int COUT>
-void wgrad(lbm_cnn* n, const void* act, const __nv_bfloat16* dzl, float* grad) {
-  constexpr int NOUT = 9 * CIN * COUT + COUT;
-  k_wgrad_tc<CIN, COUT><<<n->wblocks, WG_T, wg_smem<CIN, COUT>(), n->stream>>>(act, dzl, n->H,
-                                                                              n->W, n->wpartial);
+template <int CG, int COUT>
+void wgrad(lbm_cnn* n, const CUtensorMap& act, const CUtensorMap& dz, float* grad) {
+  constexpr int NOUT = 9 * (CG == 4 ? 32 : 4) * COUT + COUT;
+  k_wgrad<CG, COUT><<<n->wblocks, WG_T, WgShape<CG, COUT == 32 ? 32 : 16>::SMEM, n->stream>>>(
+      act, dz, n->tiles_x, n->ntiles, n->wpartial, n->timeout);
   k_sum_partials<<<(NOUT + 255) / 256, 256, 0, n->stream>>>(n->wpartial, n->wblocks, NOUT, grad);
 }
 
 // Loss against the target features and all gradients into n->grad.
 int loss_backward(lbm_cnn* n, const double* target) {
-  k_features<<<(n->npix + 255) / 256, 256, 0, n->stream>>>(target, n->npix, n->tf);
+  k_features<<<(n->npix + 255) / 256, 256, 0, n->stream>>>(target, n->npix, n->W, n->tf, nullptr);
   const int nel = 4 * n->npix, nb = (nel + 255) / 256;
   k_loss<<<nb, 256, 0, n->stream>>>(n->xf, n->z, n->tf, nel, n->dz5, n->dpart, n->scale,
                                     n->loss_kind == LBM_CNN_LOSS_L1);
   k_sum_d<<<1, 32, 0, n->stream>>>(n->dpart, nb, 1.0 / nel, n->dloss);
   float* g = n->grad;
   // layer 5 (32 -> 4): dz5 holds d loss / d z5
-  wgrad<32, 4>(n, n->act[4], n->dz5, g + param_offset(4));
+  wgrad<4, 4>(n, n->m_act[4], n->g_dz5, g + param_offset(4));
   conv<4, 32, EPI_MASK_BF16>(n, n->m_dz5, n->wb[4], nullptr, n->pos[4], n->dz[1], nullptr);
-  wgrad<32, 32>(n, n->act[3], n->dz[1], g + param_offset(3));
+  wgrad<4, 32>(n, n->m_act[3], n->g_dz[1], g + param_offset(3));
   conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[1], n->wb[3], nullptr, n->pos[3], n->dz[0], nullptr);
-  wgrad<32, 32>(n, n->act[2], n->dz[0], g + param_offset(2));
+  wgrad<4, 32>(n, n->m_act[2], n->g_dz[0], g + param_offset(2));
   conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[0], n->wb[2], nullptr, n->pos[2], n->dz[1], nullptr);
-  wgrad<32, 32>(n, n->act[1], n->dz[1], g + param_offset(1));
+  wgrad<4, 32>(n, n->m_act[1], n->g_dz[1], g + param_offset(1));
   conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[1], n->wb[1], nullptr, n->pos[1], n->dz[0], nullptr);
-  wgrad<4, 32>(n, n->xf, n->dz[0], g + param_offset(0));
+  wgrad<2, 32>(n, n->m_xs, n->g_dz[0], g + param_offset(0));
   CCK(n, cudaGetLastError());
   return LBM_OK;
 }
@@ -1013,9 +947,9 @@ int lbm_cnn_create(int H, int W, void* cuda_stream, lbm_cnn** out) {
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   };
-  allow((const void*)k_wgrad_tc<32, 32>, wg_smem<32, 32>());
-  allow((const void*)k_wgrad_tc<32, 4>, wg_smem<32, 4>());
-  allow((const void*)k_wgrad_tc<4, 32>, wg_smem<4, 32>());
+  allow((const void*)k_wgrad<4, 32>, WgShape<4, 32>::SMEM);
+  allow((const void*)k_wgrad<4, 4>, WgShape<4, 16>::SMEM);
+  allow((const void*)k_wgrad<2, 32>, WgShape<2, 32>::SMEM);
   allow((const void*)k_conv<32, 32, EPI_RELU_BF16>, ConvShape<32, 32>::SMEM);
   allow((const void*)k_conv<32, 32, EPI_MASK_BF16>, ConvShape<32, 32>::SMEM);
   allow((const void*)k_conv<32, 4, EPI_LINEAR_F32>, ConvShape<32, 4>::SMEM);
@@ -1023,8 +957,7 @@ int lbm_cnn_create(int H, int W, void* cuda_stream, lbm_cnn** out) {
   n->sms = std::max(sms, 1);
   n->tiles_x = (W + CT_X - 1) / CT_X;
   n->ntiles = n->tiles_x * ((H + CT_Y - 1) / CT_Y);
-  n->wblocks = (int)std::min<long long>((P + WG_CHUNK - 1) / WG_CHUNK,
-                                        (long long)WG_CTAS_PER_SM * std::max(sms, 1));
+  n->wblocks = std::min(n->ntiles, WG_CTAS_PER_SM * n->sms);
   auto A = [&](void** p, size_t bytes) {
     if (e == cudaSuccess) e = cudaMalloc(p, bytes);
     if (e == cudaSuccess) e = cudaMemsetAsync(*p, 0, bytes, n->stream);
@@ -1042,6 +975,7 @@ int lbm_cnn_create(int H, int W, void* cuda_stream, lbm_cnn** out) {
   A((void**)&n->dz[0], 2 * P * 32);
   A((void**)&n->dz[1], 2 * P * 32);
   A((void**)&n->dz5, 2 * P * 8);
+  A((void**)&n->xs, 2 * P * 16);
   A((void**)&n->timeout, sizeof(int));
   A((void**)&n->xf, 4 * P * 4);
   A((void**)&n->tf, 4 * P * 4);
@@ -1056,9 +990,14 @@ int lbm_cnn_create(int H, int W, void* cuda_stream, lbm_cnn** out) {
     return e == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA;
   }
   int rc = LBM_OK;
-  for (int l = 1; l < NL && rc == LBM_OK; ++l) rc = encode_image(n, n->act[l], 4, &n->m_act[l]);
-  for (int k = 0; k < 2 && rc == LBM_OK; ++k) rc = encode_image(n, n->dz[k], 4, &n->m_dz[k]);
-  if (rc == LBM_OK) rc = encode_image(n, n->dz5, 1, &n->m_dz5);
+  for (int l = 1; l < NL && rc == LBM_OK; ++l) rc = encode_image(n, n->act[l], 4, 4, true, &n->m_act[l]);
+  for (int k = 0; k < 2; ++k) {
+    if (rc == LBM_OK) rc = encode_image(n, n->dz[k], 4, 4, true, &n->m_dz[k]);
+    if (rc == LBM_OK) rc = encode_image(n, n->dz[k], 4, 4, false, &n->g_dz[k]);
+  }
+  if (rc == LBM_OK) rc = encode_image(n, n->dz5, 1, 1, true, &n->m_dz5);
+  if (rc == LBM_OK) rc = encode_image(n, n->dz5, 1, 2, false, &n->g_dz5);
+  if (rc == LBM_OK) rc = encode_image(n, n->xs, 2, 2, true, &n->m_xs);
   if (rc != LBM_OK || pack_all(n) != LBM_OK) {
     g_cnn_error = n->err;
     lbm_cnn_destroy(n);
@@ -1072,7 +1011,7 @@ int lbm_cnn_destroy(lbm_cnn* n) {
   if (!n) return LBM_OK;
   if (n->stream) cudaStreamSynchronize(n->stream);
   void* ps[] = {n->w, n->m, n->v, n->grad, n->dz[0], n->dz[1], n->xf, n->tf, n->z,
-                n->wpartial, n->dpart, n->dloss, n->dz5, n->timeout};
+                n->wpartial, n->dpart, n->dloss, n->dz5, n->xs, n->timeout};
   for (void* p : ps)
     if (p) cudaFree(p);
   for (int l = 0; l < NL; ++l) {
@@ -1175,8 +1114,8 @@ int lbm_cnn_set_loss(lbm_cnn* n, int kind) {
 int lbm_cnn_residual_rms(lbm_cnn* n, const double* coarse, const double* target, double* rms) {
   if (!n || !coarse || !target || !rms) return cfail(n, LBM_ERR_INVALID, "NULL argument");
   const int nb = (n->npix + 255) / 256;
-  k_features<<<nb, 256, 0, n->stream>>>(coarse, n->npix, n->xf);
-  k_features<<<nb, 256, 0, n->stream>>>(target, n->npix, n->tf);
+  k_features<<<nb, 256, 0, n->stream>>>(coarse, n->npix, n->W, n->xf, nullptr);
+  k_features<<<nb, 256, 0, n->stream>>>(target, n->npix, n->W, n->tf, nullptr);
   std::vector<double> part(4 * (size_t)nb);
   double* dpart = nullptr;
   CCK(n, cudaMalloc((void**)&dpart, sizeof(double) * part.size()));

@@ -34,6 +34,11 @@ __host__ __device__ constexpr unsigned idesc_f32acc(unsigned fmt, unsigned M, un
   return (1u << 4) | (fmt << 7) | (fmt << 10) | ((N >> 3) << 17) | ((M >> 4) << 24);
 }
 constexpr unsigned FMT_BF16 = 1, FMT_TF32 = 2;
+// A (B) MN-major instead (bit 15 (16)): without swizzle its core matrices are 8
+// (K) x 16 bytes (M or N), 128 contiguous bytes, the next core matrix along K
+// the descriptor's leading-dimension offset away, along M or N its
+// stride-dimension offset.
+constexpr unsigned IDESC_A_MN = 1u << 15, IDESC_B_MN = 1u << 16;
 
 __device__ __forceinline__ void mma_tf32(unsigned tmem_d, unsigned long long a, unsigned long long b,
                                          unsigned idesc, unsigned accumulate) {
