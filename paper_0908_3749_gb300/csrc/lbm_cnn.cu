@@ -45,11 +45,12 @@ __host__ __device__ constexpr int wsize(int l) { return 9 * (l == 0 ? 4 : 32) * 
 __host__ __device__ constexpr int cin_of(int l) { return l == 0 ? 4 : 32; }
 __host__ __device__ constexpr int cout_of(int l) { return l == NL - 1 ? 4 : 32; }
 
-int param_offset(int l) {  // start of layer l in the packed parameter vector
-  int o = 0;
-  for (int k = 0; k < l; ++k) o += wsize(k) + cout_of(k);
-  return o;
-}
+__host__ __device__ constexpr int nout_of(int l) { return wsize(l) + cout_of(l); }
+// Start of layer l in the packed parameter vector.
+__host__ __device__ constexpr int param_offset(int l) { return l == 0 ? 0 : param_offset(l - 1) + nout_of(l - 1); }
+static_assert(param_offset(NL) == LBM_CNN_NPARAMS, "packed parameters");
+__host__ __device__ constexpr int kp_of(int l) { return ru(9 * cin_of(l), 16); }   // K of the forward operand
+__host__ __device__ constexpr int kb_of(int l) { return ru(9 * cout_of(l), 16); }  // of the input-gradient one
 
 // ---------------------------------------------------------------------------
 // Tensor-core implicit-GEMM 3 x 3 convolution
@@ -575,16 +576,6 @@ __global__ void __launch_bounds__(C0_T) k_conv0(const float* __restrict__ xf, in
   if (bits) bits[p] = pos;
 }
 
-// grad[i] = sum over blocks b (in order) of partial[b][i].
-__global__ void k_sum_partials(const float* __restrict__ partial, int nblocks, int n,
-                               float* __restrict__ grad) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float s = 0.f;
-  for (int b = 0; b < nblocks; ++b) s += partial[(long long)b * n + i];
-  grad[i] = s;
-}
-
 // ---------------------------------------------------------------------------
 // Features, loss, Adam, packing, correction, restriction
 // ---------------------------------------------------------------------------
@@ -619,54 +610,118 @@ struct Scale4 {
   float s[4];
 };
 
-// Loss per element of out - target, d: d^2 (LBM_CNN_LOSS_MSE) or |d|
-// (LBM_CNN_LOSS_L1, whose gradient is sign(d), 0 at d = 0); summed per block.
-__global__ void k_loss(const float* __restrict__ xf, const float* __restrict__ z,
-                       const float* __restrict__ tf, int n, __nv_bfloat16* __restrict__ dz,
-                       double* __restrict__ partial, const Scale4 sc, int l1) {
-  __shared__ double sm[256];
-  const int i = blockIdx.x * 256 + threadIdx.x;
+// Loss per element of d = out - target: d^2 (LBM_CNN_LOSS_MSE) or |d|
+// (LBM_CNN_LOSS_L1, whose gradient is sign(d), 0 at d = 0), and its gradient
+// with respect to the network's output (BF16, 4 channels and 4 zeros). A pixel
+// per thread, whose target features are taken here (the logarithms, on the FP64
+// units, are most of the kernel's time); the sums in FP64, per block.
+__global__ void __launch_bounds__(256) k_loss(const float4* __restrict__ xf, const float4* __restrict__ z,
+                                              const double* __restrict__ target, int npix,
+                                              uint4* __restrict__ dz, double* __restrict__ partial,
+                                              const Scale4 sc, int l1) {
+  __shared__ double sm[8];
+  const int p = blockIdx.x * 256 + threadIdx.x;
   double s = 0.0;
-  if (i < n) {
-    const float k = sc.s[i & 3];
-    const float d = xf[i] + k * z[i] - tf[i];
-    if (l1) {
-      s = fabs((double)d);
-      const float sg = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
-      if (dz) dz[2 * (i & ~3) + (i & 3)] = __float2bfloat16(k * sg / (float)n);
-    } else {
-      s = (double)d * d;
-      if (dz) dz[2 * (i & ~3) + (i & 3)] = __float2bfloat16(2.f * k * d / (float)n);
+  if (p < npix) {
+    const float4 x4 = xf[p], z4 = z[p];
+    const float4 t4 = make_float4((float)log(target[p]), (float)target[npix + p],
+                                  (float)target[2 * npix + p], (float)log(target[3 * npix + p]));
+    const float n = (float)(4 * npix);
+    unsigned g[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const float k = sc.s[c];
+      const float d = (&x4.x)[c] + k * (&z4.x)[c] - (&t4.x)[c];
+      if (l1) {
+        s += fabs((double)d);
+        const float sg = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
+        g[c] = bf_bits(__float2bfloat16(k * sg / n));
+      } else {
+        s += (double)d * d;
+        g[c] = bf_bits(__float2bfloat16(2.f * k * d / n));
+      }
     }
+    dz[p] = make_uint4(g[0] | g[1] << 16, g[2] | g[3] << 16, 0u, 0u);
   }
-  sm[threadIdx.x] = s;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = s;
   __syncthreads();
-  for (int st = 128; st > 0; st >>= 1) {
-    if ((int)threadIdx.x < st) sm[threadIdx.x] += sm[threadIdx.x + st];
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) s += sm[w];
+    partial[blockIdx.x] = s;
   }
-  if (threadIdx.x == 0) partial[blockIdx.x] = sm[0];
 }
 
-__global__ void k_sum_d(const double* __restrict__ partial, int n, double scale, double* out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
+// After the backward pass, one launch: the gradients from the weight-gradient
+// partials, the loss from its partials and, with `adam`, the update of the
+// FP32 parameters and of their packed BF16 copies (k_pack's positions; their
+// padding stays zero). A block takes UP_N parameters, the threads of a
+// parameter every UP_S-th partial, added in a fixed order; the last block takes
+// the loss. Bound by the read of the partials (36 MB at 304 CTAs, from the L2):
+// 14 us. One thread per parameter in a launch per layer, one thread for the
+// loss, and launches of their own for Adam and each layer's packing took 117 +
+// 195 + 13 us.
+constexpr int UP_N = 32, UP_S = 8;
+struct UpdateArgs {
+  const float* part[NL];  // [blocks][nout_of(l)]
+  int nblocks;
+  float *w, *m, *v, *grad;
+  __nv_bfloat16 *wt[NL], *wb[NL];
+  const double* lpart;    // loss partials
+  int nl;
+  double lscale;
+  double* loss;
+  int adam;
+  float lr, b1, b2, eps, c1, c2;
+};
+__global__ void __launch_bounds__(UP_N * UP_S) k_update(const UpdateArgs A) {
+  const int t = threadIdx.x;
+  if (blockIdx.x == gridDim.x - 1) {
+    __shared__ double sl[UP_N * UP_S];
     double s = 0.0;
-    for (int i = 0; i < n; ++i) s += partial[i];
-    *out = s * scale;
+    for (int i = t; i < A.nl; i += UP_N * UP_S) s += A.lpart[i];
+    sl[t] = s;
+    __syncthreads();
+    for (int st = UP_N * UP_S / 2; st > 0; st >>= 1) {
+      if (t < st) sl[t] += sl[t + st];
+      __syncthreads();
+    }
+    if (t == 0) *A.loss = sl[0] * A.lscale;
+    return;
   }
-}
-
-__global__ void k_adam(float* __restrict__ w, float* __restrict__ m, float* __restrict__ v,
-                       const float* __restrict__ g, int n, float lr, float b1, float b2,
-                       float eps, float c1, float c2) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.f - b1) * gi;
-  const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  __shared__ float sm[UP_S][UP_N];
+  const int i = blockIdx.x * UP_N + (t % UP_N), slice = t / UP_N;
+  int l = 0;
+#pragma unroll
+  for (int k = 1; k < NL; ++k) l += i >= param_offset(k);
+  const int j = i - param_offset(l);
+  float s = 0.f;
+  if (i < LBM_CNN_NPARAMS) {
+    const int n = nout_of(l);
+    const float* q = A.part[l] + j;
+#pragma unroll 8
+    for (int b = slice; b < A.nblocks; b += UP_S) s += q[(long long)b * n];
+  }
+  sm[slice][t % UP_N] = s;
+  __syncthreads();
+  if (slice > 0 || i >= LBM_CNN_NPARAMS) return;
+#pragma unroll
+  for (int k = 1; k < UP_S; ++k) s += sm[k][t];
+  A.grad[i] = s;
+  if (!A.adam) return;
+  const float mi = A.b1 * A.m[i] + (1.f - A.b1) * s;
+  const float vi = A.b2 * A.v[i] + (1.f - A.b2) * s * s;
+  A.m[i] = mi;
+  A.v[i] = vi;
+  const float wi = A.w[i] - A.lr * (mi / A.c1) / (sqrtf(vi / A.c2) + A.eps);
+  A.w[i] = wi;
+  if (l == 0 || j >= wsize(l)) return;  // the first layer and the biases are used in FP32
+  const int cin = cin_of(l), cout = cout_of(l);
+  const int co = j % cout, ci = j / cout % cin, tap = j / (cout * cin);
+  const __nv_bfloat16 h = __float2bfloat16(wi);
+  A.wt[l][co * kp_of(l) + tap * cin + ci] = h;
+  A.wb[l][ci * kb_of(l) + (8 - tap) * cout + co] = h;
 }
 
 // Packs layer l's FP32 w[3][3][cin][cout] into the forward operand
@@ -685,7 +740,7 @@ __global__ void k_pack(const float* __restrict__ w, int cin, int cout, int kp, i
     }
     wt[i] = __float2bfloat16(val);
   }
-  if (wb && i < cinp * kb) {
+  if (i < cinp * kb) {
     const int ci = i / kb, k = i % kb;
     float val = 0.f;
     if (ci < cin && k < 9 * cout) {
@@ -792,7 +847,7 @@ struct lbm_cnn {
   float* grad = nullptr;
   __nv_bfloat16* wt[NL] = {};
   __nv_bfloat16* wb[NL] = {};
-  __nv_bfloat16* act[NL] = {};  // act[l] = relu output of layer l-1 (act[0] unused)
+  __nv_bfloat16* act[NL] = {};  // act[l] = relu output of layer l-1; [0] of these four is unused
   unsigned* pos[NL] = {};       // pos[l]: which channels of act[l] are positive, a word per pixel
   __nv_bfloat16* dz[2] = {};    // ping-pong output gradients (32 channels)
   __nv_bfloat16* dz5 = nullptr; // output gradients of the last layer: 4 channels and 4 zeros
@@ -805,7 +860,7 @@ struct lbm_cnn {
   float* xf = nullptr;          // input features FP32 [p][4]
   float* tf = nullptr;          // target features FP32 [p][4]
   float* z = nullptr;           // last layer output FP32 [p][4]
-  float* wpartial = nullptr;    // weight-gradient partials
+  float* wpartial = nullptr;    // weight-gradient partials, layer by layer
   double* dpart = nullptr;      // loss / mass partials
   double* dloss = nullptr;
   int wblocks = 0;              // persistent CTAs of the weight gradients
@@ -830,11 +885,8 @@ int cfail(lbm_cnn* n, int code, const std::string& msg) {
                    std::string(#call) + ": " + cudaGetErrorString(e_));          \
   } while (0)
 
-int kp_of(int l) { return ru(9 * cin_of(l), 16); }
-int kb_of(int l) { return ru(9 * cout_of(l), 16); }
-
 int pack_all(lbm_cnn* n) {
-  for (int l = 0; l < NL; ++l) {
+  for (int l = 1; l < NL; ++l) {  // the first layer uses its FP32 weights
     const int cin = cin_of(l), cout = cout_of(l);
     const int kp = kp_of(l), coutp = ru(cout, 8), kb = kb_of(l), cinp = ru(cin, 8);
     const int total = std::max(coutp * kp, cinp * kb);
@@ -894,31 +946,53 @@ int forward(lbm_cnn* n, const double* coarse, bool train) {
 }
 
 template <int CG, int COUT>
-void wgrad(lbm_cnn* n, const CUtensorMap& act, const CUtensorMap& dz, float* grad) {
-  constexpr int NOUT = 9 * (CG == 4 ? 32 : 4) * COUT + COUT;
+void wgrad(lbm_cnn* n, const CUtensorMap& act, const CUtensorMap& dz, float* partial) {
   k_wgrad<CG, COUT><<<n->wblocks, WG_T, WgShape<CG, COUT == 32 ? 32 : 16>::SMEM, n->stream>>>(
-      act, dz, n->tiles_x, n->ntiles, n->wpartial, n->timeout);
-  k_sum_partials<<<(NOUT + 255) / 256, 256, 0, n->stream>>>(n->wpartial, n->wblocks, NOUT, grad);
+      act, dz, n->tiles_x, n->ntiles, partial, n->timeout);
 }
 
-// Loss against the target features and all gradients into n->grad.
-int loss_backward(lbm_cnn* n, const double* target) {
-  k_features<<<(n->npix + 255) / 256, 256, 0, n->stream>>>(target, n->npix, n->W, n->tf, nullptr);
-  const int nel = 4 * n->npix, nb = (nel + 255) / 256;
-  k_loss<<<nb, 256, 0, n->stream>>>(n->xf, n->z, n->tf, nel, n->dz5, n->dpart, n->scale,
-                                    n->loss_kind == LBM_CNN_LOSS_L1);
-  k_sum_d<<<1, 32, 0, n->stream>>>(n->dpart, nb, 1.0 / nel, n->dloss);
-  float* g = n->grad;
+// Loss against the target features and all gradients into n->grad; with
+// `adam`, one optimiser step (n->step is its number).
+int loss_backward(lbm_cnn* n, const double* target, bool adam) {
+  const int nb = (n->npix + 255) / 256;
+  k_loss<<<nb, 256, 0, n->stream>>>((const float4*)n->xf, (const float4*)n->z, target, n->npix,
+                                    (uint4*)n->dz5, n->dpart, n->scale, n->loss_kind == LBM_CNN_LOSS_L1);
+  UpdateArgs U = {};
+  for (int l = 0; l < NL; ++l) {
+    U.part[l] = n->wpartial + (size_t)n->wblocks * param_offset(l);
+    U.wt[l] = n->wt[l];
+    U.wb[l] = n->wb[l];
+  }
+  auto part = [&](int l) { return const_cast<float*>(U.part[l]); };
   // layer 5 (32 -> 4): dz5 holds d loss / d z5
-  wgrad<4, 4>(n, n->m_act[4], n->g_dz5, g + param_offset(4));
+  wgrad<4, 4>(n, n->m_act[4], n->g_dz5, part(4));
   conv<4, 32, EPI_MASK_BF16>(n, n->m_dz5, n->wb[4], nullptr, n->pos[4], n->dz[1], nullptr);
-  wgrad<4, 32>(n, n->m_act[3], n->g_dz[1], g + param_offset(3));
+  wgrad<4, 32>(n, n->m_act[3], n->g_dz[1], part(3));
   conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[1], n->wb[3], nullptr, n->pos[3], n->dz[0], nullptr);
-  wgrad<4, 32>(n, n->m_act[2], n->g_dz[0], g + param_offset(2));
+  wgrad<4, 32>(n, n->m_act[2], n->g_dz[0], part(2));
   conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[0], n->wb[2], nullptr, n->pos[2], n->dz[1], nullptr);
-  wgrad<4, 32>(n, n->m_act[1], n->g_dz[1], g + param_offset(1));
+  wgrad<4, 32>(n, n->m_act[1], n->g_dz[1], part(1));
   conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[1], n->wb[1], nullptr, n->pos[1], n->dz[0], nullptr);
-  wgrad<2, 32>(n, n->m_xs, n->g_dz[0], g + param_offset(0));
+  wgrad<2, 32>(n, n->m_xs, n->g_dz[0], part(0));
+  U.nblocks = n->wblocks;
+  U.w = n->w;
+  U.m = n->m;
+  U.v = n->v;
+  U.grad = n->grad;
+  U.lpart = n->dpart;
+  U.nl = nb;
+  U.lscale = 1.0 / (4.0 * n->npix);
+  U.loss = n->dloss;
+  U.adam = adam;
+  U.lr = n->lr;
+  U.b1 = n->b1;
+  U.b2 = n->b2;
+  U.eps = n->eps;
+  if (adam) {
+    U.c1 = 1.f - powf(n->b1, (float)n->step);
+    U.c2 = 1.f - powf(n->b2, (float)n->step);
+  }
+  k_update<<<(LBM_CNN_NPARAMS + UP_N - 1) / UP_N + 1, UP_N * UP_S, 0, n->stream>>>(U);
   CCK(n, cudaGetLastError());
   return LBM_OK;
 }
@@ -967,6 +1041,7 @@ int lbm_cnn_create(int H, int W, void* cuda_stream, lbm_cnn** out) {
   A((void**)&n->v, sizeof(float) * LBM_CNN_NPARAMS);
   A((void**)&n->grad, sizeof(float) * LBM_CNN_NPARAMS);
   for (int l = 0; l < NL; ++l) {
+    if (l == 0) continue;  // the first layer takes the FP32 features and weights
     A((void**)&n->wt[l], 2 * (size_t)ru(cout_of(l), 8) * kp_of(l));
     A((void**)&n->wb[l], 2 * (size_t)ru(cin_of(l), 8) * kb_of(l));
     A((void**)&n->act[l], 2 * P * CH[l]);
@@ -980,7 +1055,7 @@ int lbm_cnn_create(int H, int W, void* cuda_stream, lbm_cnn** out) {
   A((void**)&n->xf, 4 * P * 4);
   A((void**)&n->tf, 4 * P * 4);
   A((void**)&n->z, 4 * P * 4);
-  A((void**)&n->wpartial, sizeof(float) * (size_t)n->wblocks * (9 * 32 * 32 + 32));
+  A((void**)&n->wpartial, sizeof(float) * (size_t)n->wblocks * LBM_CNN_NPARAMS);
   A((void**)&n->dpart, sizeof(double) * 2 * ((4 * P + 255) / 256 + 1));
   A((void**)&n->dloss, sizeof(double));
   if (e == cudaSuccess) e = cudaStreamSynchronize(n->stream);
@@ -1059,7 +1134,7 @@ int lbm_cnn_loss_grad(lbm_cnn* n, const double* coarse, const double* target, do
   nvtxRangePushA("lbm_cnn_train_step");
   struct Pop { ~Pop() { nvtxRangePop(); } } pop;
   int rc = forward(n, coarse, true);
-  if (rc == LBM_OK) rc = loss_backward(n, target);
+  if (rc == LBM_OK) rc = loss_backward(n, target, false);
   if (rc != LBM_OK) return rc;
   if (loss) CCK(n, cudaMemcpyAsync(loss, n->dloss, sizeof(double), cudaMemcpyDeviceToHost, n->stream));
   if (grads)
@@ -1074,15 +1149,9 @@ int lbm_cnn_loss_grad(lbm_cnn* n, const double* coarse, const double* target, do
 int lbm_cnn_train_step(lbm_cnn* n, const double* coarse, const double* target, double* loss) {
   if (!n || !coarse || !target) return cfail(n, LBM_ERR_INVALID, "NULL argument");
   int rc = forward(n, coarse, true);
-  if (rc == LBM_OK) rc = loss_backward(n, target);
   if (rc != LBM_OK) return rc;
   n->step += 1;
-  const float c1 = 1.f - powf(n->b1, (float)n->step), c2 = 1.f - powf(n->b2, (float)n->step);
-  k_adam<<<(LBM_CNN_NPARAMS + 255) / 256, 256, 0, n->stream>>>(n->w, n->m, n->v, n->grad,
-                                                               LBM_CNN_NPARAMS, n->lr, n->b1,
-                                                               n->b2, n->eps, c1, c2);
-  CCK(n, cudaGetLastError());
-  rc = pack_all(n);
+  rc = loss_backward(n, target, true);
   if (rc != LBM_OK) return rc;
   if (loss) {
     int flag = 0;
