@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "../../include/lbm_cnn.h"
+#include "dw.cuh"
 #include "tc05.cuh"
 
 namespace {
@@ -579,15 +580,78 @@ __global__ void __launch_bounds__(C0_T) k_conv0(const float* __restrict__ xf, in
 // ---------------------------------------------------------------------------
 // Features, loss, Adam, packing, correction, restriction
 // ---------------------------------------------------------------------------
+// log32(x) = (float)log(x), bit for bit, mostly on the FP32 units. GB300 retires
+// one FP64 instruction per warp and 19 clocks, and log() takes about 31.
+//
+// x = 2^e m, m in [sqrt(1/2), sqrt(2)); with c the reciprocal of m rounded to a
+// 1/128 grid (10 significant bits, from a table with -log c as two FP32 words)
+//   log x = e log 2 - log c + log(1 + r),   r = m c - 1, |r| < 2^-7,
+// r as an FP32 pair (m as 24 + 29 bits, the product's rounding error by an FMA,
+// p - 1 exact), e log 2 as an exact product with a 13-bit word plus the rest,
+// log(1 + r) = r + t by its Taylor series, t = r^2 (-1/2 + r/3 - r^2/4 + r^3/5 -
+// r^4/6) in FP32 (|t| < 2^-15, truncation below 2^-51), the large terms added
+// by TwoSum. What remains is the rounding of the small terms, below
+//   delta = 2^-36 (1 + |e|),  and near x = 1 (e = 0, c = 1)  2^-20 |t| + 2^-21 |r_l|,
+// with a factor of 2 to spare (5.1 roundings of t: 2^-37.3, 3 x 2^-40 per |e|). If the sum rounds to the same FP32 number with
+// delta added and subtracted, so does log(x), which is within its last FP64
+// bit of the true value; else (one value in 700 for x in [0.1, 10], and values that
+// are not positive normal numbers) log() decides.
+struct LogEntry {
+  float c, lh, ll, pad;  // 1 / m, -log c = lh + ll
+};
+constexpr int LOG_J0 = 90, LOG_N = 93;  // grid points (LOG_J0 + k) / 128
+__device__ __forceinline__ float log32(double x, const LogEntry* __restrict__ table) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  if ((unsigned)(hi - 0x00100000) >= 0x7fe00000u) return (float)log(x);
+  const int e = (hi - 0x3fe6a09e) >> 20;  // 0x3fe6a09e: the high word of sqrt(1/2)
+  const int mhi = hi - e * (1 << 20);
+  const float mh = __int_as_float((int)(((unsigned)(mhi - 0x38000000) << 3) | (lo >> 29)));
+  const float ml = (float)(lo & 0x1fffffffu) * (mhi >= 0x3ff00000 ? 0x1p-52f : 0x1p-53f);
+  const int j = __float2int_rn(__fmul_rn(mh, 128.f));
+  const float4 q = __ldg(reinterpret_cast<const float4*>(table) + (j - LOG_J0));
+  const float c = q.x;
+  const float p = __fmul_rn(mh, c);
+  const float rh = __fsub_rn(p, 1.f), rl = __fmaf_rn(ml, c, __fmaf_rn(mh, c, -p));
+  const float r = __fadd_rn(rh, rl);
+  const float t = r * r * (-0.5f + r * (1.f / 3.f + r * (-0.25f + r * (0.2f - r * (1.f / 6.f)))));
+  const float fe = (float)e;
+  constexpr float LN2_H = 0x1.62ep-1f;                             // 13 bits
+  constexpr float LN2_L = (float)(0.693147180559945309417 - (double)LN2_H);
+  float s1, e1, s2, e2;
+  d2v16::two_sum(__fmul_rn(fe, LN2_H), q.y, s1, e1);
+  d2v16::two_sum(s1, rh, s2, e2);
+  const float low = __fadd_rn(__fadd_rn(__fadd_rn(e1, e2), __fadd_rn(q.z, rl)), __fmaf_rn(fe, LN2_L, t));
+  const float delta = e == 0 && c == 1.f ? __fmaf_rn(fabsf(t), 0x1p-20f, fabsf(rl) * 0x1p-21f)
+                                         : __fmaf_rn(fabsf(fe), 0x1p-36f, 0x1p-36f);
+  const float up = __fadd_rn(s2, __fadd_rn(low, delta)), down = __fadd_rn(s2, __fsub_rn(low, delta));
+  return up == down ? up : (float)log(x);
+}
+// The table (host).
+std::vector<LogEntry> log_table() {
+  std::vector<LogEntry> t(LOG_N);
+  for (int k = 0; k < LOG_N; ++k) {
+    const double c = std::nearbyint(1024.0 * 128.0 / (LOG_J0 + k)) / 1024.0;
+    const double l = -std::log(c);
+    t[k].c = (float)c;
+    t[k].lh = (float)l;
+    t[k].ll = (float)(l - (double)t[k].lh);
+    t[k].pad = 0.f;
+  }
+  return t;
+}
+
 // Planes [4][H][W] (rho, u, v, T) -> features (log rho, u, v, log T) in FP32
 // [p][4]; with `xs`, also their three BF16 parts (channel = part * 4 + feature,
 // 12 of 16 channels, row-planar; the other 4 stay zero).
+// Bound by memory (80 bytes a pixel with xs): 512 x 512 7 us; 33 us with the FP64
+// logarithms (the loss kernel, which takes the target's, 41 -> 16 us).
 __global__ void k_features(const double* __restrict__ f, int npix, int W, float* __restrict__ xf,
-                           __nv_bfloat16* __restrict__ xs) {
+                           __nv_bfloat16* __restrict__ xs, const LogEntry* __restrict__ logs) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= npix) return;
-  const float4 q = make_float4((float)log(f[p]), (float)f[npix + p], (float)f[2 * npix + p],
-                               (float)log(f[3 * npix + p]));
+  const float4 q = make_float4(log32(f[p], logs), (float)f[npix + p], (float)f[2 * npix + p],
+                               log32(f[3 * npix + p], logs));
   reinterpret_cast<float4*>(xf)[p] = q;
   if (xs) {
     unsigned s[4][3];
@@ -613,19 +677,19 @@ struct Scale4 {
 // Loss per element of d = out - target: d^2 (LBM_CNN_LOSS_MSE) or |d|
 // (LBM_CNN_LOSS_L1, whose gradient is sign(d), 0 at d = 0), and its gradient
 // with respect to the network's output (BF16, 4 channels and 4 zeros). A pixel
-// per thread, whose target features are taken here (the logarithms, on the FP64
-// units, are most of the kernel's time); the sums in FP64, per block.
+// per thread, whose target features are taken here; the sums in FP64, per block.
 __global__ void __launch_bounds__(256) k_loss(const float4* __restrict__ xf, const float4* __restrict__ z,
                                               const double* __restrict__ target, int npix,
                                               uint4* __restrict__ dz, double* __restrict__ partial,
-                                              const Scale4 sc, int l1) {
+                                              const Scale4 sc, int l1,
+                                              const LogEntry* __restrict__ logs) {
   __shared__ double sm[8];
   const int p = blockIdx.x * 256 + threadIdx.x;
   double s = 0.0;
   if (p < npix) {
     const float4 x4 = xf[p], z4 = z[p];
-    const float4 t4 = make_float4((float)log(target[p]), (float)target[npix + p],
-                                  (float)target[2 * npix + p], (float)log(target[3 * npix + p]));
+    const float4 t4 = make_float4(log32(target[p], logs), (float)target[npix + p],
+                                  (float)target[2 * npix + p], log32(target[3 * npix + p], logs));
     const float n = (float)(4 * npix);
     unsigned g[4];
 #pragma unroll
@@ -856,6 +920,7 @@ struct lbm_cnn {
   CUtensorMap g_dz[2], g_dz5;   // the same tiles without halo
   int tiles_x = 0, ntiles = 0;  // convolution tiles
   int sms = 0;
+  LogEntry* logs = nullptr;     // table of log32
   int* timeout = nullptr;       // a bounded wait of a convolution expired
   float* xf = nullptr;          // input features FP32 [p][4]
   float* tf = nullptr;          // target features FP32 [p][4]
@@ -933,7 +998,7 @@ void conv(lbm_cnn* n, const CUtensorMap& in, const __nv_bfloat16* wt, const floa
 int forward(lbm_cnn* n, const double* coarse, bool train) {
   auto bits = [&](int l) { return train ? n->pos[l] : nullptr; };
   k_features<<<(n->npix + 255) / 256, 256, 0, n->stream>>>(coarse, n->npix, n->W, n->xf,
-                                                           train ? n->xs : nullptr);
+                                                           train ? n->xs : nullptr, n->logs);
   const float* w = n->w;
   k_conv0<<<(n->npix + C0_T - 1) / C0_T, C0_T, 0, n->stream>>>(n->xf, n->H, n->W,
                                                                w + param_offset(0), n->act[1], bits(1));
@@ -956,7 +1021,7 @@ void wgrad(lbm_cnn* n, const CUtensorMap& act, const CUtensorMap& dz, float* par
 int loss_backward(lbm_cnn* n, const double* target, bool adam) {
   const int nb = (n->npix + 255) / 256;
   k_loss<<<nb, 256, 0, n->stream>>>((const float4*)n->xf, (const float4*)n->z, target, n->npix,
-                                    (uint4*)n->dz5, n->dpart, n->scale, n->loss_kind == LBM_CNN_LOSS_L1);
+                                    (uint4*)n->dz5, n->dpart, n->scale, n->loss_kind == LBM_CNN_LOSS_L1, n->logs);
   UpdateArgs U = {};
   for (int l = 0; l < NL; ++l) {
     U.part[l] = n->wpartial + (size_t)n->wblocks * param_offset(l);
@@ -1052,6 +1117,10 @@ int lbm_cnn_create(int H, int W, void* cuda_stream, lbm_cnn** out) {
   A((void**)&n->dz5, 2 * P * 8);
   A((void**)&n->xs, 2 * P * 16);
   A((void**)&n->timeout, sizeof(int));
+  const std::vector<LogEntry> logs = log_table();
+  A((void**)&n->logs, sizeof(LogEntry) * LOG_N);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(n->logs, logs.data(), sizeof(LogEntry) * LOG_N, cudaMemcpyHostToDevice, n->stream);
   A((void**)&n->xf, 4 * P * 4);
   A((void**)&n->tf, 4 * P * 4);
   A((void**)&n->z, 4 * P * 4);
@@ -1086,7 +1155,7 @@ int lbm_cnn_destroy(lbm_cnn* n) {
   if (!n) return LBM_OK;
   if (n->stream) cudaStreamSynchronize(n->stream);
   void* ps[] = {n->w, n->m, n->v, n->grad, n->dz[0], n->dz[1], n->xf, n->tf, n->z,
-                n->wpartial, n->dpart, n->dloss, n->dz5, n->xs, n->timeout};
+                n->wpartial, n->dpart, n->dloss, n->dz5, n->xs, n->logs, n->timeout};
   for (void* p : ps)
     if (p) cudaFree(p);
   for (int l = 0; l < NL; ++l) {
@@ -1183,8 +1252,8 @@ int lbm_cnn_set_loss(lbm_cnn* n, int kind) {
 int lbm_cnn_residual_rms(lbm_cnn* n, const double* coarse, const double* target, double* rms) {
   if (!n || !coarse || !target || !rms) return cfail(n, LBM_ERR_INVALID, "NULL argument");
   const int nb = (n->npix + 255) / 256;
-  k_features<<<nb, 256, 0, n->stream>>>(coarse, n->npix, n->W, n->xf, nullptr);
-  k_features<<<nb, 256, 0, n->stream>>>(target, n->npix, n->W, n->tf, nullptr);
+  k_features<<<nb, 256, 0, n->stream>>>(coarse, n->npix, n->W, n->xf, nullptr, n->logs);
+  k_features<<<nb, 256, 0, n->stream>>>(target, n->npix, n->W, n->tf, nullptr, n->logs);
   std::vector<double> part(4 * (size_t)nb);
   double* dpart = nullptr;
   CCK(n, cudaMalloc((void**)&dpart, sizeof(double) * part.size()));
