@@ -537,44 +537,74 @@ __global__ void __launch_bounds__(WG_T, WG_CTAS_PER_SM)
 // FP32 keeps differences between neighbouring nodes that are below one BF16
 // step of the fields (smooth regions of fine-grained coarse grids).
 // w: the layer's FP32 parameters, (3, 3, 4, 32) then 32 biases.
+// A thread computes two neighbouring pixels of a row in paired FP32 (f32x2 over
+// channel pairs; taps in order, as fused multiply-adds, zeros outside the
+// image): the weights, read from shared memory four at a time by every thread
+// alike, then serve two pixels. Bound by the FP32 units (7.8 us at 512 x 512):
+// 17 us; one pixel per thread in scalar FP32 was bound by its shared-memory
+// reads, 24 us.
 constexpr int C0_T = 128;
 __global__ void __launch_bounds__(C0_T) k_conv0(const float* __restrict__ xf, int H, int W,
                                                 const float* __restrict__ w,
                                                 __nv_bfloat16* __restrict__ out,
                                                 unsigned* __restrict__ bits) {
-  __shared__ float sw[9 * 4 * 32 + 32];
+  __shared__ __align__(16) float sw[9 * 4 * 32 + 32];
   for (int i = threadIdx.x; i < 9 * 4 * 32 + 32; i += C0_T) sw[i] = w[i];
   __syncthreads();
-  const int p = blockIdx.x * C0_T + threadIdx.x;
-  if (p >= H * W) return;
-  const int y = p / W, x = p - y * W;
-  float acc[32];
+  const int W2 = (W + 1) / 2, q = blockIdx.x * C0_T + threadIdx.x;
+  if (q >= H * W2) return;
+  const int y = q / W2, x = 2 * (q - y * W2);
+  float2 acc[2][16];
 #pragma unroll
-  for (int c = 0; c < 32; ++c) acc[c] = sw[9 * 4 * 32 + c];
+  for (int c = 0; c < 16; ++c)
+    acc[0][c] = acc[1][c] = *reinterpret_cast<const float2*>(sw + 9 * 4 * 32 + 2 * c);
 #pragma unroll
-  for (int tap = 0; tap < 9; ++tap) {
-    const int yy = y + tap / 3 - 1, xx = x + tap % 3 - 1;
-    if (yy < 0 || yy >= H || xx < 0 || xx >= W) continue;
-    const float4 q = *reinterpret_cast<const float4*>(xf + 4 * ((long long)yy * W + xx));
-    const float qi[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-    for (int ci = 0; ci < 4; ++ci)
-#pragma unroll
-      for (int c = 0; c < 32; ++c) acc[c] += qi[ci] * sw[(tap * 4 + ci) * 32 + c];
-  }
-  unsigned pos = 0u;
-#pragma unroll
-  for (int cg = 0; cg < 4; ++cg) {
-    __nv_bfloat162 q[4];
+  for (int dy = 0; dy < 3; ++dy) {
+    const int yy = y + dy - 1;
+    float4 in[4];  // columns x - 1 .. x + 2
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      q[k] = __floats2bfloat162_rn(fmaxf(acc[cg * 8 + 2 * k], 0.f), fmaxf(acc[cg * 8 + 2 * k + 1], 0.f));
-      pos |= positive_bits(q[k]) >> (cg + 4 * k);
+      const int xx = x + k - 1;
+      in[k] = yy >= 0 && yy < H && xx >= 0 && xx < W
+                  ? __ldg(reinterpret_cast<const float4*>(xf) + (long long)yy * W + xx)
+                  : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    *reinterpret_cast<uint4*>(out + (((long long)y * 4 + cg) * W + x) * 8) =
-        *reinterpret_cast<const uint4*>(q);
+#pragma unroll
+    for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+      for (int ci = 0; ci < 4; ++ci) {
+        const float a = (&in[dx].x)[ci], b = (&in[dx + 1].x)[ci];
+        const float2 a2 = make_float2(a, a), b2 = make_float2(b, b);
+        const float4* row = reinterpret_cast<const float4*>(sw + ((dy * 3 + dx) * 4 + ci) * 32);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const float4 k = row[c];
+          const float2 k0 = make_float2(k.x, k.y), k1 = make_float2(k.z, k.w);
+          acc[0][2 * c] = __ffma2_rn(a2, k0, acc[0][2 * c]);
+          acc[0][2 * c + 1] = __ffma2_rn(a2, k1, acc[0][2 * c + 1]);
+          acc[1][2 * c] = __ffma2_rn(b2, k0, acc[1][2 * c]);
+          acc[1][2 * c + 1] = __ffma2_rn(b2, k1, acc[1][2 * c + 1]);
+        }
+      }
   }
-  if (bits) bits[p] = pos;
+#pragma unroll
+  for (int n = 0; n < 2; ++n) {
+    if (x + n >= W) break;
+    unsigned pos = 0u;
+#pragma unroll
+    for (int cg = 0; cg < 4; ++cg) {
+      __nv_bfloat162 v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float2 s = acc[n][cg * 4 + k];
+        v[k] = __floats2bfloat162_rn(fmaxf(s.x, 0.f), fmaxf(s.y, 0.f));
+        pos |= positive_bits(v[k]) >> (cg + 4 * k);
+      }
+      *reinterpret_cast<uint4*>(out + (((long long)y * 4 + cg) * W + x + n) * 8) =
+          *reinterpret_cast<const uint4*>(v);
+    }
+    if (bits) bits[(long long)y * W + x + n] = pos;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1000,7 +1030,7 @@ int forward(lbm_cnn* n, const double* coarse, bool train) {
   k_features<<<(n->npix + 255) / 256, 256, 0, n->stream>>>(coarse, n->npix, n->W, n->xf,
                                                            train ? n->xs : nullptr, n->logs);
   const float* w = n->w;
-  k_conv0<<<(n->npix + C0_T - 1) / C0_T, C0_T, 0, n->stream>>>(n->xf, n->H, n->W,
+  k_conv0<<<(n->H * ((n->W + 1) / 2) + C0_T - 1) / C0_T, C0_T, 0, n->stream>>>(n->xf, n->H, n->W,
                                                                w + param_offset(0), n->act[1], bits(1));
   conv<32, 32, EPI_RELU_BF16>(n, n->m_act[1], n->wt[1], w + param_offset(1) + wsize(1), nullptr, n->act[2], nullptr, bits(2));
   conv<32, 32, EPI_RELU_BF16>(n, n->m_act[2], n->wt[2], w + param_offset(2) + wsize(2), nullptr, n->act[3], nullptr, bits(3));
