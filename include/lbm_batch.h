@@ -46,12 +46,17 @@ int lbm_batch_create(const lbm_batch_config* cfg, void* cuda_stream, lbm_batch**
 int lbm_batch_set_init(lbm_batch* b, const double* rho, const double* u,
                        const double* v, const double* T, int on_device);
 
-/* Advances every tube by nsteps >= 0 steps in ONE persistent kernel launch
- * (replayed from a CUDA graph captured per distinct nsteps): each resident
- * block processes its share of the tiles, then all blocks meet at a grid
- * barrier before the next step. The barrier's spin is bounded (about 1 s);
- * if it expires the kernel records LBM_ERR_TIMEOUT (see lbm_batch_status)
- * and every block returns. Asynchronous. */
+/* Advances every tube by nsteps >= 0 steps in one CUDA-graph launch (captured
+ * per distinct nsteps), in one of two forms with the same results, bit for bit:
+ *  resident  (two steps or more, every tube of at most 3600 nodes): a block
+ *            keeps a tube in shared memory for all nsteps;
+ *  streamed  (else, and after lbm_batch_set_tiling): each block of one
+ *            persistent launch processes its share of the tiles, then all
+ *            blocks meet at a grid barrier before the next step. The
+ *            barrier's spin is bounded (about 1 s); if it expires the kernel
+ *            records LBM_ERR_TIMEOUT (see lbm_batch_status) and every block
+ *            returns.
+ * Asynchronous. */
 int lbm_batch_step(lbm_batch* b, long long nsteps);
 
 /* rho, u, v, T of every node in FP64 (conserved sums and T recovered in FP64
@@ -71,18 +76,19 @@ int lbm_batch_audit(lbm_batch* b, double* totals);
  * error of the batch). */
 int lbm_batch_status(lbm_batch* b, long long* first_bad, int* nbad, int* timeout);
 
-/* Tiling: tile = nodes per work item, threads = threads per block; each
+/* Tiling of the streamed form: tile = nodes per work item, threads = threads per block; each
  * thread updates node pairs, so tile is 2 or 4 x threads. The pairs built:
  * (128, 64), (256, 64), (256, 128), (512, 128), (512, 256), (1024, 256),
- * (1024, 512), (1024, 128); anything else is LBM_ERR_INVALID. */
+ * (1024, 512), (1024, 128); anything else is LBM_ERR_INVALID. Later steps of
+ * the batch take the streamed form with this tiling. */
 int lbm_batch_set_tiling(lbm_batch* b, int tile, int threads);
 int lbm_batch_get_tiling(lbm_batch* b, int* tile, int* threads, int* blocks);
 
-/* Autotuner: times every (tile, threads) candidate for `trial_steps` steps on
+/* Autotuner of the streamed form's tiling: times every (tile, threads) candidate for `trial_steps` steps on
  * the live GPU (restoring the populations afterwards), keeps the fastest and
  * returns it in chosen[0..1]. When cache_path is not NULL the result is read
  * from / written to that JSON file, keyed by the GPU name and a hash of the
- * tube lengths. Synchronises. */
+ * tube lengths. lbm_batch_step chooses the form by itself again. Synchronises. */
 int lbm_batch_autotune(lbm_batch* b, int trial_steps, const char* cache_path, int* chosen);
 
 /* Test hook for the bounded barrier: block `block` skips its arrival at the

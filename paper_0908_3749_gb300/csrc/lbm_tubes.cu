@@ -1,5 +1,10 @@
-// lbm_tubes.cu -- batches of quasi-1D shock tubes (include/lbm_batch.h) in one
-// persistent, graph-captured kernel launch per call.
+// lbm_tubes.cu -- batches of quasi-1D shock tubes (include/lbm_batch.h), every
+// call one graph-captured launch. Two forms with the same arithmetic: the
+// resident one (k_tubes_resident), a tube per block in shared memory for all the
+// steps of the call, and the streamed one (k_tubes), persistent blocks that
+// share the tubes' tiles out and meet at a grid barrier after every step: for
+// batches with a tube too long for shared memory, single steps, and where
+// lbm_batch_set_tiling asked for it.
 //
 // Layout: FP32 populations SoA f[i][p], p running over all tubes; tube t owns
 // nodes off[t] .. off[t] + nx[t] - 1 with off[t] a multiple of 32 (128-byte
@@ -15,7 +20,7 @@
 // constants are the relaxation weights w_k = -dt s_k and lambda = dt / dx;
 // the scaled block inverses of M are lattice constants shared by all tubes.
 //
-// The persistent kernel runs all requested steps: each resident block takes
+// The streamed form runs all requested steps in one launch: each block takes
 // items blockIdx, blockIdx + gridDim, ...; the 16 population rows of an item
 // and 4 halo nodes on each side come into shared memory by bulk TMA copies
 // (two stages: the next item's copy runs while the current one is computed);
@@ -62,6 +67,7 @@ struct BatchStatus {
   unsigned bar_gen;         // barrier generation
   int timeout;              // a barrier wait expired
   unsigned long long first_timeout_step;
+  unsigned done;            // blocks finished in a resident launch
 };
 
 struct BatchArgs {
@@ -73,6 +79,7 @@ struct BatchArgs {
   BatchStatus* st;
   long long plane;            // populations per buffer plane
   int nitems;
+  int ntubes;
   int skip_block;             // test hook: block that skips one barrier arrival
   long long skip_step;
   long long spin_cycles;      // barrier wait limit in SM clock cycles
@@ -124,6 +131,11 @@ __device__ bool grid_barrier(const BatchArgs& A, unsigned& gen, bool skip) {
   return ok != 0;
 }
 
+// Floats per row of a tube in shared memory (resident form): four columns
+// before the nodes, the nodes, the ghost after them, rounded up to 16 bytes
+// past the end of the row's copy.
+__host__ __device__ constexpr int resident_width(int nx) { return ((nx + 3) & ~3) + 8; }
+
 // Staged width of an item: its TILE nodes plus 4 halo nodes on each side.
 template <int TILE>
 __host__ __device__ constexpr int stage_width() { return TILE + 8; }
@@ -146,6 +158,78 @@ __device__ __forceinline__ void issue_item(const BatchArgs& A, const float* fin,
     bulk_load(stage + i * stage_width<TILE>(), src + i * A.plane, 4u * n, bar);
 }
 
+// The constants of one tube in registers: relaxation weights and
+// Lax-Wendroff weights per |v_x| class, a0 = 1 - 2 be, aE = be - s al, aW =
+// be + s al (s the sign of v_x).
+struct TubeConst {
+  float w[12], al[4], be[4];
+  __device__ __forceinline__ explicit TubeConst(const TubeDesc& D) {
+#pragma unroll
+    for (int k = 0; k < 12; ++k) w[k] = D.w[k];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const float c = (float)xmag(g) * D.lam;
+      al[g] = 0.5f * c;
+      be[g] = 0.5f * c * c;
+    }
+  }
+};
+
+// One step of a node pair from its populations f, in paired FP32: out(i, value)
+// takes population i's new values, east(i) and west(i) give the neighbours'
+// populations. Sets bad_a / bad_b for a non-finite state or rho <= 0.
+template <typename East, typename West, typename Out>
+__device__ __forceinline__ void tube_pair(const Coeffs<float>& E, const TubeConst& T,
+                                          const F2 (&f)[16], East east, West west, Out store,
+                                          bool& bad_a, bool& bad_b) {
+  const float (&w)[12] = T.w;
+  Groups<F2> d;
+  transform(f, d);
+  const Cons<F2> m = conserved(E, d);
+  const Eq<F2> q = equilibria(m.rho, m.jx, m.jy, m.e);
+  // deviations from equilibrium of the non-conserved moments, relaxed
+  const F2 r11 = w[6] * (row4(E.F0, 2, d.S) - q.m11);
+  const F2 r12 = w[7] * row4(E.F0, 3, d.S);
+  const F2 r7 = w[2] * (row4(E.FX, 1, d.X) - q.m7);
+  const F2 r9 = w[4] * (row4(E.FX, 2, d.X) - q.m9);
+  const F2 r15 = w[10] * row4(E.FX, 3, d.X);
+  const F2 r8 = w[3] * (row4(E.FY, 1, d.Y) - q.m8);
+  const F2 r10 = w[5] * (row4(E.FY, 2, d.Y) - q.m10);
+  const F2 r16 = w[11] * row4(E.FY, 3, d.Y);
+  const F2 r5 = w[0] * (E.FC[0][0] * d.C[0] + E.FC[0][1] * d.C[1] - q.m5);
+  const F2 r13 = w[8] * (E.FC[1][0] * d.C[0] + E.FC[1][1] * d.C[1] - q.m13);
+  const F2 r6 = w[1] * (E.FS[0][0] * d.C[2] + E.FS[0][1] * d.C[3] - q.m6);
+  const F2 r14 = w[9] * (E.FS[1][0] * d.C[2] + E.FS[1][1] * d.C[3] - q.m14);
+  F2 S[4], C[4], X[4], Y[4], df[16];
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    S[g] = E.E0[g][2] * r11 + E.E0[g][3] * r12;
+    X[g] = E.EX[g][1] * r7 + E.EX[g][2] * r9 + E.EX[g][3] * r15;
+    Y[g] = E.EY[g][1] * r8 + E.EY[g][2] * r10 + E.EY[g][3] * r16;
+  }
+  C[0] = E.EC[0][0] * r5 + E.EC[0][1] * r13;
+  C[1] = E.EC[1][0] * r5 + E.EC[1][1] * r13;
+  C[2] = E.ES[0][0] * r6 + E.ES[0][1] * r14;
+  C[3] = E.ES[1][0] * r6 + E.ES[1][1] * r14;
+  inverse_transform(S, C, X, Y, df);
+  bad_a = !(m.rho.v.x > 0.0f) || !isfinite(m.rho.v.x + m.jx.v.x + m.jy.v.x + m.e.v.x);
+  bad_b = !(m.rho.v.y > 0.0f) || !isfinite(m.rho.v.y + m.jx.v.y + m.jy.v.y + m.e.v.y);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    F2 out;
+    if (xclass(i) == 0) {
+      out = f[i] + df[i];
+    } else {
+      const int g = xclass(i) - 1;
+      const float s = xsign(i);
+      out = (1.0f - 2.0f * T.be[g]) * f[i] + df[i];
+      out = (T.be[g] - s * T.al[g]) * east(i) + out;
+      out = (T.be[g] + s * T.al[g]) * west(i) + out;
+    }
+    store(i, out);
+  }
+}
+
 // Updates one item from its staged copy: thread t takes node pairs
 // (x, x + BT) of each 2 BT-node chunk in paired arithmetic.
 template <int BT, int TILE>
@@ -156,22 +240,10 @@ __device__ __forceinline__ void tube_item(const BatchArgs& A, float* __restrict_
   const TubeDesc& D = A.tubes[it.x];
   const long long off = D.off;
   const int nx = D.nx;
-  const float lam = D.lam;
-  float w[12];
-#pragma unroll
-  for (int k = 0; k < 12; ++k) w[k] = D.w[k];
-  // Lax-Wendroff weights per |v_x| class: a0 = 1 - 2 b, aE = b - s a, aW = b + s a
-  float al[4], be[4];
-#pragma unroll
-  for (int g = 0; g < 4; ++g) {
-    const float c = (float)xmag(g) * lam;
-    al[g] = 0.5f * c;
-    be[g] = 0.5f * c * c;
-  }
+  const TubeConst T(D);
   const float* gL = A.ghost + (size_t)it.x * 32;
   const float* gR = gL + 16;
   const long long P = A.plane;
-  const Coeffs<float>& E = A.E;
   bool bad = false;
 #pragma unroll 1
   for (int c0 = 0; c0 < TILE; c0 += 2 * BT) {
@@ -184,55 +256,18 @@ __device__ __forceinline__ void tube_item(const BatchArgs& A, float* __restrict_
     F2 f[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) f[i] = F2(sa[i * W], sb[i * W]);
-    Groups<F2> d;
-    transform(f, d);
-    const Cons<F2> m = conserved(E, d);
-    const Eq<F2> q = equilibria(m.rho, m.jx, m.jy, m.e);
-    // deviations from equilibrium of the non-conserved moments, relaxed
-    const F2 r11 = w[6] * (row4(E.F0, 2, d.S) - q.m11);
-    const F2 r12 = w[7] * row4(E.F0, 3, d.S);
-    const F2 r7 = w[2] * (row4(E.FX, 1, d.X) - q.m7);
-    const F2 r9 = w[4] * (row4(E.FX, 2, d.X) - q.m9);
-    const F2 r15 = w[10] * row4(E.FX, 3, d.X);
-    const F2 r8 = w[3] * (row4(E.FY, 1, d.Y) - q.m8);
-    const F2 r10 = w[5] * (row4(E.FY, 2, d.Y) - q.m10);
-    const F2 r16 = w[11] * row4(E.FY, 3, d.Y);
-    const F2 r5 = w[0] * (E.FC[0][0] * d.C[0] + E.FC[0][1] * d.C[1] - q.m5);
-    const F2 r13 = w[8] * (E.FC[1][0] * d.C[0] + E.FC[1][1] * d.C[1] - q.m13);
-    const F2 r6 = w[1] * (E.FS[0][0] * d.C[2] + E.FS[0][1] * d.C[3] - q.m6);
-    const F2 r14 = w[9] * (E.FS[1][0] * d.C[2] + E.FS[1][1] * d.C[3] - q.m14);
-    F2 S[4], C[4], X[4], Y[4], df[16];
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      S[g] = E.E0[g][2] * r11 + E.E0[g][3] * r12;
-      X[g] = E.EX[g][1] * r7 + E.EX[g][2] * r9 + E.EX[g][3] * r15;
-      Y[g] = E.EY[g][1] * r8 + E.EY[g][2] * r10 + E.EY[g][3] * r16;
-    }
-    C[0] = E.EC[0][0] * r5 + E.EC[0][1] * r13;
-    C[1] = E.EC[1][0] * r5 + E.EC[1][1] * r13;
-    C[2] = E.ES[0][0] * r6 + E.ES[0][1] * r14;
-    C[3] = E.ES[1][0] * r6 + E.ES[1][1] * r14;
-    inverse_transform(S, C, X, Y, df);
-    bad |= !(m.rho.v.x > 0.0f) || !isfinite(m.rho.v.x + m.jx.v.x + m.jy.v.x + m.e.v.x);
-    bad |= actb && (!(m.rho.v.y > 0.0f) || !isfinite(m.rho.v.y + m.jx.v.y + m.jy.v.y + m.e.v.y));
     const bool wa = xa > 0, ea = xa < nx - 1, wb = xb > 0, eb = xb < nx - 1;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      F2 out;
-      if (xclass(i) == 0) {
-        out = f[i] + df[i];
-      } else {
-        const int g = xclass(i) - 1;
-        const float s = xsign(i);
-        const F2 fe(ea ? sa[i * W + 1] : gR[i], eb ? sb[i * W + 1] : gR[i]);
-        const F2 fw(wa ? sa[i * W - 1] : gL[i], wb ? sb[i * W - 1] : gL[i]);
-        out = (1.0f - 2.0f * be[g]) * f[i] + df[i];
-        out = (be[g] - s * al[g]) * fe + out;
-        out = (be[g] + s * al[g]) * fw + out;
-      }
-      fout[i * P + off + xa] = out.v.x;
-      if (actb) fout[i * P + off + xb] = out.v.y;
-    }
+    bool bad_a, bad_b;
+    tube_pair(
+        A.E, T, f,
+        [&](int i) { return F2(ea ? sa[i * W + 1] : gR[i], eb ? sb[i * W + 1] : gR[i]); },
+        [&](int i) { return F2(wa ? sa[i * W - 1] : gL[i], wb ? sb[i * W - 1] : gL[i]); },
+        [&](int i, F2 out) {
+          fout[i * P + off + xa] = out.v.x;
+          if (actb) fout[i * P + off + xb] = out.v.y;
+        },
+        bad_a, bad_b);
+    bad |= bad_a || (actb && bad_b);
   }
   if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0)
     atomicMin(&A.bad[it.x], level);
@@ -301,6 +336,124 @@ __global__ void __launch_bounds__(BT) k_tubes(float* f0, float* f1, const BatchA
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     A.st->step = level0 + (unsigned long long)nsteps;
     A.st->cur = (int)((cur + nsteps) & 1);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Resident form: a tube per block, in shared memory for all the steps
+// ---------------------------------------------------------------------------
+// Tubes are independent (Dirichlet ends), so a block that holds a whole tube
+// needs no grid barrier and no memory traffic between its first and its last
+// step. The block copies the tube's 16 population rows into shared memory
+// (bulk TMA), steps it nsteps times in place and stores it back into the
+// buffer it came from. A row is [1 unused][2 saved][gL][nx nodes][gR]: the
+// Dirichlet ghosts sit beside the end nodes. A step runs in chunks of 2 BT
+// nodes, thread t updating nodes (x, x + BT) with the arithmetic of the streamed
+// form (the same bits): every thread reads its nodes and their neighbours, the
+// block synchronises, every thread stores its results. The next chunk's first
+// node needs the old values of this chunk's last node: they are saved, before
+// the synchronisation, in one of the two saved columns (by chunk parity).
+//
+// Bound by instruction issue (757 per warp and step for 64 nodes, 56 % of the
+// slots at 16 warps per SM) where the streamed form is bound by HBM (128 bytes
+// per node and step). Measured: 4096 tubes of 128-2048 nodes (4.4 M) 61 us a
+// step (streamed 115), 61 such tubes 4.0 us (streamed 7.3). A single step
+// costs 190 us against 130, for the load and the store do not overlap within a
+// block; two steps 238 against 244: lbm_batch_step takes this form from two on.
+template <int BT>
+__global__ void __launch_bounds__(BT, 512 / BT) k_tubes_resident(float* f0, float* f1, const BatchArgs A,
+                                                               const int* __restrict__ order,
+                                                               long long nsteps) {
+  extern __shared__ __align__(16) unsigned char res_smem[];
+  float* const rows = reinterpret_cast<float*>(res_smem);
+  __shared__ unsigned long long bar;
+  __shared__ unsigned long long s_level;
+  __shared__ int s_cur, s_skip;
+  const int tube = order[blockIdx.x];
+  const TubeDesc& D = A.tubes[tube];
+  const int nx = D.nx, t = threadIdx.x;
+  const int W = resident_width(nx);
+  if (t == 0) {
+    mbar_init(&bar, 1);
+    s_level = *(volatile unsigned long long*)&A.st->step;
+    s_cur = *(volatile int*)&A.st->cur;
+    s_skip = *(volatile int*)&A.st->timeout;
+  }
+  __syncthreads();
+  float* const g = (s_cur ? f1 : f0) + D.off;
+  const unsigned long long level0 = s_level;
+  bool ok = s_skip == 0;  // a batch that timed out stays as it is
+  if (ok) {
+    if (t == 0) {
+      const unsigned n = 4u * (unsigned)((nx + 3) & ~3);  // bytes per row; D.off is a multiple of 32
+      mbar_expect_tx(&bar, 16u * n);
+#pragma unroll 1
+      for (int i = 0; i < 16; ++i) bulk_load(rows + i * W + 4, g + i * A.plane, n, &bar);
+    }
+    ok = __syncthreads_and(mbar_wait_bounded(&bar, 0, TMA_WAIT_CYCLES));
+    if (!ok && t == 0) {  // the copy did not land: record it, wait once more, leave
+      atomicExch(&A.st->timeout, 1);
+      atomicMin(&A.st->first_timeout_step, level0);
+      mbar_wait_bounded(&bar, 0, TMA_WAIT_CYCLES);
+    }
+  }
+  if (ok) {
+    if (t < 32) rows[(t & 15) * W + (t < 16 ? 3 : 4 + nx)] = A.ghost[(size_t)tube * 32 + t];
+    __syncthreads();
+    const TubeConst T(D);
+    bool reported = false;  // this warp has flagged the tube
+#pragma unroll 1
+    for (long long s = 0; s < nsteps; ++s) {
+#pragma unroll 1
+      for (int c = 0, c0 = 0; c0 < nx; ++c, c0 += 2 * BT) {
+        const int xa = c0 + t, xb = xa + BT;
+        F2 out[16];
+        bool bad = false;
+        if (xa < nx) {
+          const float* pa = rows + 4 + xa;
+          const float* pb = rows + 4 + min(xb, nx - 1);  // no node b: any node's values
+          const float* wa = t == 0 && c > 0 ? rows + 1 + (c & 1) : pa - 1;
+          F2 f[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) f[i] = F2(pa[i * W], pb[i * W]);
+          if (t == BT - 1 && xb < nx)
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              if (xclass(i) != 0) rows[i * W + 1 + ((c + 1) & 1)] = f[i].v.y;
+          bool bad_a, bad_b;
+          tube_pair(
+              A.E, T, f, [&](int i) { return F2(pa[i * W + 1], pb[i * W + 1]); },
+              [&](int i) { return F2(wa[i * W], pb[i * W - 1]); }, [&](int i, F2 v) { out[i] = v; },
+              bad_a, bad_b);
+          bad = bad_a || (xb < nx && bad_b);
+        }
+        __syncthreads();
+        if (xa < nx) {
+          float* pa = rows + 4 + xa;
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            pa[i * W] = out[i].v.x;
+            if (xb < nx) pa[i * W + BT] = out[i].v.y;
+          }
+        }
+        if (!reported && __any_sync(0xffffffffu, bad)) {
+          reported = true;
+          if ((t & 31) == 0) atomicMin(&A.bad[tube], level0 + (unsigned long long)s);
+        }
+      }
+      __syncthreads();
+    }
+    for (int i = 0; i < 16; ++i)
+      for (int x = t; x < nx; x += BT) g[i * A.plane + x] = rows[i * W + 4 + x];
+  }
+  // The block that finishes last moves the time level on.
+  __syncthreads();
+  if (t == 0) {
+    __threadfence();
+    if (atomicAdd(&A.st->done, 1u) == (unsigned)A.ntubes - 1) {
+      A.st->done = 0;
+      if (!*(volatile int*)&A.st->timeout) A.st->step = level0 + (unsigned long long)nsteps;
+    }
   }
 }
 
@@ -408,6 +561,26 @@ size_t variant_smem(int v) {
 }
 constexpr int NVARIANTS = sizeof(VARIANTS) / sizeof(VARIANTS[0]);
 
+// Resident form: blocks of 128, 256 or 512 threads.
+using ResidentFn = void (*)(float*, float*, const BatchArgs, const int*, long long);
+ResidentFn resident_fn(int threads) {
+  return threads == 128 ? k_tubes_resident<128> : threads == 256 ? k_tubes_resident<256> : k_tubes_resident<512>;
+}
+size_t resident_smem(int nx) { return 16 * sizeof(float) * (size_t)resident_width(nx); }
+// The longest tube that a block holds: 227 KB of shared memory less 1 KB.
+constexpr int RESIDENT_MAX_NX = 226 * 1024 / 64 - 16;
+static_assert(16 * sizeof(float) * resident_width(RESIDENT_MAX_NX) <= 226 * 1024, "shared memory");
+// Launches of the resident form group the tubes by length, in steps of
+// RESIDENT_STEP nodes (16 KB), since a launch's blocks all take the shared
+// memory of its longest tube.
+constexpr int RESIDENT_STEP = 256;
+// Fewer steps than this go through the streamed form (figures: k_tubes_resident).
+constexpr int RESIDENT_MIN_STEPS = 2;
+// Tubes per launch group: `count` tubes order[first ..], the longest nx_max.
+struct TubeGroup {
+  int first, count, nx_max, threads;
+};
+
 int find_variant(int tile, int threads) {
   for (int k = 0; k < NVARIANTS; ++k)
     if (VARIANTS[k].tile == tile && VARIANTS[k].threads == threads) return k;
@@ -443,7 +616,12 @@ struct lbm_batch {
   long long spin_cycles = 0;
   int skip_block = -1;
   long long skip_step = -1;
-  std::map<std::pair<long long, int>, cudaGraphExec_t> graphs;
+  bool streamed = false;       // lbm_batch_set_tiling asked for the streamed form
+  std::vector<TubeGroup> groups;  // resident form: launches, longest tubes first (empty: too long)
+  int* order = nullptr;           // tube indices, group by group
+  std::vector<cudaStream_t> side; // capture branches of the groups after the first
+  std::vector<cudaEvent_t> joins; // [0] the fork, [k] the end of branch k
+  std::map<std::pair<long long, int>, cudaGraphExec_t> graphs;  // key: steps, variant (-1: resident)
   std::string err = "no error";
 };
 
@@ -500,6 +678,7 @@ BatchArgs make_batch_args(lbm_batch* b) {
   A.st = b->st;
   A.plane = b->plane;
   A.nitems = b->nitems;
+  A.ntubes = b->ntubes;
   A.skip_block = b->skip_block;
   A.skip_step = b->skip_step;
   A.spin_cycles = b->spin_cycles;
@@ -523,6 +702,57 @@ int launch_tubes(lbm_batch* b, long long nsteps) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   BCK(b, cudaLaunchKernelExC(&cfg, (const void*)V.fn, args));
+  return LBM_OK;
+}
+
+// Groups the tubes for the resident form.
+int build_groups(lbm_batch* b) {
+  if (*std::max_element(b->nx.begin(), b->nx.end()) > RESIDENT_MAX_NX) return LBM_OK;
+  std::vector<int> order(b->ntubes);
+  for (int t = 0; t < b->ntubes; ++t) order[t] = t;
+  std::stable_sort(order.begin(), order.end(), [&](int p, int q) { return b->nx[p] > b->nx[q]; });
+  const bool few = b->ntubes <= b->sms;  // a tube per SM: as many threads as it has pairs
+  for (int k = 0; k < b->ntubes; ++k) {
+    const int nx = b->nx[order[k]];
+    const int threads = nx <= 256 ? 128 : nx <= 512 ? (few ? 256 : 128) : (few ? 512 : 256);
+    if (b->groups.empty() || (b->groups.back().nx_max - 1) / RESIDENT_STEP != (nx - 1) / RESIDENT_STEP ||
+        b->groups.back().threads != threads)
+      b->groups.push_back({k, 0, nx, threads});
+    ++b->groups.back().count;
+  }
+  for (int th : {128, 256, 512})
+    BCK(b, cudaFuncSetAttribute((const void*)resident_fn(th), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)resident_smem(RESIDENT_MAX_NX)));
+  BCK(b, cudaMalloc((void**)&b->order, sizeof(int) * b->ntubes));
+  BCK(b, cudaMemcpyAsync(b->order, order.data(), sizeof(int) * b->ntubes, cudaMemcpyHostToDevice, b->stream));
+  for (size_t k = 0; k < b->groups.size(); ++k) {
+    cudaEvent_t ev;
+    BCK(b, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    b->joins.push_back(ev);
+    if (k == 0) continue;
+    cudaStream_t st;
+    BCK(b, cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+    b->side.push_back(st);
+  }
+  BCK(b, cudaStreamSynchronize(b->stream));
+  return LBM_OK;
+}
+
+// The resident launches of nsteps steps: one per group, on branches of the
+// batch's stream, so that blocks of different groups share the SMs.
+int launch_resident(lbm_batch* b, long long nsteps) {
+  const BatchArgs A = make_batch_args(b);
+  if (b->groups.size() > 1) BCK(b, cudaEventRecord(b->joins[0], b->stream));
+  for (size_t k = 0; k < b->groups.size(); ++k) {
+    const TubeGroup& G = b->groups[k];
+    const cudaStream_t st = k == 0 ? b->stream : b->side[k - 1];
+    if (k > 0) BCK(b, cudaStreamWaitEvent(st, b->joins[0], 0));
+    resident_fn(G.threads)<<<G.count, G.threads, resident_smem(G.nx_max), st>>>(
+        b->f[0], b->f[1], A, b->order + G.first, nsteps);
+    BCK(b, cudaGetLastError());
+    if (k > 0) BCK(b, cudaEventRecord(b->joins[k], st));
+  }
+  for (size_t k = 1; k < b->groups.size(); ++k) BCK(b, cudaStreamWaitEvent(b->stream, b->joins[k], 0));
   return LBM_OK;
 }
 
@@ -639,7 +869,7 @@ int lbm_batch_create(const lbm_batch_config* cfg, void* cuda_stream, lbm_batch**
     lbm_batch_destroy(b);
     return rc;
   }
-  if (build_items(b) != LBM_OK || reset_batch_status(b) != LBM_OK) {
+  if (build_items(b) != LBM_OK || build_groups(b) != LBM_OK || reset_batch_status(b) != LBM_OK) {
     g_batch_create_error = b->err;
     lbm_batch_destroy(b);
     return LBM_ERR_CUDA;
@@ -680,12 +910,13 @@ int lbm_batch_step(lbm_batch* b, long long nsteps) {
   snprintf(range, sizeof(range), "lbm_batch_step n=%lld (graph)", nsteps);
   nvtxRangePushA(range);
   struct Pop { ~Pop() { nvtxRangePop(); } } pop;
-  auto key = std::make_pair(nsteps, b->variant);
+  const bool resident = !b->streamed && !b->groups.empty() && nsteps >= RESIDENT_MIN_STEPS;
+  auto key = std::make_pair(nsteps, resident ? -1 : b->variant);
   auto it = b->graphs.find(key);
   if (it == b->graphs.end()) {
     cudaGraph_t g;
     BCK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-    const int rc = launch_tubes(b, nsteps);
+    const int rc = resident ? launch_resident(b, nsteps) : launch_tubes(b, nsteps);
     cudaError_t e = cudaStreamEndCapture(b->stream, &g);
     if (rc != LBM_OK) return rc;
     if (e != cudaSuccess) return bcuda(b, e, "cudaStreamEndCapture");
@@ -765,6 +996,7 @@ int lbm_batch_set_tiling(lbm_batch* b, int tile, int threads) {
   if (k < 0) return bfail(b, LBM_ERR_INVALID, "unsupported (tile, threads)");
   // keep the populations: items only change the work split, not the layout
   b->variant = k;
+  b->streamed = true;
   return build_items(b);
 }
 
@@ -801,7 +1033,9 @@ int lbm_batch_autotune(lbm_batch* b, int trial_steps, const char* cache_path, in
         int tl = 0, th = 0;
         if (sscanf(text.c_str() + at + pat.size(), "%d, %d", &tl, &th) == 2 &&
             find_variant(tl, th) >= 0) {
-          const int rc = lbm_batch_set_tiling(b, tl, th);
+          b->variant = find_variant(tl, th);
+          b->streamed = false;
+          const int rc = build_items(b);
           if (rc != LBM_OK) return rc;
           if (chosen) { chosen[0] = tl; chosen[1] = th; }
           return LBM_OK;
@@ -855,6 +1089,7 @@ int lbm_batch_autotune(lbm_batch* b, int trial_steps, const char* cache_path, in
   if (rc != LBM_OK) return rc;
   if (best < 0) return bfail(b, LBM_ERR_TIMEOUT, "no tiling candidate completed");
   b->variant = best;
+  b->streamed = false;
   if ((rc = build_items(b)) != LBM_OK) return rc;
   if (chosen) { chosen[0] = VARIANTS[best].tile; chosen[1] = VARIANTS[best].threads; }
   if (cache_path) {
@@ -919,6 +1154,9 @@ int lbm_batch_destroy(lbm_batch* b) {
     if (b->f[k]) cudaFree(b->f[k]);
   if (b->tubes) cudaFree(b->tubes);
   if (b->items) cudaFree(b->items);
+  if (b->order) cudaFree(b->order);
+  for (cudaStream_t st : b->side) cudaStreamDestroy(st);
+  for (cudaEvent_t ev : b->joins) cudaEventDestroy(ev);
   if (b->ghost) cudaFree(b->ghost);
   if (b->bad) cudaFree(b->bad);
   if (b->st) cudaFree(b->st);
