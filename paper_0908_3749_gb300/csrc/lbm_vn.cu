@@ -6,17 +6,15 @@
 //   (d2v16::transform / conserved / collide) at f = f^eq(state); the
 //   derivative part of the result is column j of the collision Jacobian
 //   d(Delta f^coll)/df = -dt M^-1 S_hat (M - dfhat^eq/df) of Sec. IV.
-// k_vn_eig: 16 threads per matrix (8 matrices per 128-thread block, each in
-//   shared memory). G = diag(Lax-Wendroff symbol of Eq. A.1) + Jacobian, then
-//   Householder reduction to upper Hessenberg form and explicit single-shift
-//   complex QR sweeps (Wilkinson shift from the trailing 2 x 2 block,
-//   exceptional shifts after 10 and 20 sweeps without deflation, deflation
-//   where |h_{l,l-1}| <= u (|h_{l-1,l-1}| + |h_{l,l}|), u = 2^-52), the
-//   textbook complex Schur iteration (Golub and Van Loan, Matrix
+// k_vn_eig: L = 4, 8 or 16 threads per matrix (32 / L matrices per warp, a warp
+//   per block, the matrices in shared memory). G = diag(Lax-Wendroff symbol of
+//   Eq. A.1) + Jacobian, then Householder reduction to upper Hessenberg form
+//   and explicit single-shift complex QR sweeps (Wilkinson shift from the
+//   trailing 2 x 2 block, exceptional shifts after 10 and 20 sweeps without
+//   deflation, deflation where |h_{l,l-1}| <= u (|h_{l-1,l-1}| + |h_{l,l}|), u =
+//   2^-52), the textbook complex Schur iteration (Golub and Van Loan, Matrix
 //   Computations, Secs. 7.4-7.5), in FP64. Every loop is bounded; a matrix
 //   that does not converge within 30 x 16 sweeps gets NaN results.
-// The 16 threads of a matrix synchronise with __syncwarp on their own
-// half-warp mask, so the two matrices of a warp proceed independently.
 
 #include <cuda_runtime.h>
 
@@ -73,8 +71,6 @@ struct LW {
   double a0[16], aE[16], aW[16], aN[16], aS[16];
 };
 
-constexpr int VN_T = 128;           // threads per eigen block
-constexpr int MPB = VN_T / 16;      // matrices per block
 constexpr int SWEEPS_PER_EIG = 30;  // average QR sweeps allowed per eigenvalue
 
 __global__ void __launch_bounds__(16) k_vn_jacobian(const lbm_vn_case* cases, const Coeffs<double> base,
@@ -129,263 +125,388 @@ __device__ __forceinline__ cplx conj(cplx a) { return mk(a.re, -a.im); }
 __device__ __forceinline__ double cabs(cplx a) { return hypot(a.re, a.im); }
 __device__ __forceinline__ double cabs1(cplx a) { return fabs(a.re) + fabs(a.im); }
 __device__ __forceinline__ double norm2(cplx a) { return a.re * a.re + a.im * a.im; }
-// a / b by scaling with the larger component of b (Smith's method).
-__device__ __forceinline__ cplx cdiv(cplx a, cplx b) {
-  if (fabs(b.re) >= fabs(b.im)) {
-    const double r = b.im / b.re, den = b.re + b.im * r;
-    return mk((a.re + a.im * r) / den, (a.im - a.re * r) / den);
-  }
-  const double r = b.re / b.im, den = b.im + b.re * r;
-  return mk((a.re * r + a.im) / den, (a.im * r - a.re) / den);
+// 1 / sqrt(x) for positive normal x: the hardware's approximation y and one
+// third-order step of the series of (1 - e)^(-1/2), e = 1 - x y^2: y (1 + e / 2
+// + 3 e^2 / 8), which leaves e^3 (below 2^-60): five FP64 operations.
+__device__ __forceinline__ double rsq(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
 }
-// Principal square root: for z = x + i y, |z| = r, sqrt z = (t, y / (2 t)) with
-// t = sqrt((r + x) / 2) when x >= 0, else (|y| / (2 t), sign(y) t) with
-// t = sqrt((r - x) / 2).
+__device__ __forceinline__ bool is_zero(double x) {  // without the FP64 units
+  return ((__double2hiint(x) & 0x7fffffff) | __double2loint(x)) == 0;
+}
+// The solver scales its matrix to entries below 2 in magnitude, so squares
+// cannot overflow; below TINY they may underflow.
+constexpr double TINY = 0x1p-900;
+// Principal square root of z = x + i y, |z| = r: t = sqrt((r + |x|) / 2),
+// (t, y / (2 t)) when x >= 0, else (|y| / (2 t), sign(y) t); 0 for |z|^2 <
+// TINY. Used for shifts only, which may be guesses.
 __device__ __forceinline__ cplx csqrt(cplx z) {
-  const double r = cabs(z);
-  if (r == 0.0) return mk(0.0, 0.0);
-  if (z.re >= 0.0) {
-    const double t = sqrt(0.5 * (r + z.re));
-    return mk(t, z.im / (2.0 * t));
-  }
-  const double t = sqrt(0.5 * (r - z.re));
-  return mk(fabs(z.im) / (2.0 * t), copysign(t, z.im));
+  const double n2 = norm2(z);
+  if (!(n2 >= TINY)) return mk(0.0, 0.0);
+  const double u = 0.5 * fma(n2, rsq(n2), fabs(z.re));
+  const double iu = rsq(u), t = u * iu, o = 0.5 * z.im * iu;
+  return z.re >= 0.0 ? mk(t, o) : mk(fabs(o), copysign(t, z.im));
 }
 // Givens rotation G = [[c, s], [-conj(s), c]], c real, with G (a, b)^T = (r, 0)^T:
-// c = |a| / n, s = (a / |a|) conj(b) / n, r = (a / |a|) n, n^2 = |a|^2 + |b|^2,
-// from two reciprocal square roots. The solver scales its matrix to entries
-// below 2 in magnitude first, so the squares cannot overflow.
+// c = |a| / n, s = a conj(b) / (|a| n), r = a n / |a|, n^2 = |a|^2 + |b|^2: all
+// from w = 1 / (|a| n), one reciprocal square root.
 __device__ __forceinline__ void givens(cplx a, cplx b, double& c, cplx& s, cplx& r) {
-  const double na2 = norm2(a), nb2 = norm2(b);
-  if (nb2 == 0.0) {
+  const double na2 = norm2(a), nb2 = norm2(b), n2 = na2 + nb2;
+  const double q = na2 * n2;
+  if (__double2hiint(q) >= __double2hiint(TINY)) {
+    const double w = rsq(q);
+    c = na2 * w;
+    s = w * (a * conj(b));
+    r = (n2 * w) * a;
+    return;
+  }
+  // |a| n is tiny or not a number: the rotation from the components' norms
+  const double aa = cabs(a), ab = cabs(b);
+  if (ab == 0.0) {
     c = 1.0;
     s = mk(0.0, 0.0);
     r = a;
-    return;
-  }
-  if (na2 == 0.0) {
-    const double ib = rsqrt(nb2);
+  } else if (aa == 0.0) {
     c = 0.0;
-    s = ib * conj(b);
-    r = mk(nb2 * ib, 0.0);
-    return;
+    s = (1.0 / ab) * conj(b);
+    r = mk(ab, 0.0);
+  } else {
+    const double n = hypot(aa, ab);
+    const cplx ph = (1.0 / aa) * a;
+    c = aa / n;
+    s = ph * ((1.0 / n) * conj(b));
+    r = n * ph;
   }
-  const double n2 = na2 + nb2;
-  const double inv = rsqrt(n2), ia = rsqrt(na2);
-  const cplx ph = ia * a;  // a / |a|
-  c = na2 * ia * inv;
-  s = inv * (ph * conj(b));
-  r = (n2 * inv) * ph;
 }
 
+// One matrix in shared memory. Rows are one element (16 bytes) longer than the
+// matrix, so that neighbouring rows start in different banks, and the whole is
+// 64 bytes past a multiple of 512, so that the threads of a warp that access
+// the same element of their matrices do too.
 struct EigWork {
-  cplx A[16][16];
+  cplx A[16][17];
   cplx v[16];      // Householder vector
-  cplx rs[16];     // Givens sines of the current sweep
-  double rc[16];   // Givens cosines
-  double norm;     // max |a_ij|_1 after the reduction
-  double scale;    // power of two the matrix was divided by
-  int finite;
+  cplx pad[36];
 };
+static_assert(sizeof(EigWork) % 512 == 64, "bank offset between matrices");
 
-// Eigenvalues of W.A by the 16 lanes in `mask` (lane l = 0..15 of them). On
-// a true return the eigenvalues are W.A's diagonal (scaled back). Every lane
-// returns the same value.
-__device__ bool eig16(EigWork& W, int l, unsigned mask, int base) {
+// FP64 instructions of a warp cost the same whatever its number of active
+// threads (19 clocks per SM, and 64 between two of one warp), so a warp runs
+// its matrices in step: loops have bounds common to the warp, with the
+// matrices' own ranges as conditions inside.
+constexpr unsigned FULL = 0xffffffffu;
+__device__ __forceinline__ int warp_max(int v) { return __reduce_max_sync(FULL, v); }
+__device__ __forceinline__ int warp_min(int v) { return __reduce_min_sync(FULL, v); }
+__device__ __forceinline__ int exponent(double x) { return __double2hiint(x) >> 20 & 0x7ff; }
+template <int L>
+__device__ __forceinline__ int group_max(int v) {
+#pragma unroll
+  for (int o = L / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(FULL, v, o));
+  return v;
+}
+
+// Eigenvalues of W.A by the L threads of a group (thread l0 = 0 .. L - 1 of it,
+// rows and columns l0, l0 + L, ...). On a true return (the same in the group)
+// the eigenvalues are W.A's diagonal. Every thread of the warp calls it;
+// `active` is false for groups without a matrix.
+template <int L>
+__device__ bool eig16(EigWork& W, int l0, bool active) {
   constexpr double U = 2.220446049250313e-16;  // 2^-52
-  __syncwarp(mask);
-  if (l == 0) {
-    int fin = 1;
-    double amax = 0.0;
-    for (int i = 0; i < 256; ++i) {
-      const cplx a = W.A[i >> 4][i & 15];
-      fin &= isfinite(a.re) && isfinite(a.im);
-      amax = fmax(amax, fmax(fabs(a.re), fabs(a.im)));
+  constexpr int N = 16 / L;                    // rows and columns per thread
+  __syncwarp();
+  // Largest exponent of an entry (as the high words' bits) and whether any is
+  // non-zero, without the FP64 units.
+  int top = 0;
+  unsigned any = 0;
+  for (int j = 0; j < N; ++j)
+    for (int i = 0; i < 16; ++i) {
+      const cplx a = W.A[l0 + L * j][i];
+      const int hr = __double2hiint(a.re) & 0x7fffffff, hm = __double2hiint(a.im) & 0x7fffffff;
+      top = max(top, max(hr, hm));
+      any |= hr | hm | __double2loint(a.re) | __double2loint(a.im);
     }
-    W.finite = fin;
-    // 2^e with amax / 2^e in [1, 2): an exact scaling (e clamped so that
-    // 2^-e stays a normal number)
-    W.scale = (fin && amax > 0.0) ? ldexp(1.0, max(-1000, min(1000, ilogb(amax)))) : 1.0;
-  }
-  __syncwarp(mask);
-  if (!W.finite) return false;
-  {
-    const double inv_scale = 1.0 / W.scale;  // a power of two: exact
-    for (int j = 0; j < 16; ++j) W.A[l][j] = inv_scale * W.A[l][j];
-  }
+  top = group_max<L>(top);
+  any = (unsigned)group_max<L>(any != 0);
+  const bool finite = top < 0x7ff00000;
+  // 2^e with the largest component / 2^e in [1, 2): an exact scaling (e
+  // clamped so that 2^-e stays a normal number)
+  const int e = any ? max(-1000, min(1000, (top >> 20) - 1023)) : 0;
+  const double scale = __hiloint2double((1023 + e) << 20, 0);
+  const double inv_scale = __hiloint2double((1023 - e) << 20, 0);
+  active = active && finite;
+  for (int j = 0; j < N; ++j)
+    for (int i = 0; i < 16; ++i) W.A[l0 + L * j][i] = inv_scale * W.A[l0 + L * j][i];
 
   // Householder reduction to upper Hessenberg form: A <- H A H, H = I - tau v v^H.
+#pragma unroll 1
   for (int c = 0; c < 14; ++c) {
-    __syncwarp(mask);
+    __syncwarp();
     double tail = 0.0;
+#pragma unroll 1
     for (int i = c + 2; i < 16; ++i) tail += norm2(W.A[i][c]);
-    if (tail == 0.0) continue;  // the same decision in every lane
+    // Entries below 2^-450 beside ones of order 1 are left where they are (they
+    // are not read again). The same decision in the group.
+    const bool doit = tail >= TINY;
     const cplx x0 = W.A[c + 1][c];
-    const double ax0 = cabs(x0);
-    const double sigma = sqrt(ax0 * ax0 + tail);
-    const cplx ph = ax0 > 0.0 ? (1.0 / ax0) * x0 : mk(1.0, 0.0);
-    const cplx alpha = -(sigma * ph);
-    const double tau = 1.0 / (sigma * (sigma + ax0));
-    if (l >= c + 1) W.v[l] = l == c + 1 ? (ax0 + sigma) * ph : W.A[l][c];
-    __syncwarp(mask);
-    if (l == c) {
-      W.A[c + 1][c] = alpha;
-      for (int i = c + 2; i < 16; ++i) W.A[i][c] = mk(0.0, 0.0);
-    } else if (l > c) {  // column l: A[:, l] -= tau v (v^H A[:, l])
-      cplx w = mk(0.0, 0.0);
-      for (int i = c + 1; i < 16; ++i) w = w + conj(W.v[i]) * W.A[i][l];
-      w = tau * w;
-      for (int i = c + 1; i < 16; ++i) W.A[i][l] = W.A[i][l] - W.v[i] * w;
+    const double n0 = norm2(x0);
+    const double i0 = rsq(n0);
+    const bool phase = n0 >= TINY;
+    const double ax0 = phase ? n0 * i0 : 0.0;
+    const cplx ph = phase ? i0 * x0 : mk(1.0, 0.0);
+    const double s2 = n0 + tail, sigma = s2 * rsq(s2);
+    const double tau = d2v16::recip(fma(sigma, ax0, s2));
+    for (int j = 0; j < N; ++j) {
+      const int l = l0 + L * j;
+      if (l >= c + 1) W.v[l] = l == c + 1 ? (ax0 + sigma) * ph : W.A[l][c];
     }
-    __syncwarp(mask);
-    {  // row l: A[l, :] -= tau (A[l, :] v) v^H
-      cplx z = mk(0.0, 0.0);
-      for (int j = c + 1; j < 16; ++j) z = z + W.A[l][j] * W.v[j];
-      z = tau * z;
-      for (int j = c + 1; j < 16; ++j) W.A[l][j] = W.A[l][j] - z * conj(W.v[j]);
+    __syncwarp();
+    if (doit) {
+#pragma unroll 1
+      for (int j = (c + 1) / L; j < N; ++j) {  // column l: A[:, l] -= tau v (v^H A[:, l])
+        const int l = l0 + L * j;
+        if (l > c) {
+          cplx w = mk(0.0, 0.0);
+#pragma unroll 1
+          for (int i = c + 1; i < 16; ++i) w = w + conj(W.v[i]) * W.A[i][l];
+          w = tau * w;
+#pragma unroll 1
+          for (int i = c + 1; i < 16; ++i) W.A[i][l] = W.A[i][l] - W.v[i] * w;
+        }
+      }
+      for (int j = 0; j < N; ++j) {
+        const int l = l0 + L * j;
+        if (l == c + 1) W.A[l][c] = -(sigma * ph);
+        else if (l > c + 1) W.A[l][c] = mk(0.0, 0.0);
+      }
+    }
+    __syncwarp();
+    if (doit) {
+#pragma unroll 1
+      for (int j = 0; j < N; ++j) {  // row l: A[l, :] -= tau (A[l, :] v) v^H
+        const int l = l0 + L * j;
+        cplx z = mk(0.0, 0.0);
+#pragma unroll 1
+        for (int i = c + 1; i < 16; ++i) z = z + W.A[l][i] * W.v[i];
+        z = tau * z;
+#pragma unroll 1
+        for (int i = c + 1; i < 16; ++i) W.A[l][i] = W.A[l][i] - z * conj(W.v[i]);
+      }
     }
   }
-  __syncwarp(mask);
-  if (l == 0) {
-    double nrm = 0.0;
-    for (int i = 0; i < 256; ++i) nrm = fmax(nrm, cabs1(W.A[i >> 4][i & 15]));
-    W.norm = nrm;
-  }
-  __syncwarp(mask);
-  const double nrm = W.norm;
+  __syncwarp();
+  // max |a_ij|_1, as the bits of a non-negative double (their order as
+  // integers): the deflation reference of a zero diagonal.
+  long long nb = 0;
+  for (int j = 0; j < N; ++j)
+    for (int i = 0; i < 16; ++i) nb = max(nb, __double_as_longlong(cabs1(W.A[l0 + L * j][i])));
+#pragma unroll
+  for (int o = L / 2; o > 0; o >>= 1) nb = max(nb, __shfl_xor_sync(FULL, nb, o));
+  const double nrm = __longlong_as_double(nb);
 
   // Shifted QR sweeps on the active block [lo, hi].
-  int hi = 15, its = 0, total = 0;
-  while (hi > 0) {
-    if (total >= SWEEPS_PER_EIG * 16) return false;
-    __syncwarp(mask);
-    bool small = false;
-    if (l >= 1 && l <= hi) {
-      double ref = cabs1(W.A[l - 1][l - 1]) + cabs1(W.A[l][l]);
-      if (ref == 0.0) ref = nrm;
-      small = cabs1(W.A[l][l - 1]) <= U * ref;
+  int hi = active ? 15 : 0, its = 0, total = 0, lo = 0;
+  bool converged = active;
+#pragma unroll 1
+  while (true) {
+    // Deflate until every unfinished matrix has an active block of two or more.
+#pragma unroll 1
+    while (true) {
+      __syncwarp();
+      int best = 0;
+      unsigned small = 0;
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        const int l = l0 + L * j;
+        // An entry within 2^-48 of the largest component on the diagonal (by
+        // exponents, off the FP64 units) is not small; the others are looked at.
+        bool look = false;
+        if (l >= 1 && l <= hi) {
+          const cplx p = W.A[l - 1][l - 1], q = W.A[l][l], o = W.A[l][l - 1];
+          const int ed = max(max(exponent(p.re), exponent(p.im)), max(exponent(q.re), exponent(q.im)));
+          look = max(exponent(o.re), exponent(o.im)) <= ed - 48 || ed == 0;
+        }
+        if (!__any_sync(FULL, look)) continue;
+        if (look) {
+          double ref = cabs1(W.A[l - 1][l - 1]) + cabs1(W.A[l][l]);
+          if (is_zero(ref)) ref = nrm;
+          if (cabs1(W.A[l][l - 1]) <= U * ref) {
+            best = l;
+            small |= 1u << j;
+          }
+        }
+      }
+      lo = group_max<L>(best);
+      __syncwarp();
+#pragma unroll
+      for (int j = 0; j < N; ++j)
+        if (small >> j & 1u) W.A[l0 + L * j][l0 + L * j - 1] = mk(0.0, 0.0);
+      const bool deflated = hi > 0 && lo == hi;
+      if (deflated) {
+        --hi;
+        its = 0;
+      }
+      if (!__any_sync(FULL, deflated)) break;
     }
-    const unsigned bits = (__ballot_sync(mask, small) >> base) & ((2u << hi) - 1u);
-    const int lo = bits ? 31 - __clz(bits) : 0;
-    __syncwarp(mask);
-    if (small) W.A[l][l - 1] = mk(0.0, 0.0);
-    if (lo == hi) {
-      --hi;
-      its = 0;
-      continue;
+    if (hi > 0 && total >= SWEEPS_PER_EIG * 16) {
+      converged = false;
+      hi = 0;
     }
-    __syncwarp(mask);
-    cplx mu;
-    const cplx d = W.A[hi][hi], sub = W.A[hi][hi - 1];
-    if (its == 10 || its == 20) {
-      mu = mk(d.re + 0.75 * fabs(sub.re), d.im);
-    } else {
+    if (!__any_sync(FULL, hi > 0)) break;
+    __syncwarp();
+    const bool run = hi > 0;
+    cplx mu = mk(0.0, 0.0);
+    if (run) {
+      const cplx d = W.A[hi][hi], sub = W.A[hi][hi - 1];
       // Eigenvalue of [[a, b], [sub, d]] nearer d: d + h -+ sqrt(h^2 + b sub),
       // h = (a - d)/2, written as d - b sub / (h +- sqrt(...)) with the larger
-      // denominator (no cancellation).
+      // denominator (no cancellation); where that is nearly nothing, d.
       const cplx a = W.A[hi - 1][hi - 1], b = W.A[hi - 1][hi];
       const cplx h = 0.5 * (a - d);
       const cplx bc = b * sub;
       const cplx r = csqrt(h * h + bc);
       const cplx den = (h.re * r.re + h.im * r.im) >= 0.0 ? h + r : h - r;
-      mu = cabs1(den) > 0.0 ? d - cdiv(bc, den) : d;
+      const double n2 = norm2(den);
+      mu = n2 >= TINY ? d - d2v16::recip(n2) * (bc * conj(den)) : d;
+      if (its == 10 || its == 20) mu = mk(d.re + 0.75 * fabs(sub.re), d.im);
     }
-    __syncwarp(mask);
-    if (l >= lo && l <= hi) W.A[l][l] = W.A[l][l] - mu;
-    for (int k = lo; k < hi; ++k) {  // H - mu I = Q R, rows rotated in turn
-      __syncwarp(mask);
-      double c;
-      cplx s, r;
-      givens(W.A[k][k], W.A[k + 1][k], c, s, r);
-      __syncwarp(mask);
-      if (l == k) {
-        W.A[k][k] = r;
-        W.A[k + 1][k] = mk(0.0, 0.0);
-      } else if (l > k && l <= hi) {
-        const cplx x = W.A[k][l], y = W.A[k + 1][l];
-        W.A[k][l] = c * x + s * y;
-        W.A[k + 1][l] = c * y - conj(s) * x;
-      }
-      if (l == 0) {
-        W.rc[k] = c;
-        W.rs[k] = s;
-      }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const int l = l0 + L * j;
+      if (run && l >= lo && l <= hi) W.A[l][l] = W.A[l][l] - mu;
     }
-    __syncwarp(mask);
-    for (int k = lo; k < hi; ++k) {  // R Q: columns rotated in turn, lane = row
-      if (l >= lo && l <= k + 1 && l <= hi) {
-        const double c = W.rc[k];
-        const cplx s = W.rs[k];
-        const cplx x = W.A[l][k], y = W.A[l][k + 1];
-        W.A[l][k] = c * x + conj(s) * y;
-        W.A[l][k + 1] = c * y - s * x;
+    // H - mu I = Q R, rows k, k + 1 rotated in turn; R Q: columns k - 1, k
+    // rotated one turn later, once row k is final (their rows end at k).
+    const int k0 = warp_min(run ? lo : 16), k1 = warp_max(run ? hi : 0);
+    double cp = 1.0;  // the previous rotation
+    cplx sp = mk(0.0, 0.0);
+#pragma unroll 1
+    for (int k = k0; k <= k1; ++k) {
+      __syncwarp();
+      const bool rot = run && k >= lo && k < hi;       // a rotation of rows k, k + 1
+      const bool col = run && k > lo && k <= hi;       // columns k - 1, k
+      double c = 1.0;
+      cplx s = mk(0.0, 0.0), r = mk(0.0, 0.0);
+      if (rot) givens(W.A[k][k], W.A[k + 1][k], c, s, r);
+      __syncwarp();
+#pragma unroll 1
+      for (int j = k / L; j <= k1 / L; ++j) {
+        const int l = l0 + L * j;
+        if (rot && l > k && l <= hi) {
+          const cplx x = W.A[k][l], y = W.A[k + 1][l];
+          W.A[k][l] = c * x + s * y;
+          W.A[k + 1][l] = c * y - conj(s) * x;
+        } else if (rot && l == k) {
+          W.A[k][k] = r;
+          W.A[k + 1][k] = mk(0.0, 0.0);
+        }
       }
+      __syncwarp();
+#pragma unroll 1
+      for (int j = k0 / L; j <= k / L; ++j) {
+        const int l = l0 + L * j;
+        if (col && l >= lo && l <= k) {
+          const cplx x = W.A[l][k - 1], y = W.A[l][k];
+          W.A[l][k - 1] = cp * x + conj(sp) * y;
+          W.A[l][k] = cp * y - sp * x;
+        }
+      }
+      cp = c;
+      sp = s;
     }
-    __syncwarp(mask);
-    if (l >= lo && l <= hi) W.A[l][l] = W.A[l][l] + mu;
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const int l = l0 + L * j;
+      if (run && l >= lo && l <= hi) W.A[l][l] = W.A[l][l] + mu;
+    }
     ++its;
     ++total;
   }
-  __syncwarp(mask);
-  W.A[l][l] = W.scale * W.A[l][l];
-  __syncwarp(mask);
-  return true;
+  __syncwarp();
+  for (int j = 0; j < N; ++j) W.A[l0 + L * j][l0 + L * j] = scale * W.A[l0 + L * j][l0 + L * j];
+  __syncwarp();
+  return converged;
 }
 
 // Input modes of k_vn_eig.
 enum { SRC_VN = 0, SRC_MATRIX = 1 };
 
-// One matrix per 16 threads. SRC_VN: G of item (case, wave vector) from the
+// One matrix per L threads. SRC_VN: G of item (case, wave vector) from the
 // case's collision Jacobian and the Lax-Wendroff symbol; writes G if Gout,
 // else solves. SRC_MATRIX: the item's input matrix.
-__global__ void __launch_bounds__(VN_T) k_vn_eig(int src, long long nitems, int nk,
-                                                 const double* __restrict__ Jc,
-                                                 const double* __restrict__ kvec, LW lw, double dx,
-                                                 double dy, const double* __restrict__ Ain,
-                                                 double* Gout, double* omega, double* radius,
-                                                 unsigned long long* failed) {
-  __shared__ EigWork work[MPB];
-  const int half = threadIdx.x >> 4, l = threadIdx.x & 15;
-  const long long item = (long long)blockIdx.x * MPB + half;
-  if (item >= nitems) return;  // the whole half-warp leaves together
-  const int base = (threadIdx.x & 31) & ~15;
-  const unsigned mask = 0xFFFFu << base;
-  EigWork& W = work[half];
-  if (src == SRC_VN) {
+//
+// Bound by the FP64 units. With 8 matrices per warp (L = 4) the scalar part of
+// each rotation and shift serves 8 matrices and few threads idle: 3.2 M matrices/s
+// on a map of 32 x 1024 (FP64 pipe 82 % busy); two per warp
+// (16 threads each, idle outside the active block, shifts and rotations
+// computed by all, the norms by one thread) 1.2 M. Rotations from one reciprocal
+// square root instead of two, shifts and reflections from reciprocal square roots
+// and the deflation test first by exponents: 11.5 -> 10.4 ms on that map.
+template <int L>
+__global__ void __launch_bounds__(32) k_vn_eig(int src, long long nitems, int nk,
+                                               const double* __restrict__ Jc,
+                                               const double* __restrict__ kvec, LW lw, double dx,
+                                               double dy, const double* __restrict__ Ain,
+                                               double* Gout, double* omega, double* radius,
+                                               unsigned long long* failed) {
+  constexpr int M = 32 / L;  // matrices per warp
+  __shared__ EigWork work[M];
+  const int grp = threadIdx.x / L, l0 = threadIdx.x % L;
+  const long long item = (long long)blockIdx.x * M + grp;
+  const bool have = item < nitems;
+  EigWork& W = work[grp];
+  if (!have) {
+    for (int i = l0; i < 256; i += L) W.A[i >> 4][i & 15] = mk(0.0, 0.0);
+  } else if (src == SRC_VN) {
     const long long c = item / nk;
     const int q = (int)(item - c * nk);
     const double* J = Jc + c * 256;
-    for (int i = l; i < 256; i += 16) W.A[i >> 4][i & 15] = mk(J[i], 0.0);
     double sx, cx, sy, cy;
     sincos(kvec[2 * q] * dx, &sx, &cx);
     sincos(kvec[2 * q + 1] * dy, &sy, &cy);
-    // a0 + aE e^{i tx} + aW e^{-i tx} + aN e^{i ty} + aS e^{-i ty}
-    const cplx diag = mk(lw.a0[l] + (lw.aE[l] + lw.aW[l]) * cx + (lw.aN[l] + lw.aS[l]) * cy,
-                         (lw.aE[l] - lw.aW[l]) * sx + (lw.aN[l] - lw.aS[l]) * sy);
-    __syncwarp(mask);
-    W.A[l][l] = W.A[l][l] + diag;
-    if (Gout) {
-      __syncwarp(mask);
-      double* g = Gout + item * 512;
-      for (int i = l; i < 256; i += 16) {
-        g[2 * i] = W.A[i >> 4][i & 15].re;
-        g[2 * i + 1] = W.A[i >> 4][i & 15].im;
+    for (int i = l0; i < 256; i += L) {
+      cplx a = mk(J[i], 0.0);
+      const int r = i >> 4;
+      if ((i & 15) == r) {
+        // a0 + aE e^{i tx} + aW e^{-i tx} + aN e^{i ty} + aS e^{-i ty}
+        const cplx diag = mk(lw.a0[r] + (lw.aE[r] + lw.aW[r]) * cx + (lw.aN[r] + lw.aS[r]) * cy,
+                             (lw.aE[r] - lw.aW[r]) * sx + (lw.aN[r] - lw.aS[r]) * sy);
+        a = a + diag;
       }
-      return;
+      W.A[r][i & 15] = a;
     }
   } else {
     const double* a = Ain + item * 512;
-    for (int i = l; i < 256; i += 16) W.A[i >> 4][i & 15] = mk(a[2 * i], a[2 * i + 1]);
+    for (int i = l0; i < 256; i += L) W.A[i >> 4][i & 15] = mk(a[2 * i], a[2 * i + 1]);
   }
-  const bool ok = eig16(W, l, mask, base);
-  const cplx w = ok ? W.A[l][l] : mk(nan(""), nan(""));
-  if (omega) {
-    omega[item * 32 + 2 * l] = w.re;
-    omega[item * 32 + 2 * l + 1] = w.im;
+  if (Gout) {
+    __syncwarp();
+    if (!have) return;
+    double* g = Gout + item * 512;
+    for (int i = l0; i < 256; i += L) {
+      g[2 * i] = W.A[i >> 4][i & 15].re;
+      g[2 * i + 1] = W.A[i >> 4][i & 15].im;
+    }
+    return;
   }
-  double r = ok ? cabs(w) : nan("");
-  for (int off = 8; off > 0; off >>= 1) r = fmax(r, __shfl_xor_sync(mask, r, off, 16));
-  if (l == 0) {
+  const bool ok = eig16<L>(W, l0, have);
+  double r = ok ? 0.0 : nan("");
+#pragma unroll 1
+  for (int l = l0; l < 16; l += L) {
+    const cplx w = ok ? W.A[l][l] : mk(nan(""), nan(""));
+    if (omega && have) {
+      omega[item * 32 + 2 * l] = w.re;
+      omega[item * 32 + 2 * l + 1] = w.im;
+    }
+    if (ok) r = fmax(r, cabs(w));
+  }
+#pragma unroll
+  for (int off = L / 2; off > 0; off >>= 1) r = fmax(r, __shfl_xor_sync(FULL, r, off));
+  if (l0 == 0 && have) {
     if (radius) radius[item] = ok ? r : nan("");
     if (!ok && failed) atomicAdd(failed, 1ull);
   }
@@ -461,7 +582,30 @@ int copy_out(void* host, const void* dev, size_t n, int on_device, cudaStream_t 
   return LBM_OK;
 }
 
-unsigned grid_of(long long nitems) { return (unsigned)((nitems + MPB - 1) / MPB); }
+// Threads per matrix: a warp's time grows with its matrices, so batches that
+// do not give every SM four warps (one per partition) take fewer matrices per
+// warp. Measured with 16 / 8 / 4 threads (before the last change): 1200 matrices
+// 1.36 / 1.61 / 2.10 ms, 1600 1.70 / 1.59 / 2.10, 2400 2.26 / 1.82 / 2.34, 4800 3.92 /
+// 2.76 / 2.44, 32768 23.9 / 15.7 / 11.5.
+int launch_eig(int src, long long nitems, int nk, const double* Jc, const double* kvec, const LW& lw,
+               double dx, double dy, const double* Ain, double* G, double* omega, double* radius,
+               unsigned long long* failed, cudaStream_t s) {
+  int dev = 0, sms = 0;
+  VCK(cudaGetDevice(&dev));
+  VCK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const long long warps = 4ll * sms;
+  auto grid = [&](int m) { return (unsigned)((nitems + m - 1) / m); };
+  if (nitems <= 2 * warps)
+    k_vn_eig<16><<<grid(2), 32, 0, s>>>(src, nitems, nk, Jc, kvec, lw, dx, dy, Ain, G, omega, radius, failed);
+  else if (nitems <= 4 * warps)
+    k_vn_eig<8><<<grid(4), 32, 0, s>>>(src, nitems, nk, Jc, kvec, lw, dx, dy, Ain, G, omega, radius, failed);
+  else
+    k_vn_eig<4><<<grid(8), 32, 0, s>>>(src, nitems, nk, Jc, kvec, lw, dx, dy, Ain, G, omega, radius, failed);
+  VCK(cudaGetLastError());
+  return LBM_OK;
+}
+// Items of one call: the grid of eight matrices per warp must stay below 2^31.
+bool too_many(long long nitems) { return (nitems + 7) / 8 > 0x7FFFFFFFLL; }
 
 // Shared body of lbm_vn_matrices (G != nullptr) and lbm_vn_spectrum.
 int vn_run(const lbm_vn_case* cases, int ncases, const double* k, int nk, double dx, double dy,
@@ -476,7 +620,7 @@ int vn_run(const lbm_vn_case* cases, int ncases, const double* k, int nk, double
     if ((rc = check_k(k, nk)) != LBM_OK) return rc;
   }
   const long long nitems = (long long)ncases * nk;
-  if ((nitems + MPB - 1) / MPB > 0x7FFFFFFFLL) return vfail(LBM_ERR_INVALID, "too many items");
+  if (too_many(nitems)) return vfail(LBM_ERR_INVALID, "too many items");
   Coeffs<double> K;
   if (!lattice_constants(K)) return vfail(LBM_ERR_CUDA, "singular lattice block");
   set_advection(K, dt, dx, dy);
@@ -510,10 +654,9 @@ int vn_run(const lbm_vn_case* cases, int ncases, const double* k, int nk, double
   }
   k_vn_jacobian<<<ncases, 16, 0, s>>>((const lbm_vn_case*)dcases, K, dt, (double*)bj.p);
   VCK(cudaGetLastError());
-  k_vn_eig<<<grid_of(nitems), VN_T, 0, s>>>(SRC_VN, nitems, nk, (const double*)bj.p,
-                                            (const double*)dk, lw, dx, dy, nullptr,
-                                            (double*)dG, (double*)dw, (double*)dr, dfail);
-  VCK(cudaGetLastError());
+  if ((rc = launch_eig(SRC_VN, nitems, nk, (const double*)bj.p, (const double*)dk, lw, dx, dy, nullptr,
+                       (double*)dG, (double*)dw, (double*)dr, dfail, s)) != LBM_OK)
+    return rc;
   if ((rc = copy_out(G, dG, sizeof(double) * 512 * (size_t)nitems, on_device, s)) ||
       (rc = copy_out(radius, dr, sizeof(double) * (size_t)nitems, on_device, s)) ||
       (rc = copy_out(omega, dw, sizeof(double) * 32 * (size_t)nitems, on_device, s)))
@@ -549,7 +692,7 @@ int lbm_eig16(const double* A, long long n, double* omega, double* radius, int o
               void* cuda_stream, long long* nonconverged) {
   if (n < 1 || !A) return vfail(LBM_ERR_INVALID, "need n >= 1 and A");
   if (!omega && !radius && !nonconverged) return vfail(LBM_ERR_INVALID, "no output requested");
-  if ((n + MPB - 1) / MPB > 0x7FFFFFFFLL) return vfail(LBM_ERR_INVALID, "too many matrices");
+  if (too_many(n)) return vfail(LBM_ERR_INVALID, "too many matrices");
   cudaStream_t s = (cudaStream_t)cuda_stream;
   DevBuf ba, bo, br, bf;
   const void* dA = nullptr;
@@ -567,10 +710,9 @@ int lbm_eig16(const double* A, long long n, double* omega, double* radius, int o
     VCK(cudaMemsetAsync(dfail, 0, sizeof(unsigned long long), s));
   }
   LW lw = {};
-  k_vn_eig<<<grid_of(n), VN_T, 0, s>>>(SRC_MATRIX, n, 1, nullptr, nullptr, lw, 1.0, 1.0,
-                                       (const double*)dA, nullptr, (double*)dw, (double*)dr,
-                                       dfail);
-  VCK(cudaGetLastError());
+  if ((rc = launch_eig(SRC_MATRIX, n, 1, nullptr, nullptr, lw, 1.0, 1.0, (const double*)dA, nullptr,
+                       (double*)dw, (double*)dr, dfail, s)) != LBM_OK)
+    return rc;
   if ((rc = copy_out(omega, dw, sizeof(double) * 32 * (size_t)n, on_device, s)) ||
       (rc = copy_out(radius, dr, sizeof(double) * (size_t)n, on_device, s)))
     return rc;
