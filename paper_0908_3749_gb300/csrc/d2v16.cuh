@@ -141,16 +141,15 @@ inline void fill_forward(Coeffs<R>& K) {
 // ---------------------------------------------------------------------------
 #ifdef __CUDACC__
 
-// Reciprocal. FP64: hardware approximation refined by two Newton-Raphson
-// steps r <- r + r (1 - x r) (quadratic convergence of Newton's method for
-// 1/x), within about one ulp; FP32: the hardware approximation.
+// Reciprocal. FP64: the hardware approximation r with one step of the series
+// 1/x = r (1 + e + e^2 + ...), e = 1 - x r, which leaves e^3 (the approximation's
+// error is about 2^-23), within about one ulp; FP32: the hardware
+// approximation.
 __device__ __forceinline__ double recip(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  double e = fma(-x, r, 1.0);
-  r = fma(r, e, r);
-  e = fma(-x, r, 1.0);
-  return fma(r, e, r);
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
 }
 __device__ __forceinline__ float recip(float x) {
   float r;
@@ -350,6 +349,100 @@ __device__ __forceinline__ R collide(const Coeffs<KT>& K, const Groups<R>& d,
   return collide_q(K, d, equilibria(c.rho, c.jx, c.jy, c.e), df);
 }
 
+// ---------------------------------------------------------------------------
+// The FP64 step's node: conserved moments and collision in fewer operations
+// ---------------------------------------------------------------------------
+// GB300 retires one FP64 instruction per warp and 19 clocks, so the FP64 step's
+// time is its number of FP64 instructions. This is the arithmetic of
+// conserved() and collide() with the forward blocks' structure used: scaled to
+// a leading 1, pairs of rows differ in one sign only,
+//   4 m11, m12 = (S0 + 1296 S1) +- 16 (S2 + 81/16 S3)
+//   2 m7,  m9  = (X0 + 216 X1) +- 4 sqrt2 (X2 + 27/8 X3)     (m8, -m10: Y)
+// the equilibria enter the deviations as fused multiply-adds, and e is carried
+// as 2 e. 224 FP64 instructions per node with the Lax-Wendroff terms, against
+// 259 and the checks' 6 (which are integer operations now). Deviations are
+// relaxed, as in collide(), so that what is conserved does not depend on the
+// rounding of the relaxation matrices. K's relaxation columns are those of
+// scale_relaxation().
+struct Node64 {
+  double rho, jx, jy, e2, p2;  // e2 = 2 e, p2 = 2 rho T
+};
+constexpr double R2 = SQ2, R2x4 = 4.0 * SQ2, R2x16 = 16.0 * SQ2;
+
+__device__ __forceinline__ Node64 collide64(const Coeffs<double>& K, const Groups<double>& d,
+                                            double df[16]) {
+  Node64 m;
+  m.rho = (d.S[0] + d.S[1]) + (d.S[2] + d.S[3]);
+  m.e2 = fma(9.0, d.S[3], fma(4.0, d.S[2], fma(36.0, d.S[1], d.S[0])));
+  m.jx = fma(R2, fma(1.5, d.X[3], d.X[2]), fma(6.0, d.X[1], d.X[0]));
+  m.jy = fma(R2, fma(1.5, d.Y[3], d.Y[2]), fma(6.0, d.Y[1], d.Y[0]));
+  const double r = recip(m.rho);
+  const double ux = m.jx * r, uy = m.jy * r;
+  const double a = m.jx * ux;
+  const double k2 = fma(m.jy, uy, a);       // rho u^2
+  const double m5 = fma(-m.jy, uy, a), m6 = m.jx * uy, m6x2 = m6 + m6;
+  m.p2 = m.e2 - k2;
+  const double h2 = m.e2 + m.p2;            // 2 (e + P)
+  const double er2 = m.e2 * r, usq = k2 * r;
+  const double nA = fma(-3.0, er2, usq + usq);  // -(6 e / rho - 2 u^2)
+  // 4 d11 = 4 m11 - (8 e^2 / rho - (rho u^2)^2 / rho), 1 d12
+  const double su = fma(1296.0, d.S[1], d.S[0]), sv = fma(5.0625, d.S[3], d.S[2]);
+  const double d11 = fma(k2, usq, fma(-(m.e2 + m.e2), er2, fma(16.0, sv, su)));
+  const double d12 = fma(-16.0, sv, su);
+  const double d5 = fma(36.0, d.C[1], d.C[0]) - m5;
+  const double d13 = fma(nA, m5, fma(1296.0, d.C[1], d.C[0]));
+  const double d6 = fma(-0.5, m6, fma(2.25, d.C[3], d.C[2]));                 // d6 / 2
+  const double d14 = fma(0.125 * nA, m6, fma(5.0625, d.C[3], d.C[2]));        // d14 / 8
+  const double xu = fma(216.0, d.X[1], d.X[0]), xv = fma(3.375, d.X[3], d.X[2]);
+  const double d7 = fma(-h2, ux, fma(R2x4, xv, xu));                          // 2 d7
+  const double d9 = fma(m6x2, uy, fma(-m5, ux, fma(-R2x4, xv, xu)));
+  const double d15 = fma(-R2x16, fma(7.59375, d.X[3], d.X[2]), fma(7776.0, d.X[1], d.X[0]));
+  const double yu = fma(216.0, d.Y[1], d.Y[0]), yv = fma(3.375, d.Y[3], d.Y[2]);
+  const double d8 = fma(-h2, uy, fma(R2x4, yv, yu));                          // 2 d8
+  const double d10 = fma(m6x2, ux, fma(m5, uy, fma(-R2x4, yv, yu)));          // -d10
+  const double d16 = fma(-R2x16, fma(7.59375, d.Y[3], d.Y[2]), fma(7776.0, d.Y[1], d.Y[0]));  // -d16
+  double S[4], C[4], X[4], Y[4];
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    S[g] = K.K0[g][0] * d11 + K.K0[g][1] * d12;
+    X[g] = K.KX[g][0] * d7 + K.KX[g][1] * d9 + K.KX[g][2] * d15;
+    Y[g] = K.KY[g][0] * d8 + K.KY[g][1] * d10 + K.KY[g][2] * d16;
+  }
+  C[0] = K.KC[0][0] * d5 + K.KC[0][1] * d13;
+  C[1] = K.KC[1][0] * d5 + K.KC[1][1] * d13;
+  C[2] = K.KS[0][0] * d6 + K.KS[0][1] * d14;
+  C[3] = K.KS[1][0] * d6 + K.KS[1][1] * d14;
+  inverse_transform(S, C, X, Y, df);
+  return m;
+}
+
+// Checks of FP64 values on the integer units.
+__device__ __forceinline__ bool positive64(double x) {  // x > 0 (false for NaN)
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  return hi >= 0 && ((unsigned)hi | lo) != 0u && (hi < 0x7ff00000 || (hi == 0x7ff00000 && lo == 0u));
+}
+__device__ __forceinline__ int magnitude64(double x) { return __double2hiint(x) & 0x7fffffff; }
+__device__ __forceinline__ bool finite64(double a, double b, double c, double d) {
+  return max(max(magnitude64(a), magnitude64(b)), max(magnitude64(c), magnitude64(d))) < 0x7ff00000;
+}
+
 #endif  // __CUDACC__
+
+// The relaxation columns of K for collide64, whose deviations carry factors
+// (exact powers of two, and the signs of the mirrored y rows).
+inline void scale_relaxation(Coeffs<double>& K) {
+  for (int g = 0; g < 4; ++g) {
+    K.K0[g][0] *= 0.25;
+    K.KX[g][0] *= 0.5;
+    K.KY[g][0] *= 0.5;
+    K.KY[g][1] = -K.KY[g][1];
+    K.KY[g][2] = -K.KY[g][2];
+  }
+  for (int r = 0; r < 2; ++r) {
+    K.KS[r][0] *= 2.0;
+    K.KS[r][1] *= 8.0;
+  }
+}
 
 }  // namespace d2v16

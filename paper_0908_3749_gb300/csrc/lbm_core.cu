@@ -269,6 +269,7 @@ template <typename R>
 StepArgs<R> make_args(lbm_ctx* c, int slot) {
   StepArgs<R> A;
   A.K = cast_coeffs<R>(c->Kd);
+  if constexpr (std::is_same<R, double>::value) scale_relaxation(A.K);
   if (std::is_same<R, dw>::value) A.K3 = third_words(c->Kd);
   else memset(&A.K3, 0, sizeof(A.K3));
   A.nx = c->cfg.nx;

@@ -36,7 +36,7 @@ __device__ __forceinline__ void load_tile(R* stage, const CUtensorMap* tmap, uns
   tma_load_tile(stage, tmap, x0 - HALO_X, y0 - 1, bar);
 }
 
-// Updates the nodes of tile `cur` from its copy in shared memory `stage`:
+// Updates the nodes of FP64 tile `cur` from its copy in shared memory `stage`:
 // group transforms, conserved moments, Eq. 14 equilibria, relaxation and
 // back-map, f (1 - cx^2 - cy^2) + collision + Lax-Wendroff neighbour terms,
 // store. Accumulates the watchdog flags; on audit steps writes the tile's
@@ -59,15 +59,16 @@ __device__ __forceinline__ void step_tile(const StepArgs<R>& A, const R* __restr
     for (int i = 0; i < 16; ++i) f[i] = ctr[i * PS];
     Groups<R> d;
     transform(f, d);
-    const Cons<R> m = conserved(A.K, d);
     R acc[16];
-    const R press = collide(A.K, d, m, acc);
+    const Node64 n = collide64(A.K, d, acc);
+    const Cons<R> m = {n.rho, n.jx, n.jy, R(0.5) * n.e2};  // e: boundary nodes and audits only
 #pragma unroll
     for (int i = 0; i < 16; ++i) acc[i] = A.K.a0[i] * f[i] + acc[i];
 
-    const bool b = !(m.rho > R(0)) || !isfinite(m.rho + m.jx + m.jy + m.e);
+    // (2 e for e: a state within a factor of two of the largest number is bad)
+    const bool b = !positive64(n.rho) || !finite64(n.rho, n.jx, n.jy, n.e2);
     bad |= b;
-    negT |= !b && !(press > R(0));
+    negT |= !b && !positive64(n.p2);
     mc[0] = m.rho; mc[1] = m.jx; mc[2] = m.jy; mc[3] = m.e;
     neighbour_terms<R, Off, BXP>(A, fin, ctr, PS, P, pitch, c, x, y, m, t, acc);
 #pragma unroll
