@@ -313,14 +313,12 @@ int launch_persistent(lbm_ctx* c, cudaStream_t s, int from, void* fout, const St
   const R* fi = (const R*)c->f[from];
   const CUtensorMap& tm = c->tmap[from];
   if (A.nblocks >= A.ntiles) {
-    if (c->wide) k_step<R, long long, VAR><<<A.ntiles, blk, 0, s>>>(tm, fi, (R*)fout, A);
-    else k_step<R, unsigned, VAR><<<A.ntiles, blk, 0, s>>>(tm, fi, (R*)fout, A);
+    CK(c, launch_overlapped(c->wide ? k_step<R, long long, VAR> : k_step<R, unsigned, VAR>, A.ntiles, blk, 0, s,
+                            tm, fi, (R*)fout, A));
   } else {
-    const size_t smem = pipe_smem_bytes<R>();
-    if (c->wide) k_step_pipe<R, long long, VAR><<<A.nblocks, blk, smem, s>>>(tm, fi, (R*)fout, A);
-    else k_step_pipe<R, unsigned, VAR><<<A.nblocks, blk, smem, s>>>(tm, fi, (R*)fout, A);
+    CK(c, launch_overlapped(c->wide ? k_step_pipe<R, long long, VAR> : k_step_pipe<R, unsigned, VAR>, A.nblocks,
+                            blk, pipe_smem_bytes<R>(), s, tm, fi, (R*)fout, A));
   }
-  CK(c, cudaGetLastError());
   return LBM_OK;
 }
 

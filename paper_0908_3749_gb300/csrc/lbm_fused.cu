@@ -217,8 +217,10 @@ __global__ void __launch_bounds__(NT, 4)
   const int tx = threadIdx.x, ty = threadIdx.y, t = ty * FX + tx;
   const int tile = blockIdx.x;
   const int x0 = (tile % A.tiles_x) * FX, y0 = (tile / A.tiles_x) * FY;
+  dependents_may_start();
+  if (t == 0) mbar_init(&bar, 1);
+  wait_for_previous();
   if (t == 0) {
-    mbar_init(&bar, 1);
     mbar_expect_tx(&bar, S0_BYTES);
     tma_load_tile(S0, &tmap, x0 - HALO_X, y0 - 2, &bar);
     s_step = read_step2(A, &s_audit0, &s_audit1);
@@ -321,9 +323,8 @@ cudaError_t fused_prepare() {
 cudaError_t fused_launch(const CUtensorMap& tm, const float* fin, float* fout,
                          const StepArgs<float>& A, bool wide, cudaStream_t s) {
   const dim3 blk(FX, FHY);
-  if (wide) k_step2<long long><<<A.ntiles, blk, fused_smem_bytes(), s>>>(tm, fin, fout, A);
-  else k_step2<unsigned><<<A.ntiles, blk, fused_smem_bytes(), s>>>(tm, fin, fout, A);
-  return cudaGetLastError();
+  return launch_overlapped(wide ? k_step2<long long> : k_step2<unsigned>, A.ntiles, blk, fused_smem_bytes(), s,
+                           tm, fin, fout, A);
 }
 
 }  // namespace lbmk

@@ -233,10 +233,12 @@ __global__ void __launch_bounds__(Shape<R>::X * Shape<R>::TY, (step_minb<R, Off>
   __shared__ unsigned long long s_step;
   __shared__ int s_audit, s_alist[32], s_an;
   const int t = threadIdx.y * Shape<R>::X + threadIdx.x;
+  dependents_may_start();
+  if (t == 0) mbar_init(&bar, 1);
+  wait_for_previous();
   if (t == 0) {
     // Start the tile copy first so that its latency overlaps the read of
     // the step counter.
-    mbar_init(&bar, 1);
     load_tile(tile, &tmap, &bar, blockIdx.x, A.tiles_x);
     s_step = read_step(A, &s_audit);
   }
@@ -281,9 +283,13 @@ __global__ void __launch_bounds__(Shape<R>::X * Shape<R>::TY, Shape<R>::MINB_PIP
   __shared__ int s_audit, s_alist[32], s_an;
   const int t = threadIdx.y * Shape<R>::X + threadIdx.x;
   const int G = (int)gridDim.x;
+  dependents_may_start();
   if (t == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
+  }
+  wait_for_previous();
+  if (t == 0) {
     load_tile(stages, &tmap, &bar[0], blockIdx.x, A.tiles_x);  // nblocks <= ntiles
     s_step = read_step(A, &s_audit);
   }

