@@ -158,8 +158,10 @@ __global__ void __launch_bounds__(CT_T, CONV_CTAS_PER_SM)
     gbtma::mbar_expect_tx(&bar, S::TILE);
     tma_load_box(base, &map, (tile % tiles_x) * CT_X - 1, (tile / tiles_x) * CT_Y - 1, &bar);
   };
+  gbtma::dependents_may_start();
+  if (threadIdx.x == 0) gbtma::mbar_init(&bar, 1);
+  gbtma::wait_for_previous();
   if (threadIdx.x == 0) {
-    gbtma::mbar_init(&bar, 1);
     load(blockIdx.x);  // the grid has at most ntiles CTAs
   }
   constexpr int CHUNKS = S::KP / 8;  // 16-byte pieces of a weight row
@@ -393,12 +395,15 @@ __global__ void __launch_bounds__(WG_T, WG_CTAS_PER_SM)
     tma_load_box(a, &act, x - 1, y - 1, &full[st]);
     tma_load_box(a + S::A_BYTES, &dz, x, y, &full[st]);
   };
-  if (warp == 0) tc05::alloc(&s_tmem, WG_TMEM_COLS);
-  if (t == 0) {
+  gbtma::dependents_may_start();
+  if (t == 0)
     for (int k = 0; k < 2; ++k) {
       gbtma::mbar_init(&full[k], 1);
       gbtma::mbar_init(&used[k], 1);
     }
+  gbtma::wait_for_previous();
+  if (warp == 0) tc05::alloc(&s_tmem, WG_TMEM_COLS);
+  if (t == 0) {
     load(blockIdx.x, 0);  // the grid has at most ntiles CTAs
   }
   tc05::fence_before();
@@ -549,6 +554,8 @@ __global__ void __launch_bounds__(C0_T) k_conv0(const float* __restrict__ xf, in
                                                 __nv_bfloat16* __restrict__ out,
                                                 unsigned* __restrict__ bits) {
   __shared__ __align__(16) float sw[9 * 4 * 32 + 32];
+  gbtma::dependents_may_start();
+  gbtma::wait_for_previous();
   for (int i = threadIdx.x; i < 9 * 4 * 32 + 32; i += C0_T) sw[i] = w[i];
   __syncthreads();
   const int W2 = (W + 1) / 2, q = blockIdx.x * C0_T + threadIdx.x;
@@ -671,6 +678,48 @@ std::vector<LogEntry> log_table() {
   return t;
 }
 
+// exp of an FP32 number in FP64, within 0.6 units in the last place: q = n log 2 /
+// 64 + r with n log 2 / 64 as an exact product and a correction, 2^(j/64) (j = n
+// mod 64) from a table as the sum of two doubles, exp(r) - 1 by its Taylor
+// series (|r| < 0.0055, the r^7 / 5040 left out is below 2^-65), the power of two
+// 2^(n div 64) added to the exponent: 13 FP64 instructions against about 20 for
+// exp(), which takes what is not in the normal range.
+struct ExpEntry {
+  double h, l;
+};
+constexpr int EXP_N = 64;
+__device__ __forceinline__ double exp32(float q, const ExpEntry* __restrict__ table) {
+  if (!(fabsf(q) < 700.f)) return exp((double)q);
+  const float nf = rintf(q * 92.33248f);  // 64 / log 2
+  const int n = (int)nf;
+  const double2 t = __ldg(reinterpret_cast<const double2*>(table) + (n & (EXP_N - 1)));
+  constexpr double STEP = 0.693147180559945309417 / 64;
+  constexpr double STEP_H = 0x1.62e42fefp-7;                 // 33 bits: n STEP_H is exact
+  constexpr double STEP_L = 0x1.473de6af278edp-40;           // log 2 / 64 - STEP_H
+  static_assert(STEP_H + STEP_L == STEP, "log 2 / 64");
+  const double nd = (double)nf;
+  const double r = fma(-nd, STEP_L, fma(-nd, STEP_H, (double)q));
+  double c = fma(r, 1.0 / 720, 1.0 / 120);
+  c = fma(c, r, 1.0 / 24);
+  c = fma(c, r, 1.0 / 6);
+  c = fma(c, r, 0.5);
+  const double p = fma(c * r, r, r);
+  const double v = t.x + fma(t.x, p, t.y);
+  return __hiloint2double(__double2hiint(v) + ((n >> 6) << 20), __double2loint(v));
+}
+// The table (host): 2^(k/64) in extended precision as h + l.
+std::vector<ExpEntry> exp_table() {
+  std::vector<ExpEntry> t(EXP_N);
+  for (int k = 0; k < EXP_N; ++k) {
+    // l from h's own logarithm: 2^(k/64) = h exp(d), d = k log 2 / 64 - log h small,
+    // in long double (64 significant bits or more).
+    const long double x = exp2l((long double)k / 64);
+    t[k].h = (double)x;
+    t[k].l = (double)(x - (long double)t[k].h);
+  }
+  return t;
+}
+
 // Planes [4][H][W] (rho, u, v, T) -> features (log rho, u, v, log T) in FP32
 // [p][4]; with `xs`, also their three BF16 parts (channel = part * 4 + feature,
 // 12 of 16 channels, row-planar; the other 4 stay zero).
@@ -678,6 +727,8 @@ std::vector<LogEntry> log_table() {
 // logarithms (the loss kernel, which takes the target's, 41 -> 16 us).
 __global__ void k_features(const double* __restrict__ f, int npix, int W, float* __restrict__ xf,
                            __nv_bfloat16* __restrict__ xs, const LogEntry* __restrict__ logs) {
+  gbtma::dependents_may_start();
+  gbtma::wait_for_previous();
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= npix) return;
   const float4 q = make_float4(log32(f[p], logs), (float)f[npix + p], (float)f[2 * npix + p],
@@ -714,6 +765,8 @@ __global__ void __launch_bounds__(256) k_loss(const float4* __restrict__ xf, con
                                               const Scale4 sc, int l1,
                                               const LogEntry* __restrict__ logs) {
   __shared__ double sm[8];
+  gbtma::dependents_may_start();
+  gbtma::wait_for_previous();
   const int p = blockIdx.x * 256 + threadIdx.x;
   double s = 0.0;
   if (p < npix) {
@@ -770,6 +823,8 @@ struct UpdateArgs {
   float lr, b1, b2, eps, c1, c2;
 };
 __global__ void __launch_bounds__(UP_N * UP_S) k_update(const UpdateArgs A) {
+  gbtma::dependents_may_start();
+  gbtma::wait_for_previous();
   const int t = threadIdx.x;
   if (blockIdx.x == gridDim.x - 1) {
     __shared__ double sl[UP_N * UP_S];
@@ -845,38 +900,75 @@ __global__ void k_pack(const float* __restrict__ w, int cin, int cout, int kp, i
   }
 }
 
-// corrected planes from output features x + z; block partial sums of rho.
-__global__ void k_apply(const float* __restrict__ xf, const float* __restrict__ z, int npix,
-                        double* __restrict__ out, const double* __restrict__ coarse,
-                        double* __restrict__ partial, const Scale4 sc) {
+// Results that a call hands to the host, in one copy.
+struct Results {
+  double loss;
+  double mass[2];  // sums of the corrected and of the coarse density
+  int timeout;     // a bounded wait expired in some kernel (sticky)
+  unsigned done;   // blocks of k_apply finished
+};
+
+// corrected planes from output features x + z and the two masses (NaN for a
+// non-finite output): block partial sums, added by the block that finishes
+// last in a fixed order. Bound by the FP64 units (two exponentials per pixel):
+// 512 x 512 about 20 us; 32 us with exp(), FP64 finiteness checks and the partials
+// added by the host.
+__global__ void __launch_bounds__(256) k_apply(const float4* __restrict__ xf, const float4* __restrict__ z,
+                                               int npix, double* __restrict__ out,
+                                               const double* __restrict__ coarse,
+                                               double* __restrict__ partial, const Scale4 sc,
+                                               const ExpEntry* __restrict__ exps, Results* res) {
   __shared__ double sm[2][256];
-  const int p = blockIdx.x * 256 + threadIdx.x;
+  __shared__ bool s_last;
+  gbtma::dependents_may_start();
+  gbtma::wait_for_previous();
+  const int p = blockIdx.x * 256 + threadIdx.x, t = threadIdx.x;
   double r = 0.0, r0 = 0.0;
   if (p < npix) {
-    const float q0 = xf[4 * p] + sc.s[0] * z[4 * p], q1 = xf[4 * p + 1] + sc.s[1] * z[4 * p + 1];
-    const float q2 = xf[4 * p + 2] + sc.s[2] * z[4 * p + 2];
-    const float q3 = xf[4 * p + 3] + sc.s[3] * z[4 * p + 3];
-    r = exp((double)q0);
+    const float4 x4 = xf[p], z4 = z[p];
+    const float q0 = x4.x + sc.s[0] * z4.x, q1 = x4.y + sc.s[1] * z4.y;
+    const float q2 = x4.z + sc.s[2] * z4.z, q3 = x4.w + sc.s[3] * z4.w;
+    r = exp32(q0, exps);
     out[p] = r;
     out[npix + p] = q1;
     out[2 * npix + p] = q2;
-    out[3 * npix + p] = exp((double)q3);
+    out[3 * npix + p] = exp32(q3, exps);
     r0 = coarse[p];
-    if (!isfinite(r + q1 + q2 + q3)) r = nan("");
+    if ((__double2hiint(r) & 0x7fffffff) >= 0x7ff00000 || !isfinite(q1) || !isfinite(q2) || !isfinite(q3))
+      r = nan("");
   }
-  sm[0][threadIdx.x] = r;
-  sm[1][threadIdx.x] = r0;
-  __syncthreads();
-  for (int st = 128; st > 0; st >>= 1) {
-    if ((int)threadIdx.x < st) {
-      sm[0][threadIdx.x] += sm[0][threadIdx.x + st];
-      sm[1][threadIdx.x] += sm[1][threadIdx.x + st];
-    }
+  auto block_sum = [&](double a, double b) {  // into sm[.][0]
+    sm[0][t] = a;
+    sm[1][t] = b;
     __syncthreads();
-  }
-  if (threadIdx.x == 0) {
+    for (int st = 128; st > 0; st >>= 1) {
+      if (t < st) {
+        sm[0][t] += sm[0][t + st];
+        sm[1][t] += sm[1][t + st];
+      }
+      __syncthreads();
+    }
+  };
+  block_sum(r, r0);
+  if (t == 0) {
     partial[2 * blockIdx.x] = sm[0][0];
     partial[2 * blockIdx.x + 1] = sm[1][0];
+    __threadfence();
+    s_last = atomicAdd(&res->done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  double a = 0.0, b = 0.0;
+  for (int i = t; i < (int)gridDim.x; i += 256) {
+    a += __ldcg(partial + 2 * i);
+    b += __ldcg(partial + 2 * i + 1);
+  }
+  block_sum(a, b);
+  if (t == 0) {
+    res->mass[0] = sm[0][0];
+    res->mass[1] = sm[1][0];
+    res->done = 0;
   }
 }
 
@@ -951,13 +1043,14 @@ struct lbm_cnn {
   int tiles_x = 0, ntiles = 0;  // convolution tiles
   int sms = 0;
   LogEntry* logs = nullptr;     // table of log32
-  int* timeout = nullptr;       // a bounded wait of a convolution expired
+  ExpEntry* exps = nullptr;     // table of exp32
+  Results* res = nullptr;       // device
+  Results* h_res = nullptr;     // pinned host copy
   float* xf = nullptr;          // input features FP32 [p][4]
   float* tf = nullptr;          // target features FP32 [p][4]
   float* z = nullptr;           // last layer output FP32 [p][4]
   float* wpartial = nullptr;    // weight-gradient partials, layer by layer
   double* dpart = nullptr;      // loss / mass partials
-  double* dloss = nullptr;
   int wblocks = 0;              // persistent CTAs of the weight gradients
   long long step = 0;
   float lr = 1e-3f, b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
@@ -992,9 +1085,14 @@ int pack_all(lbm_cnn* n) {
   return LBM_OK;
 }
 
-// After a synchronisation: whether a bounded wait of a convolution expired.
-int check_timeout(lbm_cnn* n, int flag) {
-  return flag ? cfail(n, LBM_ERR_TIMEOUT, "a tile load (TMA) did not complete within its time limit") : LBM_OK;
+// Copies the results to the host (n->h_res), synchronises and reports an
+// expired wait.
+int fetch_results(lbm_cnn* n) {
+  CCK(n, cudaMemcpyAsync(n->h_res, n->res, sizeof(Results), cudaMemcpyDeviceToHost, n->stream));
+  CCK(n, cudaStreamSynchronize(n->stream));
+  return n->h_res->timeout
+             ? cfail(n, LBM_ERR_TIMEOUT, "a tile load (TMA) or product did not complete within its time limit")
+             : LBM_OK;
 }
 
 // Tensor map of a row-planar BF16 image of `ncg` channel groups: dims (x in
@@ -1017,41 +1115,46 @@ int encode_image(lbm_cnn* n, const void* p, int ncg, int box_cg, bool halo, CUte
 }
 
 template <int CIN, int COUT, int EPI>
-void conv(lbm_cnn* n, const CUtensorMap& in, const __nv_bfloat16* wt, const float* bias,
+int conv(lbm_cnn* n, const CUtensorMap& in, const __nv_bfloat16* wt, const float* bias,
           const unsigned* bits_in, __nv_bfloat16* ob, float* of, unsigned* bits_out = nullptr) {
   const int grid = std::min(n->ntiles, CONV_CTAS_PER_SM * n->sms);
-  k_conv<CIN, COUT, EPI><<<grid, CT_T, ConvShape<CIN, COUT>::SMEM, n->stream>>>(
-      in, n->H, n->W, n->tiles_x, n->ntiles, wt, bias, bits_in, ob, of, bits_out, n->timeout);
+  CCK(n, gbtma::launch_overlapped(k_conv<CIN, COUT, EPI>, grid, CT_T, ConvShape<CIN, COUT>::SMEM, n->stream, in,
+                                  n->H, n->W, n->tiles_x, n->ntiles, wt, bias, bits_in, ob, of, bits_out,
+                                  &n->res->timeout));
+  return LBM_OK;
 }
 
 // `train`: also store which activations are positive, for the backward pass.
 int forward(lbm_cnn* n, const double* coarse, bool train) {
+  int rc;
   auto bits = [&](int l) { return train ? n->pos[l] : nullptr; };
-  k_features<<<(n->npix + 255) / 256, 256, 0, n->stream>>>(coarse, n->npix, n->W, n->xf,
-                                                           train ? n->xs : nullptr, n->logs);
+  CCK(n, gbtma::launch_overlapped(k_features, (n->npix + 255) / 256, 256, 0, n->stream, coarse, n->npix, n->W,
+                                  n->xf, train ? n->xs : nullptr, n->logs));
   const float* w = n->w;
-  k_conv0<<<(n->H * ((n->W + 1) / 2) + C0_T - 1) / C0_T, C0_T, 0, n->stream>>>(n->xf, n->H, n->W,
-                                                               w + param_offset(0), n->act[1], bits(1));
-  conv<32, 32, EPI_RELU_BF16>(n, n->m_act[1], n->wt[1], w + param_offset(1) + wsize(1), nullptr, n->act[2], nullptr, bits(2));
-  conv<32, 32, EPI_RELU_BF16>(n, n->m_act[2], n->wt[2], w + param_offset(2) + wsize(2), nullptr, n->act[3], nullptr, bits(3));
-  conv<32, 32, EPI_RELU_BF16>(n, n->m_act[3], n->wt[3], w + param_offset(3) + wsize(3), nullptr, n->act[4], nullptr, bits(4));
-  conv<32, 4, EPI_LINEAR_F32>(n, n->m_act[4], n->wt[4], w + param_offset(4) + wsize(4), nullptr, nullptr, n->z);
-  CCK(n, cudaGetLastError());
+  CCK(n, gbtma::launch_overlapped(k_conv0, (n->H * ((n->W + 1) / 2) + C0_T - 1) / C0_T, C0_T, 0, n->stream,
+                                  n->xf, n->H, n->W, w + param_offset(0), n->act[1], bits(1)));
+  if ((rc = conv<32, 32, EPI_RELU_BF16>(n, n->m_act[1], n->wt[1], w + param_offset(1) + wsize(1), nullptr, n->act[2], nullptr, bits(2))) != LBM_OK) return rc;
+  if ((rc = conv<32, 32, EPI_RELU_BF16>(n, n->m_act[2], n->wt[2], w + param_offset(2) + wsize(2), nullptr, n->act[3], nullptr, bits(3))) != LBM_OK) return rc;
+  if ((rc = conv<32, 32, EPI_RELU_BF16>(n, n->m_act[3], n->wt[3], w + param_offset(3) + wsize(3), nullptr, n->act[4], nullptr, bits(4))) != LBM_OK) return rc;
+  if ((rc = conv<32, 4, EPI_LINEAR_F32>(n, n->m_act[4], n->wt[4], w + param_offset(4) + wsize(4), nullptr, nullptr, n->z)) != LBM_OK) return rc;
   return LBM_OK;
 }
 
 template <int CG, int COUT>
-void wgrad(lbm_cnn* n, const CUtensorMap& act, const CUtensorMap& dz, float* partial) {
-  k_wgrad<CG, COUT><<<n->wblocks, WG_T, WgShape<CG, COUT == 32 ? 32 : 16>::SMEM, n->stream>>>(
-      act, dz, n->tiles_x, n->ntiles, partial, n->timeout);
+int wgrad(lbm_cnn* n, const CUtensorMap& act, const CUtensorMap& dz, float* partial) {
+  CCK(n, gbtma::launch_overlapped(k_wgrad<CG, COUT>, n->wblocks, WG_T, WgShape<CG, COUT == 32 ? 32 : 16>::SMEM,
+                                  n->stream, act, dz, n->tiles_x, n->ntiles, partial, &n->res->timeout));
+  return LBM_OK;
 }
 
 // Loss against the target features and all gradients into n->grad; with
 // `adam`, one optimiser step (n->step is its number).
 int loss_backward(lbm_cnn* n, const double* target, bool adam) {
   const int nb = (n->npix + 255) / 256;
-  k_loss<<<nb, 256, 0, n->stream>>>((const float4*)n->xf, (const float4*)n->z, target, n->npix,
-                                    (uint4*)n->dz5, n->dpart, n->scale, n->loss_kind == LBM_CNN_LOSS_L1, n->logs);
+  int rc;
+  CCK(n, gbtma::launch_overlapped(k_loss, nb, 256, 0, n->stream, (const float4*)n->xf, (const float4*)n->z, target,
+                                  n->npix, (uint4*)n->dz5, n->dpart, n->scale,
+                                  n->loss_kind == LBM_CNN_LOSS_L1, n->logs));
   UpdateArgs U = {};
   for (int l = 0; l < NL; ++l) {
     U.part[l] = n->wpartial + (size_t)n->wblocks * param_offset(l);
@@ -1060,15 +1163,15 @@ int loss_backward(lbm_cnn* n, const double* target, bool adam) {
   }
   auto part = [&](int l) { return const_cast<float*>(U.part[l]); };
   // layer 5 (32 -> 4): dz5 holds d loss / d z5
-  wgrad<4, 4>(n, n->m_act[4], n->g_dz5, part(4));
-  conv<4, 32, EPI_MASK_BF16>(n, n->m_dz5, n->wb[4], nullptr, n->pos[4], n->dz[1], nullptr);
-  wgrad<4, 32>(n, n->m_act[3], n->g_dz[1], part(3));
-  conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[1], n->wb[3], nullptr, n->pos[3], n->dz[0], nullptr);
-  wgrad<4, 32>(n, n->m_act[2], n->g_dz[0], part(2));
-  conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[0], n->wb[2], nullptr, n->pos[2], n->dz[1], nullptr);
-  wgrad<4, 32>(n, n->m_act[1], n->g_dz[1], part(1));
-  conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[1], n->wb[1], nullptr, n->pos[1], n->dz[0], nullptr);
-  wgrad<2, 32>(n, n->m_xs, n->g_dz[0], part(0));
+  if ((rc = wgrad<4, 4>(n, n->m_act[4], n->g_dz5, part(4))) != LBM_OK) return rc;
+  if ((rc = conv<4, 32, EPI_MASK_BF16>(n, n->m_dz5, n->wb[4], nullptr, n->pos[4], n->dz[1], nullptr)) != LBM_OK) return rc;
+  if ((rc = wgrad<4, 32>(n, n->m_act[3], n->g_dz[1], part(3))) != LBM_OK) return rc;
+  if ((rc = conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[1], n->wb[3], nullptr, n->pos[3], n->dz[0], nullptr)) != LBM_OK) return rc;
+  if ((rc = wgrad<4, 32>(n, n->m_act[2], n->g_dz[0], part(2))) != LBM_OK) return rc;
+  if ((rc = conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[0], n->wb[2], nullptr, n->pos[2], n->dz[1], nullptr)) != LBM_OK) return rc;
+  if ((rc = wgrad<4, 32>(n, n->m_act[1], n->g_dz[1], part(1))) != LBM_OK) return rc;
+  if ((rc = conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[1], n->wb[1], nullptr, n->pos[1], n->dz[0], nullptr)) != LBM_OK) return rc;
+  if ((rc = wgrad<2, 32>(n, n->m_xs, n->g_dz[0], part(0))) != LBM_OK) return rc;
   U.nblocks = n->wblocks;
   U.w = n->w;
   U.m = n->m;
@@ -1077,7 +1180,7 @@ int loss_backward(lbm_cnn* n, const double* target, bool adam) {
   U.lpart = n->dpart;
   U.nl = nb;
   U.lscale = 1.0 / (4.0 * n->npix);
-  U.loss = n->dloss;
+  U.loss = &n->res->loss;
   U.adam = adam;
   U.lr = n->lr;
   U.b1 = n->b1;
@@ -1087,8 +1190,7 @@ int loss_backward(lbm_cnn* n, const double* target, bool adam) {
     U.c1 = 1.f - powf(n->b1, (float)n->step);
     U.c2 = 1.f - powf(n->b2, (float)n->step);
   }
-  k_update<<<(LBM_CNN_NPARAMS + UP_N - 1) / UP_N + 1, UP_N * UP_S, 0, n->stream>>>(U);
-  CCK(n, cudaGetLastError());
+  CCK(n, gbtma::launch_overlapped(k_update, (LBM_CNN_NPARAMS + UP_N - 1) / UP_N + 1, UP_N * UP_S, 0, n->stream, U));
   return LBM_OK;
 }
 
@@ -1146,7 +1248,6 @@ int lbm_cnn_create(int H, int W, void* cuda_stream, lbm_cnn** out) {
   A((void**)&n->dz[1], 2 * P * 32);
   A((void**)&n->dz5, 2 * P * 8);
   A((void**)&n->xs, 2 * P * 16);
-  A((void**)&n->timeout, sizeof(int));
   const std::vector<LogEntry> logs = log_table();
   A((void**)&n->logs, sizeof(LogEntry) * LOG_N);
   if (e == cudaSuccess)
@@ -1156,7 +1257,12 @@ int lbm_cnn_create(int H, int W, void* cuda_stream, lbm_cnn** out) {
   A((void**)&n->z, 4 * P * 4);
   A((void**)&n->wpartial, sizeof(float) * (size_t)n->wblocks * LBM_CNN_NPARAMS);
   A((void**)&n->dpart, sizeof(double) * 2 * ((4 * P + 255) / 256 + 1));
-  A((void**)&n->dloss, sizeof(double));
+  A((void**)&n->res, sizeof(Results));
+  const std::vector<ExpEntry> exps = exp_table();
+  A((void**)&n->exps, sizeof(ExpEntry) * EXP_N);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(n->exps, exps.data(), sizeof(ExpEntry) * EXP_N, cudaMemcpyHostToDevice, n->stream);
+  if (e == cudaSuccess) e = cudaMallocHost((void**)&n->h_res, sizeof(Results));
   if (e == cudaSuccess) e = cudaStreamSynchronize(n->stream);
   if (e != cudaSuccess) {
     g_cnn_error = std::string("lbm_cnn_create: ") + cudaGetErrorString(e);
@@ -1185,7 +1291,7 @@ int lbm_cnn_destroy(lbm_cnn* n) {
   if (!n) return LBM_OK;
   if (n->stream) cudaStreamSynchronize(n->stream);
   void* ps[] = {n->w, n->m, n->v, n->grad, n->dz[0], n->dz[1], n->xf, n->tf, n->z,
-                n->wpartial, n->dpart, n->dloss, n->dz5, n->xs, n->logs, n->timeout};
+                n->wpartial, n->dpart, n->res, n->dz5, n->xs, n->logs, n->exps};
   for (void* p : ps)
     if (p) cudaFree(p);
   for (int l = 0; l < NL; ++l) {
@@ -1194,6 +1300,7 @@ int lbm_cnn_destroy(lbm_cnn* n) {
     if (n->act[l]) cudaFree(n->act[l]);
     if (n->pos[l]) cudaFree(n->pos[l]);
   }
+  if (n->h_res) cudaFreeHost(n->h_res);
   if (n->own_stream && n->stream) cudaStreamDestroy(n->stream);
   delete n;
   return LBM_OK;
@@ -1235,14 +1342,12 @@ int lbm_cnn_loss_grad(lbm_cnn* n, const double* coarse, const double* target, do
   int rc = forward(n, coarse, true);
   if (rc == LBM_OK) rc = loss_backward(n, target, false);
   if (rc != LBM_OK) return rc;
-  if (loss) CCK(n, cudaMemcpyAsync(loss, n->dloss, sizeof(double), cudaMemcpyDeviceToHost, n->stream));
   if (grads)
     CCK(n, cudaMemcpyAsync(grads, n->grad, sizeof(float) * LBM_CNN_NPARAMS, cudaMemcpyDeviceToHost,
                            n->stream));
-  int flag = 0;
-  CCK(n, cudaMemcpyAsync(&flag, n->timeout, sizeof(int), cudaMemcpyDeviceToHost, n->stream));
-  CCK(n, cudaStreamSynchronize(n->stream));
-  return check_timeout(n, flag);
+  if ((rc = fetch_results(n)) != LBM_OK) return rc;
+  if (loss) *loss = n->h_res->loss;
+  return LBM_OK;
 }
 
 int lbm_cnn_train_step(lbm_cnn* n, const double* coarse, const double* target, double* loss) {
@@ -1253,11 +1358,8 @@ int lbm_cnn_train_step(lbm_cnn* n, const double* coarse, const double* target, d
   rc = loss_backward(n, target, true);
   if (rc != LBM_OK) return rc;
   if (loss) {
-    int flag = 0;
-    CCK(n, cudaMemcpyAsync(loss, n->dloss, sizeof(double), cudaMemcpyDeviceToHost, n->stream));
-    CCK(n, cudaMemcpyAsync(&flag, n->timeout, sizeof(int), cudaMemcpyDeviceToHost, n->stream));
-    CCK(n, cudaStreamSynchronize(n->stream));
-    return check_timeout(n, flag);
+    if ((rc = fetch_results(n)) != LBM_OK) return rc;
+    *loss = n->h_res->loss;
   }
   return LBM_OK;
 }
@@ -1309,17 +1411,10 @@ int lbm_cnn_correct(lbm_cnn* n, const double* coarse, double* corrected, double 
   int rc = forward(n, coarse, false);
   if (rc != LBM_OK) return rc;
   const int nb = (n->npix + 255) / 256;
-  k_apply<<<nb, 256, 0, n->stream>>>(n->xf, n->z, n->npix, corrected, coarse, n->dpart, n->scale);
-  CCK(n, cudaGetLastError());
-  std::vector<double> part(2 * (size_t)nb);
-  CCK(n, cudaMemcpyAsync(part.data(), n->dpart, sizeof(double) * part.size(),
-                         cudaMemcpyDeviceToHost, n->stream));
-  int flag = 0;
-  CCK(n, cudaMemcpyAsync(&flag, n->timeout, sizeof(int), cudaMemcpyDeviceToHost, n->stream));
-  CCK(n, cudaStreamSynchronize(n->stream));
-  if ((rc = check_timeout(n, flag)) != LBM_OK) return rc;
-  double m1 = 0, m0 = 0;
-  for (int b = 0; b < nb; ++b) { m1 += part[2 * b]; m0 += part[2 * b + 1]; }
+  CCK(n, gbtma::launch_overlapped(k_apply, nb, 256, 0, n->stream, (const float4*)n->xf, (const float4*)n->z,
+                                  n->npix, corrected, coarse, n->dpart, n->scale, n->exps, n->res));
+  if ((rc = fetch_results(n)) != LBM_OK) return rc;
+  const double m1 = n->h_res->mass[0], m0 = n->h_res->mass[1];
   const bool fallback = !std::isfinite(m1) || std::fabs(m1 - m0) > mass_tol * std::fabs(m0);
   if (fallback) {
     CCK(n, cudaMemcpyAsync(corrected, coarse, sizeof(double) * 4 * n->npix,

@@ -59,3 +59,48 @@ def test_log_features_of_invalid_values_are_log_s(bad):
     with np.errstate(all="ignore"):
         ref = np.abs(np.log(bad))
     assert np.isnan(r[0]) if np.isnan(ref) else r[0] == ref
+
+
+def test_corrected_fields_are_the_exponentials_of_the_features():
+    """With zero parameters the corrected density and temperature are exp of the
+    FP32 logarithms: within 0.6 units in the last place of the true value, numpy's
+    exp within one, so 2 x 2^-52 relative between them; the sums of the density
+    agree with the fallback's mass test (no fallback at 1e-6: the logarithm's FP32
+    rounding changes the density by at most 2^-24 |log|)."""
+    import torch
+    from paper_0908_3749_gb300 import lbm
+    vals = _values()
+    vals = vals[(vals > 1e-307) & (vals < 1e307)]
+    for part in (vals, np.exp(np.random.default_rng(4).uniform(-2, 2, 70000))):
+        f = np.stack([part, np.linspace(-1, 1, len(part)), np.zeros(len(part)), part[::-1]])[:, None, :]
+        coarse = torch.tensor(f, device="cuda")
+        out = torch.empty_like(coarse)
+        net = lbm.lbm_cnn_create(1, len(part))
+        try:
+            fallback = lbm.lbm_cnn_correct(net, coarse, out, mass_tol=700 * 2.0 ** -24)
+            again = torch.empty_like(coarse)
+            lbm.lbm_cnn_correct(net, coarse, again, mass_tol=700 * 2.0 ** -24)
+        finally:
+            lbm.lbm_cnn_destroy(net)
+        assert not fallback and torch.equal(out, again)
+        ref = np.exp(np.log(part).astype(np.float32).astype(np.float64))
+        got = out.cpu().numpy()
+        np.testing.assert_allclose(got[0, 0], ref, rtol=2.0 ** -51, atol=0)
+        np.testing.assert_allclose(got[3, 0], ref[::-1], rtol=2.0 ** -51, atol=0)
+        np.testing.assert_array_equal(got[1, 0], f[1, 0].astype(np.float32))
+
+
+def test_a_non_finite_output_falls_back():
+    import torch
+    from paper_0908_3749_gb300 import lbm
+    coarse = torch.ones((4, 3, 300), dtype=torch.float64, device="cuda")
+    coarse[1, 2, 299] = float("inf")
+    out = torch.zeros_like(coarse)
+    net = lbm.lbm_cnn_create(3, 300)
+    try:
+        assert lbm.lbm_cnn_correct(net, coarse, out)
+        assert torch.equal(out, coarse)
+        coarse[1, 2, 299] = 0.0
+        assert not lbm.lbm_cnn_correct(net, coarse, out)
+    finally:
+        lbm.lbm_cnn_destroy(net)
