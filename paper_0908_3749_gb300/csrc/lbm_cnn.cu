@@ -10,16 +10,15 @@
 // and of the tcgen05 operand layout, and a tap of the 3 x 3 stencil is an
 // address offset (pixels outside the image are the box's zero fill).
 // The input features stay FP32 and the first layer (4 -> 32) runs in FP32 on
-// the CUDA cores. The other 3 x 3 convolutions are implicit GEMMs on the tensor
-// cores (mma.sync m16n8k16, BF16 inputs, FP32 accumulation): rows are pixels, the
-// reduction index k = tap * CIN + ci runs over the 9 taps and the input
+// the CUDA cores. The other 3 x 3 convolutions are implicit GEMMs on the
+// 5th-generation tensor cores (tcgen05, BF16 inputs, FP32 accumulation in tensor
+// memory; mma.sync for 4 -> 32 channels): rows are pixels, the reduction index k = tap * CIN + ci runs over the 9 taps and the input
 // channels, columns are output channels. The weights of a layer are packed
 // once per update into [COUT][K] BF16 (K contiguous, the "col" operand) for
 // the forward pass and into the tap-flipped, channel-transposed [CIN][K'] for
 // the input-gradient pass, which is the same GEMM run on the output
-// gradients. Weight gradients are contractions over the pixels on the
-// 5th-generation tensor cores (tcgen05, BF16 inputs, FP32 accumulation in
-// tensor memory; the first layer's FP32 features as three BF16 parts), as
+// gradients. Weight gradients are contractions over the pixels, by tcgen05 too
+// (the first layer's FP32 features as three BF16 parts), as
 // per-CTA partials, then a fixed-order sum (reproducible). Adam keeps FP32
 // master weights.
 #include <cuda_bf16.h>
@@ -76,28 +75,7 @@ __device__ __forceinline__ unsigned positive_bits(__nv_bfloat162 v) {
 // A pixel's word of 32 such bits: channels 8 j + 2 t, + 1 (j, t = 0..3) at bits
 // 15 - s and 31 - s, s = j + 4 t.
 
-// Tiles of CT_Y x CT_X output pixels; their inputs with a halo of one pixel
-// are one TMA box of CT_HY rows x channel groups x CT_HX pixels.
-constexpr int CT_X = 32, CT_Y = 8, CT_HX = CT_X + 2, CT_HY = CT_Y + 2;
-constexpr int CT_WARPS = 4, CT_T = 32 * CT_WARPS;  // a warp computes two rows
-constexpr int CONV_CTAS_PER_SM = 3;
-constexpr unsigned PX_BYTES = 16;                  // 8 BF16 channels of a pixel
-
-__device__ __forceinline__ void ldmatrix4(unsigned (&r)[4], unsigned addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(addr));
-}
-__device__ __forceinline__ void ldmatrix2(unsigned& r0, unsigned& r1, unsigned addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];\n"
-               : "=r"(r0), "=r"(r1)
-               : "r"(addr));
-}
-__device__ __forceinline__ unsigned lds32(unsigned addr) {
-  unsigned v;
-  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr));
-  return v;
-}
+constexpr unsigned PX_BYTES = 16;  // 8 BF16 channels of a pixel
 
 // A box of `map` (3D: x in 32-bit words, channel group, row) whose first pixel
 // is (x, y), all channel groups.
@@ -111,89 +89,228 @@ __device__ __forceinline__ void tma_load_box(void* dst, const CUtensorMap* map, 
       : "memory");
 }
 
-template <int CIN, int COUT>
-struct ConvShape {
-  static constexpr int NCG = CIN == 32 ? 4 : 1;      // channel groups of the input
-  static constexpr int KP = ru(9 * CIN, 16), KS = KP / 16;
-  static constexpr int COUTP = ru(COUT, 8), NF = COUTP / 8;
-  // Weight rows in shared memory, 16 bytes longer than K: the 8 rows that an
-  // 8 x 8 ldmatrix reads then start in different 16-byte bank groups.
-  static constexpr int WPITCH = KP + 8;
-  static constexpr unsigned ROW = NCG * CT_HX * PX_BYTES;  // bytes per tile row
-  static constexpr unsigned TILE = CT_HY * ROW;
-  static constexpr unsigned STAGE = (TILE + 127) / 128 * 128;
-  static constexpr unsigned SMEM = STAGE + COUTP * WPITCH * 2 + 128;
-};
+// 32 -> COUT channels: out[p][c] = epilogue(sum_k patch(p, k) * Wt[c][k]) on the
+// 5th-generation tensor cores. A tile is 16 x 16 output pixels, its input with
+// a halo of one pixel one TMA box of 18 rows x 4 channel groups x 18 pixels. In
+// shared memory 8 pixels of a row x 8 channels are a core matrix (128
+// contiguous bytes), tile rows are CV_ROW apart: M = 128 rows of A are 8 pixels of 16
+// rows, a tap is an offset of the start address, K = 16 two channel groups; nothing
+// is gathered by threads. The packed weights stay in shared memory as core
+// matrices of 8 output channels x 8 k. One thread issues a tile's 36 products
+// (two M = 128 halves; K in order, tap by tap) and commits them; the next tile's
+// copy starts once they have completed, under the epilogue, in which a thread
+// holds all channels of a pixel. Persistent CTAs, four per SM.
+// The results are those of mma.sync m16n8k16 over the same K steps, bit for bit.
+// Bound by the tensor cores' reads of shared memory (5 KB per product, 5 us) and
+// by the latencies around each tile. Measured, 512 x 512, 32 -> 32 channels: 14
+// us, with and without the mask; as mma.sync with ldmatrix fragments (8 us at its 1024
+// multiply-adds per clock and SM) 18 us; with patches gathered from global memory
+// (L1 91 % busy) 67 us, and 72 us with the mask read from the activations.
+constexpr int CV_X = 16, CV_Y = 16, CV_HX = CV_X + 2, CV_HY = CV_Y + 2, CV_T = 128;
+constexpr int CV_CTAS_PER_SM = 4;
+constexpr int CV_KG = 9 * 32 / 8;                          // groups of 8 k
+constexpr unsigned CV_GROUP = CV_HX * PX_BYTES, CV_ROW = 4 * CV_GROUP;
+constexpr unsigned CV_TILE = CV_HY * CV_ROW, CV_STAGE = (CV_TILE + 127) / 128 * 128;
+__host__ __device__ constexpr int cv_n(int cout) { return cout == 32 ? 32 : 16; }  // N of the products (zero rows)
+__host__ __device__ constexpr unsigned cv_smem(int cout) { return CV_STAGE + CV_KG * cv_n(cout) * 16 + 128; }
 
-// out[p][c] (c < COUT) = epilogue(sum_k patch(p, k) * Wt[c][k]).
-//
-// Persistent CTAs of four warps, three per SM; a tile's input (10 x 34 pixels)
-// is copied by TMA while the CTA stores the previous tile's outputs and the
-// other CTAs compute, the packed weights stay in shared memory. A warp
-// computes two rows of 32 pixels (four 16-pixel M tiles) x COUTP channels: per
-// K step one ldmatrix.x4 per M tile (the tap is an offset into the tile), and
-// the B fragments serve all four. The K steps run in order, one accumulator per
-// fragment. Bound by the tensor pipe's mma.sync rate (8 us at 1024
-// multiply-adds per clock and SM) and the latencies around each tile.
-// Measured, 512 x 512, 32 -> 32 channels: 18 us with and without the mask;
-// reading the patches from global memory instead (four predicated 4-byte loads
-// per K step and M tile) was bound by L1 at 91 %: 67 us, and 72 us with the
-// mask read from the activations. Four and five CTAs per SM (128 and 96
-// registers, K loop partly unrolled) took 20 us, a second tile stage 18 us.
-template <int CIN, int COUT, int EPI>
-__global__ void __launch_bounds__(CT_T, CONV_CTAS_PER_SM)
+template <int COUT, int EPI>
+__global__ void __launch_bounds__(CV_T, CV_CTAS_PER_SM)
     k_conv(const __grid_constant__ CUtensorMap map, int H, int W, int tiles_x, int ntiles,
            const __nv_bfloat16* __restrict__ Wt, const float* __restrict__ bias,
            const unsigned* __restrict__ bits_in, __nv_bfloat16* __restrict__ out_bf,
            float* __restrict__ out_f, unsigned* __restrict__ bits_out, int* __restrict__ timeout) {
-  using S = ConvShape<CIN, COUT>;
+  constexpr int NP = cv_n(COUT), TM = 2 * NP;  // TMEM columns: two halves
+  constexpr unsigned IDESC = tc05::idesc_f32acc(tc05::FMT_BF16, 128, NP);
+  extern __shared__ __align__(128) unsigned char conv_raw[];
+  unsigned char* const base = conv_raw + ((128u - (gbtma::smem_addr(conv_raw) & 127u)) & 127u);
+  __shared__ unsigned long long full, done;  // copy landed; products complete
+  __shared__ unsigned s_tmem;
+  __shared__ __align__(16) float s_bias[32];
+  const int t = threadIdx.x, warp = t >> 5;
+  const int G = (int)gridDim.x;
+  auto load = [&](int tile) {
+    gbtma::mbar_expect_tx(&full, CV_TILE);
+    tma_load_box(base, &map, (tile % tiles_x) * CV_X - 1, (tile / tiles_x) * CV_Y - 1, &full);
+  };
+  gbtma::dependents_may_start();
+  if (t == 0) {
+    gbtma::mbar_init(&full, 1);
+    gbtma::mbar_init(&done, 1);
+  }
+  gbtma::wait_for_previous();
+  if (warp == 0) tc05::alloc(&s_tmem, TM);
+  if (t == 0) load(blockIdx.x);  // the grid has at most ntiles CTAs
+  // Wt [ru(COUT, 8)][288] -> [k / 8][row][8]; rows beyond it zero
+  unsigned char* const sw = base + CV_STAGE;
+  for (int i = t; i < NP * CV_KG; i += CV_T) {
+    const int n = i / CV_KG, kg = i % CV_KG;
+    *reinterpret_cast<uint4*>(sw + (kg * NP + n) * 16) =
+        n < ru(COUT, 8) ? __ldg(reinterpret_cast<const uint4*>(Wt) + i) : make_uint4(0, 0, 0, 0);
+  }
+  if (EPI != EPI_MASK_BF16 && t < COUT) s_bias[t] = bias[t];
+  tc05::fence_async_smem();
+  tc05::fence_before();
+  __syncthreads();
+  tc05::fence_after();
+  const unsigned tmem = s_tmem, a0 = gbtma::smem_addr(base), b0 = gbtma::smem_addr(sw);
+
+  bool ok = true;
+  int k = 0;
+  for (int tile = blockIdx.x; tile < ntiles; tile += G, ++k) {
+    const bool more = tile + G < ntiles;
+    const int x0 = (tile % tiles_x) * CV_X + (t & 7), y = (tile / tiles_x) * CV_Y + (t >> 3);
+    if (t == 0) {
+      ok = gbtma::mbar_wait_bounded(&full, k & 1, gbtma::TMA_WAIT_CYCLES);
+      if (ok) {
+        tc05::fence_after();
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll 1
+          for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {  // dx = q / 2, channels 16 (q % 2) ..
+              const int ks = dy * 6 + q;
+              tc05::mma_f16(tmem + m * NP,
+                            tc05::smem_desc(a0 + dy * CV_ROW + (8 * m + q / 2) * PX_BYTES + (q & 1) * 2 * CV_GROUP,
+                                            CV_GROUP, CV_ROW),
+                            tc05::smem_desc(b0 + ks * 2 * NP * 16, NP * 16, 128), IDESC, ks > 0 ? 1u : 0u);
+            }
+        tc05::commit(&done);
+      }
+    }
+    // The ReLU masks (which channels of a pixel are positive) of this thread's
+    // outputs, read while the products run.
+    unsigned keep[2] = {0u, 0u};
+    if constexpr (EPI == EPI_MASK_BF16)
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+        if (y < H && x0 + 8 * m < W) keep[m] = __ldg(bits_in + (long long)y * W + x0 + 8 * m);
+    __syncwarp();
+    ok = __syncthreads_and(ok && (t != 0 ? true : gbtma::mbar_wait_bounded(&done, k & 1, gbtma::TMA_WAIT_CYCLES)));
+    if (!ok) break;
+    if (t == 0 && more) load(tile + G);  // the products have read the tile
+    tc05::fence_after();
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      const int x = x0 + 8 * m;
+      const unsigned lanes = tmem + ((unsigned)(warp * 32) << 16) + m * NP;
+      if constexpr (EPI == EPI_LINEAR_F32) {
+        float v[16];
+        tc05::ld16(lanes, v);
+        if (y < H && x < W)
+          *reinterpret_cast<float4*>(out_f + ((long long)y * W + x) * 4) =
+              make_float4(v[0] + s_bias[0], v[1] + s_bias[1], v[2] + s_bias[2], v[3] + s_bias[3]);
+      } else {
+        float v[32];
+        tc05::ld32(lanes, v);
+        if (y < H && x < W) {
+          unsigned pos = 0u;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            __nv_bfloat162 r[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int c = 8 * j + 2 * i;
+              if constexpr (EPI == EPI_RELU_BF16) {
+                r[i] = __floats2bfloat162_rn(fmaxf(v[c] + s_bias[c], 0.f), fmaxf(v[c + 1] + s_bias[c + 1], 0.f));
+                pos |= positive_bits(r[i]) >> (j + 4 * i);
+              } else {
+                r[i] = __floats2bfloat162_rn(v[c] * (keep[m] & (0x8000u >> (j + 4 * i)) ? 1.f : 0.f),
+                                             v[c + 1] * (keep[m] & (0x80000000u >> (j + 4 * i)) ? 1.f : 0.f));
+              }
+            }
+            *reinterpret_cast<uint4*>(out_bf + (((long long)y * 4 + j) * W + x) * 8) =
+                *reinterpret_cast<const uint4*>(r);
+          }
+          if (EPI == EPI_RELU_BF16 && bits_out) bits_out[(long long)y * W + x] = pos;
+        }
+      }
+    }
+    tc05::fence_before();
+    __syncthreads();  // the accumulators are free again
+    tc05::fence_after();
+  }
+  if (!ok && t == 0) {
+    // A copy or the products did not complete in time: record it and wait once
+    // more (bounded) for both.
+    atomicExch(timeout, 1);
+    gbtma::mbar_wait_bounded(&full, k & 1, gbtma::TMA_WAIT_CYCLES);
+    gbtma::mbar_wait_bounded(&done, k & 1, gbtma::TMA_WAIT_CYCLES);
+  }
+  tc05::fence_before();
+  __syncthreads();
+  if (warp == 0) tc05::dealloc(tmem, TM);
+}
+
+// Tiles of the 4 -> 32 convolution and of the weight gradients: CT_Y x CT_X
+// output pixels; their inputs with a halo of one pixel are one TMA box of CT_HY
+// rows x channel groups x CT_HX pixels.
+constexpr int CT_X = 32, CT_Y = 8, CT_HX = CT_X + 2, CT_HY = CT_Y + 2;
+constexpr int CT_WARPS = 4, CT_T = 32 * CT_WARPS;  // a warp computes two rows
+
+__device__ __forceinline__ void ldmatrix4(unsigned (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+__device__ __forceinline__ unsigned lds32(unsigned addr) {
+  unsigned v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr));
+  return v;
+}
+
+// The input gradient of the last layer, 4 -> 32 channels with the ReLU mask: its
+// K = tap * 4 + ci (36, padded to 48) has no core matrices in the tile (8 k are
+// two taps), so the fragments of mma.sync m16n8k16 are read from the tile word by
+// word. Persistent CTAs of four warps, three per SM; a warp computes two rows of
+// 32 pixels (four 16-pixel M tiles), the B fragments serve all four. 8 us at 512 x
+// 512; 21 us with the patches and the activations' mask read from global memory.
+constexpr int C4_KS = 3, C4_KP = 16 * C4_KS, C4_CTAS_PER_SM = 3;
+// Weight rows in shared memory, 16 bytes longer than K: the 8 rows that an 8 x 8
+// ldmatrix reads then start in different 16-byte bank groups.
+constexpr int C4_PITCH = C4_KP + 8;
+constexpr unsigned C4_ROW = CT_HX * PX_BYTES, C4_TILE = CT_HY * C4_ROW, C4_STAGE = (C4_TILE + 127) / 128 * 128;
+constexpr unsigned C4_SMEM = C4_STAGE + 32 * C4_PITCH * 2 + 128;
+
+__global__ void __launch_bounds__(CT_T, C4_CTAS_PER_SM)
+    k_conv4(const __grid_constant__ CUtensorMap map, int H, int W, int tiles_x, int ntiles,
+            const __nv_bfloat16* __restrict__ Wt, const unsigned* __restrict__ bits_in,
+            __nv_bfloat16* __restrict__ out, int* __restrict__ timeout) {
   extern __shared__ __align__(128) unsigned char conv_raw[];
   unsigned char* const base = conv_raw + ((128u - (gbtma::smem_addr(conv_raw) & 127u)) & 127u);
   __shared__ unsigned long long bar;
-  const unsigned sw = gbtma::smem_addr(base) + S::STAGE;
+  const unsigned in = gbtma::smem_addr(base), sw = in + C4_STAGE;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, tig = lane & 3;
   const int G = (int)gridDim.x;
   auto load = [&](int tile) {
-    gbtma::mbar_expect_tx(&bar, S::TILE);
+    gbtma::mbar_expect_tx(&bar, C4_TILE);
     tma_load_box(base, &map, (tile % tiles_x) * CT_X - 1, (tile / tiles_x) * CT_Y - 1, &bar);
   };
   gbtma::dependents_may_start();
   if (threadIdx.x == 0) gbtma::mbar_init(&bar, 1);
   gbtma::wait_for_previous();
-  if (threadIdx.x == 0) {
-    load(blockIdx.x);  // the grid has at most ntiles CTAs
-  }
-  constexpr int CHUNKS = S::KP / 8;  // 16-byte pieces of a weight row
-  for (int i = threadIdx.x; i < S::COUTP * CHUNKS; i += CT_T)
-    *reinterpret_cast<uint4*>(base + S::STAGE + (i / CHUNKS) * (S::WPITCH * 2) + (i % CHUNKS) * 16) =
+  if (threadIdx.x == 0) load(blockIdx.x);  // the grid has at most ntiles CTAs
+  constexpr int CHUNKS = C4_KP / 8;  // 16-byte pieces of a weight row
+  for (int i = threadIdx.x; i < 32 * CHUNKS; i += CT_T)
+    *reinterpret_cast<uint4*>(base + C4_STAGE + (i / CHUNKS) * (C4_PITCH * 2) + (i % CHUNKS) * 16) =
         __ldg(reinterpret_cast<const uint4*>(Wt) + i);
   __syncthreads();
-
-  float bs[S::NF][2];
-#pragma unroll
-  for (int j = 0; j < S::NF; ++j)
-#pragma unroll
-    for (int e = 0; e < 2; ++e)
-      bs[j][e] = EPI != EPI_MASK_BF16 && j * 8 + tig * 2 + e < COUT ? __ldg(bias + j * 8 + tig * 2 + e) : 0.f;
 
   for (int k = 0, tile = blockIdx.x; tile < ntiles; tile += G, ++k) {
     const bool more = tile + G < ntiles;
     const int x0 = (tile % tiles_x) * CT_X, y0 = (tile / tiles_x) * CT_Y + 2 * warp;
-    // The ReLU masks (which channels of a pixel are positive) of this
-    // thread's outputs, read while the tile's copy is in flight. Reading the
-    // activations themselves here or in the epilogue, 32 loads of 4 bytes per
-    // thread, took 25-27 us per layer.
+    // The ReLU masks (which channels of a pixel are positive) of this thread's
+    // outputs, read while the tile's copy is in flight.
     unsigned keep[4][2];
-    if constexpr (EPI == EPI_MASK_BF16) {
 #pragma unroll
-      for (int m = 0; m < 4; ++m)
+    for (int m = 0; m < 4; ++m)
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int y = y0 + (m >> 1), x = x0 + (m & 1) * 16 + h * 8 + g;
-          keep[m][h] = y < H && x < W ? __ldg(bits_in + (long long)y * W + x) << (4 * tig) : 0u;
-        }
-    }
+      for (int h = 0; h < 2; ++h) {
+        const int y = y0 + (m >> 1), x = x0 + (m & 1) * 16 + h * 8 + g;
+        keep[m][h] = y < H && x < W ? __ldg(bits_in + (long long)y * W + x) << (4 * tig) : 0u;
+      }
     if (!__syncthreads_and(gbtma::mbar_wait_bounded(&bar, k & 1, gbtma::TMA_WAIT_CYCLES))) {
       // The copy did not land in time: record it, wait once more (bounded), leave.
       if (threadIdx.x == 0) {
@@ -202,54 +319,38 @@ __global__ void __launch_bounds__(CT_T, CONV_CTAS_PER_SM)
       }
       return;
     }
-    const unsigned in = gbtma::smem_addr(base);
-    float acc[4][S::NF][4];
+    float acc[4][4][4];
 #pragma unroll
     for (int m = 0; m < 4; ++m)
 #pragma unroll
-      for (int j = 0; j < S::NF; ++j) acc[m][j][0] = acc[m][j][1] = acc[m][j][2] = acc[m][j][3] = 0.f;
+      for (int j = 0; j < 4; ++j) acc[m][j][0] = acc[m][j][1] = acc[m][j][2] = acc[m][j][3] = 0.f;
     // M tile m: row 2 warp + m / 2, pixels 16 (m % 2) .. + 15.
-    const unsigned arow = in + 2 * warp * S::ROW;
-    // ldmatrix row addresses: lane -> pixel lane % 16, channel group lane / 16
-    const unsigned a_lane = (lane & 15) * PX_BYTES + (lane >> 4) * (CT_HX * PX_BYTES);
-    const unsigned b_lane = S::NF == 1
-                                ? ((lane & 7) * S::WPITCH + ((lane >> 3) & 1) * 8) * 2
-                                : (((lane & 7) + (lane >> 4) * 8) * S::WPITCH + ((lane >> 3) & 1) * 8) * 2;
+    const unsigned arow = in + 2 * warp * C4_ROW;
+    const unsigned b_lane = (((lane & 7) + (lane >> 4) * 8) * C4_PITCH + ((lane >> 3) & 1) * 8) * 2;
 #pragma unroll
-    for (int ks = 0; ks < S::KS; ++ks) {
-      unsigned b[S::NF][2];
-      if constexpr (S::NF == 1) {
-        ldmatrix2(b[0][0], b[0][1], sw + b_lane + ks * 32);
-      } else {
+    for (int ks = 0; ks < C4_KS; ++ks) {
+      unsigned b[4][2];
 #pragma unroll
-        for (int j = 0; j < S::NF; j += 2) {
-          unsigned r[4];
-          ldmatrix4(r, sw + b_lane + j * 8 * S::WPITCH * 2 + ks * 32);
-          b[j][0] = r[0]; b[j][1] = r[1]; b[j + 1][0] = r[2]; b[j + 1][1] = r[3];
-        }
+      for (int j = 0; j < 4; j += 2) {
+        unsigned r[4];
+        ldmatrix4(r, sw + b_lane + j * 8 * C4_PITCH * 2 + ks * 32);
+        b[j][0] = r[0]; b[j][1] = r[1]; b[j + 1][0] = r[2]; b[j + 1][1] = r[3];
       }
+      // The thread's channel pairs belong to taps 4 ks + tig / 2 and 4 ks + 2 +
+      // tig / 2 (zero beyond tap 8).
+      const int t0 = ks * 4 + (tig >> 1), t1 = t0 + 2;
+      const unsigned o0 = (t0 / 3) * C4_ROW + (t0 % 3) * PX_BYTES;
+      const unsigned o1 = (t1 / 3) * C4_ROW + (t1 % 3) * PX_BYTES;
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
+        const unsigned px = arow + (m >> 1) * C4_ROW + ((m & 1) * 16 + g) * PX_BYTES + (tig & 1) * 4;
         unsigned a[4];
-        const unsigned mt = arow + (m >> 1) * S::ROW + (m & 1) * 16 * PX_BYTES;
-        if constexpr (CIN == 32) {
-          const int tap = ks >> 1;
-          ldmatrix4(a, mt + a_lane + (tap / 3) * S::ROW + (tap % 3) * PX_BYTES +
-                           (ks & 1) * 2 * (CT_HX * PX_BYTES));
-        } else {
-          // k = tap * 4 + ci: the thread's channel pairs belong to taps
-          // 4 ks + tig / 2 and 4 ks + 2 + tig / 2 (zero beyond tap 8)
-          const int t0 = ks * 4 + (tig >> 1), t1 = t0 + 2;
-          const unsigned px = mt + g * PX_BYTES + (tig & 1) * 4;
-          const unsigned o0 = (t0 / 3) * S::ROW + (t0 % 3) * PX_BYTES;
-          const unsigned o1 = (t1 / 3) * S::ROW + (t1 % 3) * PX_BYTES;
-          a[0] = t0 < 9 ? lds32(px + o0) : 0u;
-          a[1] = t0 < 9 ? lds32(px + 8 * PX_BYTES + o0) : 0u;
-          a[2] = t1 < 9 ? lds32(px + o1) : 0u;
-          a[3] = t1 < 9 ? lds32(px + 8 * PX_BYTES + o1) : 0u;
-        }
+        a[0] = t0 < 9 ? lds32(px + o0) : 0u;
+        a[1] = t0 < 9 ? lds32(px + 8 * PX_BYTES + o0) : 0u;
+        a[2] = t1 < 9 ? lds32(px + o1) : 0u;
+        a[3] = t1 < 9 ? lds32(px + 8 * PX_BYTES + o1) : 0u;
 #pragma unroll
-        for (int j = 0; j < S::NF; ++j) mma_bf16(acc[m][j], a, b[j][0], b[j][1]);
+        for (int j = 0; j < 4; ++j) mma_bf16(acc[m][j], a, b[j][0], b[j][1]);
       }
     }
     __syncthreads();  // the tile is free again
@@ -262,39 +363,12 @@ __global__ void __launch_bounds__(CT_T, CONV_CTAS_PER_SM)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int x = x0 + (m & 1) * 16 + h * 8 + g;
-        const bool in_image = y < H && x < W;
-        unsigned pos = 0u;  // positive channels of this pixel (this thread's)
+        if (y >= H || x >= W) continue;
 #pragma unroll
-        for (int j = 0; j < S::NF; ++j) {
-          if (!in_image) continue;
-          const float v0 = acc[m][j][2 * h], v1 = acc[m][j][2 * h + 1];
-          if constexpr (EPI == EPI_LINEAR_F32) {
-            const int c = j * 8 + tig * 2;
-            if (c < COUT)
-              *reinterpret_cast<float2*>(out_f + ((long long)y * W + x) * COUT + c) =
-                  make_float2(v0 + bs[j][0], v1 + bs[j][1]);
-          } else {
-            const long long o = (((long long)y * S::NF + j) * W + x) * 8 + tig * 2;
-            float r0, r1;
-            if constexpr (EPI == EPI_RELU_BF16) {
-              r0 = fmaxf(v0 + bs[j][0], 0.f);
-              r1 = fmaxf(v1 + bs[j][1], 0.f);
-            } else {
-              r0 = v0 * (keep[m][h] & (0x8000u >> j) ? 1.f : 0.f);
-              r1 = v1 * (keep[m][h] & (0x80000000u >> j) ? 1.f : 0.f);
-            }
-            const __nv_bfloat162 r = __floats2bfloat162_rn(r0, r1);
-            *reinterpret_cast<__nv_bfloat162*>(out_bf + o) = r;
-            if (EPI == EPI_RELU_BF16)
-              pos |= positive_bits(r) >> j;
-          }
-        }
-        if (EPI == EPI_RELU_BF16 && bits_out) {  // (uniform over the grid)
-          pos >>= 4 * tig;
-          pos |= __shfl_xor_sync(0xffffffffu, pos, 1);
-          pos |= __shfl_xor_sync(0xffffffffu, pos, 2);
-          if (tig == 0 && in_image) bits_out[(long long)y * W + x] = pos;
-        }
+        for (int j = 0; j < 4; ++j)
+          *reinterpret_cast<__nv_bfloat162*>(out + (((long long)y * 4 + j) * W + x) * 8 + tig * 2) =
+              __floats2bfloat162_rn(acc[m][j][2 * h] * (keep[m][h] & (0x8000u >> j) ? 1.f : 0.f),
+                                    acc[m][j][2 * h + 1] * (keep[m][h] & (0x80000000u >> j) ? 1.f : 0.f));
       }
     }
   }
@@ -1038,9 +1112,11 @@ struct lbm_cnn {
   __nv_bfloat16* dz[2] = {};    // ping-pong output gradients (32 channels)
   __nv_bfloat16* dz5 = nullptr; // output gradients of the last layer: 4 channels and 4 zeros
   __nv_bfloat16* xs = nullptr;  // input features as three BF16 parts (16 channels)
-  CUtensorMap m_act[NL], m_dz[2], m_dz5, m_xs;  // tiles with halo of act[1..], dz[], dz5, xs
-  CUtensorMap g_dz[2], g_dz5;   // the same tiles without halo
-  int tiles_x = 0, ntiles = 0;  // convolution tiles
+  CUtensorMap c_act[NL], c_dz[2];        // convolution tiles with halo of act[1..], dz[]
+  CUtensorMap m_act[NL], m_dz5, m_xs;    // weight-gradient tiles with halo of act[1..], dz5, xs
+  CUtensorMap g_dz[2], g_dz5;            // the same without halo of dz[], dz5
+  int tiles_x = 0, ntiles = 0;    // weight-gradient tiles
+  int ctiles_x = 0, cntiles = 0;  // convolution tiles
   int sms = 0;
   LogEntry* logs = nullptr;     // table of log32
   ExpEntry* exps = nullptr;     // table of exp32
@@ -1096,15 +1172,14 @@ int fetch_results(lbm_cnn* n) {
 }
 
 // Tensor map of a row-planar BF16 image of `ncg` channel groups: dims (x in
-// 32-bit words, channel group, row); box = one tile of `box_cg` groups (those
-// beyond ncg are zero fill), with its halo or without.
-int encode_image(lbm_cnn* n, const void* p, int ncg, int box_cg, bool halo, CUtensorMap* out) {
+// 32-bit words, channel group, row); box = `px` pixels of `rows` rows and
+// `box_cg` groups (those beyond ncg are zero fill).
+int encode_image(lbm_cnn* n, const void* p, int ncg, int box_cg, int px, int rows, CUtensorMap* out) {
   gbtma::EncodeTiledFn enc = gbtma::tensor_map_encoder();
   if (!enc) return cfail(n, LBM_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
   const cuuint64_t dims[3] = {(cuuint64_t)n->W * 4, (cuuint64_t)ncg, (cuuint64_t)n->H};
   const cuuint64_t strides[2] = {(cuuint64_t)n->W * PX_BYTES, (cuuint64_t)n->W * PX_BYTES * ncg};
-  const cuuint32_t box[3] = {4u * (halo ? CT_HX : CT_X), (cuuint32_t)box_cg,
-                             (cuuint32_t)(halo ? CT_HY : CT_Y)};
+  const cuuint32_t box[3] = {4u * (cuuint32_t)px, (cuuint32_t)box_cg, (cuuint32_t)rows};
   const cuuint32_t es[3] = {1, 1, 1};
   const CUresult r = enc(out, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<void*>(p), dims, strides, box,
                          es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -1114,12 +1189,12 @@ int encode_image(lbm_cnn* n, const void* p, int ncg, int box_cg, bool halo, CUte
   return LBM_OK;
 }
 
-template <int CIN, int COUT, int EPI>
+template <int COUT, int EPI>
 int conv(lbm_cnn* n, const CUtensorMap& in, const __nv_bfloat16* wt, const float* bias,
-          const unsigned* bits_in, __nv_bfloat16* ob, float* of, unsigned* bits_out = nullptr) {
-  const int grid = std::min(n->ntiles, CONV_CTAS_PER_SM * n->sms);
-  CCK(n, gbtma::launch_overlapped(k_conv<CIN, COUT, EPI>, grid, CT_T, ConvShape<CIN, COUT>::SMEM, n->stream, in,
-                                  n->H, n->W, n->tiles_x, n->ntiles, wt, bias, bits_in, ob, of, bits_out,
+         const unsigned* bits_in, __nv_bfloat16* ob, float* of, unsigned* bits_out = nullptr) {
+  const int grid = std::min(n->cntiles, CV_CTAS_PER_SM * n->sms);
+  CCK(n, gbtma::launch_overlapped(k_conv<COUT, EPI>, grid, CV_T, cv_smem(COUT), n->stream, in, n->H, n->W,
+                                  n->ctiles_x, n->cntiles, wt, bias, bits_in, ob, of, bits_out,
                                   &n->res->timeout));
   return LBM_OK;
 }
@@ -1133,10 +1208,10 @@ int forward(lbm_cnn* n, const double* coarse, bool train) {
   const float* w = n->w;
   CCK(n, gbtma::launch_overlapped(k_conv0, (n->H * ((n->W + 1) / 2) + C0_T - 1) / C0_T, C0_T, 0, n->stream,
                                   n->xf, n->H, n->W, w + param_offset(0), n->act[1], bits(1)));
-  if ((rc = conv<32, 32, EPI_RELU_BF16>(n, n->m_act[1], n->wt[1], w + param_offset(1) + wsize(1), nullptr, n->act[2], nullptr, bits(2))) != LBM_OK) return rc;
-  if ((rc = conv<32, 32, EPI_RELU_BF16>(n, n->m_act[2], n->wt[2], w + param_offset(2) + wsize(2), nullptr, n->act[3], nullptr, bits(3))) != LBM_OK) return rc;
-  if ((rc = conv<32, 32, EPI_RELU_BF16>(n, n->m_act[3], n->wt[3], w + param_offset(3) + wsize(3), nullptr, n->act[4], nullptr, bits(4))) != LBM_OK) return rc;
-  if ((rc = conv<32, 4, EPI_LINEAR_F32>(n, n->m_act[4], n->wt[4], w + param_offset(4) + wsize(4), nullptr, nullptr, n->z)) != LBM_OK) return rc;
+  if ((rc = conv<32, EPI_RELU_BF16>(n, n->c_act[1], n->wt[1], w + param_offset(1) + wsize(1), nullptr, n->act[2], nullptr, bits(2))) != LBM_OK) return rc;
+  if ((rc = conv<32, EPI_RELU_BF16>(n, n->c_act[2], n->wt[2], w + param_offset(2) + wsize(2), nullptr, n->act[3], nullptr, bits(3))) != LBM_OK) return rc;
+  if ((rc = conv<32, EPI_RELU_BF16>(n, n->c_act[3], n->wt[3], w + param_offset(3) + wsize(3), nullptr, n->act[4], nullptr, bits(4))) != LBM_OK) return rc;
+  if ((rc = conv<4, EPI_LINEAR_F32>(n, n->c_act[4], n->wt[4], w + param_offset(4) + wsize(4), nullptr, nullptr, n->z)) != LBM_OK) return rc;
   return LBM_OK;
 }
 
@@ -1164,13 +1239,15 @@ int loss_backward(lbm_cnn* n, const double* target, bool adam) {
   auto part = [&](int l) { return const_cast<float*>(U.part[l]); };
   // layer 5 (32 -> 4): dz5 holds d loss / d z5
   if ((rc = wgrad<4, 4>(n, n->m_act[4], n->g_dz5, part(4))) != LBM_OK) return rc;
-  if ((rc = conv<4, 32, EPI_MASK_BF16>(n, n->m_dz5, n->wb[4], nullptr, n->pos[4], n->dz[1], nullptr)) != LBM_OK) return rc;
+  CCK(n, gbtma::launch_overlapped(k_conv4, std::min(n->ntiles, C4_CTAS_PER_SM * n->sms), CT_T, C4_SMEM, n->stream,
+                                  n->m_dz5, n->H, n->W, n->tiles_x, n->ntiles, n->wb[4], n->pos[4], n->dz[1],
+                                  &n->res->timeout));
   if ((rc = wgrad<4, 32>(n, n->m_act[3], n->g_dz[1], part(3))) != LBM_OK) return rc;
-  if ((rc = conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[1], n->wb[3], nullptr, n->pos[3], n->dz[0], nullptr)) != LBM_OK) return rc;
+  if ((rc = conv<32, EPI_MASK_BF16>(n, n->c_dz[1], n->wb[3], nullptr, n->pos[3], n->dz[0], nullptr)) != LBM_OK) return rc;
   if ((rc = wgrad<4, 32>(n, n->m_act[2], n->g_dz[0], part(2))) != LBM_OK) return rc;
-  if ((rc = conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[0], n->wb[2], nullptr, n->pos[2], n->dz[1], nullptr)) != LBM_OK) return rc;
+  if ((rc = conv<32, EPI_MASK_BF16>(n, n->c_dz[0], n->wb[2], nullptr, n->pos[2], n->dz[1], nullptr)) != LBM_OK) return rc;
   if ((rc = wgrad<4, 32>(n, n->m_act[1], n->g_dz[1], part(1))) != LBM_OK) return rc;
-  if ((rc = conv<32, 32, EPI_MASK_BF16>(n, n->m_dz[1], n->wb[1], nullptr, n->pos[1], n->dz[0], nullptr)) != LBM_OK) return rc;
+  if ((rc = conv<32, EPI_MASK_BF16>(n, n->c_dz[1], n->wb[1], nullptr, n->pos[1], n->dz[0], nullptr)) != LBM_OK) return rc;
   if ((rc = wgrad<2, 32>(n, n->m_xs, n->g_dz[0], part(0))) != LBM_OK) return rc;
   U.nblocks = n->wblocks;
   U.w = n->w;
@@ -1221,13 +1298,15 @@ int lbm_cnn_create(int H, int W, void* cuda_stream, lbm_cnn** out) {
   allow((const void*)k_wgrad<4, 32>, WgShape<4, 32>::SMEM);
   allow((const void*)k_wgrad<4, 4>, WgShape<4, 16>::SMEM);
   allow((const void*)k_wgrad<2, 32>, WgShape<2, 32>::SMEM);
-  allow((const void*)k_conv<32, 32, EPI_RELU_BF16>, ConvShape<32, 32>::SMEM);
-  allow((const void*)k_conv<32, 32, EPI_MASK_BF16>, ConvShape<32, 32>::SMEM);
-  allow((const void*)k_conv<32, 4, EPI_LINEAR_F32>, ConvShape<32, 4>::SMEM);
-  allow((const void*)k_conv<4, 32, EPI_MASK_BF16>, ConvShape<4, 32>::SMEM);
+  allow((const void*)k_conv<32, EPI_RELU_BF16>, cv_smem(32));
+  allow((const void*)k_conv<32, EPI_MASK_BF16>, cv_smem(32));
+  allow((const void*)k_conv<4, EPI_LINEAR_F32>, cv_smem(4));
+  allow((const void*)k_conv4, C4_SMEM);
   n->sms = std::max(sms, 1);
   n->tiles_x = (W + CT_X - 1) / CT_X;
   n->ntiles = n->tiles_x * ((H + CT_Y - 1) / CT_Y);
+  n->ctiles_x = (W + CV_X - 1) / CV_X;
+  n->cntiles = n->ctiles_x * ((H + CV_Y - 1) / CV_Y);
   n->wblocks = std::min(n->ntiles, WG_CTAS_PER_SM * n->sms);
   auto A = [&](void** p, size_t bytes) {
     if (e == cudaSuccess) e = cudaMalloc(p, bytes);
@@ -1270,14 +1349,20 @@ int lbm_cnn_create(int H, int W, void* cuda_stream, lbm_cnn** out) {
     return e == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA;
   }
   int rc = LBM_OK;
-  for (int l = 1; l < NL && rc == LBM_OK; ++l) rc = encode_image(n, n->act[l], 4, 4, true, &n->m_act[l]);
-  for (int k = 0; k < 2; ++k) {
-    if (rc == LBM_OK) rc = encode_image(n, n->dz[k], 4, 4, true, &n->m_dz[k]);
-    if (rc == LBM_OK) rc = encode_image(n, n->dz[k], 4, 4, false, &n->g_dz[k]);
+  auto map = [&](const void* p, int ncg, int box_cg, int px, int rows, CUtensorMap* out) {
+    if (rc == LBM_OK) rc = encode_image(n, p, ncg, box_cg, px, rows, out);
+  };
+  for (int l = 1; l < NL; ++l) {
+    map(n->act[l], 4, 4, CV_HX, CV_HY, &n->c_act[l]);
+    map(n->act[l], 4, 4, CT_HX, CT_HY, &n->m_act[l]);
   }
-  if (rc == LBM_OK) rc = encode_image(n, n->dz5, 1, 1, true, &n->m_dz5);
-  if (rc == LBM_OK) rc = encode_image(n, n->dz5, 1, 2, false, &n->g_dz5);
-  if (rc == LBM_OK) rc = encode_image(n, n->xs, 2, 2, true, &n->m_xs);
+  for (int k = 0; k < 2; ++k) {
+    map(n->dz[k], 4, 4, CV_HX, CV_HY, &n->c_dz[k]);
+    map(n->dz[k], 4, 4, CT_X, CT_Y, &n->g_dz[k]);
+  }
+  map(n->dz5, 1, 1, CT_HX, CT_HY, &n->m_dz5);
+  map(n->dz5, 1, 2, CT_X, CT_Y, &n->g_dz5);
+  map(n->xs, 2, 2, CT_HX, CT_HY, &n->m_xs);
   if (rc != LBM_OK || pack_all(n) != LBM_OK) {
     g_cnn_error = n->err;
     lbm_cnn_destroy(n);
