@@ -313,7 +313,8 @@ int launch_persistent(lbm_ctx* c, cudaStream_t s, int from, void* fout, const St
   const R* fi = (const R*)c->f[from];
   const CUtensorMap& tm = c->tmap[from];
   if (A.nblocks >= A.ntiles) {
-    CK(c, launch_overlapped(c->wide ? k_step<R, long long, VAR> : k_step<R, unsigned, VAR>, A.ntiles, blk, 0, s,
+    CK(c, launch_overlapped(c->wide ? k_step<R, long long, VAR> : k_step<R, unsigned, VAR>, A.ntiles, blk,
+                            tile_dynamic_bytes<R>(), s,
                             tm, fi, (R*)fout, A));
   } else {
     CK(c, launch_overlapped(c->wide ? k_step_pipe<R, long long, VAR> : k_step_pipe<R, unsigned, VAR>, A.nblocks,
@@ -346,6 +347,11 @@ cudaError_t allow_pipe_smem() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_step_pipe<R, long long, VAR>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+  const int t = (int)tile_dynamic_bytes<R>();
+  if (e == cudaSuccess && t > 0)
+    e = cudaFuncSetAttribute(k_step<R, unsigned, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, t);
+  if (e == cudaSuccess && t > 0)
+    e = cudaFuncSetAttribute(k_step<R, long long, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, t);
   return e;
 }
 

@@ -42,22 +42,28 @@ template <> struct Shape<float> {
 template <> struct Shape<double> {
   static constexpr int X = 32, Y = 2, TY = 2, MINB = 8, MINB_PIPE = 6;
 };
-// Double-word (LBM_DF64): 32 x 4 tiles of 8-byte elements (below the 48 KB
-// of static shared memory), FP32-ALU-bound. LBM_DW_LANES = 1: one node per
-// thread; 2: two rows per thread in paired f32x2 instructions (half the
-// instructions issued, twice the registers; the FP32 units retire the same
-// lanes per clock either way).
+// Double-word (LBM_DF64): 32 x 8 tiles of 8-byte elements (51 KB, in dynamic
+// shared memory), FP32-ALU-bound. LBM_DW_LANES = 1: one node per thread; 2: two
+// rows per thread in paired f32x2 instructions (half the instructions issued,
+// twice the registers; the FP32 units retire the same lanes per clock either
+// way). The update is 56 KB of straight-line code: with 32 x 4 tiles, a warp of
+// each of four unrelated blocks per scheduler, half the issue stalls were
+// instruction fetches (ncu: no_instruction 2.9 of 6.0 cycles per issue); the two
+// warps per scheduler of a 256-thread block run close behind each other and
+// share them. 2048 x 1024 301 -> 273 us a step, 600 x 200 26.8 -> 25.9, 300 x 100
+// 17.1 -> 17.5; 32 x 16 tiles (one block per SM, the copy of its next tile only
+// from the persistent form) 299, persistent 260-292; barriers inside the update
+// to keep a block's warps together cost registers (spills) and took 282-288.
 #ifndef LBM_DW_LANES
 #define LBM_DW_LANES 1
 #endif
-// Blocks per SM of the one-tile double-word form (4: 128 registers, no
-// spills; 5 spills in the node update).
+// Blocks per SM of the double-word forms (2: 128 registers, no spills).
 #ifndef LBM_DW_MINB
-#define LBM_DW_MINB 4
+#define LBM_DW_MINB 2
 #endif
 template <> struct Shape<dw> {
-  static constexpr int X = 32, Y = 4, TY = Y / LBM_DW_LANES;
-  static constexpr int MINB = LBM_DW_LANES == 1 ? LBM_DW_MINB : 6, MINB_PIPE = 3;
+  static constexpr int X = 32, Y = 8, TY = Y / LBM_DW_LANES;
+  static constexpr int MINB = LBM_DW_MINB * LBM_DW_LANES, MINB_PIPE = 2;
   static_assert(LBM_DW_LANES == 1 || LBM_DW_LANES == 2, "one or two nodes per thread");
 };
 constexpr int AUX_X = 32, AUX_Y = 8, AUX_N = AUX_X * AUX_Y;  // init / moments / audit

@@ -222,12 +222,23 @@ constexpr int step_minb() {
   return (sizeof(R) == 4 && sizeof(Off) == 8) ? Shape<R>::MINB - 1 : Shape<R>::MINB;
 }
 
+template <typename R>
+__host__ __device__ constexpr size_t tile_dynamic_bytes() {
+  return Tile<R>::BYTES <= 46 * 1024 ? 0 : (size_t)Tile<R>::BYTES + 128;
+}
+
 template <typename R, typename Off, int VAR = 0>
 __global__ void __launch_bounds__(Shape<R>::X * Shape<R>::TY, (step_minb<R, Off>()))
     k_step(const __grid_constant__ CUtensorMap tmap, const R* __restrict__ fin,
            R* __restrict__ fout, const StepArgs<R> A) {
   constexpr int N = Shape<R>::X * Shape<R>::TY;
-  __shared__ __align__(128) R tile[Tile<R>::ELEMS];
+  // The tile in static shared memory where it fits there (48 KB), else in
+  // dynamic (tile_dynamic_bytes).
+  constexpr bool DYN = tile_dynamic_bytes<R>() > 0;
+  __shared__ __align__(128) R tile_static[DYN ? 1 : Tile<R>::ELEMS];
+  extern __shared__ __align__(128) unsigned char step_smem[];
+  R* const tile = DYN ? reinterpret_cast<R*>(step_smem + ((128u - (smem_addr(step_smem) & 127u)) & 127u))
+                      : tile_static;
   __shared__ double sm[N / 4][4];
   __shared__ unsigned long long bar;
   __shared__ unsigned long long s_step;
