@@ -363,7 +363,10 @@ __device__ __forceinline__ R collide(const Coeffs<KT>& K, const Groups<R>& d,
 // 259 and the checks' 6 (which are integer operations now). Deviations are
 // relaxed, as in collide(), so that what is conserved does not depend on the
 // rounding of the relaxation matrices. K's relaxation columns are those of
-// scale_relaxation().
+// scale_relaxation(). Where a product meets a sum it is written as fma or kept
+// apart (__dmul_rn, __dadd_rn), not left to the compiler, so that k_step_lanes
+// (lbm_lanes.cuh), which computes the same operations in other lanes,
+// gives the same bits.
 struct Node64 {
   double rho, jx, jy, e2, p2;  // e2 = 2 e, p2 = 2 rho T
 };
@@ -380,11 +383,11 @@ __device__ __forceinline__ Node64 collide64(const Coeffs<double>& K, const Group
   const double ux = m.jx * r, uy = m.jy * r;
   const double a = m.jx * ux;
   const double k2 = fma(m.jy, uy, a);       // rho u^2
-  const double m5 = fma(-m.jy, uy, a), m6 = m.jx * uy, m6x2 = m6 + m6;
+  const double m5 = fma(-m.jy, uy, a), m6 = m.jx * uy, m6x2 = __dadd_rn(m6, m6);
   m.p2 = m.e2 - k2;
   const double h2 = m.e2 + m.p2;            // 2 (e + P)
   const double er2 = m.e2 * r, usq = k2 * r;
-  const double nA = fma(-3.0, er2, usq + usq);  // -(6 e / rho - 2 u^2)
+  const double nA = fma(-3.0, er2, __dadd_rn(usq, usq));  // -(6 e / rho - 2 u^2)
   // 4 d11 = 4 m11 - (8 e^2 / rho - (rho u^2)^2 / rho), 1 d12
   const double su = fma(1296.0, d.S[1], d.S[0]), sv = fma(5.0625, d.S[3], d.S[2]);
   const double d11 = fma(k2, usq, fma(-(m.e2 + m.e2), er2, fma(16.0, sv, su)));
@@ -392,7 +395,7 @@ __device__ __forceinline__ Node64 collide64(const Coeffs<double>& K, const Group
   const double d5 = fma(36.0, d.C[1], d.C[0]) - m5;
   const double d13 = fma(nA, m5, fma(1296.0, d.C[1], d.C[0]));
   const double d6 = fma(-0.5, m6, fma(2.25, d.C[3], d.C[2]));                 // d6 / 2
-  const double d14 = fma(0.125 * nA, m6, fma(5.0625, d.C[3], d.C[2]));        // d14 / 8
+  const double d14 = fma(__dmul_rn(0.125, nA), m6, fma(5.0625, d.C[3], d.C[2]));        // d14 / 8
   const double xu = fma(216.0, d.X[1], d.X[0]), xv = fma(3.375, d.X[3], d.X[2]);
   const double d7 = fma(-h2, ux, fma(R2x4, xv, xu));                          // 2 d7
   const double d9 = fma(m6x2, uy, fma(-m5, ux, fma(-R2x4, xv, xu)));
@@ -404,14 +407,15 @@ __device__ __forceinline__ Node64 collide64(const Coeffs<double>& K, const Group
   double S[4], C[4], X[4], Y[4];
 #pragma unroll
   for (int g = 0; g < 4; ++g) {
-    S[g] = K.K0[g][0] * d11 + K.K0[g][1] * d12;
-    X[g] = K.KX[g][0] * d7 + K.KX[g][1] * d9 + K.KX[g][2] * d15;
-    Y[g] = K.KY[g][0] * d8 + K.KY[g][1] * d10 + K.KY[g][2] * d16;
+    S[g] = fma(K.K0[g][1], d12, __dmul_rn(K.K0[g][0], d11));
+    X[g] = fma(K.KX[g][2], d15, fma(K.KX[g][1], d9, __dmul_rn(K.KX[g][0], d7)));
+    Y[g] = fma(K.KY[g][2], d16, fma(K.KY[g][1], d10, __dmul_rn(K.KY[g][0], d8)));
   }
-  C[0] = K.KC[0][0] * d5 + K.KC[0][1] * d13;
-  C[1] = K.KC[1][0] * d5 + K.KC[1][1] * d13;
-  C[2] = K.KS[0][0] * d6 + K.KS[0][1] * d14;
-  C[3] = K.KS[1][0] * d6 + K.KS[1][1] * d14;
+#pragma unroll
+  for (int g = 0; g < 2; ++g) {
+    C[g] = fma(K.KC[g][1], d13, __dmul_rn(K.KC[g][0], d5));
+    C[2 + g] = fma(K.KS[g][1], d14, __dmul_rn(K.KS[g][0], d6));
+  }
   inverse_transform(S, C, X, Y, df);
   return m;
 }

@@ -216,6 +216,7 @@ struct lbm_ctx {
   double* partial = nullptr;
   double* gpartial = nullptr;     // audit group sums (audit_block_done)
   unsigned* gcount = nullptr;     // audit group counters
+  unsigned* tcount = nullptr;     // audit tile counters (k_step_lanes contexts)
   int ngroups = 0;
   int agroup = 0;                 // tiles per audit group
   double* staging = nullptr;
@@ -225,6 +226,7 @@ struct lbm_ctx {
   int sms = 0;          // multiprocessors of the device
   dim3 grid, aux_grid;  // step grid; init / moments / audit grid
   bool wide = false;    // 64-bit element offsets needed
+  bool lanes = false;   // FP64 step with four lanes per node (k_step_lanes)
   Coeffs<double> Kd;
   CUtensorMap tmap[2];        // TMA descriptors of the two population buffers
   bool tc = false;            // tensor-core transforms (LBM_TC_TF32X3)
@@ -293,6 +295,8 @@ StepArgs<R> make_args(lbm_ctx* c, int slot) {
   A.geq = (const R*)c->geq;
   A.geq3 = c->dwp ? (const float*)((const dw*)c->geq + 64) : nullptr;
   A.st = c->st;
+  A.cons = c->staging;
+  A.tcount = c->tcount;
   A.partial = c->partial;
   A.gpartial = c->gpartial;
   A.gcount = c->gcount;
@@ -323,8 +327,15 @@ int launch_persistent(lbm_ctx* c, cudaStream_t s, int from, void* fout, const St
   return LBM_OK;
 }
 
+int launch_lanes(lbm_ctx* c, cudaStream_t s, int from, void* fout, const StepArgs<double>& A) {
+  CK(c, launch_overlapped(k_step_lanes, c->ntiles * LANES_BLOCKS, LANES_T, 0, s,
+                          (const double*)c->f[from], (double*)fout, A));
+  return LBM_OK;
+}
+
 int launch_step(lbm_ctx* c, cudaStream_t s, int from) {
   const int to = 1 - from;
+  if (c->lanes) return launch_lanes(c, s, from, c->f[to], make_args<double>(c, from));
   if (c->tc) {
     CK(c, tc_launch(c->tmap[from], (const float*)c->f[from], (float*)c->f[to],
                     make_args<float>(c, from), c->tc_b, c->tc_w, c->grid, s));
@@ -336,8 +347,17 @@ int launch_step(lbm_ctx* c, cudaStream_t s, int from) {
   return launch_persistent<float>(c, s, from, c->f[to], make_args<float>(c, from));
 }
 
-// Blocks of a step launch when none were chosen: one per tile (k_step).
+// Blocks of a step launch when none were chosen: one per tile (k_step); FP64
+// grids of few nodes then take k_step_lanes.
 int default_blocks(const lbm_ctx* c) { return c->ntiles; }
+bool few_nodes(const lbm_ctx* c) {
+  const lbm_config& C = c->cfg;
+  const long long nodes = (long long)C.nx * C.ny;
+  long long edge = 0;  // nodes next to a side that is not periodic
+  for (int s = 0; s < 4; ++s)
+    if (C.bc[s].kind != LBM_BC_PERIODIC) edge += s < 2 ? C.ny : C.nx;
+  return C.precision == LBM_FP64 && nodes <= LANES_MAX_NODES && (nodes <= LANES_THIN || 8 * edge <= nodes);
+}
 
 template <typename R, int VAR = 0>
 cudaError_t allow_pipe_smem() {
@@ -602,6 +622,7 @@ int lbm_create(const lbm_config* cfg, void* cuda_stream, lbm_ctx** out) {
     if (e == cudaSuccess) e = tc_prepare();
   } else {
     c->nblocks = default_blocks(c);
+    c->lanes = few_nodes(c);
     c->grid = dim3(c->nblocks);
     if (e == cudaSuccess)
       e = c->dwp ? allow_pipe_smem<dw>()
@@ -621,6 +642,10 @@ int lbm_create(const lbm_config* cfg, void* cuda_stream, lbm_ctx** out) {
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->gpartial, sizeof(double) * 4 * c->ngroups);
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->gcount, sizeof(unsigned) * c->ngroups);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->gcount, 0, sizeof(unsigned) * c->ngroups, c->stream);
+  if (e == cudaSuccess && c->lanes) {
+    e = cudaMalloc((void**)&c->tcount, sizeof(unsigned) * c->ntiles);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->tcount, 0, sizeof(unsigned) * c->ntiles, c->stream);
+  }
   if (e == cudaSuccess)
     e = cudaMalloc((void**)&c->staging, sizeof(double) * 4 * (size_t)C.nx * C.ny);
   if (e == cudaSuccess && c->tc) {
@@ -805,6 +830,7 @@ int lbm_destroy(lbm_ctx* c) {
   if (c->partial) cudaFree(c->partial);
   if (c->gpartial) cudaFree(c->gpartial);
   if (c->gcount) cudaFree(c->gcount);
+  if (c->tcount) cudaFree(c->tcount);
   if (c->staging) cudaFree(c->staging);
   if (c->pstage) cudaFree(c->pstage);
   if (c->tc_b) cudaFree(c->tc_b);
@@ -940,7 +966,7 @@ namespace {
 
 // Sets the number of blocks of the step launch: later steps are issued with
 // `g` blocks and the captured graphs are rebuilt.
-int apply_blocks(lbm_ctx* c, int g) {
+int apply_blocks(lbm_ctx* c, int g, bool lanes = false) {
   CK(c, cudaStreamSynchronize(c->stream));
   for (int k = 0; k < 2; ++k)
     if (c->graph[k]) {
@@ -948,6 +974,7 @@ int apply_blocks(lbm_ctx* c, int g) {
       c->graph[k] = nullptr;
     }
   c->nblocks = g;
+  c->lanes = lanes;
   c->grid = dim3(g);
   return LBM_OK;
 }
@@ -957,7 +984,7 @@ int apply_blocks(lbm_ctx* c, int g) {
 // state, the step counter and the audit log are untouched. Mean ms / launch.
 template <typename R, int VAR = 0>
 int time_blocks(lbm_ctx* c, int g, int launches, DevStatus* scratch, cudaEvent_t e0,
-                cudaEvent_t e1, float* ms) {
+                cudaEvent_t e1, float* ms, bool lanes = false) {
   CK(c, cudaMemsetAsync(scratch, 0, offsetof(DevStatus, audit_totals), c->stream));
   StepArgs<R> A = make_args<R>(c, 0);
   A.st = scratch;
@@ -966,7 +993,12 @@ int time_blocks(lbm_ctx* c, int g, int launches, DevStatus* scratch, cudaEvent_t
   for (int j = 0; j < 2 + launches; ++j) {
     if (j == 2) CK(c, cudaEventRecord(e0, c->stream));
     A.slot = j & 1;
-    const int rc = launch_persistent<R, VAR>(c, c->stream, c->cur, c->f[1 - c->cur], A);
+    int rc;
+    if constexpr (std::is_same<R, double>::value)
+      rc = lanes ? launch_lanes(c, c->stream, c->cur, c->f[1 - c->cur], A)
+                 : launch_persistent<R, VAR>(c, c->stream, c->cur, c->f[1 - c->cur], A);
+    else
+      rc = launch_persistent<R, VAR>(c, c->stream, c->cur, c->f[1 - c->cur], A);
     if (rc != LBM_OK) return rc;
   }
   CK(c, cudaEventRecord(e1, c->stream));
@@ -984,7 +1016,8 @@ int lbm_set_step_blocks(lbm_ctx* c, int blocks) {
   if (!c) return fail(nullptr, LBM_ERR_INVALID, "ctx is NULL");
   if (blocks < 0) return fail(c, LBM_ERR_INVALID, "blocks < 0");
   if (c->tc) return fail(c, LBM_ERR_UNSUPPORTED, "the tensor-core step sets its own launch");
-  return apply_blocks(c, blocks == 0 ? default_blocks(c) : std::min(blocks, c->ntiles));
+  return blocks == 0 ? apply_blocks(c, default_blocks(c), few_nodes(c))
+                     : apply_blocks(c, std::min(blocks, c->ntiles));
 }
 
 int lbm_step_blocks(lbm_ctx* c) { return c ? c->nblocks : -1; }
@@ -1004,7 +1037,7 @@ int lbm_autotune(lbm_ctx* c, int launches) {
   if (!c) return fail(nullptr, LBM_ERR_INVALID, "ctx is NULL");
   if (launches < 1) return fail(c, LBM_ERR_INVALID, "launches < 1");
   if (c->tc) return LBM_OK;  // nothing to choose
-  // Candidates: one tile per block (k_step), and for k_step_pipe 1 ..
+  // Candidates: (few FP64 nodes) k_step_lanes, one tile per block (k_step), and for k_step_pipe 1 ..
   // MINB_PIPE blocks per SM and ceil(ntiles / m) blocks for m = 2 .. 8 tiles
   // per block.
   const int per_sm = c->dwp ? Shape<dw>::MINB_PIPE
@@ -1034,12 +1067,21 @@ int lbm_autotune(lbm_ctx* c, int launches) {
       best = cand[i];
     }
   }
+  bool lanes = false;
+  if (rc == LBM_OK && few_nodes(c)) {
+    float ms = 0.f;
+    rc = time_blocks<double>(c, c->ntiles, launches, scratch, e0, e1, &ms, true);
+    if (rc == LBM_OK && ms < best_ms) {
+      lanes = true;
+      best = default_blocks(c);
+    }
+  }
   cudaStreamSynchronize(c->stream);
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   cudaFree(scratch);
   if (rc != LBM_OK) return rc;
-  return apply_blocks(c, best);
+  return apply_blocks(c, best, lanes);
 }
 
 const char* lbm_last_error(lbm_ctx* c) {

@@ -7,6 +7,8 @@
 #include <cuda.h>  // CUtensorMap (the encoder is fetched at run time; libcuda is not linked)
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "../../include/lbm.h"
 #include "coeffs.h"
 #include "d2v16.cuh"
@@ -103,6 +105,8 @@ struct StepArgs {
   const R* geq;       // [4][16] Dirichlet ghost populations
   const float* geq3;  // LBM_DF64: their third words; else unused
   DevStatus* st;
+  double* cons;       // k_step_lanes: [4][ny][nx] moments of an audit step
+  unsigned* tcount;   // k_step_lanes: [ntiles] blocks of the tile done in this audit step
   double* partial;    // [ntiles][4] audit scratch: one partial sum per tile
   double* gpartial;   // [ngroups][4]: the sums of groups of `agroup` tiles
   int agroup;         // tiles per audit group
@@ -319,6 +323,14 @@ struct Tile {
 // tile pointer `ctr` (population i at ctr[i * PS], rows BXP apart). Interior
 // nodes read the tile only; edge nodes wrap (periodic, global memory) or use
 // the ghost populations of their side.
+// a += k v. FP64: a fused multiply-add on every path (the compiler sinks the sums
+// of branches that join behind them and leaves products without a sum there),
+// so that interior and edge nodes, and k_step_lanes, round alike.
+template <typename R>
+__device__ __forceinline__ void add_term(R& a, R k, R v) {
+  if constexpr (std::is_same<R, double>::value) a = fma(k, v, a);
+  else a += k * v;
+}
 template <typename R, typename Off, int BXP>
 __device__ __forceinline__ void neighbour_terms(const StepArgs<R>& A, const R* __restrict__ fin,
                                                 const R* ctr, int PS, Off P, Off pitch, Off c,
@@ -329,12 +341,12 @@ __device__ __forceinline__ void neighbour_terms(const StepArgs<R>& A, const R* _
     for (int i = 0; i < 16; ++i) {
       R a = acc[i];
       if (has_x(i)) {
-        a += A.K.aW[i] * ctr[i * PS - 1];
-        a += A.K.aE[i] * ctr[i * PS + 1];
+        add_term(a, A.K.aW[i], ctr[i * PS - 1]);
+        add_term(a, A.K.aE[i], ctr[i * PS + 1]);
       }
       if (has_y(i)) {
-        a += A.K.aS[i] * ctr[i * PS - BXP];
-        a += A.K.aN[i] * ctr[i * PS + BXP];
+        add_term(a, A.K.aS[i], ctr[i * PS - BXP]);
+        add_term(a, A.K.aN[i], ctr[i * PS + BXP]);
       }
       acc[i] = a;
     }
@@ -344,69 +356,69 @@ __device__ __forceinline__ void neighbour_terms(const StepArgs<R>& A, const R* _
   if (x > 0) {
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-      if (has_x(i)) acc[i] += A.K.aW[i] * ctr[i * PS - 1];
+      if (has_x(i)) add_term(acc[i], A.K.aW[i], ctr[i * PS - 1]);
   } else if (A.bc[0] == LBM_BC_PERIODIC) {
     const Off n = c + (Off)(A.nx - 1);
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-      if (has_x(i)) acc[i] += A.K.aW[i] * fin[i * P + n];
+      if (has_x(i)) add_term(acc[i], A.K.aW[i], fin[i * P + n]);
   } else {
     R g[16];
     ghost(A, fin, P, 0, side_kind(A, 0, y, t), m, c + 1, A.nx > 1, g);
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-      if (has_x(i)) acc[i] += A.K.aW[i] * g[i];
+      if (has_x(i)) add_term(acc[i], A.K.aW[i], g[i]);
   }
   // x+ neighbour (east)
   if (x < A.nx - 1) {
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-      if (has_x(i)) acc[i] += A.K.aE[i] * ctr[i * PS + 1];
+      if (has_x(i)) add_term(acc[i], A.K.aE[i], ctr[i * PS + 1]);
   } else if (A.bc[1] == LBM_BC_PERIODIC) {
     const Off n = c - (Off)(A.nx - 1);
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-      if (has_x(i)) acc[i] += A.K.aE[i] * fin[i * P + n];
+      if (has_x(i)) add_term(acc[i], A.K.aE[i], fin[i * P + n]);
   } else {
     R g[16];
     ghost(A, fin, P, 1, side_kind(A, 1, y, t), m, c - 1, A.nx > 1, g);
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-      if (has_x(i)) acc[i] += A.K.aE[i] * g[i];
+      if (has_x(i)) add_term(acc[i], A.K.aE[i], g[i]);
   }
   // y- neighbour (south)
   if (y > 0) {
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-      if (has_y(i)) acc[i] += A.K.aS[i] * ctr[i * PS - BXP];
+      if (has_y(i)) add_term(acc[i], A.K.aS[i], ctr[i * PS - BXP]);
   } else if (A.bc[2] == LBM_BC_PERIODIC) {
     const Off n = c + (Off)(A.ny - 1) * pitch;
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-      if (has_y(i)) acc[i] += A.K.aS[i] * fin[i * P + n];
+      if (has_y(i)) add_term(acc[i], A.K.aS[i], fin[i * P + n]);
   } else {
     R g[16];
     ghost(A, fin, P, 2, side_kind(A, 2, x, t), m, c + pitch, A.ny > 1, g);
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-      if (has_y(i)) acc[i] += A.K.aS[i] * g[i];
+      if (has_y(i)) add_term(acc[i], A.K.aS[i], g[i]);
   }
   // y+ neighbour (north)
   if (y < A.ny - 1) {
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-      if (has_y(i)) acc[i] += A.K.aN[i] * ctr[i * PS + BXP];
+      if (has_y(i)) add_term(acc[i], A.K.aN[i], ctr[i * PS + BXP]);
   } else if (A.bc[3] == LBM_BC_PERIODIC) {
     const Off n = c - (Off)(A.ny - 1) * pitch;
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-      if (has_y(i)) acc[i] += A.K.aN[i] * fin[i * P + n];
+      if (has_y(i)) add_term(acc[i], A.K.aN[i], fin[i * P + n]);
   } else {
     R g[16];
     ghost(A, fin, P, 3, side_kind(A, 3, x, t), m, c - pitch, A.ny > 1, g);
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-      if (has_y(i)) acc[i] += A.K.aN[i] * g[i];
+      if (has_y(i)) add_term(acc[i], A.K.aN[i], g[i]);
   }
 }
 

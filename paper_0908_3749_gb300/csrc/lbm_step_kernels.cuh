@@ -7,6 +7,7 @@
 #include <type_traits>
 
 #include "lbm_dw_step.cuh"
+#include "lbm_lanes.cuh"
 #include "lbm_step.cuh"
 
 namespace lbmk {
@@ -63,7 +64,7 @@ __device__ __forceinline__ void step_tile(const StepArgs<R>& A, const R* __restr
     const Node64 n = collide64(A.K, d, acc);
     const Cons<R> m = {n.rho, n.jx, n.jy, R(0.5) * n.e2};  // e: boundary nodes and audits only
 #pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i] = A.K.a0[i] * f[i] + acc[i];
+    for (int i = 0; i < 16; ++i) acc[i] = fma(A.K.a0[i], f[i], acc[i]);
 
     // (2 e for e: a state within a factor of two of the largest number is bad)
     const bool b = !positive64(n.rho) || !finite64(n.rho, n.jx, n.jy, n.e2);
