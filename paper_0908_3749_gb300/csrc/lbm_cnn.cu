@@ -96,23 +96,28 @@ __device__ __forceinline__ void tma_load_box(void* dst, const CUtensorMap* map, 
 // contiguous bytes), tile rows are CV_ROW apart: M = 128 rows of A are 8 pixels of 16
 // rows, a tap is an offset of the start address, K = 16 two channel groups; nothing
 // is gathered by threads. The packed weights stay in shared memory as core
-// matrices of 8 output channels x 8 k. One thread issues a tile's 36 products
-// (two M = 128 halves; K in order, tap by tap) and commits them; the next tile's
-// copy starts once they have completed, under the epilogue, in which a thread
-// holds all channels of a pixel. Persistent CTAs, four per SM.
+// matrices of 8 output channels x 8 k. Persistent CTAs, two per SM, of six warps:
+// one thread issues the copies, one the products (36 per tile: two M = 128 halves;
+// K in order, tap by tap), four warps the epilogue, in which a thread holds all
+// channels of a pixel; CV_SLOTS slots of a tile in shared memory and its
+// accumulators in tensor memory go round between them.
 // The results are those of mma.sync m16n8k16 over the same K steps, bit for bit.
 // Bound by the tensor cores' reads of shared memory (5 KB per product, 5 us) and
-// by the latencies around each tile. Measured, 512 x 512, 32 -> 32 channels: 14
-// us, with and without the mask; as mma.sync with ldmatrix fragments (8 us at its 1024
-// multiply-adds per clock and SM) 18 us; with patches gathered from global memory
-// (L1 91 % busy) 67 us, and 72 us with the mask read from the activations.
-constexpr int CV_X = 16, CV_Y = 16, CV_HX = CV_X + 2, CV_HY = CV_Y + 2, CV_T = 128;
-constexpr int CV_CTAS_PER_SM = 4;
+// by the launch. Measured, 512 x 512, 32 -> 32 channels: 12.4 us with and without
+// the mask; with one tile at a time per CTA (copy, products, epilogue in turn) 14 us; as
+// mma.sync with ldmatrix fragments (8 us at its 1024 multiply-adds per clock and
+// SM) 18 us; with patches gathered from global memory (L1 91 % busy) 67 us, and 72 us
+// with the mask read from the activations.
+constexpr int CV_X = 16, CV_Y = 16, CV_HX = CV_X + 2, CV_HY = CV_Y + 2;
+constexpr int CV_EPI_T = 128, CV_T = CV_EPI_T + 64;  // epilogue threads; and two warps
+constexpr int CV_CTAS_PER_SM = 2, CV_SLOTS = 4;
 constexpr int CV_KG = 9 * 32 / 8;                          // groups of 8 k
 constexpr unsigned CV_GROUP = CV_HX * PX_BYTES, CV_ROW = 4 * CV_GROUP;
 constexpr unsigned CV_TILE = CV_HY * CV_ROW, CV_STAGE = (CV_TILE + 127) / 128 * 128;
 __host__ __device__ constexpr int cv_n(int cout) { return cout == 32 ? 32 : 16; }  // N of the products (zero rows)
-__host__ __device__ constexpr unsigned cv_smem(int cout) { return CV_STAGE + CV_KG * cv_n(cout) * 16 + 128; }
+__host__ __device__ constexpr unsigned cv_smem(int cout) {
+  return CV_SLOTS * CV_STAGE + CV_KG * cv_n(cout) * 16 + 128;
+}
 
 template <int COUT, int EPI>
 __global__ void __launch_bounds__(CV_T, CV_CTAS_PER_SM)
@@ -120,29 +125,36 @@ __global__ void __launch_bounds__(CV_T, CV_CTAS_PER_SM)
            const __nv_bfloat16* __restrict__ Wt, const float* __restrict__ bias,
            const unsigned* __restrict__ bits_in, __nv_bfloat16* __restrict__ out_bf,
            float* __restrict__ out_f, unsigned* __restrict__ bits_out, int* __restrict__ timeout) {
-  constexpr int NP = cv_n(COUT), TM = 2 * NP;  // TMEM columns: two halves
+  constexpr int NP = cv_n(COUT), TM = CV_SLOTS * 2 * NP;  // TMEM columns
   constexpr unsigned IDESC = tc05::idesc_f32acc(tc05::FMT_BF16, 128, NP);
   extern __shared__ __align__(128) unsigned char conv_raw[];
   unsigned char* const base = conv_raw + ((128u - (gbtma::smem_addr(conv_raw) & 127u)) & 127u);
-  __shared__ unsigned long long full, done;  // copy landed; products complete
+  // per slot: copy landed; products complete; accumulators read
+  __shared__ unsigned long long full[CV_SLOTS], done[CV_SLOTS], drained[CV_SLOTS];
   __shared__ unsigned s_tmem;
   __shared__ __align__(16) float s_bias[32];
   const int t = threadIdx.x, warp = t >> 5;
-  const int G = (int)gridDim.x;
-  auto load = [&](int tile) {
-    gbtma::mbar_expect_tx(&full, CV_TILE);
-    tma_load_box(base, &map, (tile % tiles_x) * CV_X - 1, (tile / tiles_x) * CV_Y - 1, &full);
-  };
+  const int G = (int)gridDim.x, mine = (ntiles - (int)blockIdx.x + G - 1) / G;  // tiles of this CTA
   gbtma::dependents_may_start();
-  if (t == 0) {
-    gbtma::mbar_init(&full, 1);
-    gbtma::mbar_init(&done, 1);
-  }
+  if (t == 0)
+    for (int k = 0; k < CV_SLOTS; ++k) {
+      gbtma::mbar_init(&full[k], 1);
+      gbtma::mbar_init(&done[k], 1);
+      gbtma::mbar_init(&drained[k], CV_EPI_T);
+    }
+  __syncthreads();
   gbtma::wait_for_previous();
+  auto load = [&](int k) {  // the CTA's k-th tile into slot k % CV_SLOTS
+    const int tile = (int)blockIdx.x + k * G, s = k % CV_SLOTS;
+    gbtma::mbar_expect_tx(&full[s], CV_TILE);
+    tma_load_box(base + s * CV_STAGE, &map, (tile % tiles_x) * CV_X - 1, (tile / tiles_x) * CV_Y - 1, &full[s]);
+  };
+  auto phase = [](int k) { return (unsigned)(k / CV_SLOTS) & 1u; };
+  if (t == CV_EPI_T)  // the first tiles' copies run while the CTA sets up
+    for (int k = 0; k < min(mine, CV_SLOTS); ++k) load(k);
   if (warp == 0) tc05::alloc(&s_tmem, TM);
-  if (t == 0) load(blockIdx.x);  // the grid has at most ntiles CTAs
   // Wt [ru(COUT, 8)][288] -> [k / 8][row][8]; rows beyond it zero
-  unsigned char* const sw = base + CV_STAGE;
+  unsigned char* const sw = base + CV_SLOTS * CV_STAGE;
   for (int i = t; i < NP * CV_KG; i += CV_T) {
     const int n = i / CV_KG, kg = i % CV_KG;
     *reinterpret_cast<uint4*>(sw + (kg * NP + n) * 16) =
@@ -155,88 +167,97 @@ __global__ void __launch_bounds__(CV_T, CV_CTAS_PER_SM)
   tc05::fence_after();
   const unsigned tmem = s_tmem, a0 = gbtma::smem_addr(base), b0 = gbtma::smem_addr(sw);
 
-  bool ok = true;
-  int k = 0;
-  for (int tile = blockIdx.x; tile < ntiles; tile += G, ++k) {
-    const bool more = tile + G < ntiles;
-    const int x0 = (tile % tiles_x) * CV_X + (t & 7), y = (tile / tiles_x) * CV_Y + (t >> 3);
-    if (t == 0) {
-      ok = gbtma::mbar_wait_bounded(&full, k & 1, gbtma::TMA_WAIT_CYCLES);
-      if (ok) {
-        tc05::fence_after();
+  constexpr long long LIMIT = gbtma::TMA_WAIT_CYCLES;
+  bool ok = true;  // every wait of this thread has ended in time
+  if (t == CV_EPI_T) {  // copies beyond the first CV_SLOTS: once the slot's products have read it
+    for (int k = CV_SLOTS; k < mine && ok; ++k) {
+      ok = gbtma::mbar_wait_bounded(&done[k % CV_SLOTS], phase(k - CV_SLOTS), LIMIT);
+      if (ok) load(k);
+    }
+  } else if (t == CV_EPI_T + 32) {  // products
+    for (int k = 0; k < mine && ok; ++k) {
+      const int s = k % CV_SLOTS;
+      if (k >= CV_SLOTS) ok = gbtma::mbar_wait_bounded(&drained[s], phase(k - CV_SLOTS), LIMIT);
+      ok = ok && gbtma::mbar_wait_bounded(&full[s], phase(k), LIMIT);
+      if (!ok) break;
+      tc05::fence_after();
+      const unsigned as = a0 + s * CV_STAGE, ts = tmem + s * 2 * NP;
+#pragma unroll 1
+      for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+        for (int q = 0; q < 6; ++q)  // dx = q / 2, channels 16 (q % 2) ..
+#pragma unroll
+          for (int m = 0; m < 2; ++m) {
+            const int ks = dy * 6 + q;
+            tc05::mma_f16(ts + m * NP,
+                          tc05::smem_desc(as + dy * CV_ROW + (8 * m + q / 2) * PX_BYTES + (q & 1) * 2 * CV_GROUP,
+                                          CV_GROUP, CV_ROW),
+                          tc05::smem_desc(b0 + ks * 2 * NP * 16, NP * 16, 128), IDESC, ks > 0 ? 1u : 0u);
+          }
+      tc05::commit(&done[s]);
+    }
+  } else if (t < CV_EPI_T) {  // epilogue: row t / 8 of the tile, pixels t % 8 and 8 + t % 8
+    for (int k = 0; k < mine; ++k) {
+      const int tile = (int)blockIdx.x + k * G, s = k % CV_SLOTS;
+      const int x0 = (tile % tiles_x) * CV_X + (t & 7), y = (tile / tiles_x) * CV_Y + (t >> 3);
+      // The ReLU masks (which channels of a pixel are positive), read while the
+      // products run.
+      unsigned keep[2] = {0u, 0u};
+      if constexpr (EPI == EPI_MASK_BF16)
 #pragma unroll
         for (int m = 0; m < 2; ++m)
-#pragma unroll 1
-          for (int dy = 0; dy < 3; ++dy)
+          if (y < H && x0 + 8 * m < W) keep[m] = __ldg(bits_in + (long long)y * W + x0 + 8 * m);
+      ok = __all_sync(0xffffffffu, gbtma::mbar_wait_bounded(&done[s], phase(k), LIMIT));
+      if (!ok) break;
+      tc05::fence_after();
 #pragma unroll
-            for (int q = 0; q < 6; ++q) {  // dx = q / 2, channels 16 (q % 2) ..
-              const int ks = dy * 6 + q;
-              tc05::mma_f16(tmem + m * NP,
-                            tc05::smem_desc(a0 + dy * CV_ROW + (8 * m + q / 2) * PX_BYTES + (q & 1) * 2 * CV_GROUP,
-                                            CV_GROUP, CV_ROW),
-                            tc05::smem_desc(b0 + ks * 2 * NP * 16, NP * 16, 128), IDESC, ks > 0 ? 1u : 0u);
-            }
-        tc05::commit(&done);
-      }
-    }
-    // The ReLU masks (which channels of a pixel are positive) of this thread's
-    // outputs, read while the products run.
-    unsigned keep[2] = {0u, 0u};
-    if constexpr (EPI == EPI_MASK_BF16)
-#pragma unroll
-      for (int m = 0; m < 2; ++m)
-        if (y < H && x0 + 8 * m < W) keep[m] = __ldg(bits_in + (long long)y * W + x0 + 8 * m);
-    __syncwarp();
-    ok = __syncthreads_and(ok && (t != 0 ? true : gbtma::mbar_wait_bounded(&done, k & 1, gbtma::TMA_WAIT_CYCLES)));
-    if (!ok) break;
-    if (t == 0 && more) load(tile + G);  // the products have read the tile
-    tc05::fence_after();
-#pragma unroll
-    for (int m = 0; m < 2; ++m) {
-      const int x = x0 + 8 * m;
-      const unsigned lanes = tmem + ((unsigned)(warp * 32) << 16) + m * NP;
-      if constexpr (EPI == EPI_LINEAR_F32) {
-        float v[16];
-        tc05::ld16(lanes, v);
-        if (y < H && x < W)
-          *reinterpret_cast<float4*>(out_f + ((long long)y * W + x) * 4) =
-              make_float4(v[0] + s_bias[0], v[1] + s_bias[1], v[2] + s_bias[2], v[3] + s_bias[3]);
-      } else {
-        float v[32];
-        tc05::ld32(lanes, v);
-        if (y < H && x < W) {
-          unsigned pos = 0u;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            __nv_bfloat162 r[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const int c = 8 * j + 2 * i;
-              if constexpr (EPI == EPI_RELU_BF16) {
-                r[i] = __floats2bfloat162_rn(fmaxf(v[c] + s_bias[c], 0.f), fmaxf(v[c + 1] + s_bias[c + 1], 0.f));
-                pos |= positive_bits(r[i]) >> (j + 4 * i);
-              } else {
-                r[i] = __floats2bfloat162_rn(v[c] * (keep[m] & (0x8000u >> (j + 4 * i)) ? 1.f : 0.f),
-                                             v[c + 1] * (keep[m] & (0x80000000u >> (j + 4 * i)) ? 1.f : 0.f));
-              }
-            }
-            *reinterpret_cast<uint4*>(out_bf + (((long long)y * 4 + j) * W + x) * 8) =
-                *reinterpret_cast<const uint4*>(r);
-          }
-          if (EPI == EPI_RELU_BF16 && bits_out) bits_out[(long long)y * W + x] = pos;
+      for (int m = 0; m < 2; ++m) {
+        const int x = x0 + 8 * m;
+        const unsigned lanes = tmem + ((unsigned)(warp * 32) << 16) + (s * 2 + m) * NP;
+        float v[NP];
+        if constexpr (NP == 16) tc05::ld16(lanes, v);
+        else tc05::ld32(lanes, v);
+        if (m == 1) {  // both halves are in registers
+          tc05::fence_before();
+          gbtma::mbar_arrive(&drained[s]);
         }
+        if (y < H && x < W) {
+          if constexpr (EPI == EPI_LINEAR_F32) {
+            *reinterpret_cast<float4*>(out_f + ((long long)y * W + x) * 4) =
+                make_float4(v[0] + s_bias[0], v[1] + s_bias[1], v[2] + s_bias[2], v[3] + s_bias[3]);
+          } else {
+            unsigned pos = 0u;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              __nv_bfloat162 r[4];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const int c = 8 * j + 2 * i;
+                if constexpr (EPI == EPI_RELU_BF16) {
+                  r[i] = __floats2bfloat162_rn(fmaxf(v[c] + s_bias[c], 0.f), fmaxf(v[c + 1] + s_bias[c + 1], 0.f));
+                  pos |= positive_bits(r[i]) >> (j + 4 * i);
+                } else {
+                  r[i] = __floats2bfloat162_rn(v[c] * (keep[m] & (0x8000u >> (j + 4 * i)) ? 1.f : 0.f),
+                                               v[c + 1] * (keep[m] & (0x80000000u >> (j + 4 * i)) ? 1.f : 0.f));
+                }
+              }
+              *reinterpret_cast<uint4*>(out_bf + (((long long)y * 4 + j) * W + x) * 8) =
+                  *reinterpret_cast<const uint4*>(r);
+            }
+            if (EPI == EPI_RELU_BF16 && bits_out) bits_out[(long long)y * W + x] = pos;
+          }
+        }
+        __syncwarp();
       }
     }
-    tc05::fence_before();
-    __syncthreads();  // the accumulators are free again
-    tc05::fence_after();
   }
-  if (!ok && t == 0) {
-    // A copy or the products did not complete in time: record it and wait once
-    // more (bounded) for both.
+  __syncwarp();
+  if (__syncthreads_or(!ok) && t == 0) {
+    // A copy or products did not complete in time: record it, give every copy
+    // that was issued (at most the last CV_SLOTS) a second bounded wait.
     atomicExch(timeout, 1);
-    gbtma::mbar_wait_bounded(&full, k & 1, gbtma::TMA_WAIT_CYCLES);
-    gbtma::mbar_wait_bounded(&done, k & 1, gbtma::TMA_WAIT_CYCLES);
+    for (int k = max(0, mine - CV_SLOTS); k < mine; ++k)
+      gbtma::mbar_wait_bounded(&full[k % CV_SLOTS], phase(k), LIMIT / 4);
   }
   tc05::fence_before();
   __syncthreads();
@@ -406,7 +427,7 @@ __global__ void __launch_bounds__(CT_T, C4_CTAS_PER_SM)
 // the partials of all CTAs in a fixed order.
 // Bound by the tensor cores' reads of A and B from shared memory (5 KB per
 // product; about 10 us at 512 x 512, 32 -> 32). Measured: 15 us (32 -> 32),
-// 13 us (32 -> 4), 14 us (first layer); gathering and transposing the
+// 13 us (32 -> 4), 14 us (first layer); one CTA per SM with five stages 19 us; gathering and transposing the
 // operands with threads took 83, 55 and 34 us, bound by L1 (83 %).
 constexpr int WG_T = 128;
 constexpr int WG_CTAS_PER_SM = 2;
