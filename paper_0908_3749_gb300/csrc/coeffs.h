@@ -79,6 +79,16 @@ inline bool lattice_constants(Coeffs<double>& K) {
   return true;
 }
 
+// The same constants in another arithmetic type.
+template <typename R>
+inline Coeffs<R> cast_coeffs(const Coeffs<double>& K) {
+  Coeffs<R> o;
+  const double* s = reinterpret_cast<const double*>(&K);
+  R* d = reinterpret_cast<R*>(&o);
+  for (size_t k = 0; k < sizeof(Coeffs<double>) / sizeof(double); ++k) d[k] = (R)s[k];
+  return o;
+}
+
 // K* = E* w for the non-conserved moments, w_k = -dt s_k; s holds s_1..s_16.
 __host__ __device__ inline void set_rates(Coeffs<double>& K, double dt, const double* s) {
   const double w5 = -dt * s[4], w6 = -dt * s[5], w7 = -dt * s[6], w8 = -dt * s[7];

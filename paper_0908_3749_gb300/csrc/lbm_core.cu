@@ -62,6 +62,22 @@ __global__ void k_init(R* __restrict__ f, const double* __restrict__ rho,
   for (int i = 0; i < 16; ++i) f[i * plane + c] = (R)g[i];
 }
 
+// The same for FP32 populations (feq32). 2048 x 1024: 92 us, 512 in FP64.
+__global__ void __launch_bounds__(AUX_N) k_init32(float* __restrict__ f, const double* __restrict__ rho,
+                                                  const double* __restrict__ u, const double* __restrict__ v,
+                                                  const double* __restrict__ T, const Coeffs<double> K,
+                                                  const Coeffs<dw> Kw, const Coeffs<float> K3, int nx, int ny,
+                                                  long long pitch, long long plane) {
+  const int x = blockIdx.x * AUX_X + threadIdx.x;
+  const int y = blockIdx.y * AUX_Y + threadIdx.y;
+  if (x >= nx || y >= ny) return;
+  const long long k = (long long)y * nx + x, c = (long long)y * pitch + x;
+  float g[16];
+  feq32(K, Kw, K3, rho[k], u[k], v[k], T[k], g);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) f[i * plane + c] = g[i];
+}
+
 template <typename R>
 __global__ void k_moments(const R* __restrict__ f, double* rho, double* u,
                           double* v, double* T, int nx, int ny, long long pitch,
@@ -187,15 +203,6 @@ bool build_coeffs(const lbm_config& cfg, Coeffs<double>& K) {
   return true;
 }
 
-template <typename R>
-Coeffs<R> cast_coeffs(const Coeffs<double>& K) {
-  Coeffs<R> o;
-  const double* s = reinterpret_cast<const double*>(&K);
-  R* d = reinterpret_cast<R*>(&o);
-  for (size_t k = 0; k < sizeof(Coeffs<double>) / sizeof(double); ++k) d[k] = (R)s[k];
-  return o;
-}
-
 thread_local std::string g_create_error = "no error";
 
 }  // namespace
@@ -258,15 +265,6 @@ int cuda_fail(lbm_ctx* c, cudaError_t e, const char* what) {
     cudaError_t e_ = (call);                                \
     if (e_ != cudaSuccess) return cuda_fail(ctx, e_, #call); \
   } while (0)
-
-// Third words of the double-word split of every constant (LBM_DF64).
-Coeffs<float> third_words(const Coeffs<double>& K) {
-  Coeffs<float> o;
-  const double* s = reinterpret_cast<const double*>(&K);
-  float* d = reinterpret_cast<float*>(&o);
-  for (size_t k = 0; k < sizeof(Coeffs<double>) / sizeof(double); ++k) d[k] = third_word(s[k]);
-  return o;
-}
 
 template <typename R>
 StepArgs<R> make_args(lbm_ctx* c, int slot) {
@@ -729,8 +727,9 @@ int lbm_set_init(lbm_ctx* c, const double* rho, const double* u, const double* v
     k_init<double><<<c->aux_grid, blk, 0, c->stream>>>((double*)c->f[0], p[0], p[1], p[2], p[3],
                                                     c->Kd, c->cfg.nx, c->cfg.ny, c->pitch, c->plane);
   else
-    k_init<float><<<c->aux_grid, blk, 0, c->stream>>>((float*)c->f[0], p[0], p[1], p[2], p[3],
-                                                   c->Kd, c->cfg.nx, c->cfg.ny, c->pitch, c->plane);
+    k_init32<<<c->aux_grid, blk, 0, c->stream>>>((float*)c->f[0], p[0], p[1], p[2], p[3], c->Kd,
+                                                 cast_coeffs<dw>(c->Kd), third_words(c->Kd), c->cfg.nx,
+                                                 c->cfg.ny, c->pitch, c->plane);
   CK(c, cudaGetLastError());
   const int rc = reset_status(c, 0);
   if (rc == LBM_OK && !on_device) CK(c, cudaStreamSynchronize(c->stream));  // host fields free again

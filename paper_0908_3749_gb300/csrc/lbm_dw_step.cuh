@@ -239,6 +239,87 @@ __device__ __forceinline__ void dw_feq(const Coeffs<dw>& K, const Coeffs<float>&
   dw_inverse_transform(S, C, X, Y, out);
 }
 
+// Third words of the double-word split of every constant.
+inline Coeffs<float> third_words(const Coeffs<double>& K) {
+  Coeffs<float> o;
+  const double* s = reinterpret_cast<const double*>(&K);
+  float* d = reinterpret_cast<float*>(&o);
+  for (size_t k = 0; k < sizeof(Coeffs<double>) / sizeof(double); ++k) d[k] = third_word(s[k]);
+  return o;
+}
+
+// Whether the magnitude of a double is in [2^lo, 2^10).
+__device__ __forceinline__ bool moderate(double x, int lo) {
+  const int hi = __double2hiint(x) & 0x7fffffff;
+  return hi >= (1023 + lo) << 20 && hi < (1023 + 10) << 20;
+}
+__device__ __forceinline__ bool is_zero(double x) {
+  return ((__double2hiint(x) & 0x7fffffff) | __double2loint(x)) == 0;
+}
+// Zero or such a double as an FP32 pair (its first 24 bits and the next 24 of the 29
+// left), off the FP64 units.
+__device__ __forceinline__ DWf split32(double x) {
+  if (is_zero(x)) return {0.f, 0.f};
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  const unsigned sign = (unsigned)hi & 0x80000000u;
+  const unsigned mag = ((unsigned)((hi & 0x7fffffff) - 0x38000000) << 3) | (lo >> 29);
+  const float ulp = __uint_as_float(((mag >> 23) - 52u) << 23 | sign);  // 2^(e - 52), signed
+  return {__uint_as_float(mag | sign), lmul((float)(lo & 0x1fffffffu), ulp)};
+}
+
+// f^eq of (rho, u, v, T) as (float) of the FP64 form, out[16]: the initial state of
+// FP32 populations. FP64 takes 120 instructions a node for it, at one per warp and 19
+// clocks, where the memory needs a fifth of that time. So the node is computed in
+// double-word FP32 with three-word constants, and the FP64 form is taken only where
+// the rounding to FP32 is in doubt: ten operations in a row at 2^-45.5 of their
+// terms stay below 2^-42 of the sum of the terms' magnitudes, so a value whose
+// interval of 2^-41 of that sum rounds to one FP32 number is the FP64 form's value,
+// bit for bit. The range of the states keeps the second words' underflow (2^-149 times
+// at most 2^40) far below the interval, of at least 2^-80.
+// 2048 x 1024 nodes: 92 us, 512 in FP64; 4.49 M nodes of tubes: 198 us from 1134.
+__device__ __forceinline__ bool feq32_dw(const Coeffs<dw>& K, const Coeffs<float>& K3, double rho, double u,
+                                         double v, double T, float (&out)[16]) {
+  if (!(moderate(rho, -10) && (moderate(u, -40) || is_zero(u)) && (moderate(v, -40) || is_zero(v)) &&
+        (moderate(T, -40) || is_zero(T))))
+    return false;
+  const DWf r = split32(rho), uu = split32(u), vv = split32(v), t = split32(T);
+  const DWf e = dadd(dmul(r, t), dscale(dmul(r, dadd(dmul(uu, uu), dmul(vv, vv))), 0.5f));
+  DWf g[16];
+  dw_feq(K, K3, r, dmul(r, uu), dmul(r, vv), e, g);
+  // sums of the terms' magnitudes per velocity group
+  const float ra = fabsf(r.h), ua = fabsf(uu.h), va = fabsf(vv.h), us = ua * ua + va * va;
+  const float ea = fabsf(t.h) + 0.5f * us;  // e / rho
+  const float eP = 2.f * ea + 0.5f * us, A = 6.f * ea + 2.f * us;
+  const float m11 = 2.f * ea * ea + 0.25f * us * us;
+  const float cx = ua * (ua * ua + 3.f * va * va), cy = va * (3.f * ua * ua + va * va);
+  bool sure = true;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float S = fabsf(K.E0[k][0].h) + fabsf(K.E0[k][1].h) * ea + fabsf(K.E0[k][2].h) * m11;
+    const float X = fabsf(K.EX[k][0].h) * ua + fabsf(K.EX[k][1].h) * eP * ua + fabsf(K.EX[k][2].h) * cx;
+    const float Y = fabsf(K.EY[k][0].h) * va + fabsf(K.EY[k][1].h) * eP * va + fabsf(K.EY[k][2].h) * cy;
+    const float C = k < 2 ? fabsf(K.EC[k & 1][0].h) * us + fabsf(K.EC[k & 1][1].h) * A * us
+                          : fabsf(K.ES[k & 1][0].h) * us + fabsf(K.ES[k & 1][1].h) * A * us;
+    const float band = ra * (S + C + X + Y) * 0x1p-41f;
+    sure = sure && band >= 0x1p-80f;
+#pragma unroll
+    for (int j = 4 * k; j < 4 * k + 4; ++j) {
+      out[j] = ladd(g[j].h, ladd(g[j].l, band));
+      sure = sure && out[j] == ladd(g[j].h, lsub(g[j].l, band));
+    }
+  }
+  return sure;
+}
+__device__ __forceinline__ void feq32(const Coeffs<double>& K, const Coeffs<dw>& Kw, const Coeffs<float>& K3,
+                                      double rho, double u, double v, double T, float (&out)[16]) {
+  if (feq32_dw(Kw, K3, rho, u, v, T, out)) return;
+  double g[16];
+  feq(K, rho, rho * u, rho * v, rho * T + 0.5 * rho * (u * u + v * v), g);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) out[i] = (float)g[i];
+}
+
 // Conserved moments (rho, j_x, j_y, e) of node idx of the global populations.
 template <typename Off>
 __device__ __forceinline__ void dw_load_cons(const dw* __restrict__ fin, Off plane, Off idx,

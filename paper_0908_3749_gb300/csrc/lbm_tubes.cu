@@ -42,6 +42,7 @@
 #include "../../include/lbm_batch.h"
 #include "coeffs.h"
 #include "d2v16.cuh"
+#include "lbm_dw_step.cuh"
 #include "tma.cuh"
 
 using namespace d2v16;
@@ -464,18 +465,18 @@ constexpr int AUX_T = 128;
 
 __global__ void k_tubes_init(float* f, const TubeDesc* tubes, const int2* items, long long P,
                              int tile, const double* rho, const double* u, const double* v,
-                             const double* T, const Coeffs<double> K) {
+                             const double* T, const Coeffs<double> K, const Coeffs<dw> Kw,
+                             const Coeffs<float> K3) {
   const int2 it = items[blockIdx.x];
   const TubeDesc D = tubes[it.x];
   for (int j = threadIdx.x; j < tile; j += blockDim.x) {
     const int x = it.y + j;
     if (x >= D.nx) break;
     const long long k = D.out + x;
-    const double r = rho[k], uu = u[k], vv = v[k];
-    double g[16];
-    feq(K, r, r * uu, r * vv, r * T[k] + 0.5 * r * (uu * uu + vv * vv), g);
+    float g[16];
+    lbmk::feq32(K, Kw, K3, rho[k], u[k], v[k], T[k], g);
 #pragma unroll
-    for (int i = 0; i < 16; ++i) f[i * P + D.off + x] = (float)g[i];
+    for (int i = 0; i < 16; ++i) f[i * P + D.off + x] = g[i];
   }
 }
 
@@ -891,7 +892,8 @@ int lbm_batch_set_init(lbm_batch* b, const double* rho, const double* u, const d
     }
   const int tile = VARIANTS[b->variant].tile;
   k_tubes_init<<<b->nitems, AUX_T, 0, b->stream>>>(b->f[0], b->tubes, b->items, b->plane, tile,
-                                                    p[0], p[1], p[2], p[3], b->Kd);
+                                                    p[0], p[1], p[2], p[3], b->Kd, cast_coeffs<dw>(b->Kd),
+                                                    lbmk::third_words(b->Kd));
   BCK(b, cudaGetLastError());
   return reset_batch_status(b);
 }
