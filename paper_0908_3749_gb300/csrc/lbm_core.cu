@@ -59,7 +59,10 @@ __global__ void k_init(R* __restrict__ f, const double* __restrict__ rho,
   feq(K, r, r * uu, r * vv, r * T[k] + 0.5 * r * (uu * uu + vv * vv), g);
   const long long c = (long long)y * pitch + x;
 #pragma unroll
-  for (int i = 0; i < 16; ++i) f[i * plane + c] = (R)g[i];
+  for (int i = 0; i < 16; ++i) {
+    if constexpr (std::is_same_v<R, dw>) f[i * plane + c] = d2v16::split_nearest(g[i]);
+    else f[i * plane + c] = (R)g[i];
+  }
 }
 
 // The same for FP32 populations (feq32). 2048 x 1024: 92 us, 512 in FP64.
@@ -88,7 +91,7 @@ __global__ void k_moments(const R* __restrict__ f, double* rho, double* u,
   const long long c = (long long)y * pitch + x;
   double g[16];
 #pragma unroll
-  for (int i = 0; i < 16; ++i) g[i] = (double)f[i * plane + c];
+  for (int i = 0; i < 16; ++i) g[i] = to_double(f[i * plane + c]);
   Groups<double> d;
   transform(g, d);
   const Cons<double> m = conserved(K, d);
@@ -117,7 +120,7 @@ __global__ void __launch_bounds__(AUX_N) k_audit(const R* __restrict__ f, int nx
     const long long c = (long long)y * pitch + x;
     double g[16];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) g[i] = (double)f[i * plane + c];
+    for (int i = 0; i < 16; ++i) g[i] = to_double(f[i * plane + c]);
     Groups<double> d;
     transform(g, d);
     const Cons<double> m = conserved(K, d);
