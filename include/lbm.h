@@ -208,7 +208,10 @@ int lbm_element_size(lbm_ctx* ctx);
  * block updates its tile; with fewer blocks each block takes tiles b, b + G,
  * b + 2G, ... (G blocks), copying its next tile into shared memory while it
  * computes the current one. Results do not depend on it (each node's update
- * is the same, audit partials are kept per tile); only the speed does.
+ * is the same, audit partials are kept per tile); only the speed does. LBM_FP64
+ * grids of few nodes run the default with four threads per node, blocks of eight
+ * nodes (at most 50 000 nodes, of which beyond 4864 at most one in eight lies next
+ * to a side that is not periodic).
  *  lbm_set_step_blocks: 0 = the default, one block per tile; larger values
  *    are capped at the number of tiles. Synchronises; LBM_ERR_UNSUPPORTED
  *    for LBM_TC_TF32X3 (its own persistent grid, 4 CTAs per multiprocessor).

@@ -20,7 +20,7 @@
  * step kernels run; G's eigenvalues come from a Householder reduction to
  * Hessenberg form followed by single-shift complex QR iterations (Wilkinson
  * shifts, deflation on negligible subdiagonals), all in FP64, one matrix per
- * 16 threads.
+ * 4, 8 or 16 threads (fewer the more matrices a call has).
  *
  * Layouts. Complex numbers are two doubles (re, im), as C99 double complex.
  * A 16 x 16 matrix is row-major: entry (i, j) at index 16 i + j; row i is

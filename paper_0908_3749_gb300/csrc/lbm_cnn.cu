@@ -12,9 +12,9 @@
 // The input features stay FP32 and the first layer (4 -> 32) runs in FP32 on
 // the CUDA cores. The other 3 x 3 convolutions are implicit GEMMs on the
 // 5th-generation tensor cores (tcgen05, BF16 inputs, FP32 accumulation in tensor
-// memory; mma.sync for 4 -> 32 channels): rows are pixels, the reduction index k = tap * CIN + ci runs over the 9 taps and the input
-// channels, columns are output channels. The weights of a layer are packed
-// once per update into [COUT][K] BF16 (K contiguous, the "col" operand) for
+// memory; mma.sync for 4 -> 32 channels): rows are pixels, the reduction index
+// k = tap * CIN + ci runs over the 9 taps and the input channels, columns are output
+// channels. The weights of a layer are packed once per update into [COUT][K] BF16 (K contiguous, the "col" operand) for
 // the forward pass and into the tap-flipped, channel-transposed [CIN][K'] for
 // the input-gradient pass, which is the same GEMM run on the output
 // gradients. Weight gradients are contractions over the pixels, by tcgen05 too
