@@ -66,16 +66,17 @@ METRIC = ("D2V16 MRT cell-updates/s at stated error vs FP64 oracle; "
 UNIT = "cell-updates/s"
 # Algorithmic traffic per cell-update: 16 populations read once and written once.
 BYTES_PER_CELL = {"fp64": 256, "fp32": 128}
-# Algorithmic FP64 operations per cell-update of the factorised step (FMA = 2):
-# transform 28, conserved moments 24, equilibria 40, deviations 77,
-# back-map 64, inverse transform 28, Lax-Wendroff update 128.
-FLOPS_PER_CELL = 389
+# FP64 operations per cell-update as the step executes them (FMA = 2), counted by
+# ncu: dadd 66.1 + dmul 25.1 + 2 x dfma 136.1. (The plain factorised form takes 389:
+# transform 28, conserved moments 24, equilibria 40, deviations 77, back-map 64,
+# inverse transform 28, Lax-Wendroff update 128.)
+FLOPS_PER_CELL = 363
 # FP64-pipe instructions per node update of k_step<double>, counted by ncu
 # (sm__inst_executed_pipe_fp64, profiles/k_step_f64_bubble_2048x1024.md):
 # the FP64 units retire one instruction per lane slot whether it is an add,
 # a multiply or a fused multiply-add, so this count over the measured FMA
 # rate is the step's time on those units.
-FP64_INSTR_PER_CELL = 265
+FP64_INSTR_PER_CELL = 232
 L2_FLUSH_BYTES = 256 << 20
 
 
