@@ -237,6 +237,7 @@ struct lbm_ctx {
   dim3 grid, aux_grid;  // step grid; init / moments / audit grid
   bool wide = false;    // 64-bit element offsets needed
   bool lanes = false;   // FP64 step with four lanes per node (k_step_lanes)
+  int pipe = 0;         // > 0: blocks of k_step_pipe as the default of this grid
   Coeffs<double> Kd;
   CUtensorMap tmap[2];        // TMA descriptors of the two population buffers
   bool tc = false;            // tensor-core transforms (LBM_TC_TF32X3)
@@ -304,7 +305,7 @@ StepArgs<R> make_args(lbm_ctx* c, int slot) {
   A.ngroups = c->ngroups;
   A.agroup = c->agroup;
   A.audit_every = c->cfg.audit_every;
-  A.nblocks = c->nblocks;
+  A.nblocks = c->pipe > 0 ? c->pipe : c->nblocks;
   A.ntiles = c->ntiles;
   A.tiles_x = c->tiles_x;
   A.area = c->cfg.dx * c->cfg.dy;
@@ -348,8 +349,8 @@ int launch_step(lbm_ctx* c, cudaStream_t s, int from) {
   return launch_persistent<float>(c, s, from, c->f[to], make_args<float>(c, from));
 }
 
-// Blocks of a step launch when none were chosen: one per tile (k_step); FP64
-// grids of few nodes then take k_step_lanes.
+// Blocks of a step launch when none were chosen: one per tile (k_step). FP64
+// grids of few nodes then take k_step_lanes, large FP32 and double-word ones k_step_pipe.
 int default_blocks(const lbm_ctx* c) { return c->ntiles; }
 bool few_nodes(const lbm_ctx* c) {
   const lbm_config& C = c->cfg;
@@ -358,6 +359,30 @@ bool few_nodes(const lbm_ctx* c) {
   for (int s = 0; s < 4; ++s)
     if (C.bc[s].kind != LBM_BC_PERIODIC) edge += s < 2 ? C.ny : C.nx;
   return C.precision == LBM_FP64 && nodes <= LANES_MAX_NODES && (nodes <= LANES_THIN || 8 * edge <= nodes);
+}
+// Blocks of k_step_pipe for large grids, 0 for the others. Persistent blocks of few
+// tiles hide their copies and, on audit steps, their counting; many tiles per block
+// lose the L2's reuse of rows (3 blocks per SM over 32 768 tiles: 227 us).
+//  LBM_DF64: 3 tiles per block from 4000 tiles on. k_step / this, us per step:
+//    tiles   2961         4096         8192         11750        24576       32768
+//            110.8/118.2  144.8/139.2  277.5/257.7  383.7/353.2  779.8/701.4 1036.8/927.9
+//  LBM_FP32: 6 or 7 from 5000 on, whichever takes fewer rounds of the resident blocks
+//    and whose blocks do not return to the same column of tiles (6144 tiles of 64
+//    columns: 49.3 us with 6, 39.1 with 7).
+//    tiles   4096       5311       6144       8192       11750      12288      24576        32768
+//            30.7/31.2  38.5/34.9  43.4/39.1  56.0/51.0  77.6/70.1  82.7/73.3  155.8/137.0  208.4/177.0
+//  Ten other sizes from 5421 to 17 741 tiles, wide to tall: LBM_DF64 5 to 10 % faster,
+//  LBM_FP32 2 to 13 %. LBM_FP32_DWMOM: within 6 % either way; FP64: within 0.1 %.
+int default_pipe(const lbm_ctx* c) {
+  auto blocks = [&](int m) { return (c->ntiles + m - 1) / m; };
+  if (c->wide) return 0;
+  if (c->cfg.precision == LBM_DF64 && c->ntiles >= 4000) return blocks(3);
+  if (c->cfg.precision != LBM_FP32 || c->ntiles < 5000) return 0;
+  const int resident = Shape<float>::MINB_PIPE * std::max(1, c->sms);
+  auto rounds = [&](int m) {
+    return (blocks(m) % c->tiles_x ? 0 : c->ntiles) + m * ((blocks(m) + resident - 1) / resident);
+  };
+  return blocks(rounds(7) < rounds(6) ? 7 : 6);
 }
 
 template <typename R, int VAR = 0>
@@ -624,6 +649,7 @@ int lbm_create(const lbm_config* cfg, void* cuda_stream, lbm_ctx** out) {
   } else {
     c->nblocks = default_blocks(c);
     c->lanes = few_nodes(c);
+    c->pipe = default_pipe(c);
     c->grid = dim3(c->nblocks);
     if (e == cudaSuccess)
       e = c->dwp ? allow_pipe_smem<dw>()
@@ -968,7 +994,7 @@ namespace {
 
 // Sets the number of blocks of the step launch: later steps are issued with
 // `g` blocks and the captured graphs are rebuilt.
-int apply_blocks(lbm_ctx* c, int g, bool lanes = false) {
+int apply_blocks(lbm_ctx* c, int g, bool lanes = false, int pipe = 0) {
   CK(c, cudaStreamSynchronize(c->stream));
   for (int k = 0; k < 2; ++k)
     if (c->graph[k]) {
@@ -977,6 +1003,7 @@ int apply_blocks(lbm_ctx* c, int g, bool lanes = false) {
     }
   c->nblocks = g;
   c->lanes = lanes;
+  c->pipe = pipe;
   c->grid = dim3(g);
   return LBM_OK;
 }
@@ -1018,7 +1045,7 @@ int lbm_set_step_blocks(lbm_ctx* c, int blocks) {
   if (!c) return fail(nullptr, LBM_ERR_INVALID, "ctx is NULL");
   if (blocks < 0) return fail(c, LBM_ERR_INVALID, "blocks < 0");
   if (c->tc) return fail(c, LBM_ERR_UNSUPPORTED, "the tensor-core step sets its own launch");
-  return blocks == 0 ? apply_blocks(c, default_blocks(c), few_nodes(c))
+  return blocks == 0 ? apply_blocks(c, default_blocks(c), few_nodes(c), default_pipe(c))
                      : apply_blocks(c, std::min(blocks, c->ntiles));
 }
 
