@@ -521,67 +521,6 @@ __device__ __forceinline__ void warp_sum_rows(const double* p, int first, int n,
   for (int q = 0; q < 4; ++q) out[q] = warp_total(s[q]);
 }
 
-// The sums of a group of tiles whose partials are all written, and of the groups if
-// it is the last, by one warp.
-template <typename R>
-__device__ __forceinline__ void audit_group(const StepArgs<R>& A, int gg, unsigned long long step, int lane) {
-  const int g0 = gg * A.agroup, gn = min(A.ntiles - g0, A.agroup);
-  double s4[4];
-  warp_sum_rows(A.partial, g0, gn, lane, s4);
-  if (lane < 4)
-    A.gpartial[4 * gg + lane] = lane == 0 ? s4[0] : lane == 1 ? s4[1] : lane == 2 ? s4[2] : s4[3];
-  __syncwarp();
-  int last = 0;
-  if (lane == 0) {
-    A.gcount[gg] = 0u;
-    __threadfence();
-    last = atomicAdd(&A.st->arrive_step, 1u) == (unsigned)A.ngroups - 1;
-  }
-  if (__shfl_sync(0xffffffffu, last, 0)) {
-    __syncwarp();
-    __threadfence();
-    double tot[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int c = 0; c < A.ngroups; c += AUDIT_GROUP_MAX) {  // chunks of groups, in order
-      double part[4];
-      warp_sum_rows(A.gpartial, c, min(A.ngroups - c, AUDIT_GROUP_MAX), lane, part);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) tot[q] += part[q];
-    }
-    const unsigned slot = (unsigned)(A.st->audit_count & (LBM_AUDIT_RING - 1));
-    if (lane < 4)
-      A.st->audit_totals[slot][lane] =
-          (lane == 0 ? tot[0] : lane == 1 ? tot[1] : lane == 2 ? tot[2] : tot[3]) * A.area;
-    __syncwarp();
-    if (lane == 0) {
-      A.st->audit_steps[slot] = (long long)step;
-      A.st->audit_count += 1;
-      A.st->arrive_step = 0u;
-    }
-  }
-}
-
-// One tile per block: warp 0 counts the tile once its lanes 0 .. 3 have written the
-// partial, before the block's populations are stored (a fence waits for every earlier
-// store), and sums the tile's group at the block's end (audit_tile_done) if it was the
-// group's last (*s_n, in shared memory).
-template <typename R>
-__device__ __forceinline__ void audit_tile_arrive(const StepArgs<R>& A, int tile, int* s_n) {
-  __syncwarp();
-  if (threadIdx.x == 0) {
-    const int g = tile / A.agroup, gn = min(A.ntiles - g * A.agroup, A.agroup);
-    __threadfence();
-    *s_n = atomicAdd(&A.gcount[g], 1u) == (unsigned)gn - 1;
-  }
-}
-template <typename R>
-__device__ __forceinline__ void audit_tile_done(const StepArgs<R>& A, int tile, unsigned long long step,
-                                                const int* s_n) {
-  __syncwarp();
-  if (*s_n == 0) return;
-  __threadfence();
-  audit_group(A, tile / A.agroup, step, threadIdx.x);
-}
-
 // Audit steps, once per block after its last tile (every thread calls it;
 // the block's tiles are first, first + stride, ...): two levels of
 // fixed-order sums, so that no warp sums more than A.agroup partials.
@@ -618,7 +557,40 @@ __device__ __forceinline__ void audit_block_done(const StepArgs<R>& A, int first
     if (n > 0) {
       __threadfence();  // the groups' partials, released by the blocks that wrote them
       for (int k = warp; k < n; k += nwarps) {
-        audit_group(A, s_list[k], step, lane);
+        const int gg = s_list[k];
+        const int g0 = gg * A.agroup, gn = min(A.ntiles - g0, A.agroup);
+        double s4[4];
+        warp_sum_rows(A.partial, g0, gn, lane, s4);
+        if (lane < 4)
+          A.gpartial[4 * gg + lane] = lane == 0 ? s4[0] : lane == 1 ? s4[1] : lane == 2 ? s4[2] : s4[3];
+        __syncwarp();
+        int last = 0;
+        if (lane == 0) {
+          A.gcount[gg] = 0u;
+          __threadfence();
+          last = atomicAdd(&A.st->arrive_step, 1u) == (unsigned)A.ngroups - 1;
+        }
+        if (__shfl_sync(0xffffffffu, last, 0)) {
+          __syncwarp();
+          __threadfence();
+          double tot[4] = {0.0, 0.0, 0.0, 0.0};
+          for (int c = 0; c < A.ngroups; c += AUDIT_GROUP_MAX) {  // chunks of groups, in order
+            double part[4];
+            warp_sum_rows(A.gpartial, c, min(A.ngroups - c, AUDIT_GROUP_MAX), lane, part);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) tot[q] += part[q];
+          }
+          const unsigned slot = (unsigned)(A.st->audit_count & (LBM_AUDIT_RING - 1));
+          if (lane < 4)
+            A.st->audit_totals[slot][lane] =
+                (lane == 0 ? tot[0] : lane == 1 ? tot[1] : lane == 2 ? tot[2] : tot[3]) * A.area;
+          __syncwarp();
+          if (lane == 0) {
+            A.st->audit_steps[slot] = (long long)step;
+            A.st->audit_count += 1;
+            A.st->arrive_step = 0u;
+          }
+        }
       }
     }
     __syncthreads();  // s_list and s_n are reused in the next round

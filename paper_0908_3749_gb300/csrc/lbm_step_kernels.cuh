@@ -91,16 +91,11 @@ __device__ __forceinline__ void step_tile(const StepArgs<R>& A, const R* __restr
 // FP32 populations, the Eq. 14 equilibria and P = rho T in double-word
 // arithmetic (lbm_dw_step.cuh), rounded to FP32 only where they enter the
 // FP32 relaxation; audits sum the double-word moments.
-// ONE: the block's only tile. Its audit partial is written and counted before the
-// populations are stored, as warp 0's fence waits for every store before it: an
-// audit step of 2048 x 1024 takes 33 us longer than another, counted at the block's
-// end (audit_block_done) 38 us. The FP64 step has other blocks' arithmetic to hide it;
-// the double-word step spilled with it (300 from 290 us a step).
-template <typename Off, bool MAC, bool ONE>
+template <typename Off, bool MAC = false>
 __device__ __forceinline__ void step_tile_x2(const StepArgs<float>& A, const float* __restrict__ fin,
                                              float* __restrict__ fout, const float* stage, int cur,
                                              bool audit, float t, double (*sm)[4], bool& bad,
-                                             bool& negT, int* s_n) {
+                                             bool& negT) {
   constexpr int BXD = Shape<float>::X, BYD = Shape<float>::Y, HY = BYD / 2;
   constexpr int BXP = Tile<float>::BXP, PS = Tile<float>::ROWS * BXP;
   static_assert(Shape<float>::TY == HY, "two rows per thread");
@@ -109,18 +104,18 @@ __device__ __forceinline__ void step_tile_x2(const StepArgs<float>& A, const flo
   const bool act_a = x < A.nx && ya < A.ny, act_b = x < A.nx && yb < A.ny;  // act_b => act_a
   float mca[4] = {0.f, 0.f, 0.f, 0.f}, mcb[4] = {0.f, 0.f, 0.f, 0.f};
   dw wca[4], wcb[4];  // MAC: the double-word conserved moments for the audit
-  const Off P = (Off)A.plane, pitch = (Off)A.pitch;
-  const Off ca = (Off)ya * pitch + (Off)x, cb = ca + (Off)HY * pitch;
-  const float* sa = stage + (threadIdx.y + 1) * BXP + threadIdx.x + HALO_X;
-  const float* sb = sa + HY * BXP;
-  Cons<F2> m;
-  F2 acc[16];
   if (act_a) {
+    const Off P = (Off)A.plane, pitch = (Off)A.pitch;
+    const Off ca = (Off)ya * pitch + (Off)x, cb = ca + (Off)HY * pitch;
+    const float* sa = stage + (threadIdx.y + 1) * BXP + threadIdx.x + HALO_X;
+    const float* sb = sa + HY * BXP;
     F2 f[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) f[i] = F2(sa[i * PS], sb[i * PS]);
     Groups<F2> d;
     transform(f, d);
+    Cons<F2> m;
+    F2 acc[16];
     F2 press;
     if constexpr (MAC) {
       float2 fv[16];
@@ -154,29 +149,7 @@ __device__ __forceinline__ void step_tile_x2(const StepArgs<float>& A, const flo
     negT |= (!ba && !(press.v.x > 0.f)) || (act_b && !bb && !(press.v.y > 0.f));
     mca[0] = m.rho.v.x; mca[1] = m.jx.v.x; mca[2] = m.jy.v.x; mca[3] = m.e.v.x;
     if (act_b) { mcb[0] = m.rho.v.y; mcb[1] = m.jx.v.y; mcb[2] = m.jy.v.y; mcb[3] = m.e.v.y; }
-  }
-  auto audit_sums = [&] {  // double-word warp sums, FP64 across warps, only on audit steps
-    float ha[4], la[4], hb[4], lb[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if constexpr (MAC) {
-        ha[q] = act_a ? wca[q].h : 0.f;
-        la[q] = act_a ? wca[q].l : 0.f;
-        hb[q] = act_b ? wcb[q].h : 0.f;
-        lb[q] = act_b ? wcb[q].l : 0.f;
-      } else {
-        ha[q] = mca[q];
-        hb[q] = mcb[q];
-        la[q] = lb[q] = 0.f;
-      }
-    }
-    audit_pair_rows<BXD, BYD>(A, cur, ha, la, hb, lb, sm);
-  };
-  if (ONE && audit) {
-    audit_sums();
-    if (threadIdx.y == 0) audit_tile_arrive(A, cur, s_n);
-  }
-  if (act_a) {
+
     if (act_b && x > 0 && x < A.nx - 1 && ya > 0 && yb < A.ny - 1) {
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
@@ -210,21 +183,37 @@ __device__ __forceinline__ void step_tile_x2(const StepArgs<float>& A, const flo
       }
     }
   }
-  if (!ONE && audit) audit_sums();
+  if (audit) {  // double-word warp sums, FP64 across warps, only on audit steps
+    float ha[4], la[4], hb[4], lb[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if constexpr (MAC) {
+        ha[q] = act_a ? wca[q].h : 0.f;
+        la[q] = act_a ? wca[q].l : 0.f;
+        hb[q] = act_b ? wcb[q].h : 0.f;
+        lb[q] = act_b ? wcb[q].l : 0.f;
+      } else {
+        ha[q] = mca[q];
+        hb[q] = mcb[q];
+        la[q] = lb[q] = 0.f;
+      }
+    }
+    audit_pair_rows<BXD, BYD>(A, cur, ha, la, hb, lb, sm);
+  }
 }
 
 // VAR selects a variant of the FP32 step: 0 the plain one, 1 the one with
 // double-word conserved moments and equilibria (LBM_FP32_DWMOM).
-template <typename R, typename Off, int VAR, bool ONE>
+template <typename R, typename Off, int VAR>
 __device__ __forceinline__ void step_any(const StepArgs<R>& A, const R* __restrict__ fin,
                                          R* __restrict__ fout, const R* stage, int cur, bool audit,
-                                         R t, double (*sm)[4], bool& bad, bool& negT, int* s_n) {
+                                         R t, double (*sm)[4], bool& bad, bool& negT) {
   if constexpr (std::is_same<R, dw>::value)
     step_tile_dw<Off>(A, fin, fout, stage, cur, audit, t, sm, bad, negT);
   else if constexpr (Shape<R>::TY == Shape<R>::Y)
     step_tile<R, Off>(A, fin, fout, stage, cur, audit, t, sm, bad, negT);
   else
-    step_tile_x2<Off, VAR == 1, ONE>(A, fin, fout, stage, cur, audit, t, sm, bad, negT, s_n);
+    step_tile_x2<Off, VAR == 1>(A, fin, fout, stage, cur, audit, t, sm, bad, negT);
 }
 
 // Blocks per SM the one-tile form is compiled for: the FP32 form with 64-bit
@@ -279,14 +268,10 @@ __global__ void __launch_bounds__(Shape<R>::X * Shape<R>::TY, (step_minb<R, Off>
     return;
   }
   bool bad = false, negT = false;
-  step_any<R, Off, VAR, true>(A, fin, fout, tile, blockIdx.x, audit, A.dtr * R(s_step), sm, bad, negT, &s_an);
+  step_any<R, Off, VAR>(A, fin, fout, tile, blockIdx.x, audit, A.dtr * R(s_step), sm, bad, negT);
   const unsigned long long step = s_step;
   watchdog_flags(A.st, step, bad, negT);
-  if constexpr (!std::is_same<R, float>::value) {
-    if (audit) audit_block_done(A, (int)blockIdx.x, A.ntiles, step, s_alist, &s_an);
-  } else {
-    if (audit && threadIdx.y == 0) audit_tile_done(A, (int)blockIdx.x, step, &s_an);
-  }
+  if (audit) audit_block_done(A, (int)blockIdx.x, A.ntiles, step, s_alist, &s_an);
 }
 
 // Two tile stages (each a multiple of 128 bytes) plus room to align the first
@@ -341,8 +326,8 @@ __global__ void __launch_bounds__(Shape<R>::X * Shape<R>::TY, Shape<R>::MINB_PIP
       }
       return;
     }
-    step_any<R, Off, VAR, false>(A, fin, fout, stages + s * Tile<R>::ELEMS, cur, s_audit != 0,
-                                 A.dtr * R(s_step), sm, bad, negT, &s_an);
+    step_any<R, Off, VAR>(A, fin, fout, stages + s * Tile<R>::ELEMS, cur, s_audit != 0,
+                     A.dtr * R(s_step), sm, bad, negT);
     __syncthreads();  // stage s and sm are free again
   }
   watchdog_flags(A.st, s_step, bad, negT);
