@@ -213,11 +213,15 @@ int lbm_element_size(lbm_ctx* ctx);
  * nodes (at most 50 000 nodes, of which beyond 4864 at most one in eight lies next
  * to a side that is not periodic); LBM_FP32 and LBM_DF64 grids of many tiles (from
  * 5000 and 4000 on) run it with 6 or 7 and with 3 tiles per block.
- *  lbm_set_step_blocks: 0 = the default, one block per tile; larger values
- *    are capped at the number of tiles. Synchronises; LBM_ERR_UNSUPPORTED
+ *  lbm_set_step_blocks: 0 = the default, as above; the default's own number
+ *    selects it too; other values above the number of tiles are one block per
+ *    tile. Synchronises; LBM_ERR_UNSUPPORTED
  *    for LBM_TC_TF32X3 (its own persistent grid, 4 CTAs per multiprocessor).
- *  lbm_step_blocks: the current value (-1 for a NULL ctx).
- *  lbm_autotune: times `launches` step launches for each candidate (one
+ *  lbm_step_blocks: the blocks of a step's launch (with four threads per node:
+ *    8 blocks per tile); set again it selects
+ *    the same launch. -1 for a NULL ctx.
+ *  lbm_autotune: times `launches` step launches for each candidate (the
+ *    four-thread form where it is the default; one
  *    block per tile; 1 .. k blocks per multiprocessor; ceil(tiles / m) blocks
  *    for m = 2 .. 8) and keeps the fastest. The timed launches read the
  *    current populations and write the spare buffer against scratch

@@ -237,7 +237,6 @@ struct lbm_ctx {
   dim3 grid, aux_grid;  // step grid; init / moments / audit grid
   bool wide = false;    // 64-bit element offsets needed
   bool lanes = false;   // FP64 step with four lanes per node (k_step_lanes)
-  int pipe = 0;         // > 0: blocks of k_step_pipe as the default of this grid
   Coeffs<double> Kd;
   CUtensorMap tmap[2];        // TMA descriptors of the two population buffers
   bool tc = false;            // tensor-core transforms (LBM_TC_TF32X3)
@@ -305,7 +304,7 @@ StepArgs<R> make_args(lbm_ctx* c, int slot) {
   A.ngroups = c->ngroups;
   A.agroup = c->agroup;
   A.audit_every = c->cfg.audit_every;
-  A.nblocks = c->pipe > 0 ? c->pipe : c->nblocks;
+  A.nblocks = c->nblocks;
   A.ntiles = c->ntiles;
   A.tiles_x = c->tiles_x;
   A.area = c->cfg.dx * c->cfg.dy;
@@ -357,9 +356,7 @@ int launch_step(lbm_ctx* c, cudaStream_t s, int from) {
   return launch_persistent<float>(c, s, from, c->f[to], make_args<float>(c, from));
 }
 
-// Blocks of a step launch when none were chosen: one per tile (k_step). FP64
-// grids of few nodes then take k_step_lanes, large FP32 and double-word ones k_step_pipe.
-int default_blocks(const lbm_ctx* c) { return c->ntiles; }
+// FP64 grids that take k_step_lanes when no number of blocks was chosen.
 bool few_nodes(const lbm_ctx* c) {
   const lbm_config& C = c->cfg;
   const long long nodes = (long long)C.nx * C.ny;
@@ -391,6 +388,12 @@ int default_pipe(const lbm_ctx* c) {
     return (blocks(m) % c->tiles_x ? 0 : c->ntiles) + m * ((blocks(m) + resident - 1) / resident);
   };
   return blocks(rounds(7) < rounds(6) ? 7 : 6);
+}
+// Blocks of a step launch when none were chosen: those of k_step_lanes or of
+// k_step_pipe where the grid takes one of them, else one per tile (k_step).
+int default_blocks(const lbm_ctx* c) {
+  const int pipe = default_pipe(c);
+  return few_nodes(c) ? c->ntiles * LANES_BLOCKS : pipe > 0 ? pipe : c->ntiles;
 }
 
 template <typename R, int VAR = 0>
@@ -657,7 +660,6 @@ int lbm_create(const lbm_config* cfg, void* cuda_stream, lbm_ctx** out) {
   } else {
     c->nblocks = default_blocks(c);
     c->lanes = few_nodes(c);
-    c->pipe = default_pipe(c);
     c->grid = dim3(c->nblocks);
     if (e == cudaSuccess)
       e = c->dwp ? allow_pipe_smem<dw>()
@@ -1002,7 +1004,7 @@ namespace {
 
 // Sets the number of blocks of the step launch: later steps are issued with
 // `g` blocks and the captured graphs are rebuilt.
-int apply_blocks(lbm_ctx* c, int g, bool lanes = false, int pipe = 0) {
+int apply_blocks(lbm_ctx* c, int g, bool lanes = false) {
   CK(c, cudaStreamSynchronize(c->stream));
   for (int k = 0; k < 2; ++k)
     if (c->graph[k]) {
@@ -1011,7 +1013,6 @@ int apply_blocks(lbm_ctx* c, int g, bool lanes = false, int pipe = 0) {
     }
   c->nblocks = g;
   c->lanes = lanes;
-  c->pipe = pipe;
   c->grid = dim3(g);
   return LBM_OK;
 }
@@ -1053,8 +1054,9 @@ int lbm_set_step_blocks(lbm_ctx* c, int blocks) {
   if (!c) return fail(nullptr, LBM_ERR_INVALID, "ctx is NULL");
   if (blocks < 0) return fail(c, LBM_ERR_INVALID, "blocks < 0");
   if (c->tc) return fail(c, LBM_ERR_UNSUPPORTED, "the tensor-core step sets its own launch");
-  return blocks == 0 ? apply_blocks(c, default_blocks(c), few_nodes(c), default_pipe(c))
-                     : apply_blocks(c, std::min(blocks, c->ntiles));
+  const int d = default_blocks(c);
+  if (blocks == 0 || blocks == d) return apply_blocks(c, d, few_nodes(c));
+  return apply_blocks(c, std::min(blocks, c->ntiles));
 }
 
 int lbm_step_blocks(lbm_ctx* c) { return c ? c->nblocks : -1; }

@@ -47,7 +47,7 @@ def main(argv=None):
     ap.add_argument("--steps", type=int, default=100)
     ap.add_argument("--audit-every", type=int, default=0)
     ap.add_argument("--blocks", type=int, default=0,
-                    help="step launch blocks (0: one per tile); see lbm_set_step_blocks")
+                    help="step launch blocks (0: the default for the grid); see lbm_set_step_blocks")
     ap.add_argument("--fused", type=int, default=1, choices=(1, 2),
                     help="time steps per FP32 launch (lbm_set_fused_steps)")
     ap.add_argument("--autotune", type=int, default=0,
