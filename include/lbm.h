@@ -210,7 +210,7 @@ int lbm_element_size(lbm_ctx* ctx);
  * computes the current one. Results do not depend on it (each node's update
  * is the same, audit partials are kept per tile); only the speed does. LBM_FP64
  * grids of few nodes run the default with four threads per node, blocks of eight
- * nodes (at most 50 000 nodes, of which beyond 4864 at most one in eight lies next
+ * nodes (at most 9728 nodes, of which beyond 4864 at most one in eight lies next
  * to a side that is not periodic); LBM_FP32 and LBM_DF64 grids of many tiles (from
  * 5000 and 4000 on) run it with 6 or 7 and with 3 tiles per block.
  *  lbm_set_step_blocks: 0 = the default, as above; the default's own number

@@ -317,15 +317,7 @@ int launch_persistent(lbm_ctx* c, cudaStream_t s, int from, void* fout, const St
   const dim3 blk(Shape<R>::X, Shape<R>::TY);
   const R* fi = (const R*)c->f[from];
   const CUtensorMap& tm = c->tmap[from];
-  if (VAR == 1 && A.nblocks >= A.ntiles && A.ntiles > c->sms && 4 * A.ntiles < 9 * c->sms) {
-    // LBM_FP32_DWMOM, one to two tiles per SM or just above: blocks that start early
-    // find the SMs of the last launch's second blocks taken and pile up elsewhere. Step
-    // with overlapped launches / without: 190 tiles 8.2 / 7.5 us, 320 tiles 8.8 / 7.9, 416
-    // tiles 8.8 / 9.3, 475 tiles 8.9 / 10.1; the FP32 step gains at all of these.
-    (c->wide ? k_step<R, long long, VAR> : k_step<R, unsigned, VAR>)<<<A.ntiles, blk, tile_dynamic_bytes<R>(), s>>>(
-        tm, fi, (R*)fout, A);
-    CK(c, cudaGetLastError());
-  } else if (A.nblocks >= A.ntiles) {
+  if (A.nblocks >= A.ntiles) {
     CK(c, launch_overlapped(c->wide ? k_step<R, long long, VAR> : k_step<R, unsigned, VAR>, A.ntiles, blk,
                             tile_dynamic_bytes<R>(), s,
                             tm, fi, (R*)fout, A));

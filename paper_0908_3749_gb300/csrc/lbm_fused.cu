@@ -217,7 +217,6 @@ __global__ void __launch_bounds__(NT, 4)
   const int tx = threadIdx.x, ty = threadIdx.y, t = ty * FX + tx;
   const int tile = blockIdx.x;
   const int x0 = (tile % A.tiles_x) * FX, y0 = (tile / A.tiles_x) * FY;
-  dependents_may_start();
   if (t == 0) mbar_init(&bar, 1);
   wait_for_previous();
   if (t == 0) {
@@ -303,6 +302,7 @@ __global__ void __launch_bounds__(NT, 4)
     watchdog_flags(A.st, step + 1, bad, negT);
     if (audit1) audit_pair(A, tile, nb, nbb, sm);
   }
+  if (!audit0 && !audit1) dependents_may_start();
   if (audit0 || audit1)
     audit_block_done(A, tile, A.ntiles, audit0 ? step : step + 1, s_alist, &s_an);
 }

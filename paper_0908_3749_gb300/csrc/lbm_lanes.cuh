@@ -15,10 +15,17 @@
 // b, -0), which round alike).
 //
 // Bound by the latency of those instructions and of the loads from L2.
-// Measured per step, this form / k_step:
-//   nodes   800      4800     9600   14400    19200  30000  45000  60000  90000
-//   (us)    6.3/12.8 6.3/12.9 12.7/22.9 13.2/33.8 24.7/45.1 30.8/51.0 42.1/55.7 51.5/54.3 65.8/63.8
-// (200 x 4 to 3600 x 4 Sod tubes, then shock bubbles, whose sides take ghosts).
+// Measured per step, one thread per node in plain launches / in overlapped ones (k_step) /
+// this form:
+//   nodes         800   4800   9600  14000  19200  20000  30000  45000
+//   periodic (us) 13.7  13.7   13.7   15.2   15.2   21.2   26.5   35.1
+//                 11.6  11.6   12.1   12.9   12.9   17.8   21.8   28.7
+//                  6.0   6.1    8.1   11.7   13.1   21.4   23.2   34.1
+//   walled (us)     -     -      -    21.6   22.9   29.4   34.3   49.9
+//                   -     -      -    20.1   20.5   25.2   28.7   43.8
+//                   -     -      -    21.1   23.1   27.8   30.4   41.8
+// (200 x 4, 1200 x 4, 2400 x 4, 140 x 100, 160 x 120, 200 x 100, 200 x 150, 250 x 180; the
+// first three with Dirichlet ends, walled ones with ghosts on all four sides.)
 #pragma once
 
 #include "lbm_step.cuh"
@@ -30,11 +37,13 @@ namespace lbmk {
 constexpr int LANES_T = 32, LANES_NODES = LANES_T / 4;
 constexpr int LANES_ROW = Shape<double>::X / LANES_NODES, LANES_BLOCKS = LANES_ROW * Shape<double>::Y;
 
-// Grids that take this form: at most LANES_MAX_NODES nodes, and beyond LANES_THIN of
-// them (four blocks per SM) only where few are next to a side that is not
+// Grids that take this form: at most LANES_MAX_NODES nodes (two blocks per partition of
+// every SM; more share the FP64 units, of whose instructions this form has 1.27 times
+// as many in all), and beyond LANES_THIN of
+// them (one per partition) only where few are next to a side that is not
 // periodic: such a node's ghosts cost a block as many instructions as its eight
 // nodes' own update. (1800 x 4 nodes between reflecting walls: 25.7 us against 23.2.)
-constexpr long long LANES_MAX_NODES = 50000, LANES_THIN = 4864;
+constexpr long long LANES_MAX_NODES = 9728, LANES_THIN = 4864;
 
 __device__ __forceinline__ double lane_value(double v, int src) { return __shfl_sync(0xffffffffu, v, src, 4); }
 
@@ -80,7 +89,6 @@ __global__ void __launch_bounds__(LANES_T)
   __shared__ unsigned long long s_step;
   __shared__ int s_audit, s_alist[32], s_an;
   const int lane = threadIdx.x, g = lane & 3;
-  dependents_may_start();
   wait_for_previous();
   if (lane == 0) s_step = read_step(A, &s_audit);
   const int tile = blockIdx.x / LANES_BLOCKS, sub = blockIdx.x % LANES_BLOCKS;
@@ -201,6 +209,7 @@ __global__ void __launch_bounds__(LANES_T)
     if (gs) put(2, x, c + pitch, A.ny > 1, s);
     if (gn) put(3, x, c - pitch, A.ny > 1, n);
   }
+  if (!audit) dependents_may_start();
   __syncwarp();
 #pragma unroll
   for (int k = 0; k < 4; ++k) {

@@ -245,7 +245,6 @@ __global__ void __launch_bounds__(Shape<R>::X * Shape<R>::TY, (step_minb<R, Off>
   __shared__ unsigned long long s_step;
   __shared__ int s_audit, s_alist[32], s_an;
   const int t = threadIdx.y * Shape<R>::X + threadIdx.x;
-  dependents_may_start();
   if (t == 0) mbar_init(&bar, 1);
   wait_for_previous();
   if (t == 0) {
@@ -269,6 +268,7 @@ __global__ void __launch_bounds__(Shape<R>::X * Shape<R>::TY, (step_minb<R, Off>
   }
   bool bad = false, negT = false;
   step_any<R, Off, VAR>(A, fin, fout, tile, blockIdx.x, audit, A.dtr * R(s_step), sm, bad, negT);
+  if (!audit) dependents_may_start();
   const unsigned long long step = s_step;
   watchdog_flags(A.st, step, bad, negT);
   if (audit) audit_block_done(A, (int)blockIdx.x, A.ntiles, step, s_alist, &s_an);
@@ -295,7 +295,6 @@ __global__ void __launch_bounds__(Shape<R>::X * Shape<R>::TY, Shape<R>::MINB_PIP
   __shared__ int s_audit, s_alist[32], s_an;
   const int t = threadIdx.y * Shape<R>::X + threadIdx.x;
   const int G = (int)gridDim.x;
-  dependents_may_start();
   if (t == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
@@ -330,6 +329,7 @@ __global__ void __launch_bounds__(Shape<R>::X * Shape<R>::TY, Shape<R>::MINB_PIP
                      A.dtr * R(s_step), sm, bad, negT);
     __syncthreads();  // stage s and sm are free again
   }
+  if (!s_audit) dependents_may_start();
   watchdog_flags(A.st, s_step, bad, negT);
   if (s_audit) audit_block_done(A, (int)blockIdx.x, G, s_step, s_alist, &s_an);
 }

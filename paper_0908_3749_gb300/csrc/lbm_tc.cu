@@ -157,21 +157,27 @@ __global__ void __launch_bounds__(TC_T, TC_CTAS_PER_SM)
   const int tx = threadIdx.x, ty = threadIdx.y, t = ty * TC_X + tx, warp = ty;
   const int G = (int)gridDim.x;
 
-  dependents_may_start();
   if (t == 0) {
     for (int i = 0; i < TC_STAGES; ++i) mbar_init(&S.bar_tma[i], 1);
     mbar_init(&S.bar_mma, 1);
   }
-  // transform constants into shared memory (16 KB)
-  for (int i = t; i < 4 * (int)TC_B_BYTES / 16; i += TC_T)
-    reinterpret_cast<uint4*>(&S.b[0][0])[i] = reinterpret_cast<const uint4*>(bconst)[i];
-  // The previous step's tensor memory is free once it has completed.
+  // The transform constants (16 KB) are on their way before the wait; the tile's
+  // copy starts before they are stored. (Stored first, then tensor memory, then the
+  // copy: 400 x 225 9.4 us a step, 1500 x 900 41.8; so 6.7 and 39.3.)
+  constexpr int NB = 4 * (int)TC_B_BYTES / 16 / TC_T;
+  uint4 bc[NB];
+#pragma unroll
+  for (int k = 0; k < NB; ++k) bc[k] = reinterpret_cast<const uint4*>(bconst)[k * TC_T + t];
   wait_for_previous();
-  if (warp == 0) tc05::alloc(&S.tmem_base, TC_TMEM_COLS);  // for all this CTA's tiles
   if (t == 0) {
     tc_load_tile(S.tile[0], &tmap, &S.bar_tma[0], blockIdx.x, A.tiles_x);  // grid <= ntiles
     S.step = read_step(A, &S.audit);
   }
+  // The previous step's tensor memory is free once it has completed.
+  if (warp == 1) tc05::alloc(&S.tmem_base, TC_TMEM_COLS);  // for all this CTA's tiles
+#pragma unroll
+  for (int k = 0; k < NB; ++k) reinterpret_cast<uint4*>(&S.b[0][0])[k * TC_T + t] = bc[k];
+  tc05::fence_async_smem();
   tc05::fence_before();
   __syncthreads();
   tc05::fence_after();
@@ -334,14 +340,15 @@ __global__ void __launch_bounds__(TC_T, TC_CTAS_PER_SM)
     }
     tc05::fence_before();
     __syncthreads();
-    if (warp == 0) tc05::dealloc(tmem, TC_TMEM_COLS);
+    if (warp == 1) tc05::dealloc(tmem, TC_TMEM_COLS);
     return;
   }
 
+  if (!audit) dependents_may_start();
   // free tensor memory (every tcgen05.ld of this CTA is complete)
   tc05::fence_before();
   __syncthreads();
-  if (warp == 0) tc05::dealloc(tmem, TC_TMEM_COLS);
+  if (warp == 1) tc05::dealloc(tmem, TC_TMEM_COLS);
 
   watchdog_flags(A.st, step, bad, negT);
   if (audit) audit_block_done(A, (int)blockIdx.x, G, step, S.alist, &S.an);

@@ -78,10 +78,19 @@ __device__ __forceinline__ void fence_proxy_async() {
 // of that one has called dependents_may_start() (or has ended): its blocks then
 // set up their barriers and wait in wait_for_previous() until the previous
 // kernel has completed and its writes are visible. Every thread calls that
-// before it touches memory that the previous kernel may write or read. Measured on the
-// step kernels (a launch and its tile's first copy otherwise follow the previous
-// step's last block): 600 x 200 FP32 6.9 -> 6.4 us a step, 200 x 4 FP64 13.3 -> 12.8,
-// 2048 x 1024 FP32 57.8 -> 56.8, tensor cores 68.4 -> 66.7.
+// before it touches memory that the previous kernel may write or read.
+//
+// The step kernels call dependents_may_start() when a block has only its stores
+// left. Called at their top, the next step's blocks take whatever slots are free
+// then, so that some SMs get several of them and others none: a grid of two blocks
+// or so per SM takes the time of the fullest. Measured, us a step, plain launches /
+// early / late:
+//   FP64, one thread per node, 2400 x 4: 13.7 / 22.9 / 12.1;
+//   FP32 200 x 150 4.4 / 5.1 / 4.1, 300 x 200 5.0 / 5.3 / 4.7, 600 x 200 6.5 / 6.1 / 6.1;
+//   LBM_FP32_DWMOM 256 x 128 4.9 / 6.7 / 4.6, 400 x 225 7.1 / 7.5 / 6.6.
+// Audit steps leave it out: their blocks end in a chain of fences and counters, beside
+// which the next step's blocks would only wait (audits on every step, FP32 160 x 120:
+// 11.5 us plainly, 11.9 with it, 11.3 without).
 __device__ __forceinline__ void dependents_may_start() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
