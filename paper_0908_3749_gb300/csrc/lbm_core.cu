@@ -237,6 +237,7 @@ struct lbm_ctx {
   dim3 grid, aux_grid;  // step grid; init / moments / audit grid
   bool wide = false;    // 64-bit element offsets needed
   bool lanes = false;   // FP64 step with four lanes per node (k_step_lanes)
+  bool rows4 = false;   // LBM_DF64 on 32 x 4 tiles
   Coeffs<double> Kd;
   CUtensorMap tmap[2];        // TMA descriptors of the two population buffers
   bool tc = false;            // tensor-core transforms (LBM_TC_TF32X3)
@@ -306,24 +307,41 @@ StepArgs<R> make_args(lbm_ctx* c, int slot) {
   A.audit_every = c->cfg.audit_every;
   A.nblocks = c->nblocks;
   A.ntiles = c->ntiles;
+  // The double-word step of few tiles: a block that starts early starts on another SM, which
+  // has to fetch the 56 KB of instructions (1200 x 4: 9.4 us a step, overlapped 9.8).
+  A.overlapped = !c->rows4 || c->ntiles >= c->sms;
   A.tiles_x = c->tiles_x;
   A.area = c->cfg.dx * c->cfg.dy;
   A.slot = slot;
   return A;
 }
 
+// The step kernels of a context with 64-bit element offsets, or without (V_ROWS4 grids are
+// small).
+template <typename R, int VAR>
+auto step_kernel(bool wide) {
+  if constexpr (VAR != V_ROWS4)
+    if (wide) return k_step<R, long long, VAR>;
+  return k_step<R, unsigned, VAR>;
+}
+template <typename R, int VAR>
+auto pipe_kernel(bool wide) {
+  if constexpr (VAR != V_ROWS4)
+    if (wide) return k_step_pipe<R, long long, VAR>;
+  return k_step_pipe<R, unsigned, VAR>;
+}
+
 template <typename R, int VAR = 0>
 int launch_persistent(lbm_ctx* c, cudaStream_t s, int from, void* fout, const StepArgs<R>& A) {
-  const dim3 blk(Shape<R>::X, Shape<R>::TY);
+  const dim3 blk(Shape<R, VAR>::X, Shape<R, VAR>::TY);
   const R* fi = (const R*)c->f[from];
   const CUtensorMap& tm = c->tmap[from];
   if (A.nblocks >= A.ntiles) {
-    CK(c, launch_overlapped(c->wide ? k_step<R, long long, VAR> : k_step<R, unsigned, VAR>, A.ntiles, blk,
-                            tile_dynamic_bytes<R>(), s,
-                            tm, fi, (R*)fout, A));
+    CK(c, launch(A.overlapped, step_kernel<R, VAR>(c->wide), A.ntiles, blk,
+                 tile_dynamic_bytes<R, VAR>(), s, tm, fi, (R*)fout, A));
   } else {
-    CK(c, launch_overlapped(c->wide ? k_step_pipe<R, long long, VAR> : k_step_pipe<R, unsigned, VAR>, A.nblocks,
-                            blk, pipe_smem_bytes<R>(), s, tm, fi, (R*)fout, A));
+    CK(c, launch(A.overlapped, pipe_kernel<R, VAR>(c->wide), A.nblocks, blk,
+                 pipe_smem_bytes<R, VAR>(), s, tm, fi, (R*)fout, A));
   }
   return LBM_OK;
 }
@@ -342,12 +360,25 @@ int launch_step(lbm_ctx* c, cudaStream_t s, int from) {
                     make_args<float>(c, from), c->tc_b, c->tc_w, c->grid, s));
     return LBM_OK;
   }
+  if (c->rows4) return launch_persistent<dw, V_ROWS4>(c, s, from, c->f[to], make_args<dw>(c, from));
   if (c->dwp) return launch_persistent<dw>(c, s, from, c->f[to], make_args<dw>(c, from));
-  if (c->dwmom) return launch_persistent<float, 1>(c, s, from, c->f[to], make_args<float>(c, from));
+  if (c->dwmom) return launch_persistent<float, V_DWMOM>(c, s, from, c->f[to], make_args<float>(c, from));
   if (c->esize == 8) return launch_persistent<double>(c, s, from, c->f[to], make_args<double>(c, from));
   return launch_persistent<float>(c, s, from, c->f[to], make_args<float>(c, from));
 }
 
+// Double-word grids on 32 x 4 tiles instead of 32 x 8. Few tiles: the blocks have SMs
+// to themselves, and walls take fewer of a block's warps. From one to one and a half
+// 32 x 8 tiles per SM: some SMs would have two and the others one. us a step, 32 x 8 / 32 x 4
+// in overlapped launches, grids walled and periodic (1800 x 4: Dirichlet ends):
+//   90 x 70   300 x 16   1800 x 4  128 x 64   140 x 100  220 x 160  250 x 180  300 x 200
+//   27 tiles  20         57        32         65         140        184        250
+//   14.0/12.8 13.9/12.9            12.8/13.2  13.2/13.6  13.7/14.8  16.8/15.1  16.7/17.8
+//    8.9/9.1   8.2/8.2    9.0/8.3   8.9/9.5    9.1/9.8    9.9/10.5  13.4/11.5  13.5/13.9
+bool rows4(const lbm_config& C, int sms) {
+  const long long t = ((C.nx + 31ll) / 32) * ((C.ny + 7ll) / 8);
+  return C.precision == LBM_DF64 && (t < 64 || (t >= sms && 2 * t <= 3ll * sms));
+}
 // FP64 grids that take k_step_lanes when no number of blocks was chosen.
 bool few_nodes(const lbm_ctx* c) {
   const lbm_config& C = c->cfg;
@@ -390,17 +421,14 @@ int default_blocks(const lbm_ctx* c) {
 
 template <typename R, int VAR = 0>
 cudaError_t allow_pipe_smem() {
-  const int b = (int)pipe_smem_bytes<R>();
-  cudaError_t e = cudaFuncSetAttribute(k_step_pipe<R, unsigned, VAR>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_step_pipe<R, long long, VAR>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-  const int t = (int)tile_dynamic_bytes<R>();
-  if (e == cudaSuccess && t > 0)
-    e = cudaFuncSetAttribute(k_step<R, unsigned, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, t);
-  if (e == cudaSuccess && t > 0)
-    e = cudaFuncSetAttribute(k_step<R, long long, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, t);
+  const int b = (int)pipe_smem_bytes<R, VAR>(), t = (int)tile_dynamic_bytes<R, VAR>();
+  cudaError_t e = cudaSuccess;
+  for (bool wide : {false, true}) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(pipe_kernel<R, VAR>(wide), cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+    if (e == cudaSuccess && t > 0)
+      e = cudaFuncSetAttribute(step_kernel<R, VAR>(wide), cudaFuncAttributeMaxDynamicSharedMemorySize, t);
+  }
   return e;
 }
 
@@ -472,7 +500,7 @@ int encode_map(lbm_ctx* c, int b, cuuint32_t rows, CUtensorMap* out) {
 int encode_tile_map(lbm_ctx* c, int b) {
   const bool dbl = c->esize == 8;
   const cuuint32_t rows = c->tc ? (cuuint32_t)(TC_Y + 2)
-                    : (cuuint32_t)(c->dwp ? Tile<dw>::ROWS
+                    : (cuuint32_t)(c->rows4 ? Tile<dw, V_ROWS4>::ROWS : c->dwp ? Tile<dw>::ROWS
                                           : (dbl ? Tile<double>::ROWS : Tile<float>::ROWS));
   int rc = encode_map(c, b, rows, &c->tmap[b]);
   if (rc == LBM_OK && !dbl && !c->tc)
@@ -632,19 +660,20 @@ int lbm_create(const lbm_config* cfg, void* cuda_stream, lbm_ctx** out) {
     e = cudaStreamCreate(&c->stream);  // blocking: ordered with the default stream
     c->own_stream = true;
   }
-  c->pitch = ((long long)C.nx + 31) / 32 * 32;
-  c->plane = c->pitch * C.ny;
-  const int bx = c->tc ? TC_X : (c->dwp ? Shape<dw>::X : (c->esize == 8 ? Shape<double>::X : Shape<float>::X));
-  const int by = c->tc ? TC_Y : (c->dwp ? Shape<dw>::Y : (c->esize == 8 ? Shape<double>::Y : Shape<float>::Y));
-  c->tiles_x = (C.nx + bx - 1) / bx;
-  c->ntiles = c->tiles_x * ((C.ny + by - 1) / by);
-  c->aux_grid = dim3((C.nx + AUX_X - 1) / AUX_X, (C.ny + AUX_Y - 1) / AUX_Y);
-  c->wide = 16ll * c->plane >= (1ll << 32);
   {
     int dev = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
   }
+  c->pitch = ((long long)C.nx + 31) / 32 * 32;
+  c->plane = c->pitch * C.ny;
+  const int bx = c->tc ? TC_X : (c->dwp ? Shape<dw>::X : (c->esize == 8 ? Shape<double>::X : Shape<float>::X));
+  c->rows4 = rows4(C, c->sms);
+  const int by = c->tc ? TC_Y : c->rows4 ? Shape<dw, V_ROWS4>::Y : (c->dwp ? Shape<dw>::Y : (c->esize == 8 ? Shape<double>::Y : Shape<float>::Y));
+  c->tiles_x = (C.nx + bx - 1) / bx;
+  c->ntiles = c->tiles_x * ((C.ny + by - 1) / by);
+  c->aux_grid = dim3((C.nx + AUX_X - 1) / AUX_X, (C.ny + AUX_Y - 1) / AUX_Y);
+  c->wide = 16ll * c->plane >= (1ll << 32);
   if (c->tc) {  // persistent CTAs, each taking every G-th tile
     c->nblocks = std::max(1, std::min(c->ntiles, TC_CTAS_PER_SM * std::max(1, c->sms)));
     c->grid = dim3(c->nblocks);
@@ -654,8 +683,9 @@ int lbm_create(const lbm_config* cfg, void* cuda_stream, lbm_ctx** out) {
     c->lanes = few_nodes(c);
     c->grid = dim3(c->nblocks);
     if (e == cudaSuccess)
-      e = c->dwp ? allow_pipe_smem<dw>()
-                 : c->dwmom ? allow_pipe_smem<float, 1>()
+      e = c->rows4 ? allow_pipe_smem<dw, V_ROWS4>()
+          : c->dwp ? allow_pipe_smem<dw>()
+                 : c->dwmom ? allow_pipe_smem<float, V_DWMOM>()
                             : (c->esize == 8 ? allow_pipe_smem<double>() : allow_pipe_smem<float>());
     if (e == cudaSuccess && c->esize == 4) e = fused_prepare();
   }
@@ -1071,7 +1101,8 @@ int lbm_autotune(lbm_ctx* c, int launches) {
   // Candidates: (few FP64 nodes) k_step_lanes, one tile per block (k_step), and for k_step_pipe 1 ..
   // MINB_PIPE blocks per SM and ceil(ntiles / m) blocks for m = 2 .. 8 tiles
   // per block.
-  const int per_sm = c->dwp ? Shape<dw>::MINB_PIPE
+  const int per_sm = c->rows4 ? Shape<dw, V_ROWS4>::MINB_PIPE
+                     : c->dwp ? Shape<dw>::MINB_PIPE
                             : (c->esize == 8 ? Shape<double>::MINB_PIPE : Shape<float>::MINB_PIPE);
   std::vector<int> cand;
   auto add = [&](long long g) {
@@ -1089,8 +1120,9 @@ int lbm_autotune(lbm_ctx* c, int launches) {
     rc = fail(c, LBM_ERR_CUDA, "cudaEventCreate failed");
   for (size_t i = 0; i < cand.size() && rc == LBM_OK; ++i) {
     float ms = 0.f;
-    rc = c->dwp ? time_blocks<dw>(c, cand[i], launches, scratch, e0, e1, &ms)
-         : c->dwmom ? time_blocks<float, 1>(c, cand[i], launches, scratch, e0, e1, &ms)
+    rc = c->rows4 ? time_blocks<dw, V_ROWS4>(c, cand[i], launches, scratch, e0, e1, &ms)
+         : c->dwp ? time_blocks<dw>(c, cand[i], launches, scratch, e0, e1, &ms)
+         : c->dwmom ? time_blocks<float, V_DWMOM>(c, cand[i], launches, scratch, e0, e1, &ms)
          : c->esize == 8 ? time_blocks<double>(c, cand[i], launches, scratch, e0, e1, &ms)
                          : time_blocks<float>(c, cand[i], launches, scratch, e0, e1, &ms);
     if (rc == LBM_OK && (i == 0 || ms < best_ms)) {

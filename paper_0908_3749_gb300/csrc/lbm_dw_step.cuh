@@ -469,14 +469,15 @@ __device__ __forceinline__ DWf lane_dw(DW<V> v, int k) {
 // memory in the lane form; a thread with a node on the domain edge finishes
 // node by node through the generic neighbour_terms (ghosts and periodic wraps
 // on the normalised scalar type dw). Watchdog and audit as in the FP32 update.
-template <typename Off>
+template <typename Off, int VAR>
 __device__ __forceinline__ void step_tile_dw(const StepArgs<dw>& A, const dw* __restrict__ fin,
                                              dw* __restrict__ fout, const dw* stage, int cur,
                                              bool audit, dw t, double (*sm)[4], bool& bad,
                                              bool& negT) {
-  constexpr int BXD = Shape<dw>::X, BYD = Shape<dw>::Y, TY = Shape<dw>::TY, NL = BYD / TY;
+  using S = Shape<dw, VAR>;
+  constexpr int BXD = S::X, BYD = S::Y, TY = S::TY, NL = BYD / TY;
   using V = typename std::conditional<NL == 2, float2, float>::type;
-  constexpr int BXP = Tile<dw>::BXP, PS = Tile<dw>::ROWS * BXP;
+  constexpr int BXP = Tile<dw, VAR>::BXP, PS = Tile<dw, VAR>::ROWS * BXP;
   static_assert(NL == 1 || NL == 2, "one or two nodes per thread");
   const int x = (cur % A.tiles_x) * BXD + threadIdx.x;
   int y[NL];

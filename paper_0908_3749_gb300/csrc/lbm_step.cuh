@@ -28,20 +28,22 @@ constexpr unsigned long long NONE = ~0ull;
 // FP32 arithmetic (memory-bound: fewer instructions per node). FP64: 32 x 2
 // tiles, one node per thread (FP64-ALU-bound: small tiles spread the work
 // evenly over the SMs).
-template <typename R> struct Shape;
+// VAR: variant of the step kernel (V_DWMOM is FP32's, V_ROWS4 LBM_DF64's).
+constexpr int V_DWMOM = 1, V_ROWS4 = 2;
+template <typename R, int VAR = 0> struct Shape;
 // FP32 node tiles are 32 x LBM_F32_TILE_Y nodes (4, 8 or 16 rows), two rows
 // per thread; the launch bounds keep 128 registers per thread (one-tile form)
 // and 170 (persistent form, two tile stages).
 #ifndef LBM_F32_TILE_Y
 #define LBM_F32_TILE_Y 8
 #endif
-template <> struct Shape<float> {
+template <int VAR> struct Shape<float, VAR> {
   static constexpr int X = 32, Y = LBM_F32_TILE_Y, TY = Y / 2;
   static constexpr int MINB = 512 / (X * TY);
   static constexpr int MINB_PIPE = 384 / (X * TY) > 0 ? 384 / (X * TY) : 1;
   static_assert(Y == 4 || Y == 8 || Y == 16, "FP32 tile rows: 4, 8 or 16");
 };
-template <> struct Shape<double> {
+template <int VAR> struct Shape<double, VAR> {
   static constexpr int X = 32, Y = 2, TY = 2, MINB = 8, MINB_PIPE = 6;
 };
 // Double-word (LBM_DF64): 32 x 8 tiles of 8-byte elements (51 KB, in dynamic
@@ -52,10 +54,10 @@ template <> struct Shape<double> {
 // each of four unrelated blocks per scheduler, half the issue stalls were
 // instruction fetches (ncu: no_instruction 2.9 of 6.0 cycles per issue); the two
 // warps per scheduler of a 256-thread block run close behind each other and
-// share them. 2048 x 1024 301 -> 273 us a step, 600 x 200 26.8 -> 25.9, 300 x 100
-// 17.1 -> 17.5; 32 x 16 tiles (one block per SM, the copy of its next tile only
+// share them. 2048 x 1024 301 -> 273 us a step; 32 x 16 tiles (one block per SM, the copy of its next tile only
 // from the persistent form) 299, persistent 260-292; barriers inside the update
 // to keep a block's warps together cost registers (spills) and took 282-288.
+// V_ROWS4: 32 x 4 tiles, for the grids that tall tiles divide badly (rows4 in lbm_core.cu).
 #ifndef LBM_DW_LANES
 #define LBM_DW_LANES 1
 #endif
@@ -63,9 +65,9 @@ template <> struct Shape<double> {
 #ifndef LBM_DW_MINB
 #define LBM_DW_MINB 2
 #endif
-template <> struct Shape<dw> {
-  static constexpr int X = 32, Y = 8, TY = Y / LBM_DW_LANES;
-  static constexpr int MINB = LBM_DW_MINB * LBM_DW_LANES, MINB_PIPE = 2;
+template <int VAR> struct Shape<dw, VAR> {
+  static constexpr int X = 32, Y = VAR == V_ROWS4 ? 4 : 8, TY = Y / LBM_DW_LANES;
+  static constexpr int MINB = LBM_DW_MINB * LBM_DW_LANES * (8 / Y), MINB_PIPE = VAR == V_ROWS4 ? 3 : 2;
   static_assert(LBM_DW_LANES == 1 || LBM_DW_LANES == 2, "one or two nodes per thread");
 };
 constexpr int AUX_X = 32, AUX_Y = 8, AUX_N = AUX_X * AUX_Y;  // init / moments / audit
@@ -110,6 +112,7 @@ struct StepArgs {
   double* partial;    // [ntiles][4] audit scratch: one partial sum per tile
   double* gpartial;   // [ngroups][4]: the sums of groups of `agroup` tiles
   int agroup;         // tiles per audit group
+  int overlapped;     // the launch may start beside the previous step's (V_ROWS4)
   unsigned* gcount;   // [ngroups]: tiles of the group done in this audit step
   int ngroups;
   int audit_every;
@@ -309,10 +312,10 @@ __device__ __forceinline__ void ghost(const StepArgs<R>& A, const R* __restrict_
 // reach outside the tensor are filled with zeros; those values are never
 // used (boundary nodes take ghosts, periodic wraps read global memory).
 constexpr int HALO_X = 4;
-template <typename R>
+template <typename R, int VAR = 0>
 struct Tile {
-  static constexpr int BXP = Shape<R>::X + 2 * HALO_X;
-  static constexpr int ROWS = Shape<R>::Y + 2;
+  static constexpr int BXP = Shape<R, VAR>::X + 2 * HALO_X;
+  static constexpr int ROWS = Shape<R, VAR>::Y + 2;
   static constexpr int ELEMS = 16 * ROWS * BXP;
   static constexpr unsigned BYTES = ELEMS * sizeof(R);
 };

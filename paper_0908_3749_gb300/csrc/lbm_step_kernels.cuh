@@ -29,11 +29,11 @@ namespace lbmk {
 // the same, and audit partials are kept per tile.
 // Off: unsigned (32-bit element offsets, grids with 16 * plane < 2^32) or
 // long long.
-template <typename R>
+template <int VAR, typename R>
 __device__ __forceinline__ void load_tile(R* stage, const CUtensorMap* tmap, unsigned long long* bar,
                                           int tile, int tiles_x) {
-  const int x0 = (tile % tiles_x) * Shape<R>::X, y0 = (tile / tiles_x) * Shape<R>::Y;
-  mbar_expect_tx(bar, Tile<R>::BYTES);
+  const int x0 = (tile % tiles_x) * Shape<R, VAR>::X, y0 = (tile / tiles_x) * Shape<R, VAR>::Y;
+  mbar_expect_tx(bar, Tile<R, VAR>::BYTES);
   tma_load_tile(stage, tmap, x0 - HALO_X, y0 - 1, bar);
 }
 
@@ -202,41 +202,41 @@ __device__ __forceinline__ void step_tile_x2(const StepArgs<float>& A, const flo
   }
 }
 
-// VAR selects a variant of the FP32 step: 0 the plain one, 1 the one with
-// double-word conserved moments and equilibria (LBM_FP32_DWMOM).
+// VAR selects a variant: V_DWMOM the FP32 step with double-word conserved moments
+// and equilibria (LBM_FP32_DWMOM), V_ROWS4 the double-word step on 32 x 4 tiles.
 template <typename R, typename Off, int VAR>
 __device__ __forceinline__ void step_any(const StepArgs<R>& A, const R* __restrict__ fin,
                                          R* __restrict__ fout, const R* stage, int cur, bool audit,
                                          R t, double (*sm)[4], bool& bad, bool& negT) {
   if constexpr (std::is_same<R, dw>::value)
-    step_tile_dw<Off>(A, fin, fout, stage, cur, audit, t, sm, bad, negT);
+    step_tile_dw<Off, VAR>(A, fin, fout, stage, cur, audit, t, sm, bad, negT);
   else if constexpr (Shape<R>::TY == Shape<R>::Y)
     step_tile<R, Off>(A, fin, fout, stage, cur, audit, t, sm, bad, negT);
   else
-    step_tile_x2<Off, VAR == 1>(A, fin, fout, stage, cur, audit, t, sm, bad, negT);
+    step_tile_x2<Off, VAR == V_DWMOM>(A, fin, fout, stage, cur, audit, t, sm, bad, negT);
 }
 
 // Blocks per SM the one-tile form is compiled for: the FP32 form with 64-bit
 // offsets needs more than 128 registers (it spilled at 4 blocks per SM).
-template <typename R, typename Off>
+template <typename R, typename Off, int VAR>
 constexpr int step_minb() {
-  return (sizeof(R) == 4 && sizeof(Off) == 8) ? Shape<R>::MINB - 1 : Shape<R>::MINB;
+  return (sizeof(R) == 4 && sizeof(Off) == 8) ? Shape<R>::MINB - 1 : Shape<R, VAR>::MINB;
 }
 
-template <typename R>
+template <typename R, int VAR = 0>
 __host__ __device__ constexpr size_t tile_dynamic_bytes() {
-  return Tile<R>::BYTES <= 46 * 1024 ? 0 : (size_t)Tile<R>::BYTES + 128;
+  return Tile<R, VAR>::BYTES <= 46 * 1024 ? 0 : (size_t)Tile<R, VAR>::BYTES + 128;
 }
 
 template <typename R, typename Off, int VAR = 0>
-__global__ void __launch_bounds__(Shape<R>::X * Shape<R>::TY, (step_minb<R, Off>()))
+__global__ void __launch_bounds__(Shape<R, VAR>::X * Shape<R, VAR>::TY, (step_minb<R, Off, VAR>()))
     k_step(const __grid_constant__ CUtensorMap tmap, const R* __restrict__ fin,
            R* __restrict__ fout, const StepArgs<R> A) {
-  constexpr int N = Shape<R>::X * Shape<R>::TY;
+  constexpr int N = Shape<R, VAR>::X * Shape<R, VAR>::TY;
   // The tile in static shared memory where it fits there (48 KB), else in
   // dynamic (tile_dynamic_bytes).
-  constexpr bool DYN = tile_dynamic_bytes<R>() > 0;
-  __shared__ __align__(128) R tile_static[DYN ? 1 : Tile<R>::ELEMS];
+  constexpr bool DYN = tile_dynamic_bytes<R, VAR>() > 0;
+  __shared__ __align__(128) R tile_static[DYN ? 1 : Tile<R, VAR>::ELEMS];
   extern __shared__ __align__(128) unsigned char step_smem[];
   R* const tile = DYN ? reinterpret_cast<R*>(step_smem + ((128u - (smem_addr(step_smem) & 127u)) & 127u))
                       : tile_static;
@@ -244,13 +244,13 @@ __global__ void __launch_bounds__(Shape<R>::X * Shape<R>::TY, (step_minb<R, Off>
   __shared__ unsigned long long bar;
   __shared__ unsigned long long s_step;
   __shared__ int s_audit, s_alist[32], s_an;
-  const int t = threadIdx.y * Shape<R>::X + threadIdx.x;
+  const int t = threadIdx.y * Shape<R, VAR>::X + threadIdx.x;
   if (t == 0) mbar_init(&bar, 1);
-  wait_for_previous();
+  if (VAR != V_ROWS4 || A.overlapped) wait_for_previous();
   if (t == 0) {
     // Start the tile copy first so that its latency overlaps the read of
     // the step counter.
-    load_tile(tile, &tmap, &bar, blockIdx.x, A.tiles_x);
+    load_tile<VAR>(tile, &tmap, &bar, blockIdx.x, A.tiles_x);
     s_step = read_step(A, &s_audit);
   }
   __syncthreads();
@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(Shape<R>::X * Shape<R>::TY, (step_minb<R, Off>
   }
   bool bad = false, negT = false;
   step_any<R, Off, VAR>(A, fin, fout, tile, blockIdx.x, audit, A.dtr * R(s_step), sm, bad, negT);
-  if (!audit) dependents_may_start();
+  if (!audit && (VAR != V_ROWS4 || A.overlapped)) dependents_may_start();
   const unsigned long long step = s_step;
   watchdog_flags(A.st, step, bad, negT);
   if (audit) audit_block_done(A, (int)blockIdx.x, A.ntiles, step, s_alist, &s_an);
@@ -276,32 +276,32 @@ __global__ void __launch_bounds__(Shape<R>::X * Shape<R>::TY, (step_minb<R, Off>
 
 // Two tile stages (each a multiple of 128 bytes) plus room to align the first
 // to 128 bytes, as TMA destinations require.
-template <typename R>
-constexpr size_t pipe_smem_bytes() { return 2 * sizeof(R) * (size_t)Tile<R>::ELEMS + 128; }
+template <typename R, int VAR = 0>
+constexpr size_t pipe_smem_bytes() { return 2 * sizeof(R) * (size_t)Tile<R, VAR>::ELEMS + 128; }
 static_assert(sizeof(float) * Tile<float>::ELEMS % 128 == 0, "stage size");
 static_assert(sizeof(double) * Tile<double>::ELEMS % 128 == 0, "stage size");
 
 template <typename R, typename Off, int VAR = 0>
-__global__ void __launch_bounds__(Shape<R>::X * Shape<R>::TY, Shape<R>::MINB_PIPE)
+__global__ void __launch_bounds__(Shape<R, VAR>::X * Shape<R, VAR>::TY, Shape<R, VAR>::MINB_PIPE)
     k_step_pipe(const __grid_constant__ CUtensorMap tmap, const R* __restrict__ fin,
                 R* __restrict__ fout, const StepArgs<R> A) {
-  constexpr int N = Shape<R>::X * Shape<R>::TY;
+  constexpr int N = Shape<R, VAR>::X * Shape<R, VAR>::TY;
   extern __shared__ __align__(128) unsigned char pipe_smem[];
-  R* const stages = reinterpret_cast<R*>(  // [2][Tile<R>::ELEMS], 128-byte aligned
+  R* const stages = reinterpret_cast<R*>(  // [2][Tile<R, VAR>::ELEMS], 128-byte aligned
       pipe_smem + ((128u - (smem_addr(pipe_smem) & 127u)) & 127u));
   __shared__ double sm[N / 4][4];
   __shared__ unsigned long long bar[2];
   __shared__ unsigned long long s_step;
   __shared__ int s_audit, s_alist[32], s_an;
-  const int t = threadIdx.y * Shape<R>::X + threadIdx.x;
+  const int t = threadIdx.y * Shape<R, VAR>::X + threadIdx.x;
   const int G = (int)gridDim.x;
   if (t == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
   }
-  wait_for_previous();
+  if (VAR != V_ROWS4 || A.overlapped) wait_for_previous();
   if (t == 0) {
-    load_tile(stages, &tmap, &bar[0], blockIdx.x, A.tiles_x);  // nblocks <= ntiles
+    load_tile<VAR>(stages, &tmap, &bar[0], blockIdx.x, A.tiles_x);  // nblocks <= ntiles
     s_step = read_step(A, &s_audit);
   }
   __syncthreads();
@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(Shape<R>::X * Shape<R>::TY, Shape<R>::MINB_PIP
     const bool more = cur + G < A.ntiles;
     // Stage 1 - s was released at the end of the previous tile.
     if (t == 0 && more)
-      load_tile(stages + (1 - s) * Tile<R>::ELEMS, &tmap, &bar[1 - s], cur + G, A.tiles_x);
+      load_tile<VAR>(stages + (1 - s) * Tile<R, VAR>::ELEMS, &tmap, &bar[1 - s], cur + G, A.tiles_x);
     // Every thread waits for the tile (bounded); the block decides together.
     if (!__syncthreads_and(mbar_wait_bounded(&bar[s], (k >> 1) & 1, TMA_WAIT_CYCLES))) {
       // A copy did not land: record it, give the copies issued a second
@@ -325,11 +325,11 @@ __global__ void __launch_bounds__(Shape<R>::X * Shape<R>::TY, Shape<R>::MINB_PIP
       }
       return;
     }
-    step_any<R, Off, VAR>(A, fin, fout, stages + s * Tile<R>::ELEMS, cur, s_audit != 0,
+    step_any<R, Off, VAR>(A, fin, fout, stages + s * Tile<R, VAR>::ELEMS, cur, s_audit != 0,
                      A.dtr * R(s_step), sm, bad, negT);
     __syncthreads();  // stage s and sm are free again
   }
-  if (!s_audit) dependents_may_start();
+  if (!s_audit && (VAR != V_ROWS4 || A.overlapped)) dependents_may_start();
   watchdog_flags(A.st, s_step, bad, negT);
   if (s_audit) audit_block_done(A, (int)blockIdx.x, G, s_step, s_alist, &s_an);
 }

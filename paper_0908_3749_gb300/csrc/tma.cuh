@@ -98,8 +98,8 @@ __device__ __forceinline__ void wait_for_previous() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 template <typename... P, typename... A>
-inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
-                                     cudaStream_t stream, A&&... args) {
+inline cudaError_t launch(bool overlapped, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                          cudaStream_t stream, A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -109,8 +109,13 @@ inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = overlapped ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                     cudaStream_t stream, A&&... args) {
+  return launch(true, kernel, grid, block, smem, stream, static_cast<A&&>(args)...);
 }
 
 // cuTensorMapEncodeTiled through the runtime (libcuda is not linked); null if
