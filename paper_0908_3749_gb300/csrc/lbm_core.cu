@@ -584,6 +584,23 @@ int repitch(lbm_ctx* c, const void* src, long long sp, void* dst, long long dp) 
   return LBM_OK;
 }
 
+// The same for an array of the caller's on the device (`own`: the context's side, of row
+// pitch c->pitch). The kernel takes memory of this device whose elements are aligned;
+// any other pointer (LBM_DF64's pairs at a 4-byte boundary, managed, mapped or another
+// device's memory) goes through the copy engine, which checks it.
+int copy_user_rows(lbm_ctx* c, void* dst, const void* src, bool to_user) {
+  const void* user = to_user ? dst : src;
+  cudaPointerAttributes at;
+  int dev = 0;
+  const bool direct = (uintptr_t)user % c->esize == 0 && cudaPointerGetAttributes(&at, user) == cudaSuccess &&
+                      at.type == cudaMemoryTypeDevice && cudaGetDevice(&dev) == cudaSuccess && at.device == dev;
+  if (direct) return to_user ? repitch(c, src, c->pitch, dst, c->cfg.nx) : repitch(c, src, c->cfg.nx, dst, c->pitch);
+  const size_t w = (size_t)c->cfg.nx * c->esize, own = (size_t)c->pitch * c->esize;
+  CK(c, cudaMemcpy2DAsync(dst, to_user ? w : own, src, to_user ? own : w, w, (size_t)16 * c->cfg.ny,
+                          cudaMemcpyDeviceToDevice, c->stream));
+  return LBM_OK;
+}
+
 // Device buffer for one contiguous copy of the populations (host transfers).
 int population_stage(lbm_ctx* c) {
   if (!c->pstage)
@@ -976,7 +993,7 @@ int lbm_get_populations(lbm_ctx* c, void* f, long long* step, int on_device) {
   const size_t w = (size_t)c->cfg.nx * c->esize;
   const size_t bytes = w * 16 * c->cfg.ny;
   if (on_device) {
-    const int rc = repitch(c, c->f[c->cur], c->pitch, f, c->cfg.nx);
+    const int rc = copy_user_rows(c, f, c->f[c->cur], true);
     if (rc != LBM_OK) return rc;
   } else if (c->pitch == c->cfg.nx) {  // rows unpadded: one contiguous copy
     CK(c, cudaMemcpyAsync(f, c->f[c->cur], bytes, cudaMemcpyDeviceToHost, c->stream));
@@ -1003,7 +1020,7 @@ int lbm_set_populations(lbm_ctx* c, const void* f, long long step, int on_device
   const size_t bytes = w * 16 * c->cfg.ny;
   c->cur = 0;
   if (on_device) {
-    const int rc = repitch(c, f, c->cfg.nx, c->f[0], c->pitch);
+    const int rc = copy_user_rows(c, c->f[0], f, false);
     if (rc != LBM_OK) return rc;
   } else if (c->pitch == c->cfg.nx) {
     CK(c, cudaMemcpyAsync(c->f[0], f, bytes, cudaMemcpyHostToDevice, c->stream));
