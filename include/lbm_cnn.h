@@ -41,6 +41,13 @@ int lbm_cnn_set_params(lbm_cnn* n, const float* params, int on_device);
 int lbm_cnn_get_params(lbm_cnn* n, float* params, int on_device);
 int lbm_cnn_set_adam(lbm_cnn* n, double lr, double beta1, double beta2, double eps);
 
+/* The kernels' waits for their own copies and products are bounded (about 1 s). When
+ * one expires, lbm_cnn_loss_grad, lbm_cnn_train_step with a loss, or lbm_cnn_correct
+ * returns LBM_ERR_TIMEOUT, the first of them after it, and its outputs are not valid.
+ * The parameters and the Adam state are then those before the step in which the
+ * wait expired: that step and those issued after it, up to the report, were left
+ * out. The next call starts anew; lbm_cnn_set_params forgets an expired wait. */
+
 /* Loss (mean squared or absolute feature error against the target fields,
  * lbm_cnn_set_loss) and the
  * gradient of every parameter (packed, FP32) for one coarse / target pair,
@@ -88,6 +95,10 @@ int lbm_cnn_correct(lbm_cnn* n, const double* coarse, double* corrected,
  * Hf and Wf must be multiples of r. Asynchronous on cuda_stream. */
 int lbm_restrict(const double* fine, int Hf, int Wf, int r, double* coarse,
                  void* cuda_stream);
+
+/* Test hook for the bounded waits: those for copies (bit 0) and for products (bit 1)
+ * of the following calls expire at once; 0 switches it off. */
+int lbm_cnn_debug_give_up(lbm_cnn* n, int which);
 
 const char* lbm_cnn_last_error(lbm_cnn* n);
 

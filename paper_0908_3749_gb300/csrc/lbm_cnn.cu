@@ -27,6 +27,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -51,6 +52,24 @@ __host__ __device__ constexpr int param_offset(int l) { return l == 0 ? 0 : para
 static_assert(param_offset(NL) == LBM_CNN_NPARAMS, "packed parameters");
 __host__ __device__ constexpr int kp_of(int l) { return ru(9 * cin_of(l), 16); }   // K of the forward operand
 __host__ __device__ constexpr int kb_of(int l) { return ru(9 * cout_of(l), 16); }  // of the input-gradient one
+
+// Results that a call hands to the host, in one copy.
+struct Results {
+  double loss;
+  double mass[2];  // sums of the corrected and of the coarse density
+  int timeout;     // a bounded wait expired in some kernel since the last report
+  int skipped;     // updates left out since then
+  unsigned done;   // blocks of k_apply finished
+};
+
+// Waits of the convolution and weight-gradient kernels: bounded; when one expires,
+// the block sets Results::timeout, waits once more for the copies and products that
+// it has in flight, frees its tensor memory and leaves. k_update then leaves
+// the parameters alone. give_up (test hook): the waits that expire at once.
+enum GiveUp { GIVE_UP_COPIES = 1, GIVE_UP_PRODUCTS = 2 };
+__device__ __forceinline__ bool wait_for(unsigned long long* bar, unsigned parity, bool give_up) {
+  return !give_up && gbtma::mbar_wait_bounded(bar, parity, gbtma::TMA_WAIT_CYCLES);
+}
 
 // ---------------------------------------------------------------------------
 // Tensor-core implicit-GEMM 3 x 3 convolution
@@ -124,7 +143,8 @@ __global__ void __launch_bounds__(CV_T, CV_CTAS_PER_SM)
     k_conv(const __grid_constant__ CUtensorMap map, int H, int W, int tiles_x, int ntiles,
            const __nv_bfloat16* __restrict__ Wt, const float* __restrict__ bias,
            const unsigned* __restrict__ bits_in, __nv_bfloat16* __restrict__ out_bf,
-           float* __restrict__ out_f, unsigned* __restrict__ bits_out, int* __restrict__ timeout) {
+           float* __restrict__ out_f, unsigned* __restrict__ bits_out, int* __restrict__ timeout,
+           int give_up) {
   constexpr int NP = cv_n(COUT), TM = CV_SLOTS * 2 * NP;  // TMEM columns
   constexpr unsigned IDESC = tc05::idesc_f32acc(tc05::FMT_BF16, 128, NP);
   extern __shared__ __align__(128) unsigned char conv_raw[];
@@ -167,18 +187,20 @@ __global__ void __launch_bounds__(CV_T, CV_CTAS_PER_SM)
   tc05::fence_after();
   const unsigned tmem = s_tmem, a0 = gbtma::smem_addr(base), b0 = gbtma::smem_addr(sw);
 
-  constexpr long long LIMIT = gbtma::TMA_WAIT_CYCLES;
+  const bool no_copy = give_up & GIVE_UP_COPIES, no_product = give_up != 0;  // no products without copies
   bool ok = true;  // every wait of this thread has ended in time
+  int issued = 0;  // by this thread: tiles copied, tiles multiplied
   if (t == CV_EPI_T) {  // copies beyond the first CV_SLOTS: once the slot's products have read it
-    for (int k = CV_SLOTS; k < mine && ok; ++k) {
-      ok = gbtma::mbar_wait_bounded(&done[k % CV_SLOTS], phase(k - CV_SLOTS), LIMIT);
-      if (ok) load(k);
+    for (issued = min(mine, CV_SLOTS); issued < mine; ++issued) {
+      ok = wait_for(&done[issued % CV_SLOTS], phase(issued - CV_SLOTS), no_product);
+      if (!ok) break;
+      load(issued);
     }
   } else if (t == CV_EPI_T + 32) {  // products
-    for (int k = 0; k < mine && ok; ++k) {
+    for (int k = 0; k < mine; ++k) {
       const int s = k % CV_SLOTS;
-      if (k >= CV_SLOTS) ok = gbtma::mbar_wait_bounded(&drained[s], phase(k - CV_SLOTS), LIMIT);
-      ok = ok && gbtma::mbar_wait_bounded(&full[s], phase(k), LIMIT);
+      if (k >= CV_SLOTS) ok = wait_for(&drained[s], phase(k - CV_SLOTS), no_product);
+      ok = ok && wait_for(&full[s], phase(k), no_copy);
       if (!ok) break;
       tc05::fence_after();
       const unsigned as = a0 + s * CV_STAGE, ts = tmem + s * 2 * NP;
@@ -195,6 +217,7 @@ __global__ void __launch_bounds__(CV_T, CV_CTAS_PER_SM)
                           tc05::smem_desc(b0 + ks * 2 * NP * 16, NP * 16, 128), IDESC, ks > 0 ? 1u : 0u);
           }
       tc05::commit(&done[s]);
+      issued = k + 1;
     }
   } else if (t < CV_EPI_T) {  // epilogue: row t / 8 of the tile, pixels t % 8 and 8 + t % 8
     for (int k = 0; k < mine; ++k) {
@@ -207,7 +230,7 @@ __global__ void __launch_bounds__(CV_T, CV_CTAS_PER_SM)
 #pragma unroll
         for (int m = 0; m < 2; ++m)
           if (y < H && x0 + 8 * m < W) keep[m] = __ldg(bits_in + (long long)y * W + x0 + 8 * m);
-      ok = __all_sync(0xffffffffu, gbtma::mbar_wait_bounded(&done[s], phase(k), LIMIT));
+      ok = __all_sync(0xffffffffu, wait_for(&done[s], phase(k), no_product));
       if (!ok) break;
       tc05::fence_after();
 #pragma unroll
@@ -252,12 +275,15 @@ __global__ void __launch_bounds__(CV_T, CV_CTAS_PER_SM)
     }
   }
   __syncwarp();
-  if (__syncthreads_or(!ok) && t == 0) {
-    // A copy or products did not complete in time: record it, give every copy
-    // that was issued (at most the last CV_SLOTS) a second bounded wait.
-    atomicExch(timeout, 1);
-    for (int k = max(0, mine - CV_SLOTS); k < mine; ++k)
-      gbtma::mbar_wait_bounded(&full[k % CV_SLOTS], phase(k), LIMIT / 4);
+  if (__syncthreads_or(!ok)) {
+    // A copy or products did not complete in time: record it; the threads that issued
+    // them give the last of each slot (the others have been waited for) a second
+    // bounded wait, so that nothing reads or writes this CTA's memory after it.
+    if (t == 0) atomicExch(timeout, 1);
+    for (int k = max(0, issued - CV_SLOTS); k < issued; ++k)
+      gbtma::mbar_wait_bounded(t == CV_EPI_T ? &full[k % CV_SLOTS] : &done[k % CV_SLOTS], phase(k),
+                               gbtma::TMA_WAIT_CYCLES);
+    __syncwarp();
   }
   tc05::fence_before();
   __syncthreads();
@@ -297,7 +323,7 @@ constexpr unsigned C4_SMEM = C4_STAGE + 32 * C4_PITCH * 2 + 128;
 __global__ void __launch_bounds__(CT_T, C4_CTAS_PER_SM)
     k_conv4(const __grid_constant__ CUtensorMap map, int H, int W, int tiles_x, int ntiles,
             const __nv_bfloat16* __restrict__ Wt, const unsigned* __restrict__ bits_in,
-            __nv_bfloat16* __restrict__ out, int* __restrict__ timeout) {
+            __nv_bfloat16* __restrict__ out, int* __restrict__ timeout, int give_up) {
   extern __shared__ __align__(128) unsigned char conv_raw[];
   unsigned char* const base = conv_raw + ((128u - (gbtma::smem_addr(conv_raw) & 127u)) & 127u);
   __shared__ unsigned long long bar;
@@ -332,7 +358,7 @@ __global__ void __launch_bounds__(CT_T, C4_CTAS_PER_SM)
         const int y = y0 + (m >> 1), x = x0 + (m & 1) * 16 + h * 8 + g;
         keep[m][h] = y < H && x < W ? __ldg(bits_in + (long long)y * W + x) << (4 * tig) : 0u;
       }
-    if (!__syncthreads_and(gbtma::mbar_wait_bounded(&bar, k & 1, gbtma::TMA_WAIT_CYCLES))) {
+    if (!__syncthreads_and(wait_for(&bar, k & 1, give_up & GIVE_UP_COPIES))) {
       // The copy did not land in time: record it, wait once more (bounded), leave.
       if (threadIdx.x == 0) {
         atomicExch(timeout, 1);
@@ -470,7 +496,7 @@ __device__ __forceinline__ void split3(float x, unsigned (&p)[3]) {
 template <int CG, int COUT>
 __global__ void __launch_bounds__(WG_T, WG_CTAS_PER_SM)
     k_wgrad(const __grid_constant__ CUtensorMap act, const __grid_constant__ CUtensorMap dz,
-            int tiles_x, int ntiles, float* __restrict__ partial, int* __restrict__ timeout) {
+            int tiles_x, int ntiles, float* __restrict__ partial, int* __restrict__ timeout, int give_up) {
   constexpr int NP = COUT == 32 ? 32 : 16;  // N of the MMA
   constexpr int CIN = CG == 4 ? 32 : 4;
   constexpr int NOUT = 9 * CIN * COUT + COUT;
@@ -507,17 +533,21 @@ __global__ void __launch_bounds__(WG_T, WG_CTAS_PER_SM)
   const unsigned tmem = s_tmem;
 
   float db[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // bias sums: pixel column `lane`, group `warp`
+  const bool no_copy = give_up & GIVE_UP_COPIES, no_product = give_up & GIVE_UP_PRODUCTS;
   bool ok = true;
-  int k = 0;
+  int k = 0, loaded = 1, multiplied = 0;  // tiles copied and multiplied (thread 0)
   for (int tile = blockIdx.x; tile < ntiles; tile += G, ++k) {
     const int st = k & 1;
     if (t == 0) {
       // Stage 1 - st: tile k - 1's products must have read it (the bias sums
       // have, by the barrier at the end of the loop body).
-      if (k > 0) ok = gbtma::mbar_wait_bounded(&used[1 - st], ((k - 1) >> 1) & 1, gbtma::TMA_WAIT_CYCLES);
-      if (ok && tile + G < ntiles) load(tile + G, 1 - st);
+      if (k > 0) ok = wait_for(&used[1 - st], ((k - 1) >> 1) & 1, no_product);
+      if (ok && tile + G < ntiles) {
+        load(tile + G, 1 - st);
+        ++loaded;
+      }
     }
-    ok = __syncthreads_and(ok && gbtma::mbar_wait_bounded(&full[st], (k >> 1) & 1, gbtma::TMA_WAIT_CYCLES));
+    ok = __syncthreads_and(ok && wait_for(&full[st], (k >> 1) & 1, no_copy));
     if (!ok) break;
     const unsigned a = gbtma::smem_addr(base) + st * S::STAGE, b = a + S::A_BYTES;
     if (t == 0) {
@@ -533,6 +563,7 @@ __global__ void __launch_bounds__(WG_T, WG_CTAS_PER_SM)
                           tc05::smem_desc(b + r * S::BROW + kg * 16 * PX_BYTES, 128, S::BGROUP), IDESC,
                           (k > 0 || r > 0 || kg > 0) ? 1u : 0u);
       tc05::commit(&used[st]);
+      ++multiplied;
     }
     if (warp < COUT / 8 || warp == 0) {
 #pragma unroll
@@ -550,17 +581,19 @@ __global__ void __launch_bounds__(WG_T, WG_CTAS_PER_SM)
     __syncthreads();
   }
   // The last tile's products (every earlier one was waited for).
-  if (ok) ok = gbtma::mbar_wait_bounded(&used[(k - 1) & 1], ((k - 1) >> 1) & 1, gbtma::TMA_WAIT_CYCLES);
+  if (ok) ok = wait_for(&used[(k - 1) & 1], ((k - 1) >> 1) & 1, no_product);
   ok = __syncthreads_and(ok);
   float* out = partial + (long long)blockIdx.x * NOUT;
   if (!ok) {
-    // A copy or the products did not complete in time: record it, wait once
-    // more (bounded) for both, free tensor memory.
+    // A copy or the products did not complete in time: record it, wait once more
+    // (bounded) for the last copy and the last products of each stage (the others
+    // have been waited for), free tensor memory.
     if (t == 0) {
       atomicExch(timeout, 1);
-      const int st = k & 1;
-      gbtma::mbar_wait_bounded(&full[st], (k >> 1) & 1, gbtma::TMA_WAIT_CYCLES);
-      if (k > 0) gbtma::mbar_wait_bounded(&used[1 - st], ((k - 1) >> 1) & 1, gbtma::TMA_WAIT_CYCLES);
+      for (int j = max(0, loaded - 2); j < loaded; ++j)
+        gbtma::mbar_wait_bounded(&full[j & 1], (j >> 1) & 1, gbtma::TMA_WAIT_CYCLES);
+      for (int j = max(0, multiplied - 2); j < multiplied; ++j)
+        gbtma::mbar_wait_bounded(&used[j & 1], (j >> 1) & 1, gbtma::TMA_WAIT_CYCLES);
     }
     tc05::fence_before();
     __syncthreads();
@@ -913,7 +946,7 @@ struct UpdateArgs {
   const double* lpart;    // loss partials
   int nl;
   double lscale;
-  double* loss;
+  Results* res;           // loss, timeout, skipped
   int adam;
   float lr, b1, b2, eps, c1, c2;
 };
@@ -921,6 +954,12 @@ __global__ void __launch_bounds__(UP_N * UP_S) k_update(const UpdateArgs A) {
   gbtma::dependents_may_start();
   gbtma::wait_for_previous();
   const int t = threadIdx.x;
+  // A wait of a kernel before expired: its partials are not this step's. Nothing
+  // is updated; the host learns of it from the flag.
+  if (*(volatile int*)&A.res->timeout) {
+    if (blockIdx.x == 0 && t == 0 && A.adam) ++A.res->skipped;
+    return;
+  }
   if (blockIdx.x == gridDim.x - 1) {
     __shared__ double sl[UP_N * UP_S];
     double s = 0.0;
@@ -931,7 +970,7 @@ __global__ void __launch_bounds__(UP_N * UP_S) k_update(const UpdateArgs A) {
       if (t < st) sl[t] += sl[t + st];
       __syncthreads();
     }
-    if (t == 0) *A.loss = sl[0] * A.lscale;
+    if (t == 0) A.res->loss = sl[0] * A.lscale;
     return;
   }
   __shared__ float sm[UP_S][UP_N];
@@ -994,14 +1033,6 @@ __global__ void k_pack(const float* __restrict__ w, int cin, int cout, int kp, i
     wb[i] = __float2bfloat16(val);
   }
 }
-
-// Results that a call hands to the host, in one copy.
-struct Results {
-  double loss;
-  double mass[2];  // sums of the corrected and of the coarse density
-  int timeout;     // a bounded wait expired in some kernel (sticky)
-  unsigned done;   // blocks of k_apply finished
-};
 
 // corrected planes from output features x + z and the two masses (NaN for a
 // non-finite output): block partial sums, added by the block that finishes
@@ -1153,6 +1184,7 @@ struct lbm_cnn {
   float lr = 1e-3f, b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   Scale4 scale = {{1.f, 1.f, 1.f, 1.f}};
   int loss_kind = LBM_CNN_LOSS_MSE;
+  int give_up = 0;  // test hook: GiveUp
   std::string err = "no error";
 };
 
@@ -1182,14 +1214,24 @@ int pack_all(lbm_cnn* n) {
   return LBM_OK;
 }
 
+// Forgets an expired wait.
+int clear_timeout(lbm_cnn* n) {
+  static_assert(offsetof(Results, skipped) == offsetof(Results, timeout) + sizeof(int), "one memset");
+  CCK(n, cudaMemsetAsync(&n->res->timeout, 0, 2 * sizeof(int), n->stream));
+  return LBM_OK;
+}
+
 // Copies the results to the host (n->h_res), synchronises and reports an
-// expired wait.
+// expired wait, once: the updates since it were left out, and their numbers are
+// taken back.
 int fetch_results(lbm_cnn* n) {
   CCK(n, cudaMemcpyAsync(n->h_res, n->res, sizeof(Results), cudaMemcpyDeviceToHost, n->stream));
   CCK(n, cudaStreamSynchronize(n->stream));
-  return n->h_res->timeout
-             ? cfail(n, LBM_ERR_TIMEOUT, "a tile load (TMA) or product did not complete within its time limit")
-             : LBM_OK;
+  if (!n->h_res->timeout) return LBM_OK;
+  n->step -= n->h_res->skipped;
+  const int rc = clear_timeout(n);
+  return rc != LBM_OK ? rc
+                      : cfail(n, LBM_ERR_TIMEOUT, "a tile load (TMA) or product did not complete within its time limit");
 }
 
 // Tensor map of a row-planar BF16 image of `ncg` channel groups: dims (x in
@@ -1216,7 +1258,7 @@ int conv(lbm_cnn* n, const CUtensorMap& in, const __nv_bfloat16* wt, const float
   const int grid = std::min(n->cntiles, CV_CTAS_PER_SM * n->sms);
   CCK(n, gbtma::launch_overlapped(k_conv<COUT, EPI>, grid, CV_T, cv_smem(COUT), n->stream, in, n->H, n->W,
                                   n->ctiles_x, n->cntiles, wt, bias, bits_in, ob, of, bits_out,
-                                  &n->res->timeout));
+                                  &n->res->timeout, n->give_up));
   return LBM_OK;
 }
 
@@ -1239,7 +1281,7 @@ int forward(lbm_cnn* n, const double* coarse, bool train) {
 template <int CG, int COUT>
 int wgrad(lbm_cnn* n, const CUtensorMap& act, const CUtensorMap& dz, float* partial) {
   CCK(n, gbtma::launch_overlapped(k_wgrad<CG, COUT>, n->wblocks, WG_T, WgShape<CG, COUT == 32 ? 32 : 16>::SMEM,
-                                  n->stream, act, dz, n->tiles_x, n->ntiles, partial, &n->res->timeout));
+                                  n->stream, act, dz, n->tiles_x, n->ntiles, partial, &n->res->timeout, n->give_up));
   return LBM_OK;
 }
 
@@ -1262,7 +1304,7 @@ int loss_backward(lbm_cnn* n, const double* target, bool adam) {
   if ((rc = wgrad<4, 4>(n, n->m_act[4], n->g_dz5, part(4))) != LBM_OK) return rc;
   CCK(n, gbtma::launch_overlapped(k_conv4, std::min(n->ntiles, C4_CTAS_PER_SM * n->sms), CT_T, C4_SMEM, n->stream,
                                   n->m_dz5, n->H, n->W, n->tiles_x, n->ntiles, n->wb[4], n->pos[4], n->dz[1],
-                                  &n->res->timeout));
+                                  &n->res->timeout, n->give_up));
   if ((rc = wgrad<4, 32>(n, n->m_act[3], n->g_dz[1], part(3))) != LBM_OK) return rc;
   if ((rc = conv<32, EPI_MASK_BF16>(n, n->c_dz[1], n->wb[3], nullptr, n->pos[3], n->dz[0], nullptr)) != LBM_OK) return rc;
   if ((rc = wgrad<4, 32>(n, n->m_act[2], n->g_dz[0], part(2))) != LBM_OK) return rc;
@@ -1278,7 +1320,7 @@ int loss_backward(lbm_cnn* n, const double* target, bool adam) {
   U.lpart = n->dpart;
   U.nl = nb;
   U.lscale = 1.0 / (4.0 * n->npix);
-  U.loss = &n->res->loss;
+  U.res = n->res;
   U.adam = adam;
   U.lr = n->lr;
   U.b1 = n->b1;
@@ -1419,7 +1461,8 @@ int lbm_cnn_set_params(lbm_cnn* n, const float* params, int on_device) {
   CCK(n, cudaMemsetAsync(n->m, 0, sizeof(float) * LBM_CNN_NPARAMS, n->stream));
   CCK(n, cudaMemsetAsync(n->v, 0, sizeof(float) * LBM_CNN_NPARAMS, n->stream));
   n->step = 0;
-  const int rc = pack_all(n);
+  int rc = pack_all(n);
+  if (rc == LBM_OK) rc = clear_timeout(n);
   if (rc != LBM_OK) return rc;
   if (!on_device) CCK(n, cudaStreamSynchronize(n->stream));
   return LBM_OK;
@@ -1467,6 +1510,13 @@ int lbm_cnn_train_step(lbm_cnn* n, const double* coarse, const double* target, d
     if ((rc = fetch_results(n)) != LBM_OK) return rc;
     *loss = n->h_res->loss;
   }
+  return LBM_OK;
+}
+
+int lbm_cnn_debug_give_up(lbm_cnn* n, int which) {
+  if (!n || which < 0 || which > (GIVE_UP_COPIES | GIVE_UP_PRODUCTS))
+    return cfail(n, LBM_ERR_INVALID, "lbm_cnn_debug_give_up: which must be 0 .. 3");
+  n->give_up = which;
   return LBM_OK;
 }
 

@@ -486,6 +486,7 @@ _SIGS.update({
     "lbm_cnn_set_loss": (ctypes.c_int, [_vp, ctypes.c_int]),
     "lbm_cnn_residual_rms": (ctypes.c_int, [_vp, _vp, _vp, _vp]),
     "lbm_restrict": (ctypes.c_int, [_vp, ctypes.c_int, ctypes.c_int, ctypes.c_int, _vp, _vp]),
+    "lbm_cnn_debug_give_up": (ctypes.c_int, [_vp, ctypes.c_int]),
     "lbm_cnn_last_error": (ctypes.c_char_p, [_vp]),
 })
 
@@ -547,6 +548,10 @@ CNN_LOSS = {"mse": 0, "l1": 1}
 
 def lbm_cnn_set_loss(n, kind):
     _ccheck(load().lbm_cnn_set_loss(n, CNN_LOSS[kind]), n)
+
+
+def lbm_cnn_debug_give_up(n, which):
+    _ccheck(load().lbm_cnn_debug_give_up(n, int(which)), n)
 
 
 def lbm_cnn_set_output_scale(n, scale):
