@@ -141,9 +141,9 @@ __host__ __device__ constexpr unsigned cv_smem(int cout) {
 template <int COUT, int EPI>
 __global__ void __launch_bounds__(CV_T, CV_CTAS_PER_SM)
     k_conv(const __grid_constant__ CUtensorMap map, int H, int W, int tiles_x, int ntiles,
-           const __nv_bfloat16* __restrict__ Wt, const float* __restrict__ bias,
-           const unsigned* __restrict__ bits_in, __nv_bfloat16* __restrict__ out_bf,
-           float* __restrict__ out_f, unsigned* __restrict__ bits_out, int* __restrict__ timeout,
+           const __nv_bfloat16* Wt, const float* bias,
+           const unsigned* bits_in, __nv_bfloat16* out_bf,
+           float* out_f, unsigned* bits_out, int* timeout,
            int give_up) {
   constexpr int NP = cv_n(COUT), TM = CV_SLOTS * 2 * NP;  // TMEM columns
   constexpr unsigned IDESC = tc05::idesc_f32acc(tc05::FMT_BF16, 128, NP);
@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(CV_T, CV_CTAS_PER_SM)
   for (int i = t; i < NP * CV_KG; i += CV_T) {
     const int n = i / CV_KG, kg = i % CV_KG;
     *reinterpret_cast<uint4*>(sw + (kg * NP + n) * 16) =
-        n < ru(COUT, 8) ? __ldg(reinterpret_cast<const uint4*>(Wt) + i) : make_uint4(0, 0, 0, 0);
+        n < ru(COUT, 8) ? reinterpret_cast<const uint4*>(Wt)[i] : make_uint4(0, 0, 0, 0);
   }
   if (EPI != EPI_MASK_BF16 && t < COUT) s_bias[t] = bias[t];
   tc05::fence_async_smem();
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(CV_T, CV_CTAS_PER_SM)
       if constexpr (EPI == EPI_MASK_BF16)
 #pragma unroll
         for (int m = 0; m < 2; ++m)
-          if (y < H && x0 + 8 * m < W) keep[m] = __ldg(bits_in + (long long)y * W + x0 + 8 * m);
+          if (y < H && x0 + 8 * m < W) keep[m] = bits_in[(long long)y * W + x0 + 8 * m];
       ok = __all_sync(0xffffffffu, wait_for(&done[s], phase(k), no_product));
       if (!ok) break;
       tc05::fence_after();
@@ -322,8 +322,8 @@ constexpr unsigned C4_SMEM = C4_STAGE + 32 * C4_PITCH * 2 + 128;
 
 __global__ void __launch_bounds__(CT_T, C4_CTAS_PER_SM)
     k_conv4(const __grid_constant__ CUtensorMap map, int H, int W, int tiles_x, int ntiles,
-            const __nv_bfloat16* __restrict__ Wt, const unsigned* __restrict__ bits_in,
-            __nv_bfloat16* __restrict__ out, int* __restrict__ timeout, int give_up) {
+            const __nv_bfloat16* Wt, const unsigned* bits_in,
+            __nv_bfloat16* out, int* timeout, int give_up) {
   extern __shared__ __align__(128) unsigned char conv_raw[];
   unsigned char* const base = conv_raw + ((128u - (gbtma::smem_addr(conv_raw) & 127u)) & 127u);
   __shared__ unsigned long long bar;
@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(CT_T, C4_CTAS_PER_SM)
   constexpr int CHUNKS = C4_KP / 8;  // 16-byte pieces of a weight row
   for (int i = threadIdx.x; i < 32 * CHUNKS; i += CT_T)
     *reinterpret_cast<uint4*>(base + C4_STAGE + (i / CHUNKS) * (C4_PITCH * 2) + (i % CHUNKS) * 16) =
-        __ldg(reinterpret_cast<const uint4*>(Wt) + i);
+        reinterpret_cast<const uint4*>(Wt)[i];
   __syncthreads();
 
   for (int k = 0, tile = blockIdx.x; tile < ntiles; tile += G, ++k) {
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(CT_T, C4_CTAS_PER_SM)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int y = y0 + (m >> 1), x = x0 + (m & 1) * 16 + h * 8 + g;
-        keep[m][h] = y < H && x < W ? __ldg(bits_in + (long long)y * W + x) << (4 * tig) : 0u;
+        keep[m][h] = y < H && x < W ? bits_in[(long long)y * W + x] << (4 * tig) : 0u;
       }
     if (!__syncthreads_and(wait_for(&bar, k & 1, give_up & GIVE_UP_COPIES))) {
       // The copy did not land in time: record it, wait once more (bounded), leave.
@@ -496,7 +496,7 @@ __device__ __forceinline__ void split3(float x, unsigned (&p)[3]) {
 template <int CG, int COUT>
 __global__ void __launch_bounds__(WG_T, WG_CTAS_PER_SM)
     k_wgrad(const __grid_constant__ CUtensorMap act, const __grid_constant__ CUtensorMap dz,
-            int tiles_x, int ntiles, float* __restrict__ partial, int* __restrict__ timeout, int give_up) {
+            int tiles_x, int ntiles, float* partial, int* timeout, int give_up) {
   constexpr int NP = COUT == 32 ? 32 : 16;  // N of the MMA
   constexpr int CIN = CG == 4 ? 32 : 4;
   constexpr int NOUT = 9 * CIN * COUT + COUT;
@@ -677,10 +677,10 @@ __global__ void __launch_bounds__(WG_T, WG_CTAS_PER_SM)
 // 17 us; one pixel per thread in scalar FP32 was bound by its shared-memory
 // reads, 24 us.
 constexpr int C0_T = 128;
-__global__ void __launch_bounds__(C0_T) k_conv0(const float* __restrict__ xf, int H, int W,
-                                                const float* __restrict__ w,
-                                                __nv_bfloat16* __restrict__ out,
-                                                unsigned* __restrict__ bits) {
+__global__ void __launch_bounds__(C0_T) k_conv0(const float* xf, int H, int W,
+                                                const float* w,
+                                                __nv_bfloat16* out,
+                                                unsigned* bits) {
   __shared__ __align__(16) float sw[9 * 4 * 32 + 32];
   gbtma::dependents_may_start();
   gbtma::wait_for_previous();
@@ -701,7 +701,7 @@ __global__ void __launch_bounds__(C0_T) k_conv0(const float* __restrict__ xf, in
     for (int k = 0; k < 4; ++k) {
       const int xx = x + k - 1;
       in[k] = yy >= 0 && yy < H && xx >= 0 && xx < W
-                  ? __ldg(reinterpret_cast<const float4*>(xf) + (long long)yy * W + xx)
+                  ? reinterpret_cast<const float4*>(xf)[(long long)yy * W + xx]
                   : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 #pragma unroll
@@ -853,8 +853,8 @@ std::vector<ExpEntry> exp_table() {
 // 12 of 16 channels, row-planar; the other 4 stay zero).
 // Bound by memory (80 bytes a pixel with xs): 512 x 512 7 us; 33 us with the FP64
 // logarithms (the loss kernel, which takes the target's, 41 -> 16 us).
-__global__ void k_features(const double* __restrict__ f, int npix, int W, float* __restrict__ xf,
-                           __nv_bfloat16* __restrict__ xs, const LogEntry* __restrict__ logs) {
+__global__ void k_features(const double* f, int npix, int W, float* xf,
+                           __nv_bfloat16* xs, const LogEntry* __restrict__ logs) {
   gbtma::dependents_may_start();
   gbtma::wait_for_previous();
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -887,9 +887,9 @@ struct Scale4 {
 // (LBM_CNN_LOSS_L1, whose gradient is sign(d), 0 at d = 0), and its gradient
 // with respect to the network's output (BF16, 4 channels and 4 zeros). A pixel
 // per thread, whose target features are taken here; the sums in FP64, per block.
-__global__ void __launch_bounds__(256) k_loss(const float4* __restrict__ xf, const float4* __restrict__ z,
-                                              const double* __restrict__ target, int npix,
-                                              uint4* __restrict__ dz, double* __restrict__ partial,
+__global__ void __launch_bounds__(256) k_loss(const float4* xf, const float4* z,
+                                              const double* target, int npix,
+                                              uint4* dz, double* partial,
                                               const Scale4 sc, int l1,
                                               const LogEntry* __restrict__ logs) {
   __shared__ double sm[8];
@@ -1039,10 +1039,10 @@ __global__ void k_pack(const float* __restrict__ w, int cin, int cout, int kp, i
 // last in a fixed order. Bound by the FP64 units (two exponentials per pixel):
 // 512 x 512 about 20 us; 32 us with exp(), FP64 finiteness checks and the partials
 // added by the host.
-__global__ void __launch_bounds__(256) k_apply(const float4* __restrict__ xf, const float4* __restrict__ z,
-                                               int npix, double* __restrict__ out,
-                                               const double* __restrict__ coarse,
-                                               double* __restrict__ partial, const Scale4 sc,
+__global__ void __launch_bounds__(256) k_apply(const float4* xf, const float4* z,
+                                               int npix, double* out,
+                                               const double* coarse,
+                                               double* partial, const Scale4 sc,
                                                const ExpEntry* __restrict__ exps, Results* res) {
   __shared__ double sm[2][256];
   __shared__ bool s_last;

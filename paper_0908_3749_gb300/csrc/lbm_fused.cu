@@ -205,8 +205,8 @@ __device__ __forceinline__ void audit_pair(const StepArgs<float>& A, int tile,
 
 template <typename Off>
 __global__ void __launch_bounds__(NT, 4)
-    k_step2(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ fin,
-            float* __restrict__ fout, const StepArgs<float> A) {
+    k_step2(const __grid_constant__ CUtensorMap tmap, const float* fin,
+            float* fout, const StepArgs<float> A) {
   extern __shared__ __align__(128) unsigned char fused_smem[];
   float* const S0 = reinterpret_cast<float*>(
       fused_smem + ((128u - (smem_addr(fused_smem) & 127u)) & 127u));

@@ -85,7 +85,7 @@ __device__ __forceinline__ void lanes_arrive(const StepArgs<double>& A, int tile
 }
 
 __global__ void __launch_bounds__(LANES_T)
-    k_step_lanes(const double* __restrict__ fin, double* __restrict__ fout, const StepArgs<double> A) {
+    k_step_lanes(const double* fin, double* fout, const StepArgs<double> A) {
   __shared__ unsigned long long s_step;
   __shared__ int s_audit, s_alist[32], s_an;
   const int lane = threadIdx.x, g = lane & 3;

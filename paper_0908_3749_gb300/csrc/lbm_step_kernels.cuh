@@ -230,8 +230,8 @@ __host__ __device__ constexpr size_t tile_dynamic_bytes() {
 
 template <typename R, typename Off, int VAR = 0>
 __global__ void __launch_bounds__(Shape<R, VAR>::X * Shape<R, VAR>::TY, (step_minb<R, Off, VAR>()))
-    k_step(const __grid_constant__ CUtensorMap tmap, const R* __restrict__ fin,
-           R* __restrict__ fout, const StepArgs<R> A) {
+    k_step(const __grid_constant__ CUtensorMap tmap, const R* fin,
+           R* fout, const StepArgs<R> A) {
   constexpr int N = Shape<R, VAR>::X * Shape<R, VAR>::TY;
   // The tile in static shared memory where it fits there (48 KB), else in
   // dynamic (tile_dynamic_bytes).
@@ -283,8 +283,8 @@ static_assert(sizeof(double) * Tile<double>::ELEMS % 128 == 0, "stage size");
 
 template <typename R, typename Off, int VAR = 0>
 __global__ void __launch_bounds__(Shape<R, VAR>::X * Shape<R, VAR>::TY, Shape<R, VAR>::MINB_PIPE)
-    k_step_pipe(const __grid_constant__ CUtensorMap tmap, const R* __restrict__ fin,
-                R* __restrict__ fout, const StepArgs<R> A) {
+    k_step_pipe(const __grid_constant__ CUtensorMap tmap, const R* fin,
+                R* fout, const StepArgs<R> A) {
   constexpr int N = Shape<R, VAR>::X * Shape<R, VAR>::TY;
   extern __shared__ __align__(128) unsigned char pipe_smem[];
   R* const stages = reinterpret_cast<R*>(  // [2][Tile<R, VAR>::ELEMS], 128-byte aligned

@@ -149,8 +149,8 @@ __device__ __forceinline__ void tc_load_tile(float* dst, const CUtensorMap* tmap
 }
 
 __global__ void __launch_bounds__(TC_T, TC_CTAS_PER_SM)
-    k_step_tc(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ fin,
-              float* __restrict__ fout, const StepArgs<float> A,
+    k_step_tc(const __grid_constant__ CUtensorMap tmap, const float* fin,
+              float* fout, const StepArgs<float> A,
               const unsigned char* __restrict__ bconst, const TcWeights wk) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   TcSmem& S = *reinterpret_cast<TcSmem*>(smem_raw);

@@ -78,7 +78,10 @@ __device__ __forceinline__ void fence_proxy_async() {
 // of that one has called dependents_may_start() (or has ended): its blocks then
 // set up their barriers and wait in wait_for_previous() until the previous
 // kernel has completed and its writes are visible. Every thread calls that
-// before it touches memory that the previous kernel may write or read.
+// before it touches memory that the previous kernel may write or read. A kernel's
+// pointers to such memory are not __restrict__ and not read with __ldg: either
+// promises that the memory does not change while the kernel runs, and lets the compiler
+// move reads (and, for __restrict__, writes) above the wait.
 //
 // The step kernels call dependents_may_start() when a block has only its stores
 // left. Called at their top, the next step's blocks take whatever slots are free
