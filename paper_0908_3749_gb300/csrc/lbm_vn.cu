@@ -138,8 +138,9 @@ __device__ __forceinline__ bool is_zero(double x) {  // without the FP64 units
   return ((__double2hiint(x) & 0x7fffffff) | __double2loint(x)) == 0;
 }
 // The solver scales its matrix to entries below 2 in magnitude, so squares
-// cannot overflow; below TINY they may underflow.
-constexpr double TINY = 0x1p-900;
+// cannot overflow; sums of squares from TINY on have lost nothing to underflow (their
+// bits end above 2^-1022).
+constexpr double TINY = 0x1p-960;
 // Principal square root of z = x + i y, |z| = r: t = sqrt((r + |x|) / 2),
 // (t, y / (2 t)) when x >= 0, else (|y| / (2 t), sign(y) t); 0 for |z|^2 <
 // TINY. Used for shifts only, which may be guesses.
@@ -247,13 +248,16 @@ __device__ bool eig16(EigWork& W, int l0, bool active) {
     double tail = 0.0;
 #pragma unroll 1
     for (int i = c + 2; i < 16; ++i) tail += norm2(W.A[i][c]);
-    // Entries below 2^-450 beside ones of order 1 are left where they are (they
+    // Entries below 2^-480 beside ones of order 1 are left where they are (they
     // are not read again). The same decision in the group.
     const bool doit = tail >= TINY;
     const cplx x0 = W.A[c + 1][c];
-    const double n0 = norm2(x0);
-    const double i0 = rsq(n0);
-    const bool phase = n0 >= TINY;
+    // An x0 that small counts as zero in everything that follows: the reflection has to
+    // be one (its own inverse), or it changes the eigenvalues of the whole matrix.
+    const double x2 = norm2(x0);
+    const bool phase = x2 >= TINY;
+    const double n0 = phase ? x2 : 0.0;
+    const double i0 = rsq(x2);
     const double ax0 = phase ? n0 * i0 : 0.0;
     const cplx ph = phase ? i0 * x0 : mk(1.0, 0.0);
     const double s2 = n0 + tail, sigma = s2 * rsq(s2);
