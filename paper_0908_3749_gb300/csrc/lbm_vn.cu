@@ -325,12 +325,13 @@ __device__ bool eig16(EigWork& W, int l0, bool active) {
       for (int j = 0; j < N; ++j) {
         const int l = l0 + L * j;
         // An entry within 2^-48 of the largest component on the diagonal (by
-        // exponents, off the FP64 units) is not small; the others are looked at.
+        // exponents, off the FP64 units) is not small; the others are looked at, and all
+        // beside a diagonal so small that the difference has no meaning.
         bool look = false;
         if (l >= 1 && l <= hi) {
           const cplx p = W.A[l - 1][l - 1], q = W.A[l][l], o = W.A[l][l - 1];
           const int ed = max(max(exponent(p.re), exponent(p.im)), max(exponent(q.re), exponent(q.im)));
-          look = max(exponent(o.re), exponent(o.im)) <= ed - 48 || ed == 0;
+          look = max(exponent(o.re), exponent(o.im)) <= ed - 48 || ed <= 48;
         }
         if (!__any_sync(FULL, look)) continue;
         if (look) {
