@@ -48,7 +48,9 @@ int lbm_batch_set_init(lbm_batch* b, const double* rho, const double* u,
 
 /* Advances every tube by nsteps >= 0 steps in one CUDA-graph launch (captured
  * per distinct nsteps), in one of two forms with the same results, bit for bit:
- *  resident  (two steps or more, every tube of at most 3600 nodes): a block
+ *  resident  (every tube of at most 3600 nodes, and enough steps: 2 up to 1024
+ *            nodes, 3 up to 2048, beyond that 4 or 8 and enough nodes in all to
+ *            outlast the longest tube): a block
  *            keeps a tube in shared memory for all nsteps;
  *  streamed  (else, and after lbm_batch_set_tiling): each block of one
  *            persistent launch processes its share of the tiles, then all
@@ -91,8 +93,12 @@ int lbm_batch_get_tiling(lbm_batch* b, int* tile, int* threads, int* blocks);
  * tube lengths. lbm_batch_step chooses the form by itself again. Synchronises. */
 int lbm_batch_autotune(lbm_batch* b, int trial_steps, const char* cache_path, int* chosen);
 
+/* How lbm_batch_step(b, nsteps) runs: *resident 1 or 0 (streamed), *launches its kernel
+ * launches (resident: one per group of tubes of similar length). Either may be NULL. */
+int lbm_batch_plan(lbm_batch* b, long long nsteps, int* resident, int* launches);
+
 /* Test hook for the bounded barrier: block `block` skips its arrival at the
- * barrier after step `step` of the next launch (-1 disables). Used to check
+ * barrier after step `step` of the next launch, which is a streamed one (-1 disables). Used to check
  * that an expired wait is reported as LBM_ERR_TIMEOUT without hanging. */
 int lbm_batch_debug_skip_arrival(lbm_batch* b, int block, long long step);
 

@@ -357,9 +357,8 @@ __global__ void __launch_bounds__(BT) k_tubes(float* f0, float* f1, const BatchA
 // Bound by instruction issue (757 per warp and step for 64 nodes, 56 % of the
 // slots at 16 warps per SM) where the streamed form is bound by HBM (128 bytes
 // per node and step). Measured: 4096 tubes of 128-2048 nodes (4.4 M) 61 us a
-// step (streamed 115), 61 such tubes 4.0 us (streamed 7.3). A single step
-// costs 190 us against 130, for the load and the store do not overlap within a
-// block; two steps 238 against 244: lbm_batch_step takes this form from two on.
+// step (streamed 115), 61 such tubes 4.0 us (streamed 7.3). takes_resident has
+// the calls that take this form.
 template <int BT>
 __global__ void __launch_bounds__(BT, 512 / BT) k_tubes_resident(float* f0, float* f1, const BatchArgs A,
                                                                const int* __restrict__ order,
@@ -572,8 +571,6 @@ static_assert(16 * sizeof(float) * resident_width(RESIDENT_MAX_NX) <= 226 * 1024
 // RESIDENT_STEP nodes (16 KB), since a launch's blocks all take the shared
 // memory of its longest tube.
 constexpr int RESIDENT_STEP = 256;
-// Fewer steps than this go through the streamed form (figures: k_tubes_resident).
-constexpr int RESIDENT_MIN_STEPS = 2;
 // Tubes per launch group: `count` tubes order[first ..], the longest nx_max.
 struct TubeGroup {
   int first, count, nx_max, threads;
@@ -734,6 +731,26 @@ int build_groups(lbm_batch* b) {
   }
   BCK(b, cudaStreamSynchronize(b->stream));
   return LBM_OK;
+}
+
+// Whether a call of nsteps steps takes the resident form. A call's load and store do not
+// overlap the steps, so it takes a few of them; and a step takes at least as long as the
+// longest tube's block, 4.2 us up to 2048 nodes, 6 to 8 us beyond, where the streamed form
+// takes 6 us and 20 us per million nodes. Measured, streamed / resident:
+//   steps            2          3          4          8          64
+//   1024 nodes x 153 1.19       1.28       1.41       1.60       1.96
+//   2048 x 1, 153    0.94 0.93  0.99 1.01  1.2  1.05  1.3  1.17  1.5  1.3
+//   2500 x 1, 61     0.79 0.96  0.81 1.03  0.83 1.07  0.87 1.16  0.92 1.27
+//   3600 x 8, 61     0.73 1.1   0.75 1.18  0.75 1.24  0.77 1.35  0.81 1.51
+//   3600 x 153, 304  0.77 1.22  0.81 1.37  0.84 1.44  0.88 1.61  0.94 1.81
+bool takes_resident(const lbm_batch* b, long long nsteps) {
+  if (b->streamed || b->groups.empty()) return false;
+  const int longest = b->groups.front().nx_max;
+  if (longest <= 1024) return nsteps >= 2;
+  if (longest <= 2048) return nsteps >= 3;
+  long long nodes = 0;
+  for (int nx : b->nx) nodes += nx;
+  return b->ntubes <= b->sms ? nsteps >= 4 && nodes >= 1000ll * b->sms : nsteps >= 8 && nodes >= 4096ll * b->sms;
 }
 
 // The resident launches of nsteps steps: one per group, on branches of the
@@ -909,7 +926,7 @@ int lbm_batch_step(lbm_batch* b, long long nsteps) {
   snprintf(range, sizeof(range), "lbm_batch_step n=%lld (graph)", nsteps);
   nvtxRangePushA(range);
   struct Pop { ~Pop() { nvtxRangePop(); } } pop;
-  const bool resident = !b->streamed && !b->groups.empty() && nsteps >= RESIDENT_MIN_STEPS;
+  const bool resident = takes_resident(b, nsteps);
   auto key = std::make_pair(nsteps, resident ? -1 : b->variant);
   auto it = b->graphs.find(key);
   if (it == b->graphs.end()) {
@@ -1127,6 +1144,14 @@ int lbm_batch_debug_skip_arrival(lbm_batch* b, int block, long long step) {
   if (block >= b->blocks) return bfail(b, LBM_ERR_INVALID, "block out of range");
   b->skip_block = block;
   b->skip_step = step;
+  return LBM_OK;
+}
+
+int lbm_batch_plan(lbm_batch* b, long long nsteps, int* resident, int* launches) {
+  if (!b || nsteps < 1) return bfail(b, LBM_ERR_INVALID, "bad argument");
+  const bool r = takes_resident(b, nsteps);
+  if (resident) *resident = r;
+  if (launches) *launches = r ? (int)b->groups.size() : 1;
   return LBM_OK;
 }
 

@@ -281,6 +281,7 @@ _BATCH_SIGS = {
                                             ctypes.POINTER(ctypes.c_int)]),
     "lbm_batch_autotune": (ctypes.c_int, [_vp, ctypes.c_int, ctypes.c_char_p, ctypes.POINTER(ctypes.c_int)]),
     "lbm_batch_debug_skip_arrival": (ctypes.c_int, [_vp, ctypes.c_int, _ll]),
+    "lbm_batch_plan": (ctypes.c_int, [_vp, _ll, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)]),
     "lbm_batch_step_count": (_ll, [_vp]),
     "lbm_batch_total_nodes": (ctypes.c_int, [_vp, ctypes.POINTER(_ll)]),
     "lbm_batch_destroy": (ctypes.c_int, [_vp]),
@@ -446,6 +447,13 @@ def lbm_batch_autotune(b, trial_steps=20, cache_path=None):
 
 def lbm_batch_debug_skip_arrival(b, block, step):
     _bcheck(load().lbm_batch_debug_skip_arrival(b, int(block), int(step)), b)
+
+
+def lbm_batch_plan(b, nsteps):
+    """(resident, launches) of lbm_batch_step(b, nsteps)."""
+    r, n = ctypes.c_int(), ctypes.c_int()
+    _bcheck(load().lbm_batch_plan(b, int(nsteps), ctypes.byref(r), ctypes.byref(n)), b)
+    return bool(r.value), n.value
 
 
 def lbm_batch_step_count(b):
