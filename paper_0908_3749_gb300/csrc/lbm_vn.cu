@@ -440,9 +440,59 @@ __device__ bool eig16(EigWork& W, int l0, bool active) {
 // Input modes of k_vn_eig.
 enum { SRC_VN = 0, SRC_MATRIX = 1 };
 
+// The phases (sin, cos of k_x dx and of k_y dy) of a wave vector.
+struct Phases {
+  double sx, cx, sy, cy;
+};
+__device__ __forceinline__ Phases phases(const double* k, double dx, double dy) {
+  Phases p;
+  sincos(k[0] * dx, &p.sx, &p.cx);
+  sincos(k[1] * dy, &p.sy, &p.cy);
+  return p;
+}
+// Entry r of the Lax-Wendroff symbol: a0 + aE e^{i tx} + aW e^{-i tx} + aN e^{i ty} +
+// aS e^{-i ty}
+__device__ __forceinline__ cplx symbol(const LW& lw, int r, const Phases& p) {
+  return mk(lw.a0[r] + (lw.aE[r] + lw.aW[r]) * p.cx + (lw.aN[r] + lw.aS[r]) * p.cy,
+            (lw.aE[r] - lw.aW[r]) * p.sx + (lw.aN[r] - lw.aS[r]) * p.sy);
+}
+
+// G of every (case, wave vector): the case's Jacobian and the symbol on the diagonal.
+// Bound by the writes (4 KB a matrix, 8-byte stores since G may be aligned to doubles
+// only). A block writes GM matrices, whose phases and diagonals are computed in full
+// warps first: an FP64 instruction costs a warp the same whatever its active threads.
+// 32 x 1024 matrices with the call's allocations: 264 us; 408 us when k_vn_eig wrote them
+// in blocks of a warp, 300 in blocks of four.
+constexpr int GM = 8, GM_T = 256;
+__global__ void __launch_bounds__(GM_T) k_vn_matrices(long long nitems, int nk, const double* __restrict__ Jc,
+                                                      const double* __restrict__ kvec, LW lw, double dx,
+                                                      double dy, double* __restrict__ G) {
+  __shared__ Phases ph[GM];
+  __shared__ cplx diag[GM][16];
+  const long long item0 = (long long)blockIdx.x * GM;
+  const int n = (int)min((long long)GM, nitems - item0), t = threadIdx.x;
+  if (t < n) ph[t] = phases(kvec + 2 * ((item0 + t) % nk), dx, dy);
+  __syncthreads();
+  if (t < 16 * n) {
+    const int m = t >> 4, r = t & 15;
+    diag[m][r] = mk(Jc[(item0 + m) / nk * 256 + 17 * r], 0.0) + symbol(lw, r, ph[m]);
+  }
+  __syncthreads();
+  for (int m = 0; m < n; ++m) {
+    const double* J = Jc + (item0 + m) / nk * 256;
+    double* g = G + (item0 + m) * 512;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = (t + h * GM_T) >> 1, r = i >> 4;  // entry i, its real (t even) or imaginary part
+      const bool on = (i & 15) == r;
+      g[t + h * GM_T] = t & 1 ? (on ? diag[m][r].im : 0.0) : (on ? diag[m][r].re : J[i]);
+    }
+  }
+}
+
 // One matrix per L threads. SRC_VN: G of item (case, wave vector) from the
-// case's collision Jacobian and the Lax-Wendroff symbol; writes G if Gout,
-// else solves. SRC_MATRIX: the item's input matrix.
+// case's collision Jacobian and the Lax-Wendroff symbol. SRC_MATRIX: the item's input
+// matrix.
 //
 // Bound by the FP64 units. With 8 matrices per warp (L = 4) the scalar part of
 // each rotation and shift serves 8 matrices and few threads idle: 3.2 M matrices/s
@@ -456,7 +506,7 @@ __global__ void __launch_bounds__(32) k_vn_eig(int src, long long nitems, int nk
                                                const double* __restrict__ Jc,
                                                const double* __restrict__ kvec, LW lw, double dx,
                                                double dy, const double* __restrict__ Ain,
-                                               double* Gout, double* omega, double* radius,
+                                               double* omega, double* radius,
                                                unsigned long long* failed) {
   constexpr int M = 32 / L;  // matrices per warp
   __shared__ EigWork work[M];
@@ -470,33 +520,16 @@ __global__ void __launch_bounds__(32) k_vn_eig(int src, long long nitems, int nk
     const long long c = item / nk;
     const int q = (int)(item - c * nk);
     const double* J = Jc + c * 256;
-    double sx, cx, sy, cy;
-    sincos(kvec[2 * q] * dx, &sx, &cx);
-    sincos(kvec[2 * q + 1] * dy, &sy, &cy);
+    const Phases p = phases(kvec + 2 * q, dx, dy);
     for (int i = l0; i < 256; i += L) {
       cplx a = mk(J[i], 0.0);
       const int r = i >> 4;
-      if ((i & 15) == r) {
-        // a0 + aE e^{i tx} + aW e^{-i tx} + aN e^{i ty} + aS e^{-i ty}
-        const cplx diag = mk(lw.a0[r] + (lw.aE[r] + lw.aW[r]) * cx + (lw.aN[r] + lw.aS[r]) * cy,
-                             (lw.aE[r] - lw.aW[r]) * sx + (lw.aN[r] - lw.aS[r]) * sy);
-        a = a + diag;
-      }
+      if ((i & 15) == r) a = a + symbol(lw, r, p);
       W.A[r][i & 15] = a;
     }
   } else {
     const double* a = Ain + item * 512;
     for (int i = l0; i < 256; i += L) W.A[i >> 4][i & 15] = mk(a[2 * i], a[2 * i + 1]);
-  }
-  if (Gout) {
-    __syncwarp();
-    if (!have) return;
-    double* g = Gout + item * 512;
-    for (int i = l0; i < 256; i += L) {
-      g[2 * i] = W.A[i >> 4][i & 15].re;
-      g[2 * i + 1] = W.A[i >> 4][i & 15].im;
-    }
-    return;
   }
   const bool ok = eig16<L>(W, l0, have);
   double r = ok ? 0.0 : nan("");
@@ -593,7 +626,7 @@ int copy_out(void* host, const void* dev, size_t n, int on_device, cudaStream_t 
 // 1.36 / 1.61 / 2.10 ms, 1600 1.70 / 1.59 / 2.10, 2400 2.26 / 1.82 / 2.34, 4800 3.92 /
 // 2.76 / 2.44, 32768 23.9 / 15.7 / 11.5.
 int launch_eig(int src, long long nitems, int nk, const double* Jc, const double* kvec, const LW& lw,
-               double dx, double dy, const double* Ain, double* G, double* omega, double* radius,
+               double dx, double dy, const double* Ain, double* omega, double* radius,
                unsigned long long* failed, cudaStream_t s) {
   int dev = 0, sms = 0;
   VCK(cudaGetDevice(&dev));
@@ -601,11 +634,11 @@ int launch_eig(int src, long long nitems, int nk, const double* Jc, const double
   const long long warps = 4ll * sms;
   auto grid = [&](int m) { return (unsigned)((nitems + m - 1) / m); };
   if (nitems <= 2 * warps)
-    k_vn_eig<16><<<grid(2), 32, 0, s>>>(src, nitems, nk, Jc, kvec, lw, dx, dy, Ain, G, omega, radius, failed);
+    k_vn_eig<16><<<grid(2), 32, 0, s>>>(src, nitems, nk, Jc, kvec, lw, dx, dy, Ain, omega, radius, failed);
   else if (nitems <= 4 * warps)
-    k_vn_eig<8><<<grid(4), 32, 0, s>>>(src, nitems, nk, Jc, kvec, lw, dx, dy, Ain, G, omega, radius, failed);
+    k_vn_eig<8><<<grid(4), 32, 0, s>>>(src, nitems, nk, Jc, kvec, lw, dx, dy, Ain, omega, radius, failed);
   else
-    k_vn_eig<4><<<grid(8), 32, 0, s>>>(src, nitems, nk, Jc, kvec, lw, dx, dy, Ain, G, omega, radius, failed);
+    k_vn_eig<4><<<grid(8), 32, 0, s>>>(src, nitems, nk, Jc, kvec, lw, dx, dy, Ain, omega, radius, failed);
   VCK(cudaGetLastError());
   return LBM_OK;
 }
@@ -659,9 +692,14 @@ int vn_run(const lbm_vn_case* cases, int ncases, const double* k, int nk, double
   }
   k_vn_jacobian<<<ncases, 16, 0, s>>>((const lbm_vn_case*)dcases, K, dt, (double*)bj.p);
   VCK(cudaGetLastError());
-  if ((rc = launch_eig(SRC_VN, nitems, nk, (const double*)bj.p, (const double*)dk, lw, dx, dy, nullptr,
-                       (double*)dG, (double*)dw, (double*)dr, dfail, s)) != LBM_OK)
+  if (G) {
+    k_vn_matrices<<<(unsigned)((nitems + GM - 1) / GM), GM_T, 0, s>>>(nitems, nk, (const double*)bj.p, (const double*)dk,
+                                                                    lw, dx, dy, (double*)dG);
+    VCK(cudaGetLastError());
+  } else if ((rc = launch_eig(SRC_VN, nitems, nk, (const double*)bj.p, (const double*)dk, lw, dx, dy, nullptr,
+                              (double*)dw, (double*)dr, dfail, s)) != LBM_OK) {
     return rc;
+  }
   if ((rc = copy_out(G, dG, sizeof(double) * 512 * (size_t)nitems, on_device, s)) ||
       (rc = copy_out(radius, dr, sizeof(double) * (size_t)nitems, on_device, s)) ||
       (rc = copy_out(omega, dw, sizeof(double) * 32 * (size_t)nitems, on_device, s)))
@@ -715,7 +753,7 @@ int lbm_eig16(const double* A, long long n, double* omega, double* radius, int o
     VCK(cudaMemsetAsync(dfail, 0, sizeof(unsigned long long), s));
   }
   LW lw = {};
-  if ((rc = launch_eig(SRC_MATRIX, n, 1, nullptr, nullptr, lw, 1.0, 1.0, (const double*)dA, nullptr,
+  if ((rc = launch_eig(SRC_MATRIX, n, 1, nullptr, nullptr, lw, 1.0, 1.0, (const double*)dA,
                        (double*)dw, (double*)dr, dfail, s)) != LBM_OK)
     return rc;
   if ((rc = copy_out(omega, dw, sizeof(double) * 32 * (size_t)n, on_device, s)) ||
