@@ -622,8 +622,6 @@ struct lbm_batch {
   bool streamed = false;       // lbm_batch_set_tiling asked for the streamed form
   std::vector<TubeGroup> groups;  // resident form: launches, longest tubes first (empty: too long)
   int* order = nullptr;           // tube indices, group by group
-  std::vector<cudaStream_t> side; // capture branches of the groups after the first
-  std::vector<cudaEvent_t> joins; // [0] the fork, [k] the end of branch k
   std::map<std::pair<long long, int>, cudaGraphExec_t> graphs;  // key: steps, variant (-1: resident)
   std::string err = "no error";
 };
@@ -711,9 +709,11 @@ int launch_tubes(lbm_batch* b, long long nsteps) {
 // Groups the tubes for the resident form.
 int build_groups(lbm_batch* b) {
   if (*std::max_element(b->nx.begin(), b->nx.end()) > RESIDENT_MAX_NX) return LBM_OK;
-  std::vector<int> order(b->ntubes);
-  for (int t = 0; t < b->ntubes; ++t) order[t] = t;
-  std::stable_sort(order.begin(), order.end(), [&](int p, int q) { return b->nx[p] > b->nx[q]; });
+  // longest first: tubes counted by length
+  std::vector<int> at(RESIDENT_MAX_NX + 2, 0), order(b->ntubes);
+  for (int nx : b->nx) ++at[nx - 1];
+  for (int nx = RESIDENT_MAX_NX; nx >= 0; --nx) at[nx] += at[nx + 1];
+  for (int t = 0; t < b->ntubes; ++t) order[at[b->nx[t]]++] = t;
   const bool few = b->ntubes <= b->sms;  // a tube per SM: as many threads as it has pairs
   for (int k = 0; k < b->ntubes; ++k) {
     const int nx = b->nx[order[k]];
@@ -728,15 +728,6 @@ int build_groups(lbm_batch* b) {
                                 (int)resident_smem(RESIDENT_MAX_NX)));
   BCK(b, cudaMalloc((void**)&b->order, sizeof(int) * b->ntubes));
   BCK(b, cudaMemcpyAsync(b->order, order.data(), sizeof(int) * b->ntubes, cudaMemcpyHostToDevice, b->stream));
-  for (size_t k = 0; k < b->groups.size(); ++k) {
-    cudaEvent_t ev;
-    BCK(b, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-    b->joins.push_back(ev);
-    if (k == 0) continue;
-    cudaStream_t st;
-    BCK(b, cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
-    b->side.push_back(st);
-  }
   BCK(b, cudaStreamSynchronize(b->stream));
   return LBM_OK;
 }
@@ -761,21 +752,37 @@ bool takes_resident(const lbm_batch* b, long long nsteps) {
   return b->ntubes <= b->sms ? nsteps >= 4 && nodes >= 1000ll * b->sms : nsteps >= 8 && nodes >= 4096ll * b->sms;
 }
 
-// The resident launches of nsteps steps: one per group, on branches of the
-// batch's stream, so that blocks of different groups share the SMs.
-int launch_resident(lbm_batch* b, long long nsteps) {
-  const BatchArgs A = make_batch_args(b);
-  if (b->groups.size() > 1) BCK(b, cudaEventRecord(b->joins[0], b->stream));
-  for (size_t k = 0; k < b->groups.size(); ++k) {
-    const TubeGroup& G = b->groups[k];
-    const cudaStream_t st = k == 0 ? b->stream : b->side[k - 1];
-    if (k > 0) BCK(b, cudaStreamWaitEvent(st, b->joins[0], 0));
-    resident_fn(G.threads)<<<G.count, G.threads, resident_smem(G.nx_max), st>>>(
-        b->f[0], b->f[1], A, b->order + G.first, nsteps);
-    BCK(b, cudaGetLastError());
-    if (k > 0) BCK(b, cudaEventRecord(b->joins[k], st));
+// A graph of the resident launches of nsteps steps: one per group, none after another,
+// so that blocks of different groups share the SMs.
+int resident_graph(lbm_batch* b, long long nsteps, cudaGraph_t* out) {
+  BatchArgs A = make_batch_args(b);
+  BCK(b, cudaGraphCreate(out, 0));
+  for (const TubeGroup& G : b->groups) {
+    const int* order = b->order + G.first;
+    void* args[] = {&b->f[0], &b->f[1], &A, &order, &nsteps};
+    cudaKernelNodeParams p = {};
+    p.func = (void*)resident_fn(G.threads);
+    p.gridDim = dim3(G.count);
+    p.blockDim = dim3(G.threads);
+    p.sharedMemBytes = (unsigned)resident_smem(G.nx_max);
+    p.kernelParams = args;
+    cudaGraphNode_t node;
+    const cudaError_t e = cudaGraphAddKernelNode(&node, *out, nullptr, 0, &p);
+    if (e != cudaSuccess) {
+      cudaGraphDestroy(*out);
+      return bcuda(b, e, "cudaGraphAddKernelNode");
+    }
   }
-  for (size_t k = 1; k < b->groups.size(); ++k) BCK(b, cudaStreamWaitEvent(b->stream, b->joins[k], 0));
+  return LBM_OK;
+}
+
+// The graph of the streamed launch, captured.
+int streamed_graph(lbm_batch* b, long long nsteps, cudaGraph_t* out) {
+  BCK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
+  const int rc = launch_tubes(b, nsteps);
+  const cudaError_t e = cudaStreamEndCapture(b->stream, out);
+  if (rc != LBM_OK) return rc;
+  if (e != cudaSuccess) return bcuda(b, e, "cudaStreamEndCapture");
   return LBM_OK;
 }
 
@@ -939,13 +946,10 @@ int lbm_batch_step(lbm_batch* b, long long nsteps) {
   auto it = b->graphs.find(key);
   if (it == b->graphs.end()) {
     cudaGraph_t g;
-    BCK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-    const int rc = resident ? launch_resident(b, nsteps) : launch_tubes(b, nsteps);
-    cudaError_t e = cudaStreamEndCapture(b->stream, &g);
+    const int rc = resident ? resident_graph(b, nsteps, &g) : streamed_graph(b, nsteps, &g);
     if (rc != LBM_OK) return rc;
-    if (e != cudaSuccess) return bcuda(b, e, "cudaStreamEndCapture");
     cudaGraphExec_t ex;
-    e = cudaGraphInstantiate(&ex, g, 0);
+    cudaError_t e = cudaGraphInstantiate(&ex, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return bcuda(b, e, "cudaGraphInstantiate");
     it = b->graphs.emplace(key, ex).first;
@@ -1187,8 +1191,6 @@ int lbm_batch_destroy(lbm_batch* b) {
   if (b->tubes) cudaFree(b->tubes);
   if (b->items) cudaFree(b->items);
   if (b->order) cudaFree(b->order);
-  for (cudaStream_t st : b->side) cudaStreamDestroy(st);
-  for (cudaEvent_t ev : b->joins) cudaEventDestroy(ev);
   if (b->ghost) cudaFree(b->ghost);
   if (b->bad) cudaFree(b->bad);
   if (b->st) cudaFree(b->st);
