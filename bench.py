@@ -517,22 +517,27 @@ def e2e_steps(torch, lbm, ctx, w, K, W):
     return times, f.numel() * f.element_size(), outs.numel() * 8
 
 
-def tubes_measure(torch, lbm, stream, args, hbm_peak):
-    """4096 seeded quasi-1D Riemann problems (Nx ~ U[128, 2048]) in one
-    persistent launch per call: the autotuned tiling, then timed calls of
-    ``--tube-steps`` steps each (inputs larger than L2). The watchdog's
-    per-tube status after the timed calls splits the tubes into stable and
-    unstable ones; a second batch then runs the configuration's whole 10 000
-    steps (t = 0.1) and is counted the same way."""
+# Floating-point operations per node-update of the quasi-1D FP32 step (the 2D
+# count without the y terms), FMA = 2.
+FLOPS_PER_TUBE_NODE = 325
+
+
+def tubes_measure(torch, lbm, stream, args, hbm_peak, fp32_fma):
+    """4096 seeded quasi-1D Riemann problems (Nx ~ U[128, 2048]), timed calls of
+    ``--tube-steps`` steps each (inputs larger than L2) in the form that the
+    library takes for them (each tube in shared memory for all the steps of a
+    call, so that the populations cross HBM once per call: bound by instruction
+    issue) and, as ``streamed``, with every step's populations through HBM, with
+    the autotuned tiling. The watchdog's per-tube status after the timed calls
+    splits the tubes into stable and unstable ones; a second batch then runs the
+    configuration's whole 10 000 steps (t = 0.1) and is counted the same way."""
     import workloads
     B = workloads.tube_batch()
     nt = len(B["nx"])
     nx = np.asarray(B["nx"])
-    b = lbm.lbm_batch_create(B["nx"], B["dx"], B["dt"], B["s"], B["left"], B["right"], stream)
-    try:
-        lbm.lbm_batch_set_init(b, *workloads.tube_fields(B))
-        chosen = lbm.lbm_batch_autotune(b, 20, None)
-        n = args.tube_steps
+    n = args.tube_steps
+
+    def call_ms(b):
         lbm.lbm_batch_step(b, n)               # capture + warm-up
         torch.cuda.synchronize()
         ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
@@ -544,27 +549,46 @@ def tubes_measure(torch, lbm, stream, args, hbm_peak):
                 ev[1].record(stream)
                 stream.synchronize()
                 times.append(ev[0].elapsed_time(ev[1]))
+        return min(times)
+
+    b = lbm.lbm_batch_create(B["nx"], B["dx"], B["dt"], B["s"], B["left"], B["right"], stream)
+    try:
+        lbm.lbm_batch_set_init(b, *workloads.tube_fields(B))
+        resident, launches = lbm.lbm_batch_plan(b, n)
+        call = call_ms(b)
         steps_run = lbm.lbm_batch_step_count(b)
         rc, bad, nbad, to = lbm.lbm_batch_status(b, nt)
         total = lbm.lbm_batch_total_nodes(b)
+        chosen = lbm.lbm_batch_autotune(b, 20, None)
+        lbm.lbm_batch_set_tiling(b, *chosen)
+        streamed = call_ms(b)
     finally:
         lbm.lbm_batch_destroy(b)
-    ms = min(times) / n
+    ms = call / n
     stable_nodes = int(nx[bad < 0].sum())
-    out = {"workload": "4096_tubes_nx_128_2048", "nodes": total, "steps_per_launch": n,
+    per_call = BYTES_PER_CELL["fp32"] * total * (1 if resident else n)
+
+    def gbs(nbytes, t):
+        return nbytes / (t * 1e-3) / 1e9
+    out = {"workload": "4096_tubes_nx_128_2048", "nodes": total, "steps_per_call": n,
            "value": total / (ms * 1e-3), "unit": UNIT, "ms_per_step": ms,
-           "achieved_gbs": BYTES_PER_CELL["fp32"] * total / (ms * 1e-3) / 1e9,
-           "frac_of_hbm": BYTES_PER_CELL["fp32"] * total / (ms * 1e-3) / 1e9 / hbm_peak,
-           "tiling": list(chosen), "timeout": to, "graph": True, "launches_per_call": 1,
+           "form": "resident" if resident else "streamed", "launches_per_call": launches,
+           "hbm_bytes_per_call": per_call, "achieved_gbs": gbs(per_call, call),
+           "frac_of_hbm": gbs(per_call, call) / hbm_peak,
+           "frac_of_fp32": FLOPS_PER_TUBE_NODE * total / (ms * 1e-3) / (2 * fp32_fma),
+           "bound": "issue" if resident else "hbm",
+           "timeout": to, "graph": True,
            "steps_run": steps_run, "unstable_tubes": nbad, "stable_tubes": nt - nbad,
            "value_stable": stable_nodes / (ms * 1e-3),
            "value_stable_note": "node-updates of the tubes that stayed physical, per second of "
-                                "the whole batch's step"}
+                                "the whole batch's step",
+           "streamed": {"tiling": list(chosen), "launches_per_call": 1, "ms_per_step": streamed / n,
+                        "achieved_gbs": gbs(BYTES_PER_CELL["fp32"] * total * n, streamed),
+                        "frac_of_hbm": gbs(BYTES_PER_CELL["fp32"] * total * n, streamed) / hbm_peak}}
     # the configuration's whole run, counted
     b = lbm.lbm_batch_create(B["nx"], B["dx"], B["dt"], B["s"], B["left"], B["right"], stream)
     try:
         lbm.lbm_batch_set_init(b, *workloads.tube_fields(B))
-        lbm.lbm_batch_set_tiling(b, chosen[0], chosen[1])
         lbm.lbm_batch_step(b, B["nsteps"])
         rc, bad, nbad, to = lbm.lbm_batch_status(b, nt)
         out["full_run"] = {"steps": B["nsteps"], "unstable_tubes": nbad, "stable_tubes": nt - nbad,
@@ -727,7 +751,8 @@ def run_ours(args):
     large = None if args.no_large else large_grid_measure(torch, lbm, stream, args.audit_every, hbm_peak)
     refl = None if args.no_small else reflection_measure(torch, lbm, stream, flush, args.audit_every,
                                                          hbm_peak, max(K, 20), W)
-    tubes = None if args.no_tubes else tubes_measure(torch, lbm, stream, args, hbm_peak)
+    tubes = None if args.no_tubes else tubes_measure(torch, lbm, stream, args, hbm_peak,
+                                                      peaks["fp32_fma_per_s"])
     vn = None if args.no_vn else vn_measure(torch, lbm, stream)
     corr = None if args.no_corrector else corrector_measure(torch)
     clocks.stop()

@@ -54,9 +54,10 @@ template <int VAR> struct Shape<double, VAR> {
 // each of four unrelated blocks per scheduler, half the issue stalls were
 // instruction fetches (ncu: no_instruction 2.9 of 6.0 cycles per issue); the two
 // warps per scheduler of a 256-thread block run close behind each other and
-// share them. 2048 x 1024 301 -> 273 us a step; 32 x 16 tiles (one block per SM, the copy of its next tile only
-// from the persistent form) 299, persistent 260-292; barriers inside the update
-// to keep a block's warps together cost registers (spills) and took 282-288.
+// share them. 2048 x 1024 301 -> 273 us a step; 32 x 16 tiles (one block per SM, the
+// copy of its next tile only from the persistent form) 299, persistent 260-292;
+// barriers inside the update to keep a block's warps together cost registers
+// (spills) and took 282-288.
 // V_ROWS4: 32 x 4 tiles, for the grids that tall tiles divide badly (rows4 in lbm_core.cu).
 #ifndef LBM_DW_LANES
 #define LBM_DW_LANES 1
