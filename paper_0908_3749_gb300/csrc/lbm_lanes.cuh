@@ -9,7 +9,7 @@
 // its group; then lanes 0, 1, 2, 3 take the S, X, Y and C values of all groups (the
 // rows of the moment blocks have the same form with other coefficients), share
 // the steps of the equilibria, and each relaxes, transforms back and advects its
-// own group: 71 FP64 instructions of a warp. Every value is computed by the
+// own group: 68 FP64 instructions of a warp. Every value is computed by the
 // operations of collide64 and neighbour_terms, in some lane, so the results are
 // those of k_step bit for bit (a sum a + b as fma(1, a, b), a product a b as fma(a,
 // b, -0), which round alike).
