@@ -316,13 +316,19 @@ StepArgs<R> make_args(lbm_ctx* c, int slot) {
   return A;
 }
 
-// The step kernels of a context with 64-bit element offsets, or without (V_ROWS4 grids are
-// small).
+// The step kernels of a context. 64-bit element offsets: not V_ROWS4, whose grids are small.
+// The next step's blocks start at once beside an FP32 step of three tiles per SM on (as all
+// grids with 64-bit offsets have), which fill the SMs evenly all the same, else at its stores.
+// us a step, at the stores / at once: tiles 377 (400 x 225) 5.70/6.07, 475 (600 x 200)
+// 6.19/6.12, 528 (500 x 260) 6.26/6.18, 1653 (900 x 450) 11.8/11.6, 2850 (1200 x 600) 21.4/20.9;
+// LBM_FP32_DWMOM 528 8.49/8.10. (FP64, 1000 tiles: 44.7/51.3.) Two kernels: one with both places
+// and a condition takes 2 % more.
 template <typename R, int VAR>
-auto step_kernel(bool wide) {
+auto step_kernel(bool wide, bool early) {
+  constexpr bool E = sizeof(R) == 4;
   if constexpr (VAR != V_ROWS4)
-    if (wide) return k_step<R, long long, VAR>;
-  return k_step<R, unsigned, VAR>;
+    if (wide) return k_step<R, long long, VAR, E>;
+  return early ? k_step<R, unsigned, VAR, E> : k_step<R, unsigned, VAR>;
 }
 template <typename R, int VAR>
 auto pipe_kernel(bool wide) {
@@ -337,7 +343,7 @@ int launch_persistent(lbm_ctx* c, cudaStream_t s, int from, void* fout, const St
   const R* fi = (const R*)c->f[from];
   const CUtensorMap& tm = c->tmap[from];
   if (A.nblocks >= A.ntiles) {
-    CK(c, launch(A.overlapped, step_kernel<R, VAR>(c->wide), A.ntiles, blk,
+    CK(c, launch(A.overlapped, step_kernel<R, VAR>(c->wide, A.ntiles >= 3 * c->sms), A.ntiles, blk,
                  tile_dynamic_bytes<R, VAR>(), s, tm, fi, (R*)fout, A));
   } else {
     CK(c, launch(A.overlapped, pipe_kernel<R, VAR>(c->wide), A.nblocks, blk,
@@ -426,8 +432,8 @@ cudaError_t allow_pipe_smem() {
   for (bool wide : {false, true}) {
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(pipe_kernel<R, VAR>(wide), cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    if (e == cudaSuccess && t > 0)
-      e = cudaFuncSetAttribute(step_kernel<R, VAR>(wide), cudaFuncAttributeMaxDynamicSharedMemorySize, t);
+    if (e == cudaSuccess && t > 0)  // (double-word: no early form)
+      e = cudaFuncSetAttribute(step_kernel<R, VAR>(wide, false), cudaFuncAttributeMaxDynamicSharedMemorySize, t);
   }
   return e;
 }

@@ -228,7 +228,9 @@ __host__ __device__ constexpr size_t tile_dynamic_bytes() {
   return Tile<R, VAR>::BYTES <= 46 * 1024 ? 0 : (size_t)Tile<R, VAR>::BYTES + 128;
 }
 
-template <typename R, typename Off, int VAR = 0>
+// EARLY: the next step's blocks may start at once, beside this one's (FP32 grids of three
+// tiles per SM on, launch_persistent in lbm_core.cu); else at the stores.
+template <typename R, typename Off, int VAR = 0, bool EARLY = false>
 __global__ void __launch_bounds__(Shape<R, VAR>::X * Shape<R, VAR>::TY, (step_minb<R, Off, VAR>()))
     k_step(const __grid_constant__ CUtensorMap tmap, const R* fin,
            R* fout, const StepArgs<R> A) {
@@ -245,6 +247,7 @@ __global__ void __launch_bounds__(Shape<R, VAR>::X * Shape<R, VAR>::TY, (step_mi
   __shared__ unsigned long long s_step;
   __shared__ int s_audit, s_alist[32], s_an;
   const int t = threadIdx.y * Shape<R, VAR>::X + threadIdx.x;
+  if (EARLY) dependents_may_start();
   if (t == 0) mbar_init(&bar, 1);
   if (VAR != V_ROWS4 || A.overlapped) wait_for_previous();
   if (t == 0) {
@@ -268,7 +271,7 @@ __global__ void __launch_bounds__(Shape<R, VAR>::X * Shape<R, VAR>::TY, (step_mi
   }
   bool bad = false, negT = false;
   step_any<R, Off, VAR>(A, fin, fout, tile, blockIdx.x, audit, A.dtr * R(s_step), sm, bad, negT);
-  if (!audit && (VAR != V_ROWS4 || A.overlapped)) dependents_may_start();
+  if (!EARLY && !audit && (VAR != V_ROWS4 || A.overlapped)) dependents_may_start();
   const unsigned long long step = s_step;
   watchdog_flags(A.st, step, bad, negT);
   if (audit) audit_block_done(A, (int)blockIdx.x, A.ntiles, step, s_alist, &s_an);
@@ -295,6 +298,7 @@ __global__ void __launch_bounds__(Shape<R, VAR>::X * Shape<R, VAR>::TY, Shape<R,
   __shared__ int s_audit, s_alist[32], s_an;
   const int t = threadIdx.y * Shape<R, VAR>::X + threadIdx.x;
   const int G = (int)gridDim.x;
+  if (sizeof(R) == 4) dependents_may_start();  // (before the last tile: 0.5 % slower)
   if (t == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
@@ -325,11 +329,11 @@ __global__ void __launch_bounds__(Shape<R, VAR>::X * Shape<R, VAR>::TY, Shape<R,
       }
       return;
     }
+    if (sizeof(R) != 4 && !more && !s_audit && (VAR != V_ROWS4 || A.overlapped)) dependents_may_start();
     step_any<R, Off, VAR>(A, fin, fout, stages + s * Tile<R, VAR>::ELEMS, cur, s_audit != 0,
                      A.dtr * R(s_step), sm, bad, negT);
     __syncthreads();  // stage s and sm are free again
   }
-  if (!s_audit && (VAR != V_ROWS4 || A.overlapped)) dependents_may_start();
   watchdog_flags(A.st, s_step, bad, negT);
   if (s_audit) audit_block_done(A, (int)blockIdx.x, G, s_step, s_alist, &s_an);
 }

@@ -84,7 +84,8 @@ __device__ __forceinline__ void fence_proxy_async() {
 // move reads (and, for __restrict__, writes) above the wait.
 //
 // The step kernels call dependents_may_start() when a block has only its stores
-// left. Called at their top, the next step's blocks take whatever slots are free
+// left (FP64 and double-word persistent ones before their last tile, FP32 ones of
+// many tiles at once). Called at their top, the next step's blocks take whatever slots are free
 // then, so that some SMs get several of them and others none: a grid of two blocks
 // or so per SM takes the time of the fullest. Measured, us a step, plain launches /
 // early / late:
