@@ -67,7 +67,8 @@ struct Results {
 // Waits of the convolution and weight-gradient kernels: bounded; when one expires,
 // the block sets Results::timeout, waits once more for the copies and products that
 // it has in flight, frees its tensor memory and leaves. k_update then leaves
-// the parameters alone. give_up (test hook): the waits that expire at once.
+// the parameters alone. give_up (test hook): the waits that expire at once, in instances
+// of the kernels of their own (HOOK): a look at it beside every wait takes 2 %.
 enum GiveUp { GIVE_UP_COPIES = 1, GIVE_UP_PRODUCTS = 2 };
 __device__ __forceinline__ bool wait_for(unsigned long long* bar, unsigned parity, bool give_up) {
   return !give_up && gbtma::mbar_wait_bounded(bar, parity, gbtma::TMA_WAIT_CYCLES);
@@ -140,7 +141,7 @@ __host__ __device__ constexpr unsigned cv_smem(int cout) {
   return CV_SLOTS * CV_STAGE + CV_KG * cv_n(cout) * 16 + 128;
 }
 
-template <int COUT, int EPI>
+template <int COUT, int EPI, bool HOOK>
 __global__ void __launch_bounds__(CV_T, CV_CTAS_PER_SM)
     k_conv(const __grid_constant__ CUtensorMap map, int H, int W, int tiles_x, int ntiles,
            const __nv_bfloat16* Wt, const float* bias,
@@ -189,7 +190,8 @@ __global__ void __launch_bounds__(CV_T, CV_CTAS_PER_SM)
   tc05::fence_after();
   const unsigned tmem = s_tmem, a0 = gbtma::smem_addr(base), b0 = gbtma::smem_addr(sw);
 
-  const bool no_copy = give_up & GIVE_UP_COPIES, no_product = give_up != 0;  // no products without copies
+  // (no products without copies)
+  const bool no_copy = HOOK && (give_up & GIVE_UP_COPIES), no_product = HOOK && give_up != 0;
   bool ok = true;  // every wait of this thread has ended in time
   int issued = 0;  // by this thread: tiles copied, tiles multiplied
   if (t == CV_EPI_T) {  // copies beyond the first CV_SLOTS: once the slot's products have read it
@@ -322,6 +324,7 @@ constexpr int C4_PITCH = C4_KP + 8;
 constexpr unsigned C4_ROW = CT_HX * PX_BYTES, C4_TILE = CT_HY * C4_ROW, C4_STAGE = (C4_TILE + 127) / 128 * 128;
 constexpr unsigned C4_SMEM = C4_STAGE + 32 * C4_PITCH * 2 + 128;
 
+template <bool HOOK>
 __global__ void __launch_bounds__(CT_T, C4_CTAS_PER_SM)
     k_conv4(const __grid_constant__ CUtensorMap map, int H, int W, int tiles_x, int ntiles,
             const __nv_bfloat16* Wt, const unsigned* bits_in,
@@ -360,7 +363,7 @@ __global__ void __launch_bounds__(CT_T, C4_CTAS_PER_SM)
         const int y = y0 + (m >> 1), x = x0 + (m & 1) * 16 + h * 8 + g;
         keep[m][h] = y < H && x < W ? bits_in[(long long)y * W + x] << (4 * tig) : 0u;
       }
-    if (!__syncthreads_and(wait_for(&bar, k & 1, give_up & GIVE_UP_COPIES))) {
+    if (!__syncthreads_and(wait_for(&bar, k & 1, HOOK && (give_up & GIVE_UP_COPIES)))) {
       // The copy did not land in time: record it, wait once more (bounded), leave.
       if (threadIdx.x == 0) {
         atomicExch(timeout, 1);
@@ -495,7 +498,7 @@ __device__ __forceinline__ void split3(float x, unsigned (&p)[3]) {
 
 // CG: channel groups of A (4: a 32-channel layer, 2: the split features); COUT
 // output channels.
-template <int CG, int COUT>
+template <int CG, int COUT, bool HOOK>
 __global__ void __launch_bounds__(WG_T, WG_CTAS_PER_SM)
     k_wgrad(const __grid_constant__ CUtensorMap act, const __grid_constant__ CUtensorMap dz,
             int tiles_x, int ntiles, float* partial, int* timeout, int give_up) {
@@ -535,7 +538,7 @@ __global__ void __launch_bounds__(WG_T, WG_CTAS_PER_SM)
   const unsigned tmem = s_tmem;
 
   float db[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // bias sums: pixel column `lane`, group `warp`
-  const bool no_copy = give_up & GIVE_UP_COPIES, no_product = give_up & GIVE_UP_PRODUCTS;
+  const bool no_copy = HOOK && (give_up & GIVE_UP_COPIES), no_product = HOOK && (give_up & GIVE_UP_PRODUCTS);
   bool ok = true;
   int k = 0, loaded = 1, multiplied = 0;  // tiles copied and multiplied (thread 0)
   for (int tile = blockIdx.x; tile < ntiles; tile += G, ++k) {
@@ -957,11 +960,8 @@ __global__ void __launch_bounds__(UP_N * UP_S) k_update(const UpdateArgs A) {
   gbtma::wait_for_previous();
   const int t = threadIdx.x;
   // A wait of a kernel before expired: its partials are not this step's. Nothing
-  // is updated; the host learns of it from the flag.
-  if (*(volatile int*)&A.res->timeout) {
-    if (blockIdx.x == 0 && t == 0 && A.adam) ++A.res->skipped;
-    return;
-  }
+  // is updated; the host learns of it from the flag (which arrives beside the partials).
+  const int expired = *(volatile int*)&A.res->timeout;
   if (blockIdx.x == gridDim.x - 1) {
     __shared__ double sl[UP_N * UP_S];
     double s = 0.0;
@@ -972,7 +972,8 @@ __global__ void __launch_bounds__(UP_N * UP_S) k_update(const UpdateArgs A) {
       if (t < st) sl[t] += sl[t + st];
       __syncthreads();
     }
-    if (t == 0) A.res->loss = sl[0] * A.lscale;
+    if (t == 0 && !expired) A.res->loss = sl[0] * A.lscale;
+    if (t == 0 && expired && A.adam) ++A.res->skipped;
     return;
   }
   __shared__ float sm[UP_S][UP_N];
@@ -990,7 +991,7 @@ __global__ void __launch_bounds__(UP_N * UP_S) k_update(const UpdateArgs A) {
   }
   sm[slice][t % UP_N] = s;
   __syncthreads();
-  if (slice > 0 || i >= LBM_CNN_NPARAMS) return;
+  if (slice > 0 || i >= LBM_CNN_NPARAMS || expired) return;
 #pragma unroll
   for (int k = 1; k < UP_S; ++k) s += sm[k][t];
   A.grad[i] = s;
@@ -1296,7 +1297,7 @@ template <int COUT, int EPI>
 int conv(lbm_cnn* n, const CUtensorMap& in, const __nv_bfloat16* wt, const float* bias,
          const unsigned* bits_in, __nv_bfloat16* ob, float* of, unsigned* bits_out = nullptr) {
   const int grid = std::min(n->cntiles, CV_CTAS_PER_SM * n->sms);
-  CCK(n, gbtma::launch_overlapped(k_conv<COUT, EPI>, grid, CV_T, cv_smem(COUT), n->stream, in, n->H, n->W,
+  CCK(n, gbtma::launch_overlapped(n->give_up ? k_conv<COUT, EPI, true> : k_conv<COUT, EPI, false>, grid, CV_T, cv_smem(COUT), n->stream, in, n->H, n->W,
                                   n->ctiles_x, n->cntiles, wt, bias, bits_in, ob, of, bits_out,
                                   &n->res->timeout, n->give_up));
   return LBM_OK;
@@ -1320,7 +1321,7 @@ int forward(lbm_cnn* n, const double* coarse, bool train) {
 
 template <int CG, int COUT>
 int wgrad(lbm_cnn* n, const CUtensorMap& act, const CUtensorMap& dz, float* partial) {
-  CCK(n, gbtma::launch_overlapped(k_wgrad<CG, COUT>, n->wblocks, WG_T, WgShape<CG, COUT == 32 ? 32 : 16>::SMEM,
+  CCK(n, gbtma::launch_overlapped(n->give_up ? k_wgrad<CG, COUT, true> : k_wgrad<CG, COUT, false>, n->wblocks, WG_T, WgShape<CG, COUT == 32 ? 32 : 16>::SMEM,
                                   n->stream, act, dz, n->tiles_x, n->ntiles, partial, &n->res->timeout, n->give_up));
   return LBM_OK;
 }
@@ -1342,7 +1343,7 @@ int loss_backward(lbm_cnn* n, const double* target, bool adam) {
   auto part = [&](int l) { return const_cast<float*>(U.part[l]); };
   // layer 5 (32 -> 4): dz5 holds d loss / d z5
   if ((rc = wgrad<4, 4>(n, n->m_act[4], n->g_dz5, part(4))) != LBM_OK) return rc;
-  CCK(n, gbtma::launch_overlapped(k_conv4, std::min(n->ntiles, C4_CTAS_PER_SM * n->sms), CT_T, C4_SMEM, n->stream,
+  CCK(n, gbtma::launch_overlapped(n->give_up ? k_conv4<true> : k_conv4<false>, std::min(n->ntiles, C4_CTAS_PER_SM * n->sms), CT_T, C4_SMEM, n->stream,
                                   n->m_dz5, n->H, n->W, n->tiles_x, n->ntiles, n->wb[4], n->pos[4], n->dz[1],
                                   &n->res->timeout, n->give_up));
   if ((rc = wgrad<4, 32>(n, n->m_act[3], n->g_dz[1], part(3))) != LBM_OK) return rc;
@@ -1398,13 +1399,20 @@ int lbm_cnn_create(int H, int W, void* cuda_stream, lbm_cnn** out) {
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   };
-  allow((const void*)k_wgrad<4, 32>, WgShape<4, 32>::SMEM);
-  allow((const void*)k_wgrad<4, 4>, WgShape<4, 16>::SMEM);
-  allow((const void*)k_wgrad<2, 32>, WgShape<2, 32>::SMEM);
-  allow((const void*)k_conv<32, EPI_RELU_BF16>, cv_smem(32));
-  allow((const void*)k_conv<32, EPI_MASK_BF16>, cv_smem(32));
-  allow((const void*)k_conv<4, EPI_LINEAR_F32>, cv_smem(4));
-  allow((const void*)k_conv4, C4_SMEM);
+  allow((const void*)k_wgrad<4, 32, false>, WgShape<4, 32>::SMEM);
+  allow((const void*)k_wgrad<4, 32, true>, WgShape<4, 32>::SMEM);
+  allow((const void*)k_wgrad<4, 4, false>, WgShape<4, 16>::SMEM);
+  allow((const void*)k_wgrad<4, 4, true>, WgShape<4, 16>::SMEM);
+  allow((const void*)k_wgrad<2, 32, false>, WgShape<2, 32>::SMEM);
+  allow((const void*)k_wgrad<2, 32, true>, WgShape<2, 32>::SMEM);
+  allow((const void*)k_conv<32, EPI_RELU_BF16, false>, cv_smem(32));
+  allow((const void*)k_conv<32, EPI_RELU_BF16, true>, cv_smem(32));
+  allow((const void*)k_conv<32, EPI_MASK_BF16, false>, cv_smem(32));
+  allow((const void*)k_conv<32, EPI_MASK_BF16, true>, cv_smem(32));
+  allow((const void*)k_conv<4, EPI_LINEAR_F32, false>, cv_smem(4));
+  allow((const void*)k_conv<4, EPI_LINEAR_F32, true>, cv_smem(4));
+  allow((const void*)k_conv4<false>, C4_SMEM);
+  allow((const void*)k_conv4<true>, C4_SMEM);
   n->sms = std::max(sms, 1);
   n->tiles_x = (W + CT_X - 1) / CT_X;
   n->ntiles = n->tiles_x * ((H + CT_Y - 1) / CT_Y);
