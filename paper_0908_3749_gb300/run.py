@@ -87,8 +87,8 @@ def main(argv=None):
 
 
 def run_tubes(args):
-    """The seeded tube batch (``--nx`` tubes, default 4096) in one persistent
-    launch per ``lbm_batch_step`` call of ``--steps`` steps."""
+    """The seeded tube batch (``--nx`` tubes, default 4096) in one
+    ``lbm_batch_step`` call of ``--steps`` steps."""
     import workloads as W
     B = W.tube_batch(ntubes=args.nx or 4096)
     nt = len(B["nx"])
