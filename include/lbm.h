@@ -204,7 +204,8 @@ int lbm_element_size(lbm_ctx* ctx);
 
 /* Launch shape of the step (LBM_FP64 / LBM_FP32 / LBM_DF64 / LBM_FP32_DWMOM).
  * The grid is cut into node tiles (32 x 8 nodes in FP32, 32 x 2 in FP64,
- * 32 x 8 or, where these fill the multiprocessors badly, 32 x 4 in LBM_DF64). With one block per tile each
+ * 32 x 8 in LBM_DF64 or, where these fill the multiprocessors badly,
+ * 32 x 4). With one block per tile each
  * block updates its tile; with fewer blocks each block takes tiles b, b + G,
  * b + 2G, ... (G blocks), copying its next tile into shared memory while it
  * computes the current one. Results do not depend on it (each node's update
